@@ -28,7 +28,7 @@
  * appended token that names no valid slot) set bits in the device status word and never trap: a bad
  * page id is replaced by page 0 (every access stays in bounds, the affected sequence's output is
  * unspecified), a bad length is clamped, a bad token is skipped.  Read the word with
- * novakv_last_device_status.  The kernels contain no spin wait.
+ * novakv_last_device_status.  No wait in a kernel is unbounded: one that gives up (about a second) sets a bit.
  *
  * Determinism: for fixed inputs, shapes and device, outputs are bitwise reproducible.
  */
@@ -59,9 +59,9 @@ typedef enum {
 /* Bits of the device status word. */
 #define NOVAKV_DEV_BAD_PAGE      1u   /* a page id was outside [0, n_pages) */
 #define NOVAKV_DEV_BAD_LENGTH    2u   /* a sequence length exceeded 64 * max_pages_per_seq */
-#define NOVAKV_DEV_WAIT_TIMEOUT  4u   /* reserved: no kernel of this build waits on another thread or copy */
+#define NOVAKV_DEV_WAIT_TIMEOUT  4u   /* a wait of the prompt encoder inside a thread block gave up (that call's output is unspecified) */
 #define NOVAKV_DEV_BAD_TOKEN     8u   /* an appended token named a sequence slot or position out of range */
-#define NOVAKV_DEV_SMEM_LAYOUT  16u   /* the scan kernel could not place its tables in shared memory (no output was produced) */
+#define NOVAKV_DEV_SMEM_LAYOUT  16u   /* a kernel could not place its tables in shared memory (no output was produced) */
 
 typedef struct {
     int n_layers;
@@ -121,14 +121,14 @@ size_t novakv_decode_workspace_bytes(const novakv_ctx* ctx, int batch);
 /*
  * Write path (Algorithm 1 line 7; Sec. 4 "Complexity"): for each new token t and KV head,
  *     r = (k_t - k_mean) rk,   s = (v_t - v_mean) rv          exact products accumulated in binary64
- * (append-sized batches: blocks of the input dimension in index order, the blocks added pairwise; larger
- * ones: blocks of four input dimensions on the fp64 tensor path; the results differ by less than an ulp of
- * binary64), then for every group l the index of
+ * (blocks of the input dimension in index order, the blocks added pairwise; the order moves the result by less
+ * than an ulp of binary64), then for every group l the index of
  * the nearest codeword: exact Euclidean search (Sec. 2.2 "Quantization", App. B "Calibration"), the
  * lowest index winning a tie.  The stored index is the minimiser of the binary64 squared distance
- * sum_i (coef_i - codeword_i)^2 of the binary64 coefficient.  (Both kernels evaluate the 256 distances
- * in binary32 first and keep that result only where the two smallest distances are further apart than
- * binary32 rounding can have moved them; every other group is searched again in binary64.  The result
+ * sum_i (coef_i - codeword_i)^2 of the binary64 coefficient.  (The kernels rank
+ * the 256 distances first - append-sized batches in binary32, larger ones on the tensor cores from coefficients of
+ * about 22 bits - and keep that result only where the two smallest distances are further apart than the errors of
+ * coefficient and distance can have moved them; every other group is searched again in binary64.  The result
  * can differ from a binary64 reference only where the two nearest codewords are within ~1e-12 relative.)
  * The 2L index bytes go to page page_table[tok_seq[t]][tok_pos[t]/64] at slot tok_pos[t]%64, and
  * seq_lens[tok_seq[t]] becomes max(seq_lens[tok_seq[t]], tok_pos[t]+1).

@@ -17,7 +17,7 @@
 
 #include <cooperative_groups.h>
 
-#include "novakv_internal.cuh"
+#include "novakv_search.cuh"
 
 namespace {
 
@@ -156,15 +156,6 @@ __device__ __noinline__ int exact_search_group(const float* r_row_s, const __nv_
     return bi;
 }
 
-// What the binary32 evaluation can have moved a squared distance by: the coefficient vector of the group
-// is off by at most delta in norm (its rounding to binary32), the eight operations of the distance add a
-// relative 6 * 2^-24.  |d32 - d| <= 2 sqrt(d) delta + delta^2 + 6 * 2^-24 d; the test below uses twice the
-// bound at the larger of the two distances (both have moved) with some slack on the constants.
-__device__ __forceinline__ bool needs_exact_search(float best, float second, float delta) {
-    const float thr = 4.5f * sqrtf(second) * delta + 2.5f * delta * delta + 9.6e-7f * second;     // 9.6e-7 > 16 * 2^-24
-    return !(second - best > thr);
-}
-
 // Search of the tile's coefficients (r_s, [ENC_TILE][RSTRIDE] float) against the paired codebook image.
 // Warp w of n_warps owns groups w, w+n_warps, ...; lane t owns tokens t and t+32.
 // The binary32 pass finds the first minimum in ascending codeword order (what a scan with a strict '<' keeps)
@@ -269,302 +260,8 @@ __device__ __forceinline__ void search_tile(const float* r_s, const float4* cb_s
     }
 }
 
-// Named barriers of the tiled encode kernel (hardware barriers; bar.arrive does not block).
-__device__ __forceinline__ void nbar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void nbar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-constexpr int BAR_T = 1, BAR_S = 2, BAR_FULL = 3 /* +buf */, BAR_EMPTY = 5 /* +buf */;
-constexpr int ENC_HALF_THREADS = ENC_THREADS / 2;
-
-// Shared-memory plan of the pipelined encode kernel.
-template <int D>
-struct EncPipe {
-    static constexpr int L = D / NOVAKV_G;
-    static constexpr int RS = D + 4;
-    static constexpr int KS = 8;                               // rows of the transform matrix per slab
-    static constexpr size_t cb_bytes = (size_t)L * NOVAKV_C * NOVAKV_G * sizeof(float);
-    static constexpr size_t r_bytes = (size_t)ENC_TILE * RS * sizeof(float);       // one buffer
-    static constexpr size_t slab_x_bytes = (size_t)ENC_TILE * KS * sizeof(double);  // centred inputs [64][KS]
-    static constexpr size_t slab_r_bytes = (size_t)KS * D * sizeof(double);         // KS rows of R
-    static constexpr size_t slab_bytes = slab_x_bytes + slab_r_bytes;
-    static constexpr size_t idx_bytes = (size_t)ENC_TILE * L;
-    static constexpr size_t off_r = cb_bytes;
-    static constexpr size_t off_slab = off_r + 2 * r_bytes;                         // 2 slab buffers
-    static constexpr size_t off_idx = off_slab + 2 * slab_bytes;
-    static constexpr size_t off_pos = off_idx + idx_bytes;                          // [2][2][ENC_TILE] ints
-    static constexpr size_t off_mean = off_pos + 4 * ENC_TILE * sizeof(int);        // [D] doubles
-    static constexpr size_t off_rho = off_mean + D * sizeof(double);                // [2][2][ENC_TILE] floats (key scale | value scale, zero)
-    static constexpr size_t total = off_rho + 4 * ENC_TILE * sizeof(float);
-    static_assert(total <= 232448, "shared memory budget");
-};
-
-// Tiled (prefill) encode, one CTA per (run of 64-token tiles, KV head, side), the codebook of the
-// (head, side) resident in shared memory.  The two phases of a tile use different units of the SM:
-// the binary64 transform runs on the fp64 pipe and the load/store unit, the 256-way search on the FMA
-// pipe.  Half of the warps therefore transform tile i+1 while the other half searches tile i
-// (coefficients double-buffered in shared memory, hand-over by named hardware barriers).
-// KSC (key format with a per-token scale, Algorithm 3 "Normalize"): after the key transform of a tile
-// the transform warps compute rho = ||r||_2 / sqrt(d) of each token's binary32 coefficients (sum of squares
-// in binary64), round it to binary32 and then to bfloat16 (a scale that is not positive and finite becomes
-// 1), divide the coefficients by it in binary32 (IEEE division) and hand rho to the search warps, which
-// store it beside the indices (k_scales [n_pages][Hkv][64]).  Values are not scaled.
-// VSQ (scalar INT2 value codec of the deployed format): after the value transform of a tile the transform
-// warps form zero = bf16(min) and scale = bf16((max - zero) / 3) per token, replace each coefficient by its
-// level clamp(rint((s - zero) / scale), 0, 3), and the other warps pack four levels per byte (the byte of a
-// group) instead of searching; (scale, zero) go to v_meta [n_pages][Hkv][64][2].
-// FMT: 0 = 2-bit keys and values (vector quantised), 1 = KSC, 2 = KSC and VSQ.
-template <int D, int FMT>
-__global__ void __launch_bounds__(ENC_THREADS, 1)
-novakv_encode_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
-                     const int32_t* __restrict__ tok_seq, const int32_t* __restrict__ tok_pos, int n_tokens,
-                     const double* __restrict__ rk_d, const double* __restrict__ rv_d,
-                     const double* __restrict__ rk_plain, const double* __restrict__ rv_plain,
-                     const double* __restrict__ k_mean_d, const double* __restrict__ v_mean_d,
-                     const float* __restrict__ cb_k, const float* __restrict__ cb_v,
-                     uint8_t* __restrict__ k_pages, uint8_t* __restrict__ v_pages,
-                     __nv_bfloat16* __restrict__ k_scales, __nv_bfloat16* __restrict__ v_meta, int n_pages,
-                     const int32_t* __restrict__ page_table, int max_pages_per_seq, int n_seq,
-                     int32_t* __restrict__ seq_lens, int n_kv_heads, int tiles_per_cta_k, int tiles_per_cta_v,
-                     uint32_t* __restrict__ dev_status) {
-    // rk_d / rv_d: the transforms in tensor-core fragment order [d/4][d][4]; rk_plain / rv_plain: the same
-    // matrices row-major [d][d] (read only by the certified search's binary64 recomputation)
-    constexpr bool KSC = FMT >= 1, VSQ = FMT == 2;
-    using P = EncPipe<D>;
-    constexpr int L = D / NOVAKV_G, RS = P::RS, NT = ENC_HALF_THREADS;
-    extern __shared__ __align__(16) unsigned char smem[];
-    float4* cb_s = reinterpret_cast<float4*>(smem);
-    uint8_t* idx_s = smem + P::off_idx;
-    int* pos_s = reinterpret_cast<int*>(smem + P::off_pos);                // [buf][page|slot][ENC_TILE]
-    double* mean_s = reinterpret_cast<double*>(smem + P::off_mean);
-    float* rho_s = reinterpret_cast<float*>(smem + P::off_rho);            // [buf][2][ENC_TILE]
-
-    const int kvh = blockIdx.y, side = blockIdx.z;
-    const __nv_bfloat16* x_new = side == 0 ? k_new : v_new;
-    const double* R = (side == 0 ? rk_d : rv_d) + (size_t)kvh * D * D;      // fragment order [d/4][d][4]
-    const double* mean = (side == 0 ? k_mean_d : v_mean_d) + (size_t)kvh * D;
-    const float4* cb_g = reinterpret_cast<const float4*>((side == 0 ? cb_k : cb_v) + (size_t)kvh * L * NOVAKV_C * NOVAKV_G);
-
-    const int n_tiles = (n_tokens + ENC_TILE - 1) / ENC_TILE;
-    const int tiles_per_cta = blockIdx.z == 0 ? tiles_per_cta_k : tiles_per_cta_v;     // (the two sides may be cut differently)
-    const int tile0 = blockIdx.x * tiles_per_cta;
-    const int n_local = max(0, min(n_tiles, tile0 + tiles_per_cta) - tile0);
-    {
-        // a CTA whose token entries are all unused (sequence -1) has nothing to do
-        int any = 0;
-        const int t_end = min(n_tokens, (tile0 + n_local) * ENC_TILE);
-        for (int t = tile0 * ENC_TILE + threadIdx.x; t < t_end; t += ENC_THREADS) any |= tok_seq[t] != -1;
-        if (!__syncthreads_or(any)) return;
-    }
-
-    // codebook of this (head, side) -> shared memory, once per CTA
-    if (!(VSQ && side == 1)) fill_codebook_pairs(reinterpret_cast<float*>(cb_s), cb_g, L);
-    for (int i = threadIdx.x; i < D; i += ENC_THREADS) mean_s[i] = mean[i];
-    __syncthreads();
-    const bool is_transform = threadIdx.x < NT;
-    const int tid = is_transform ? threadIdx.x : threadIdx.x - NT;
-
-    if (is_transform) {
-        // ---------------- transform warps: fill r_s[buf] and the destinations of tile i ----------------
-        // r[t][c] = sum_i xc[t][i] R[i][c] in binary64 on the tensor cores (mma.sync m8n8k4, f64): exact
-        // products, binary64 accumulation in blocks of 4 input dimensions taken in index order, one rounding
-        // to binary32 at the end.  Warp w owns the 16 columns 16w .. 16w+15 of all 64 tokens: 8 x 2 fragments
-        // of 8 tokens x 8 columns, 2 accumulator registers each.  The input dimension is walked in slabs of
-        // KS rows: a slab is KS rows of R in fragment order (one contiguous block, asynchronous copy) and the
-        // centred inputs xc[64][KS]; slabs are double buffered and slab s + 1 is fetched while slab s is
-        // consumed, one barrier of the transform warps per slab.
-        constexpr int KS = P::KS, NSLAB = D / KS;
-        constexpr int NWT = NT / 32;                    // transform warps
-        constexpr int NTILE_N = D / 8 / NWT;            // column fragments per warp: 2 (D=128) or 1 (D=64)
-        constexpr int NTILE_M = ENC_TILE / 8;           // token fragments: 8
-        static_assert(NSLAB % 2 == 0 && ENC_TILE * KS / 2 == NT && NTILE_N >= 1, "slab mapping");
-        const int wt = tid >> 5, lane = tid & 31, fr = lane >> 2, fk = lane & 3;
-        const int xt = tid / (KS / 2), xk = (tid % (KS / 2)) * 2;      // this thread's two inputs of a slab
-        uint32_t xraw = 0u;
-        auto slab_issue = [&](int tile_t0, int tile_valid, int sl) {
-            unsigned char* buf_b = smem + P::off_slab + (sl & 1) * P::slab_bytes;
-            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(buf_b + P::slab_x_bytes);
-            const char* src = reinterpret_cast<const char*>(R + (size_t)sl * KS * D);
-#pragma unroll
-            for (int q = 0; q < (int)(P::slab_r_bytes / 16 / NT); ++q)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (tid + q * NT) * 16),
-                             "l"(src + (size_t)(tid + q * NT) * 16) : "memory");
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            xraw = 0u;
-            if (xt < tile_valid)
-                xraw = *reinterpret_cast<const uint32_t*>(x_new + ((size_t)(tile_t0 + xt) * n_kv_heads + kvh) * D + sl * KS + xk);
-        };
-        if (n_local > 0) slab_issue(tile0 * ENC_TILE, min(ENC_TILE, n_tokens - tile0 * ENC_TILE), 0);
-        for (int i = 0; i < n_local; ++i) {
-            const int buf = i & 1;
-            const int t0 = (tile0 + i) * ENC_TILE;
-            const int n_valid = min(ENC_TILE, n_tokens - t0);
-            float* r_s = reinterpret_cast<float*>(smem + P::off_r + buf * P::r_bytes);
-            // destination of each token (validated once); written to shared memory when the buffer is free
-            int page = -1, slot = 0;
-            if (tid < n_valid) {
-                const int sq = tok_seq[t0 + tid], pos = tok_pos[t0 + tid];
-                if (sq == -1) {
-                    // unused entry of the token list: skipped
-                } else if (sq < 0 || sq >= n_seq || pos < 0 || pos / NOVAKV_PAGE_TOKENS >= max_pages_per_seq) {
-                    atomicOr(dev_status, NOVAKV_DEV_BAD_TOKEN);
-                } else {
-                    page = page_table[(size_t)sq * max_pages_per_seq + pos / NOVAKV_PAGE_TOKENS];
-                    slot = pos % NOVAKV_PAGE_TOKENS;
-                    if (page < 0 || page >= n_pages) {
-                        atomicOr(dev_status, NOVAKV_DEV_BAD_PAGE);
-                        page = -1;
-                    } else if (kvh == 0 && side == 0) {
-                        atomicMax(&seq_lens[sq], pos + 1);
-                    }
-                }
-            }
-            double acc[NTILE_M][NTILE_N][2];
-#pragma unroll
-            for (int mt = 0; mt < NTILE_M; ++mt)
-#pragma unroll
-                for (int nt = 0; nt < NTILE_N; ++nt) { acc[mt][nt][0] = 0.0; acc[mt][nt][1] = 0.0; }
-#pragma unroll 1
-            for (int sl = 0; sl < NSLAB; ++sl) {
-                unsigned char* buf_b = smem + P::off_slab + (sl & 1) * P::slab_bytes;
-                double* xs = reinterpret_cast<double*>(buf_b);
-                const double* Rs = reinterpret_cast<const double*>(buf_b + P::slab_x_bytes);
-                // slab sl: its rows of R have landed, its inputs are centred in binary64 (exact) and stored
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-                {
-                    const __nv_bfloat162 xb = *reinterpret_cast<const __nv_bfloat162*>(&xraw);
-                    const bool valid = xt < n_valid;
-                    double2 v;
-                    v.x = valid ? (double)__bfloat162float(xb.x) - mean_s[sl * KS + xk] : 0.0;
-                    v.y = valid ? (double)__bfloat162float(xb.y) - mean_s[sl * KS + xk + 1] : 0.0;
-                    *reinterpret_cast<double2*>(xs + ((size_t)(xk >> 2) * ENC_TILE + xt) * 4 + (xk & 3)) = v;   // [k/4][t][k%4]
-                }
-                nbar_sync(BAR_T, NT);       // slab sl visible; everyone is done with slab sl - 1 (the other buffer)
-                if (sl + 1 < NSLAB) slab_issue(t0, n_valid, sl + 1);
-                else if (i + 1 < n_local) slab_issue(t0 + ENC_TILE, min(ENC_TILE, n_tokens - t0 - ENC_TILE), 0);
-#pragma unroll
-                for (int kq = 0; kq < KS / 4; ++kq) {
-                    // B fragments: R[4 kq + fk][column 16 wt + 8 nt + fr]; A fragments: xc[token 8 mt + fr][4 kq + fk]
-                    double bf[NTILE_N];
-#pragma unroll
-                    for (int nt = 0; nt < NTILE_N; ++nt) bf[nt] = Rs[((size_t)kq * D + (wt * NTILE_N + nt) * 8 + fr) * 4 + fk];
-#pragma unroll
-                    for (int mt = 0; mt < NTILE_M; ++mt) {
-                        const double af = xs[((size_t)kq * ENC_TILE + mt * 8 + fr) * 4 + fk];
-#pragma unroll
-                        for (int nt = 0; nt < NTILE_N; ++nt)
-                            asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-                                         : "+d"(acc[mt][nt][0]), "+d"(acc[mt][nt][1]) : "d"(af), "d"(bf[nt]));
-                    }
-                }
-            }
-            if (i >= 2) nbar_sync(BAR_EMPTY + buf, ENC_THREADS);          // the search of tile i-2 has released the buffer
-            if (tid < ENC_TILE) {
-                pos_s[(buf * 2 + 0) * ENC_TILE + tid] = page;
-                pos_s[(buf * 2 + 1) * ENC_TILE + tid] = slot;
-            }
-            // accumulator fragment: token 8 mt + fr, columns 16 wt + 8 nt + 2 fk, + 1
-#pragma unroll
-            for (int mt = 0; mt < NTILE_M; ++mt)
-#pragma unroll
-                for (int nt = 0; nt < NTILE_N; ++nt)
-                    *reinterpret_cast<float2*>(r_s + (size_t)(mt * 8 + fr) * RS + (wt * NTILE_N + nt) * 8 + 2 * fk) =
-                        make_float2((float)acc[mt][nt][0], (float)acc[mt][nt][1]);
-            if (KSC && side == 0) {
-                // 4 threads per token, thread `part` takes the columns = part (mod 4): conflict-free rows
-                nbar_sync(BAR_T, NT);
-                const int t = tid >> 2, part = tid & 3;
-                float* row = r_s + (size_t)t * RS + part;
-                double ss = 0.0;
-#pragma unroll 8
-                for (int i = 0; i < D / 4; ++i) {
-                    const double r = (double)row[4 * i];
-                    ss = fma(r, r, ss);
-                }
-                ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-                ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-                float rho = __bfloat162float(__float2bfloat16_rn((float)sqrt(ss / (double)D)));
-                if (!(rho > 0.f) || !isfinite(rho)) rho = 1.f;
-#pragma unroll 8
-                for (int i = 0; i < D / 4; ++i) row[4 * i] = __fdiv_rn(row[4 * i], rho);
-                if (part == 0) rho_s[(buf * 2) * ENC_TILE + t] = rho;
-            }
-            if (VSQ && side == 1) {
-                nbar_sync(BAR_T, NT);
-                const int t = tid >> 2, part = tid & 3;
-                float* row = r_s + (size_t)t * RS + part;
-                float mn = row[0], mx = row[0];
-#pragma unroll 8
-                for (int i = 1; i < D / 4; ++i) { mn = fminf(mn, row[4 * i]); mx = fmaxf(mx, row[4 * i]); }
-                mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 1)); mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 2)); mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                const float zero = __bfloat162float(__float2bfloat16_rn(mn));
-                float scale = __bfloat162float(__float2bfloat16_rn(__fdiv_rn(__fsub_rn(mx, zero), 3.0f)));
-                if (!(scale > 0.f) || !isfinite(scale)) scale = 1.f;
-#pragma unroll 8
-                for (int i = 0; i < D / 4; ++i) {
-                    float u = rintf(__fdiv_rn(__fsub_rn(row[4 * i], zero), scale));
-                    if (!(u > 0.f)) u = 0.f;
-                    row[4 * i] = fminf(u, 3.f);
-                }
-                if (part == 0) { rho_s[(buf * 2) * ENC_TILE + t] = scale; rho_s[(buf * 2 + 1) * ENC_TILE + t] = zero; }
-            }
-            __threadfence_block();
-            nbar_arrive(BAR_FULL + buf, ENC_THREADS);            // hand tile i to the search warps
-        }
-    } else {
-        // ---------------- search warps: nearest codewords of tile i, paged store ------------------------
-        for (int i = 0; i < n_local; ++i) {
-            const int buf = i & 1;
-            const int t0 = (tile0 + i) * ENC_TILE;
-            const int n_valid = min(ENC_TILE, n_tokens - t0);
-            const float* r_s = reinterpret_cast<const float*>(smem + P::off_r + buf * P::r_bytes);
-            nbar_sync(BAR_FULL + buf, ENC_THREADS);
-            if (VSQ && side == 1) {
-                // four levels (0..3, held as floats) per byte: the byte of group l
-                for (int e = tid; e < ENC_TILE * L; e += NT) {
-                    const int t = e / L, l = e - t * L;
-                    const float4 c = *reinterpret_cast<const float4*>(r_s + (size_t)t * RS + l * 4);
-                    idx_s[e] = (uint8_t)((int)c.x | ((int)c.y << 2) | ((int)c.z << 4) | ((int)c.w << 6));
-                }
-            } else {
-                const __nv_bfloat16* x_tile = x_new + ((size_t)t0 * n_kv_heads + kvh) * D;
-                const double* R_plain = (side == 0 ? rk_plain : rv_plain) + (size_t)kvh * D * D;
-                // normalised keys are defined in binary32: the values in r_s are the vector to encode
-                if (KSC && side == 0)
-                    search_tile<D, true>(r_s, cb_s, idx_s, n_valid, tid >> 5, NT / 32, x_tile, (size_t)n_kv_heads * D, mean_s, R_plain);
-                else
-                    search_tile<D, false>(r_s, cb_s, idx_s, n_valid, tid >> 5, NT / 32, x_tile, (size_t)n_kv_heads * D, mean_s, R_plain);
-            }
-            nbar_sync(BAR_S, NT);
-            for (int e = tid; e < n_valid * L; e += NT) {
-                const int t = e / L, l = e - t * L;
-                const int page = pos_s[(buf * 2 + 0) * ENC_TILE + t];
-                if (page < 0) continue;
-                const int slot = pos_s[(buf * 2 + 1) * ENC_TILE + t];
-                const size_t base = ((size_t)page * n_kv_heads + kvh) * (NOVAKV_PAGE_TOKENS * L);
-                if (side == 0) k_pages[base + novakv_k_offset<L>(slot, l)] = idx_s[e];
-                else v_pages[base + novakv_v_offset<L>(slot, l)] = idx_s[e];
-            }
-            if (KSC && side == 0 && tid < n_valid) {
-                const int page = pos_s[(buf * 2 + 0) * ENC_TILE + tid];
-                if (page >= 0)
-                    k_scales[((size_t)page * n_kv_heads + kvh) * NOVAKV_PAGE_TOKENS + pos_s[(buf * 2 + 1) * ENC_TILE + tid]] =
-                        __float2bfloat16_rn(rho_s[(buf * 2) * ENC_TILE + tid]);
-            }
-            if (VSQ && side == 1 && tid < n_valid) {
-                const int page = pos_s[(buf * 2 + 0) * ENC_TILE + tid];
-                if (page >= 0)
-                    reinterpret_cast<__nv_bfloat162*>(v_meta)[((size_t)page * n_kv_heads + kvh) * NOVAKV_PAGE_TOKENS +
-                                                              pos_s[(buf * 2 + 1) * ENC_TILE + tid]] =
-                        __floats2bfloat162_rn(rho_s[(buf * 2) * ENC_TILE + tid], rho_s[(buf * 2 + 1) * ENC_TILE + tid]);
-            }
-            nbar_sync(BAR_S, NT);                                // idx_s and the buffer are free again
-            if (i + 2 < n_local) nbar_arrive(BAR_EMPTY + buf, ENC_THREADS);
-        }
-    }
-}
-
-// Append-sized batches (a decode step appends one token per sequence): the tiled kernel above would
-// pad every (head, side) to a 64-token tile and fill a 128 KB codebook per CTA.  Here one warp owns one
+// Append-sized batches (a decode step appends one token per sequence): the prompt encoder would
+// pad every (head, side) to a 256-token tile.  Here one warp owns one
 // group of one (head, side) and stages only its 4 columns of the transform (4 KB of binary64) and its
 // group's codebook (4 KB), so the work spreads over L/4 * Hkv * 2 CTAs.  A pass covers tp tokens
 // (tp = 1, 2, ... 32, the smallest power of two that holds the batch, at most 32): lane = grp * tp + token.
@@ -964,43 +661,8 @@ novakv_status launch_encode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
         ctx->launches++;
         return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
     }
-    auto kern = v_meta ? novakv_encode_kernel<D, 2> : (k_scales ? novakv_encode_kernel<D, 1> : novakv_encode_kernel<D, 0>);
-    const size_t smem = EncPipe<D>::total;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return NOVAKV_ECUDA;
-    const int n_tiles = (n_tokens + ENC_TILE - 1) / ENC_TILE;
-    const int hs = ctx->cfg.n_kv_heads * 2;
-    // enough CTAs per (head, side) to fill the machine about twice, each amortising its codebook fill
-    // CTAs per (head, side): whole waves of the machine, each CTA amortising its 128 KB codebook fill
-    // (counted as 1.5 tiles) over several tiles
-    int ctas_x = 1, tiles_per_cta = n_tiles;
-    double best = 1e30;
-    for (int w = 1; w <= 8; ++w) {
-        int cx = min(n_tiles, max(1, (w * ctx->n_sm) / hs));
-        const int tp = (n_tiles + cx - 1) / cx;
-        cx = (n_tiles + tp - 1) / tp;
-        const int waves = (cx * hs + ctx->n_sm - 1) / ctx->n_sm;
-        const double cost = waves * (tp + 1.5);
-        if (cost < best) { best = cost; ctas_x = cx; tiles_per_cta = tp; }
-    }
-    int tiles_k = tiles_per_cta, tiles_v = tiles_per_cta;
-    if (v_meta != nullptr && ctas_x > 1) {
-        // scalar INT2 values need no codeword search: a value tile costs about 3/8 of a key tile, so the CTAs of a head
-        // are shared out 8 : 3 between the two sides instead of evenly (the value side then takes longer runs)
-        const int per_head = 2 * ctas_x;
-        const int ck = max(1, min(n_tiles, (per_head * 8 + 5) / 11)), cv = max(1, min(n_tiles, per_head - ck));
-        tiles_k = (n_tiles + ck - 1) / ck;
-        tiles_v = (n_tiles + cv - 1) / cv;
-        ctas_x = max((n_tiles + tiles_k - 1) / tiles_k, (n_tiles + tiles_v - 1) / tiles_v);
-    }
-    dim3 grid(ctas_x, ctx->cfg.n_kv_heads, 2);
-    novakv_prof_scope ps(ctx, 1, stream);
-    kern<<<grid, ENC_THREADS, smem, stream>>>(k_new, v_new, tok_seq, tok_pos, n_tokens, ly.rk_d_mma, ly.rv_d_mma,
-                                               ly.rk_d, ly.rv_d, ly.k_mean_d, ly.v_mean_d, ly.cb_k, ly.cb_v, k_pages, v_pages, k_scales,
-                                               v_meta, n_pages, page_table, max_pages_per_seq, n_seq, seq_lens,
-                                               ctx->cfg.n_kv_heads, tiles_k, tiles_v, ctx->dev_status);
-    ps.end();
-    ctx->launches++;
-    return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
+    return novakv_launch_prefill(ctx, ly, k_new, v_new, tok_seq, tok_pos, n_tokens, k_pages, v_pages, n_pages, page_table,
+                                 max_pages_per_seq, n_seq, seq_lens, stream, k_scales, v_meta);
 }
 
 template <int D>

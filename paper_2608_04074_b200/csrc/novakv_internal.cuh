@@ -13,6 +13,8 @@
 #define NOVAKV_G 4
 #define NOVAKV_C 256
 #define NOVAKV_VBLOCK 16
+#define NOVAKV_PF_GROUP_BYTES 12288                    // prompt encoder: 8 KB search operand + 4 KB binary32 codewords of a group
+#define NOVAKV_PF_CONSTS(d) ((d) + 2 * ((d) / 4) + 4)
 
 // Device copies of one layer's tables, in the layouts the kernels read.
 struct novakv_layer {
@@ -20,8 +22,9 @@ struct novakv_layer {
     // write path (binary64 transforms, see the encode entry of the public header)
     double* rk_d = nullptr;       // [Hkv][d][d]
     double* rv_d = nullptr;       // [Hkv][d][d]
-    double* rk_d_mma = nullptr;   // [Hkv][d/4][d][4]: rk_d with the input dimension blocked by 4 (tensor-core fragments)
-    double* rv_d_mma = nullptr;   // same for rv_d
+    uint8_t* pf_r = nullptr;      // [2 sides][Hkv][3 d d 2]: bfloat16 slices of rk / rv as tensor-core operands (prompt encoder)
+    uint8_t* pf_cb = nullptr;     // [2][Hkv][L][NOVAKV_PF_GROUP_BYTES]: codebooks as search operand and in binary32
+    float* pf_const = nullptr;    // [2][Hkv][NOVAKV_PF_CONSTS]: mean share, column norms, scales
     double* k_mean_d = nullptr;   // [Hkv][d]
     float* k_mean = nullptr;      // [Hkv][d] (offset q . k_mean of a sink logit / the BF16 band, scaled key format)
     float* k_mean_eff = nullptr;  // [Hkv][d] k_mean + centre R_K^{-1}: the same offset when the table is built from centred codewords
@@ -58,6 +61,7 @@ struct novakv_ctx {
     int seg_weight = 24;          // pages one (sequence, KV head) segment weighs extra in the scan kernel's work split
     bool fused_merge = false;     // true: the scan kernel merges the partials itself where it can (no sink, no band)
     unsigned smem_opt_in = 0;     // scan-kernel instantiations whose shared-memory opt-in was set on this device
+    unsigned prefill_opt_in = 0;  // the same for the prompt encoder's formats
 };
 
 // RAII-free helper: brackets a launch with events when profiling is on.
@@ -78,6 +82,12 @@ novakv_status novakv_launch_encode(novakv_ctx* ctx, const novakv_layer& ly, cons
     int max_pages_per_seq, int n_seq, int32_t* seq_lens, cudaStream_t stream,
     __nv_bfloat16* k_scales = nullptr /* scaled key format: [n_pages][Hkv][64] */,
     __nv_bfloat16* v_meta = nullptr /* INT2 value codec: (scale, zero) [n_pages][Hkv][64][2] */);
+novakv_status novakv_launch_prefill(novakv_ctx* ctx, const novakv_layer& ly, const __nv_bfloat16* k_new, const __nv_bfloat16* v_new,
+    const int32_t* tok_seq, const int32_t* tok_pos, int n_tokens, uint8_t* k_pages, uint8_t* v_pages, int n_pages,
+    const int32_t* page_table, int max_pages_per_seq, int n_seq, int32_t* seq_lens, cudaStream_t stream, __nv_bfloat16* k_scales,
+    __nv_bfloat16* v_meta);
+// host: the prompt encoder's images of one (KV head, side)
+void novakv_build_prefill_image(int d, const float* R, const float* mean, const float* cb, uint8_t* r_img, uint8_t* cb_img, float* consts);
 novakv_status novakv_launch_search(novakv_ctx* ctx, const novakv_layer& ly, int which, const float* coef,
     int n, uint8_t* idx_out, cudaStream_t stream);
 

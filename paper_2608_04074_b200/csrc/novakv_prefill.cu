@@ -1,0 +1,998 @@
+// Write path for prompt-sized batches: transform and nearest-codeword search on the 5th-generation tensor cores.
+//
+// Work unit: 256 tokens of one (KV head, side) and 16 (or 8) groups; one persistent CTA per SM walks a contiguous run of
+// units.  Per 128-token half tile (TMEM lane = token):
+//   transform   D[128 x 64] = x R, three bfloat16 slices of the binary32 matrix R, binary32 accumulators in TMEM.  The
+//               token's thread subtracts the mean's share m R and parks the coefficients in shared memory.
+//   search      per group D[128 x 256] = |r - c|^2 / 2 for all codewords as ONE K = 16 product
+//                   [rh rh rl 1 1 qh ql] . [-ch -cl -ch ph pl 1 1],   q = |r|^2 / 2, p = |c|^2 / 2,
+//               (h, l: a binary16 number and its binary16 remainder), binary16 accumulators in TMEM; the thread takes the
+//               minima of 32 rows of 8 codewords with packed three-input minima (a quarter instruction per codeword),
+//               keeps every row that could hold the nearest codeword, and evaluates those rows - almost always one -
+//               directly in binary32.
+//   certificate the direct distances are trusted only where the two smallest are further apart than the error bounds of
+//               coefficient and distance; every other (token, group) goes to one of two helper warps, which search it in
+//               binary64 from the binary64 coefficient.  The stored index is the nearest codeword of the binary64
+//               coefficient.
+//
+// Roles: four token warpgroups, two per half tile (thread = token, each takes half of the groups), whose first warp
+// issues the search MMAs; one warp loads token rows and issues the transforms; one feeds the codebook ring; two search
+// in binary64.  A chunk of 128 codewords makes a round trip token warps -> MMA -> token warps (about 300 cycles, whatever
+// its width), so chunks are as wide as TMEM allows (four warpgroups x 128 columns: the coefficients live in shared
+// memory for that), the first chunk of the next group is computed behind the selection of this one, and four token warps
+// per scheduler hide the rest.  Every wait is bounded (novakv_tcgen05.cuh): a wait that gives up sets
+// NOVAKV_DEV_WAIT_TIMEOUT, and the CTA runs through its remaining steps without waiting.  (The named barriers among token
+// warps are never skipped.)
+#include <math_constants.h>
+
+#include <cmath>
+#include <cstring>
+
+#include "novakv_search.cuh"
+#include "novakv_tcgen05.cuh"
+
+namespace {
+
+constexpr int PF_TOKEN_WARPS = 16;
+constexpr int PF_HELPERS = 2;
+constexpr int PF_THREADS = (PF_TOKEN_WARPS + 2 + PF_HELPERS) * 32;
+constexpr int PF_TILE = 256;                 // tokens per unit: two half tiles
+constexpr int PF_HALF = 128;
+constexpr int PF_STAGES = 4;                 // codebook ring
+constexpr int PF_STAGE_BYTES = NOVAKV_PF_GROUP_BYTES;
+constexpr int PF_QUEUE = 16;                 // entries of a helper's queue
+// durations the work split reckons with, microseconds per unit
+constexpr double PF_US_UNIT = 2.0, PF_US_GROUP = 0.6, PF_US_INT2 = 4.0;
+// |coefficient - binary64 coefficient| <= KAPPA (|x| + |mean|) |R column|.  The accumulation order of the tensor core is
+// not specified; all-positive inputs (every truncation in the same direction) showed 2^-21.6, random signs 2^-23.3.
+constexpr float KAPPA = 1.4e-6f;             // > 2^-19.5
+// |D - |r - c|^2 / 2| <= EPS_S (|r| + |c|)^2: dropped rl.cl and remainders (3 2^-22 |r||c|) plus the accumulation
+// (5.3e-7 of the largest term seen on random operands), with a factor of 4.
+constexpr float EPS_S = 1.0e-6f;
+constexpr float KEY_REL = 9.6e-7f;           // > 2^-20: the direct distances carry a codeword number in their low 3 bits
+
+template <int D, int FMT>
+struct PF {
+    static constexpr int L = D / NOVAKV_G;
+    static constexpr int KSTEPS = D / 16;
+    static constexpr int GU = 16;                                 // groups of a unit, at most
+    // a per-token scale needs the token's whole row: then all columns of R are resident, which leaves room for two slots
+    static constexpr int R_COLS = FMT == 0 ? GU * NOVAKV_G : D;
+    static constexpr int NX = D == 128 && FMT != 0 ? 2 : 3;
+    static constexpr uint32_t R_SLICE = R_COLS * D * 2;
+    static constexpr uint32_t R_IMG_SLICE = D * D * 2;
+    static constexpr uint32_t X_BYTES = PF_HALF * D * 2;          // token rows of a half tile
+    static constexpr uint32_t SLOT_BYTES = PF_HALF * GU * 16;     // the same memory later holds its coefficients [GU][128][4]
+    static constexpr uint32_t A_BYTES = PF_HALF * 32;             // search operand of one group
+    static constexpr int NCONST = NOVAKV_PF_CONSTS(D);            // mean share [D] | column norm [L] | scale [L] | 4 norms
+    static constexpr uint32_t OFF_R = 0;
+    static constexpr uint32_t OFF_X = OFF_R + 3 * R_SLICE;
+    static constexpr uint32_t OFF_RING = OFF_X + NX * SLOT_BYTES;
+    static constexpr uint32_t OFF_A = OFF_RING + PF_STAGES * PF_STAGE_BYTES;
+    static constexpr uint32_t OFF_QUEUE = OFF_A + 4 * A_BYTES;
+    static constexpr uint32_t OFF_CONST = OFF_QUEUE + PF_HELPERS * PF_QUEUE * 16;
+    static constexpr uint32_t OFF_BAR = OFF_CONST + ((NCONST * 4 + 15) & ~15);
+    static constexpr uint32_t OFF_MISC = OFF_BAR + 256;           // TMEM base, abort flag, finished token warps, queue counters
+    static constexpr uint32_t BYTES = OFF_MISC + 64;
+    static_assert(BYTES <= 232448, "shared memory budget");
+    static_assert(X_BYTES <= SLOT_BYTES && R_SLICE % 1024 == 0 && SLOT_BYTES % 1024 == 0, "swizzled operands start on 1024 bytes");
+};
+// mbarriers
+enum { B_R = 0, B_X = 1 /* +slot */, B_XFREE = 4 /* +slot */, B_T = 7 /* +half */, B_TFREE = 9 /* +half */, B_S = 11 /* +wg */,
+       B_RING = 15 /* +stage */, B_RINGFREE = B_RING + PF_STAGES, B_COUNT = B_RING + 2 * PF_STAGES };
+static_assert(B_COUNT * 8 <= 256, "barrier block");
+// named barriers: 1 + wg among the four warps of a warpgroup, 5 + half among the eight of a half tile
+__device__ __forceinline__ void nbar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void nbar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+struct PrefillArgs {
+    const __nv_bfloat16 *k_new, *v_new;
+    const int32_t *tok_seq, *tok_pos;
+    int n_tokens;
+    const uint8_t* r_img;       // [2][Hkv][3 d d 2]
+    const uint8_t* cb_img;      // [2][Hkv][L][stage]
+    const float* consts;        // [2][Hkv][NCONST]
+    const double *rk_d, *rv_d, *k_mean_d, *v_mean_d;
+    const float *cb_k, *cb_v;   // [Hkv][L][256][4]
+    uint8_t *k_pages, *v_pages;
+    __nv_bfloat16 *k_scales, *v_meta;
+    int n_pages;
+    const int32_t* page_table;
+    int max_pages_per_seq, n_seq;
+    int32_t* seq_lens;
+    int n_kv_heads;
+    int gs;                     // parts a head's groups are cut into
+    int cost_k, cost_v;         // relative cost of a key / value unit (the cut of the walk)
+    uint32_t* dev_status;
+};
+
+__device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
+    uint32_t d;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+__device__ __forceinline__ float2 unpack_half2(uint32_t h) { return __half22float2(*reinterpret_cast<const __half2*>(&h)); }
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+__device__ __forceinline__ uint64_t dup2(float x) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1,%1};" : "=l"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Binary32 codeword image of a group: rows of 8 codewords (128 bytes), a row as 4 codeword pairs of two 16-byte chunks:
+// chunk 2 p + h of a row holds components 2 h, 2 h + 1 of its codewords 2 p, 2 p + 1, [c0.a c1.a c0.b c1.b].
+__host__ __device__ __forceinline__ int codeword_offset(int code, int comp) {       // in floats
+    return (code >> 3) * 32 + (((code & 7) >> 1) * 2 + (comp >> 1)) * 4 + (comp & 1) * 2 + (code & 1);
+}
+
+// Warp-cooperative exact search of one (token, group): all lanes call it with the same arguments and get the same result.
+// rho > 0: the vector to encode is the binary32 quotient of the binary32 coefficient and rho (scaled key format).
+// Lane i evaluates the codewords i, i + 32, ... in ascending order with a strict '<'; the warp then keeps the smallest
+// distance and, among equal distances, the lowest index.
+template <int D>
+__device__ __noinline__ int exact_search_token(const __nv_bfloat16* __restrict__ x_row, const double* __restrict__ mean,
+                                               const double* __restrict__ R /* [D][D] */, int l, const float4* __restrict__ cb /* [256] */,
+                                               float rho) {
+    const int lane = threadIdx.x & 31;
+    double r[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) r[c] = 0.0;
+#pragma unroll
+    for (int j = 0; j < D / 32; ++j) {
+        const int k = lane + 32 * j;
+        const double xc = (double)__bfloat162float(x_row[k]) - mean[k];
+        const double2 r01 = *reinterpret_cast<const double2*>(R + (size_t)k * D + l * 4);
+        const double2 r23 = *reinterpret_cast<const double2*>(R + (size_t)k * D + l * 4 + 2);
+        r[0] = fma(xc, r01.x, r[0]); r[1] = fma(xc, r01.y, r[1]);
+        r[2] = fma(xc, r23.x, r[2]); r[3] = fma(xc, r23.y, r[3]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r[c] += __shfl_xor_sync(0xffffffffu, r[c], o);
+    if (rho > 0.f) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) r[c] = (double)__fdiv_rn((float)r[c], rho);
+    }
+    double best = CUDART_INF;
+    int bi = lane;
+#pragma unroll 4
+    for (int j = 0; j < NOVAKV_C / 32; ++j) {
+        const float4 c = cb[lane + 32 * j];
+        const double e0 = r[0] - (double)c.x, e1 = r[1] - (double)c.y, e2 = r[2] - (double)c.z, e3 = r[3] - (double)c.w;
+        const double dd = __dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(e0, e0), __dmul_rn(e1, e1)), __dmul_rn(e2, e2)), __dmul_rn(e3, e3));
+        if (dd < best) { best = dd; bi = lane + 32 * j; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    return bi;
+}
+
+// All binary32 coefficients of one token from binary64 sums: lane i gets columns D / 32 * i .. (same arguments in all lanes).
+template <int D>
+__device__ __noinline__ void exact_row(const __nv_bfloat16* __restrict__ x_row, const double* __restrict__ mean,
+                                       const double* __restrict__ R, float (&out)[D / 32]) {
+    constexpr int N = D / 32;
+    const int lane = threadIdx.x & 31;
+    double acc[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < D; ++k) {
+        const double xc = (double)__bfloat162float(x_row[k]) - mean[k];
+#pragma unroll
+        for (int i = 0; i < N; i += 2) {
+            const double2 r = *reinterpret_cast<const double2*>(R + (size_t)k * D + lane * N + i);
+            acc[i] = fma(xc, r.x, acc[i]);
+            acc[i + 1] = fma(xc, r.y, acc[i + 1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) out[i] = (float)acc[i];
+}
+
+// Stores the codes of groups l .. l + 3 of this lane's token (group l in the low byte); l a multiple of 4.
+template <int L>
+__device__ __forceinline__ void store_key_word(uint8_t* chunk, int slot, int l, uint32_t w) {
+    const int x = slot & (l < 16 ? 7 : 15);
+    const int jw = (l >> 2) ^ (x >> 2);
+    *reinterpret_cast<uint32_t*>(chunk + ((((slot >> 5) * (L / 16) + (jw >> 2)) * 32 + (slot & 31)) * 16 + (jw & 3) * 4)) =
+        __byte_perm(w, 0u, 0x3210u ^ ((x & 3) * 0x1111u));
+}
+// Values keep the codes of four tokens (4 apart) of one group in a word.  aligned: the warp's lanes are whole 16-token
+// blocks in order, so that a 4 x 4 byte transpose among the lanes (4 apart) makes those words; otherwise single bytes.
+template <int L>
+__device__ __forceinline__ void store_value_word(uint8_t* chunk, int slot, int l, uint32_t w, bool aligned, bool valid, int lane) {
+    if (aligned) {
+        uint32_t t = __shfl_xor_sync(0xffffffffu, w, 8);
+        w = __byte_perm(w, t, lane & 8 ? 0x3276u : 0x5410u);
+        t = __shfl_xor_sync(0xffffffffu, w, 4);
+        w = __byte_perm(w, t, lane & 4 ? 0x3715u : 0x6240u);
+        const int gl = l + ((lane >> 2) & 3), fc = lane & 3;
+        *reinterpret_cast<uint32_t*>(chunk + ((slot >> 4) * (L * 16) + ((gl & 7) * 4 + fc) * (L / 2) + ((gl >> 3) ^ (fc & 1)) * 4)) = w;
+    } else if (valid) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) chunk[novakv_v_offset<L>(slot, l + i)] = (uint8_t)(w >> (8 * i));
+    }
+}
+
+// FMT: 0 = 2-bit keys and values (vector quantised), 1 = keys with a per-token scale, 2 = those and scalar INT2 values.
+// Per-token scale (keys): rho = bf16(sqrt(sum r^2 / d)) of the binary32 coefficients; it is taken from the tensor-core
+// coefficients where no error within their bound can move the bfloat16 rounding, else from the binary64 row.
+// INT2 values: zero, scale and the levels likewise; a token with any decision inside the bound takes the binary64 row.
+template <int D, int FMT>
+__global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const PrefillArgs a) {
+    using P = PF<D, FMT>;
+    constexpr int L = P::L;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const uint32_t sb = smem_u32(smem);
+    if ((sb & 1023u) != 0u) {          // cannot happen without static shared memory; reported, never trapped
+        if (threadIdx.x == 0) atomicOr(a.dev_status, NOVAKV_DEV_SMEM_LAYOUT);
+        return;
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    volatile int* const misc = reinterpret_cast<volatile int*>(smem + P::OFF_MISC);
+    volatile int* const abort_flag = misc + 1;
+    int* const s_done = reinterpret_cast<int*>(smem + P::OFF_MISC) + 2;               // token warps that have finished the segment
+    int* const s_count = reinterpret_cast<int*>(smem + P::OFF_MISC) + 4;              // [helper] entries in the queue
+    int* const s_head = reinterpret_cast<int*>(smem + P::OFF_MISC) + 4 + PF_HELPERS;  // [helper] entries ever queued
+    float* const cst = reinterpret_cast<float*>(smem + P::OFF_CONST);
+    auto bar = [&](int i) -> uint32_t { return sb + P::OFF_BAR + i * 8; };
+
+    // the walk: key units, then value units, cut evenly in cost
+    const int n_tiles = (a.n_tokens + PF_TILE - 1) / PF_TILE;
+    const int units_k = a.n_kv_heads * a.gs * n_tiles, gs_v = FMT == 2 ? 1 : a.gs, units_v = a.n_kv_heads * gs_v * n_tiles;
+    auto first_unit = [&](int c) -> int {
+        const long tk = (long)units_k * a.cost_k, t = (tk + (long)units_v * a.cost_v) * c / gridDim.x;
+        return t < tk ? (int)(t / a.cost_k) : units_k + (int)((t - tk) / a.cost_v);
+    };
+    const int u_end = first_unit(blockIdx.x + 1);
+    int u_next = first_unit(blockIdx.x);
+    if (u_next >= u_end) return;
+
+    if (warp == 0) tmem_alloc<512>(sb + P::OFF_MISC);
+    if (threadIdx.x == 0) {
+        misc[1] = 0;
+#pragma unroll
+        for (int h = 0; h < PF_HELPERS; ++h) { s_count[h] = 0; s_head[h] = 0; }
+        mbar_init(bar(B_R), 1);
+#pragma unroll
+        for (int x = 0; x < P::NX; ++x) { mbar_init(bar(B_X + x), 1); mbar_init(bar(B_XFREE + x), 8); }
+#pragma unroll
+        for (int w = 0; w < 2; ++w) { mbar_init(bar(B_T + w), 1); mbar_init(bar(B_TFREE + w), 4); }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) mbar_init(bar(B_S + g), 1);
+#pragma unroll
+        for (int s = 0; s < PF_STAGES; ++s) {
+            mbar_init(bar(B_RING + s), 1);
+            mbar_init(bar(B_RINGFREE + s), 10);        // MMAs and token warps of the two half tiles
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_proxy_async();
+    }
+    for (int i = threadIdx.x; i < PF_HELPERS * PF_QUEUE; i += PF_THREADS) reinterpret_cast<uint4*>(smem + P::OFF_QUEUE)[i] = make_uint4(0, 0, 0, 0);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = (uint32_t)misc[0];
+
+    // running phase counts of the barriers, over all segments
+    int n_it = 0, n_use = 0, n_seg = 0;               // tiles; ring uses; segments
+    uint32_t n_s = 0;                                 // token warps: chunks seen
+    int q_tail = 0;                                   // helpers: entries taken
+
+    // ---- segments: units of one (KV head, side, part of the groups)
+    while (u_next < u_end) {
+        const bool is_v = u_next >= units_k;
+        const int ul = is_v ? u_next - units_k : u_next, row_u = ul / n_tiles, tile0 = ul - row_u * n_tiles;
+        const int gs = is_v ? gs_v : a.gs, kvh = row_u / gs, part = row_u - kvh * gs, side = is_v ? 1 : 0;
+        const int n_local = min(n_tiles - tile0, (is_v ? u_end : min(u_end, units_k)) - u_next);
+        const bool ksc = FMT >= 1 && side == 0, vsq = FMT == 2 && side == 1;
+        const int ngh = vsq ? 0 : L / gs / 2;                              // groups a token warpgroup searches
+        const int g0 = part * (L / gs);
+        // columns of the transform: all of them where a token's whole row is needed
+        const int c0 = ksc || vsq ? 0 : g0 * 4, nc = ksc || vsq ? D : L / gs * 4;
+        u_next += n_local;
+        const size_t sh = (size_t)side * a.n_kv_heads + kvh;
+        const __nv_bfloat16* x_new = side == 0 ? a.k_new : a.v_new;
+        const double* R_plain = (side == 0 ? a.rk_d : a.rv_d) + (size_t)kvh * D * D;
+        const double* mean = (side == 0 ? a.k_mean_d : a.v_mean_d) + (size_t)kvh * D;
+        const float4* cb_g = reinterpret_cast<const float4*>(side == 0 ? a.cb_k : a.cb_v) + (size_t)kvh * L * NOVAKV_C;
+        uint8_t* const pages = side == 0 ? a.k_pages : a.v_pages;
+        for (int i = threadIdx.x; i < P::NCONST; i += PF_THREADS) cst[i] = a.consts[sh * P::NCONST + i];
+        if (threadIdx.x == 0) *s_done = 0;
+        __syncthreads();
+
+        if (warp == PF_TOKEN_WARPS) {
+            // ---- token rows ([128][D] bfloat16 of a half tile, 128-byte rows per panel, 16-byte chunks swizzled by the
+            //      row), one half tile ahead of the transforms.  Half tile q of the CTA uses slot q % NX.
+            const int q0 = 2 * n_it, q1 = q0 + 2 * n_local;
+            bool ok = true;
+            auto load_rows = [&](int q) {
+                const int slot = q % P::NX;
+                if (q >= P::NX) ok = mbar_wait(bar(B_XFREE + slot), (q / P::NX - 1) & 1, abort_flag);
+                if (!__all_sync(0xffffffffu, ok)) { ok = false; return; }
+                const int t0 = tile0 * PF_TILE + (q - q0) * PF_HALF;
+                const uint32_t dst0 = sb + P::OFF_X + slot * P::SLOT_BYTES;
+#pragma unroll 8
+                for (int e = lane; e < PF_HALF * (D / 8); e += 32) {
+                    const int t = e / (D / 8), c = e - t * (D / 8);
+                    const uint32_t dst = dst0 + (c >> 3) * (PF_HALF * 128) + t * 128 + (((c & 7) ^ (t & 7)) * 16);
+                    const bool in = t0 + t < a.n_tokens;
+                    const __nv_bfloat16* src = x_new + ((size_t)(in ? t0 + t : 0) * a.n_kv_heads + kvh) * D + c * 8;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+                }
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(B_X + slot));
+                __syncwarp();
+            };
+            load_rows(q0);
+            ok = __all_sync(0xffffffffu, ok && mbar_wait(bar(B_R), n_seg & 1, abort_flag));
+            const uint32_t id_t = umma_idesc(true, true, 128, 0) | ((uint32_t)(nc >> 3) << 17);
+            for (int q = q0; q < q1 && ok; ++q) {
+                const int w = q & 1, slot = q % P::NX;
+                if (q >= 2) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_TFREE + w), ((q >> 1) - 1) & 1, abort_flag));
+                if (!ok) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    bool first = true;
+                    // small slices first: their sums are added while the accumulator is small
+#pragma unroll 1
+                    for (int s = 2; s >= 0; --s)
+#pragma unroll
+                        for (int k = 0; k < P::KSTEPS; ++k) {
+                            const uint32_t off = P::OFF_X + slot * P::SLOT_BYTES + (k >> 2) * (PF_HALF * 128) + (k & 3) * 32;
+                            const uint32_t offr = P::OFF_R + s * P::R_SLICE + (k >> 2) * (P::R_COLS * 128) + (k & 3) * 32;
+                            umma_f16(tmem + w * 256, umma_desc(sb + off, 16, 1024, 2), umma_desc(sb + offr, 16, 1024, 2), id_t, !first);
+                            first = false;
+                        }
+                    umma_commit(bar(B_T + w));
+                }
+                __syncwarp();
+                if (q + 1 < q1) load_rows(q + 1);
+            }
+            n_it += n_local;
+        } else if (warp == PF_TOKEN_WARPS + 1) {
+            if (lane == 0) {
+                // ---- the matrix slices (columns c0 .. c0 + nc - 1) once, then the codebook ring
+                mbar_expect_tx(bar(B_R), 3 * (uint32_t)nc * D * 2);
+#pragma unroll 1
+                for (int s = 0; s < 3; ++s)
+#pragma unroll 1
+                    for (int p = 0; p < D / 64; ++p)
+                        bulk_copy(sb + P::OFF_R + s * P::R_SLICE + p * (P::R_COLS * 128),
+                                  a.r_img + sh * (3 * P::R_IMG_SLICE) + s * P::R_IMG_SLICE + p * (D * 128) + c0 * 128, (uint32_t)nc * 128, bar(B_R));
+                const uint8_t* src = a.cb_img + (sh * L + g0) * PF_STAGE_BYTES;
+                const int n = n_local * 2 * ngh;
+                bool ok = true;
+                // use 2 g + h: group g of the half of the groups that warpgroups h take
+                for (int j = 0, g = 0; j < n && ok; ++j, ++n_use) {
+                    const int s = n_use % PF_STAGES;
+                    if (n_use >= PF_STAGES) ok = mbar_wait(bar(B_RINGFREE + s), (n_use / PF_STAGES - 1) & 1, abort_flag);
+                    if (!ok) break;
+                    mbar_expect_tx(bar(B_RING + s), PF_STAGE_BYTES);
+                    bulk_copy(sb + P::OFF_RING + s * PF_STAGE_BYTES, src + (size_t)((j & 1) * ngh + g) * PF_STAGE_BYTES, PF_STAGE_BYTES,
+                              bar(B_RING + s));
+                    if (j & 1) g = g + 1 == ngh ? 0 : g + 1;
+                }
+                // no copy and no commit may be in flight when the segment (and the CTA's memory) goes away
+                mbar_wait(bar(B_R), n_seg & 1, abort_flag);
+                for (int j = max(0, n_use - PF_STAGES); j < n_use; ++j) {
+                    int tries = 0;
+                    while (!mbar_try(bar(B_RING + j % PF_STAGES), (j / PF_STAGES) & 1) && ++tries < 1000000) {}
+                    mbar_wait(bar(B_RINGFREE + j % PF_STAGES), (j / PF_STAGES) & 1, abort_flag);
+                }
+            }
+            __syncwarp();
+        } else if (warp > PF_TOKEN_WARPS + 1) {
+            // ---- helpers: binary64 searches queued by the token warps
+            const int h = warp - (PF_TOKEN_WARPS + 2);
+            volatile uint32_t* const queue = reinterpret_cast<volatile uint32_t*>(smem + P::OFF_QUEUE) + h * PF_QUEUE * 4;
+            for (;;) {
+                const bool last = *reinterpret_cast<volatile int*>(s_done) == PF_TOKEN_WARPS;      // (read before the entry)
+                volatile uint32_t* const e = queue + (q_tail % PF_QUEUE) * 4;
+                const uint32_t tag = e[0];
+                if (!__any_sync(0xffffffffu, tag != 0u)) {
+                    if (__any_sync(0xffffffffu, last)) break;
+                    __nanosleep(200);
+                    continue;
+                }
+                __threadfence_block();
+                const uint32_t t0 = __shfl_sync(0xffffffffu, e[0], 0);
+                const int l = t0 & 63, slot = (t0 >> 6) & 63, tkn = (int)e[1], page = (int)e[2];
+                const float rho = __uint_as_float(e[3]);
+                __syncwarp();
+                const int bi = exact_search_token<D>(x_new + ((size_t)tkn * a.n_kv_heads + kvh) * D, mean, R_plain, l, cb_g + l * NOVAKV_C, rho);
+                if (lane == 0) {
+                    pages[((size_t)page * a.n_kv_heads + kvh) * (NOVAKV_PAGE_TOKENS * L) +
+                          (side == 0 ? novakv_k_offset<L>(slot, l) : novakv_v_offset<L>(slot, l))] = (uint8_t)bi;
+                    e[0] = 0u;
+                    __threadfence_block();
+                    atomicSub(&s_count[h], 1);
+                }
+                __syncwarp();
+                ++q_tail;
+            }
+        } else {
+            // ---- token warps: thread = token; warpgroup wg = 2 * half tile + half of the groups
+            const int wg = warp >> 2, w = wg >> 1, hf = wg & 1, row = threadIdx.x & (PF_HALF - 1);
+            const uint32_t lane_base = (uint32_t)(warp & 3) << 21;
+            const uint32_t d_t = tmem + w * 256 + lane_base, d_s = tmem + wg * 128;
+            const uint32_t a_s = sb + P::OFF_A + wg * P::A_BYTES;
+            float* const x2_s = reinterpret_cast<float*>(smem + P::OFF_A);               // partial |x|^2, [wg][A_BYTES / 4]
+            const float *mr = cst, *rnorm = cst + D, *gscale = cst + D + L;
+            const float mean_norm = cst[D + 2 * L], r_fro = cst[D + 2 * L + 1], r_colmax = cst[D + 2 * L + 2];
+            const int lx = lane & 7;
+            bool ok = true;
+#pragma unroll 1
+            for (int i = 0; i < n_local; ++i, ++n_it) {
+                const int t0 = (tile0 + i) * PF_TILE + w * PF_HALF;            // first token of the half tile
+                const int tw = t0 + (warp & 3) * 32;                           // first token of the warp
+                const int tkn = t0 + row;
+                const int q = 2 * n_it + w, xslot = q % P::NX;
+                unsigned char* const x_s = smem + P::OFF_X + xslot * P::SLOT_BYTES;
+                int sq = -1, pos = 0;
+                if (tkn < a.n_tokens) { sq = a.tok_seq[tkn]; pos = a.tok_pos[tkn]; }
+                // |x| of the token; each warpgroup sums its half of the row
+                ok = ok && mbar_wait(bar(B_X + xslot), (q / P::NX) & 1, abort_flag);
+                {
+                    float x2 = 0.f;
+#pragma unroll
+                    for (int cc = 0; cc < D / 16; ++cc) {
+                        const int c = hf * (D / 16) + cc;
+                        const uint4 v = *reinterpret_cast<const uint4*>(x_s + (c >> 3) * (PF_HALF * 128) + row * 128 + (((c & 7) ^ (row & 7)) * 16));
+                        const uint32_t qv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float lo = __uint_as_float(qv[j] << 16), hi = __uint_as_float(qv[j] & 0xffff0000u);
+                            x2 = fmaf(lo, lo, fmaf(hi, hi, x2));
+                        }
+                    }
+                    x2_s[wg * (P::A_BYTES / 4) + row] = x2;
+                }
+                // destination of the token
+                int page = -1, slot = 0;
+                const bool named = sq >= 0 && sq < a.n_seq && pos >= 0 && pos / NOVAKV_PAGE_TOKENS < a.max_pages_per_seq;
+                if (named) {
+                    page = a.page_table[(size_t)sq * a.max_pages_per_seq + pos / NOVAKV_PAGE_TOKENS];
+                    slot = pos % NOVAKV_PAGE_TOKENS;
+                } else if (sq != -1) {                                         // (-1: unused entry of the token list, skipped)
+                    atomicOr(a.dev_status, NOVAKV_DEV_BAD_TOKEN);
+                }
+                nbar_sync(5 + w, PF_TILE);                                     // the row has been read by everyone; partial sums visible
+                float bound;                                                   // times a column norm: error of that coefficient
+                {
+                    const float x2 = x2_s[(2 * w) * (P::A_BYTES / 4) + row] + x2_s[(2 * w + 1) * (P::A_BYTES / 4) + row];
+                    bound = KAPPA * (sqrtf(x2) * 1.00001f + mean_norm);
+                }
+                ok = ok && mbar_wait(bar(B_T + w), n_it & 1, abort_flag);
+                tc_fence_after();
+                __syncwarp();
+
+                float rho = 0.f, inv_rho = 1.f;
+                if (ksc) {
+                    float ss = 0.f;
+#pragma unroll 1
+                    for (int c = 0; c < D; c += 16) {
+                        float f[16];
+                        tmem_ld16(d_t + c, f);
+                        tmem_wait_ld();
+                        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                        for (int j = 0; j < 16; j += 2) {
+                            const float v0 = f[j] - mr[c + j], v1 = f[j + 1] - mr[c + j + 1];
+                            s0 = fmaf(v0, v0, s0);
+                            s1 = fmaf(v1, v1, s1);
+                        }
+                        ss += s0 + s1;
+                    }
+                    // relative error of the norm: that of the coefficients, their rounding, and the binary32 sum
+                    const float nrm = sqrtf(ss), rel = bound * r_fro / nrm + 4.0e-6f;
+                    const float f = sqrtf(ss / (float)D);
+                    rho = bf16_round(f);
+                    const bool sure = bf16_round(f * (1.f - rel)) == rho && bf16_round(f * (1.f + rel)) == rho && rho > 0.f && rho < CUDART_INF_F;
+                    unsigned todo = __ballot_sync(0xffffffffu, sq >= 0 && !sure);
+                    while (todo) {
+                        const int src = __ffs(todo) - 1;
+                        todo &= todo - 1;
+                        float r[D / 32];
+                        exact_row<D>(x_new + ((size_t)(tw + src) * a.n_kv_heads + kvh) * D, mean, R_plain, r);
+                        double s2 = 0.0;
+#pragma unroll
+                        for (int j = 0; j < D / 32; ++j) s2 = fma((double)r[j], (double)r[j], s2);
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+                        float e = bf16_round((float)sqrt(s2 / (double)D));
+                        if (!(e > 0.f) || !isfinite(e)) e = 1.f;
+                        if (lane == src) rho = e;
+                    }
+                    if (!(rho > 0.f) || !isfinite(rho)) rho = 1.f;             // (lanes without a token)
+                    inv_rho = __fdividef(1.f, rho);
+                    bound *= inv_rho * 1.00001f;
+                }
+                // coefficients of this warpgroup's groups lb .. lb + ngh - 1 -> shared memory, [group][token][4]
+                const int lb = g0 + hf * ngh;
+                float4* const c_s = reinterpret_cast<float4*>(x_s) + (hf * (P::GU / 2)) * PF_HALF + row;
+#pragma unroll 1
+                for (int g = 0; g < ngh; g += 4) {
+                    float f[16];
+                    tmem_ld16(d_t + 4 * (lb + g) - c0, f);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 m = *reinterpret_cast<const float4*>(mr + 4 * (lb + g + j));
+                        float4 r = make_float4(f[4 * j] - m.x, f[4 * j + 1] - m.y, f[4 * j + 2] - m.z, f[4 * j + 3] - m.w);
+                        if (ksc) { r.x *= inv_rho; r.y *= inv_rho; r.z *= inv_rho; r.w *= inv_rho; }
+                        c_s[(g + j) * PF_HALF] = r;
+                    }
+                }
+                // destination, second part (the page id has arrived by now)
+                if (named) {
+                    if (page < 0 || page >= a.n_pages) {
+                        atomicOr(a.dev_status, NOVAKV_DEV_BAD_PAGE);
+                        page = -1;
+                    } else if (sh == 0 && g0 == 0 && hf == 0) {
+                        atomicMax(&a.seq_lens[sq], pos + 1);
+                    }
+                }
+                const bool valid = page >= 0;
+                const int page0 = __shfl_sync(0xffffffffu, page, lane & 16), slot0 = __shfl_sync(0xffffffffu, slot, lane & 16);
+                const bool aligned = __all_sync(0xffffffffu, valid && page == page0 && (slot & 15) == (lane & 15) && (slot ^ slot0) < 16);
+                uint8_t* const chunk = pages + ((size_t)(valid ? page : 0) * a.n_kv_heads + kvh) * (NOVAKV_PAGE_TOKENS * L);
+                if (ksc && valid && g0 == 0 && hf == 0)
+                    a.k_scales[((size_t)page * a.n_kv_heads + kvh) * NOVAKV_PAGE_TOKENS + slot] = __float2bfloat16_rn(rho);
+                if (vsq) {
+                    float mn = CUDART_INF_F, mx = -CUDART_INF_F;
+#pragma unroll 1
+                    for (int c = 0; c < D; c += 16) {
+                        float f[16];
+                        tmem_ld16(d_t + c, f);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const float v = f[j] - mr[c + j];
+                            mn = fminf(mn, v);
+                            mx = fmaxf(mx, v);
+                        }
+                    }
+                    const float err = bound * r_colmax + 1.2e-7f * fmaxf(fabsf(mn), fabsf(mx));
+                    float zero = bf16_round(mn);
+                    float scale = bf16_round(__fdiv_rn(__fsub_rn(mx, zero), 3.0f));
+                    bool sure = bf16_round(mn - err) == zero && bf16_round(mn + err) == zero &&
+                                bf16_round(((mx - err) - zero) * 0.33333328f) == scale && bf16_round(((mx + err) - zero) * 0.33333339f) == scale &&
+                                scale > 0.f && scale < CUDART_INF_F;
+                    const float inv_scale = __fdividef(1.f, scale), uerr = err * inv_scale + 2.0e-6f;
+                    uint32_t word[L / 8];                                      // this warpgroup's half of the levels
+#pragma unroll
+                    for (int qw = 0; qw < L / 8; ++qw) {
+                        const int c = hf * (D / 2) + qw * 16;
+                        float f[16];
+                        tmem_ld16(d_t + c, f);
+                        tmem_wait_ld();
+                        uint32_t wd = 0;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            // level = clamp(rint(t), 0, 3); t near a boundary 0.5, 1.5, 2.5 is inside the bound
+                            const float t = (f[j] - mr[c + j] - zero) * inv_scale;
+                            const float lv = fminf(fmaxf(rintf(t), 0.f), 3.f);
+                            sure &= fminf(fminf(fabsf(t - 0.5f), fabsf(t - 1.5f)), fabsf(t - 2.5f)) > uerr;
+                            wd |= (uint32_t)lv << (2 * j);
+                        }
+                        word[qw] = wd;
+                    }
+                    tc_fence_before();
+                    nbar_sync(5 + w, PF_TILE);                                 // the accumulators are read out, the row slot is free
+                    if (lane == 0) {
+                        mbar_arrive(bar(B_XFREE + xslot));
+                        if (hf == 0) mbar_arrive(bar(B_TFREE + w));
+                    }
+                    unsigned todo = __ballot_sync(0xffffffffu, valid && !sure);
+                    while (todo) {
+                        const int src = __ffs(todo) - 1;
+                        todo &= todo - 1;
+                        float r[D / 32];
+                        exact_row<D>(x_new + ((size_t)(tw + src) * a.n_kv_heads + kvh) * D, mean, R_plain, r);
+                        float rmn = r[0], rmx = r[0];
+#pragma unroll
+                        for (int j = 1; j < D / 32; ++j) { rmn = fminf(rmn, r[j]); rmx = fmaxf(rmx, r[j]); }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            rmn = fminf(rmn, __shfl_xor_sync(0xffffffffu, rmn, o));
+                            rmx = fmaxf(rmx, __shfl_xor_sync(0xffffffffu, rmx, o));
+                        }
+                        const float ez = bf16_round(rmn);
+                        float es = bf16_round(__fdiv_rn(__fsub_rn(rmx, ez), 3.0f));
+                        if (!(es > 0.f) || !isfinite(es)) es = 1.f;
+                        uint32_t mine = 0;                                     // this lane's D / 32 levels, 2 bits each
+#pragma unroll
+                        for (int j = 0; j < D / 32; ++j) {
+                            float t = rintf(__fdiv_rn(__fsub_rn(r[j], ez), es));
+                            if (!(t > 0.f)) t = 0.f;
+                            mine |= (uint32_t)fminf(t, 3.f) << (2 * j);
+                        }
+#pragma unroll
+                        for (int qw = 0; qw < L / 8; ++qw) {                   // 16 levels per word: 512 / D lanes each
+                            uint32_t wd = 0;
+#pragma unroll
+                            for (int j = 0; j < 512 / D; ++j)
+                                wd |= __shfl_sync(0xffffffffu, mine, hf * 16 + qw * (512 / D) + j) << (j * (D / 16));
+                            if (lane == src) word[qw] = wd;
+                        }
+                        if (lane == src) { zero = ez; scale = es; }
+                    }
+#pragma unroll
+                    for (int qw = 0; qw < L / 8; ++qw) store_value_word<L>(chunk, slot, hf * (L / 2) + 4 * qw, word[qw], aligned, valid, lane);
+                    if (valid && hf == 0)
+                        reinterpret_cast<__nv_bfloat162*>(a.v_meta)[((size_t)page * a.n_kv_heads + kvh) * NOVAKV_PAGE_TOKENS + slot] =
+                            __floats2bfloat162_rn(scale, zero);
+                    continue;
+                }
+                tc_fence_before();
+                nbar_sync(5 + w, PF_TILE);                                     // the transform's accumulators are read out
+
+                // ---- search of groups lb .. lb + ngh - 1
+                // the coefficients of group g, and its search operand into shared memory
+                auto publish = [&](int g, float4& r, float& qq) {
+                    r = c_s[g * PF_HALF];
+                    const float sc = gscale[lb + g];
+                    const float s0 = r.x * sc, s1 = r.y * sc, s2 = r.z * sc, s3 = r.w * sc;
+                    qq = fmaf(s0, s0, fmaf(s1, s1, fmaf(s2, s2, s3 * s3)));
+                    const uint32_t h01 = pack_half2(s0, s1), h23 = pack_half2(s2, s3);
+                    const float2 f01 = unpack_half2(h01), f23 = unpack_half2(h23);
+                    const uint32_t l01 = pack_half2(s0 - f01.x, s1 - f01.y), l23 = pack_half2(s2 - f23.x, s3 - f23.y);
+                    const float qh = 0.5f * qq, qhh = __half2float(__float2half_rn(qh));
+                    const uint32_t qp = pack_half2(qhh, qh - qhh);
+                    const uint32_t dst = a_s + row * 16;
+                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(h01), "r"(h23), "r"(h01), "r"(h23) : "memory");
+                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst + PF_HALF * 16), "r"(l01), "r"(l23), "r"(0x3c003c00u), "r"(qp) : "memory");
+                    fence_proxy_async();
+                };
+                // The warp is done with the accumulators (and has written its operand rows); when the four warps of the
+                // warpgroup are, its first warp issues the distances of chunk c of the group in ring stage st.
+                const int use0 = n_use + hf;
+                auto release_and_issue = [&](int c, int g) {
+                    tc_fence_before();
+                    if ((warp & 3) != 0) {
+                        nbar_arrive(1 + wg, PF_HALF);
+                    } else {
+                        const int use = use0 + 2 * g, st = use % PF_STAGES;
+                        if (c == 0) ok = ok && mbar_wait(bar(B_RING + st), (use / PF_STAGES) & 1, abort_flag);
+                        nbar_sync(1 + wg, PF_HALF);
+                        tc_fence_after();
+                        if (elect_one()) {
+                            umma_f16(d_s, umma_desc(a_s, PF_HALF * 16, 128, 0),
+                                     umma_desc(sb + P::OFF_RING + st * PF_STAGE_BYTES + c * 2048, 4096, 128, 0), umma_idesc(false, false, 128, 128), false);
+                            umma_commit(bar(B_S + wg));
+                            if (c == 1) umma_commit(bar(B_RINGFREE + st));
+                        }
+                        __syncwarp();
+                    }
+                };
+                float4 r, rn = make_float4(0.f, 0.f, 0.f, 0.f);                // coefficients of this group and the next
+                float q2, q2n = 0.f;                                           // |r|^2 in the group's scale
+                publish(0, r, q2);
+                release_and_issue(0, 0);
+                uint32_t codes = 0, pend = 0;
+#pragma unroll 1
+                for (int g = 0; g < ngh; ++g) {
+                    const int l = lb + g, use = use0 + 2 * g, st = use % PF_STAGES;
+                    uint32_t rmin[16];                                         // minima of 32 rows of 8 codewords, two per register
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        if ((c & 1) == 0) {
+                            ok = ok && mbar_wait(bar(B_S + wg), n_s & 1, abort_flag);
+                            ++n_s;
+                            tc_fence_after();
+                            __syncwarp();
+                        }
+                        uint32_t v[32];
+                        tmem_ld64_h2(d_s + lane_base + (c & 1) * 64, v);
+                        tmem_wait_ld();
+                        if (c == 1) {
+                            release_and_issue(1, g);
+                        } else if (c == 3) {
+                            if (g + 1 < ngh) {
+                                publish(g + 1, rn, q2n);
+                                release_and_issue(0, g + 1);
+                                if (g + 2 == ngh) {
+                                    __syncwarp();
+                                    if (lane == 0) mbar_arrive(bar(B_XFREE + xslot));      // the coefficients are read out
+                                }
+                            } else {
+                                tc_fence_before();
+                                __syncwarp();
+                                if (lane == 0 && hf == 0) mbar_arrive(bar(B_TFREE + w));
+                            }
+                        }
+                        // (distances are not negative, or tiny: their binary16 patterns compare like integers.  A negative
+                        // one sorts below every positive one, and every negative row minimum passes the test below.)
+#pragma unroll
+                        for (int qd = 0; qd < 4; ++qd)
+                            rmin[4 * c + qd] = __vimin3_s16x2(__vimin3_s16x2(v[8 * qd], v[8 * qd + 1], v[8 * qd + 2]),
+                                                              __vimin3_s16x2(v[8 * qd + 3], v[8 * qd + 4], v[8 * qd + 5]),
+                                                              __vmins2(v[8 * qd + 6], v[8 * qd + 7]));
+                    }
+                    float mf;
+                    {
+                        uint32_t m = __vimin3_s16x2(__vimin3_s16x2(rmin[0], rmin[1], rmin[2]), __vimin3_s16x2(rmin[3], rmin[4], rmin[5]),
+                                                    __vimin3_s16x2(rmin[6], rmin[7], rmin[8]));
+                        m = __vimin3_s16x2(m, __vimin3_s16x2(rmin[9], rmin[10], rmin[11]), __vimin3_s16x2(rmin[12], rmin[13], rmin[14]));
+                        const float2 f = unpack_half2(__vmins2(m, rmin[15]));
+                        mf = fminf(f.x, f.y);
+                        if (!(f.x == f.x) || !(f.y == f.y)) mf = CUDART_INF_F;
+                    }
+                    // A row can hold the nearest codeword only if its binary16 minimum is at most t: the rounding of two
+                    // binary16 numbers (2^-11 each; below their normal range 2^-25, also of the operands), the error of the
+                    // product (EPS_S) for both, and what the error of the coefficient moves the difference of two distances by.
+                    const float rlen2 = fmaf(r.x, r.x, fmaf(r.y, r.y, fmaf(r.z, r.z, r.w * r.w)));
+                    const float delta = fmaf(bound, rnorm[l], (ksc ? 3.0e-7f : 6.0e-8f) * sqrt_approx(rlen2));
+                    const float dl = delta * gscale[l], sq2 = sqrt_approx(2.f * fmaxf(mf, 0.f)), rl = sqrt_approx(q2);
+                    const float s2 = 2.f * rl + 1.1f * sq2;
+                    float t = fmaf(2.1f * EPS_S, s2 * s2, fmaf(fmaxf(mf, 0.f), 1.0025f, 2.5f * dl * (sq2 + dl) + 4.0e-7f));
+                    t *= 1.0005f;
+                    const uint32_t t1 = pack_half2(t, t);
+                    uint32_t bits = 0;
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const uint32_t le = __hle2_mask(*reinterpret_cast<const __half2*>(&rmin[k]), *reinterpret_cast<const __half2*>(&t1));
+                        bits |= le & (0x00010001u << k);
+                    }
+                    bool exact = !(mf < 60000.f) || bits == 0u;
+                    // Direct binary32 distances of the rows that are left, two codewords per operation.  A lane reads the 8
+                    // chunks of its row in the order j ^ (lane % 8), so that the 8 lanes of a quarter warp read 8 different
+                    // 16-byte columns: odd lanes meet the chunk of components 2, 3 first.  The low 3 bits of a distance are
+                    // replaced by the codeword's number in the row.
+                    uint32_t best = 0x7f800000u, second = 0x7f800000u;
+                    int brow = 0;
+                    ok = ok && mbar_wait(bar(B_RING + st), (use / PF_STAGES) & 1, abort_flag);
+                    __syncwarp();
+                    const uint32_t cb = sb + P::OFF_RING + st * PF_STAGE_BYTES + 8192;
+                    {
+                        const bool odd = lane & 1;
+                        const uint64_t ra0 = dup2(odd ? r.z : r.x), ra1 = dup2(odd ? r.w : r.y);
+                        const uint64_t rb0 = dup2(odd ? r.x : r.z), rb1 = dup2(odd ? r.y : r.w);
+                        do {
+                            const int k = bits ? __ffs(bits) - 1 : 0;
+                            const bool take = bits != 0u;
+                            const int rowi = ((k & 15) << 1) | (k >> 4);
+                            const uint32_t base = cb + rowi * 128;
+                            uint32_t key[8];
+#pragma unroll
+                            for (int p = 0; p < 4; ++p) {
+                                uint64_t a0, a1, b0, b1;
+                                asm volatile("ld.shared.v2.u64 {%0,%1}, [%2];" : "=l"(a0), "=l"(a1) : "r"(base + (((2 * p) ^ lx) * 16)));
+                                asm volatile("ld.shared.v2.u64 {%0,%1}, [%2];" : "=l"(b0), "=l"(b1) : "r"(base + (((2 * p + 1) ^ lx) * 16)));
+                                a0 = f2_sub(ra0, a0); a1 = f2_sub(ra1, a1); b0 = f2_sub(rb0, b0); b1 = f2_sub(rb1, b1);
+                                const uint64_t d = f2_fma(b1, b1, f2_fma(b0, b0, f2_fma(a1, a1, f2_mul(a0, a0))));
+                                key[2 * p] = ((uint32_t)d & ~7u) | (2 * p);
+                                key[2 * p + 1] = ((uint32_t)(d >> 32) & ~7u) | (2 * p + 1);
+                            }
+                            // two smallest of the 8: pairs, then merges
+                            uint32_t lo[4], hi[4];
+#pragma unroll
+                            for (int p = 0; p < 4; ++p) { lo[p] = min(key[2 * p], key[2 * p + 1]); hi[p] = max(key[2 * p], key[2 * p + 1]); }
+#pragma unroll
+                            for (int p = 0; p < 4; p += 2) {
+                                hi[p] = __vimin3_u32(max(lo[p], lo[p + 1]), hi[p], hi[p + 1]);
+                                lo[p] = min(lo[p], lo[p + 1]);
+                            }
+                            hi[0] = __vimin3_u32(max(lo[0], lo[2]), hi[0], hi[2]);
+                            lo[0] = min(lo[0], lo[2]);
+                            if (take) {
+                                second = __vimin3_u32(max(best, lo[0]), second, hi[0]);
+                                if (lo[0] < best) { best = lo[0]; brow = rowi; }
+                            }
+                            bits &= bits - 1;
+                        } while (__any_sync(0xffffffffu, bits != 0u));
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_RINGFREE + st));
+                    const int bi = brow * 8 + (int)((best & 7u) ^ (lx & 6));
+                    // where the two nearest codewords are closer than the errors can resolve, the search is repeated in binary64
+                    exact |= needs_exact_search(__uint_as_float(best & ~7u), __uint_as_float(second | 7u), delta, KEY_REL);
+                    codes = (codes >> 8) | ((uint32_t)bi << 24);
+                    pend = (pend >> 1) | (exact && valid ? 8u : 0u);
+                    if ((l & 3) == 3) {
+                        if (side == 0) { if (valid) store_key_word<L>(chunk, slot, l - 3, codes); }
+                        else store_value_word<L>(chunk, slot, l - 3, codes, aligned, valid, lane);
+                        // binary64 searches of the four groups: to the helper's queue, or here when it is full
+                        unsigned todo;
+                        while ((todo = __ballot_sync(0xffffffffu, pend != 0u)) != 0u) {
+                            const int h = warp & (PF_HELPERS - 1), n = __popc(todo);
+                            int base = -1;
+                            if (lane == 0) {
+                                if (atomicAdd(&s_count[h], n) + n <= PF_QUEUE) base = atomicAdd(&s_head[h], n);
+                                else atomicSub(&s_count[h], n);
+                            }
+                            base = __shfl_sync(0xffffffffu, base, 0);
+                            const int lq = l - 3 + (pend ? __ffs(pend) - 1 : 0);
+                            if (base >= 0) {
+                                if (pend) {
+                                    volatile uint32_t* e = reinterpret_cast<volatile uint32_t*>(smem + P::OFF_QUEUE) +
+                                                           (h * PF_QUEUE + (base + __popc(todo & ((1u << lane) - 1))) % PF_QUEUE) * 4;
+                                    e[1] = (uint32_t)tkn; e[2] = (uint32_t)page; e[3] = __float_as_uint(rho);
+                                    __threadfence_block();
+                                    e[0] = 0x80000000u | ((uint32_t)slot << 6) | (uint32_t)lq;
+                                }
+                            } else {
+                                while (todo) {
+                                    const int src = __ffs(todo) - 1;
+                                    todo &= todo - 1;
+                                    const int ls = __shfl_sync(0xffffffffu, lq, src);
+                                    const int res = exact_search_token<D>(x_new + ((size_t)(tw + src) * a.n_kv_heads + kvh) * D, mean, R_plain, ls,
+                                                                          cb_g + ls * NOVAKV_C, __shfl_sync(0xffffffffu, rho, src));
+                                    if (lane == src) chunk[side == 0 ? novakv_k_offset<L>(slot, ls) : novakv_v_offset<L>(slot, ls)] = (uint8_t)res;
+                                }
+                            }
+                            pend &= pend - 1;
+                            __syncwarp();
+                        }
+                    }
+                    r = rn;
+                    q2 = q2n;
+                }
+                n_use += 2 * ngh;
+            }
+            __syncwarp();
+            if (lane == 0) { __threadfence_block(); atomicAdd(s_done, 1); }
+        }
+        ++n_seg;
+        tc_fence_before();
+        __syncthreads();                               // constants, matrix slices and TMEM are free for the next segment
+        tc_fence_after();
+    }
+    if (warp == 0) tmem_dealloc<512>(tmem);
+    if (threadIdx.x == 0 && misc[1] != 0) atomicOr(a.dev_status, NOVAKV_DEV_WAIT_TIMEOUT);
+}
+
+template <int D, int FMT>
+novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStream_t stream) {
+    using P = PF<D, FMT>;
+    constexpr int L = P::L;
+    PrefillArgs a = args;
+    auto kern = novakv_prefill_kernel<D, FMT>;
+    if (!(ctx->prefill_opt_in & (1u << FMT))) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::BYTES) != cudaSuccess) return NOVAKV_ECUDA;
+        ctx->prefill_opt_in |= 1u << FMT;
+    }
+    const int n_tiles = (a.n_tokens + PF_TILE - 1) / PF_TILE, hkv = ctx->cfg.n_kv_heads;
+    // Units of 16 groups; of 8 (each repeats the transform's fixed costs) where that makes the longest run of units
+    // cheaper: when there are too few units to give every SM one, or a few whole ones.
+    double best = 1e30;
+    int grid = 1;
+    for (int gs = L / P::GU; gs <= L / 8; gs *= 2) {
+        const double ck = PF_US_UNIT + PF_US_GROUP * (L / gs), cv = FMT == 2 ? PF_US_INT2 : ck;
+        const int uk = hkv * gs * n_tiles, uv = FMT == 2 ? hkv * n_tiles : uk;
+        const int g = uk + uv < ctx->n_sm ? uk + uv : ctx->n_sm;
+        double longest = (uk * ck + uv * cv) / g;
+        if (longest < ck) longest = ck;
+        const double n_k = ceil(longest / ck - 1e-6);                          // units are whole
+        if (n_k * ck < best) {
+            best = n_k * ck;
+            grid = g;
+            a.gs = gs;
+            a.cost_k = (int)(ck * 64.0);
+            a.cost_v = (int)(cv * 64.0);
+        }
+    }
+    novakv_prof_scope ps(ctx, 1, stream);
+    kern<<<grid, PF_THREADS, P::BYTES, stream>>>(a);
+    ps.end();
+    ctx->launches++;
+    return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
+}
+
+}  // namespace
+
+novakv_status novakv_launch_prefill(novakv_ctx* ctx, const novakv_layer& ly, const __nv_bfloat16* k_new, const __nv_bfloat16* v_new,
+    const int32_t* tok_seq, const int32_t* tok_pos, int n_tokens, uint8_t* k_pages, uint8_t* v_pages, int n_pages,
+    const int32_t* page_table, int max_pages_per_seq, int n_seq, int32_t* seq_lens, cudaStream_t stream, __nv_bfloat16* k_scales,
+    __nv_bfloat16* v_meta) {
+    const PrefillArgs a = {k_new, v_new, tok_seq, tok_pos, n_tokens, ly.pf_r, ly.pf_cb, ly.pf_const, ly.rk_d, ly.rv_d, ly.k_mean_d,
+                           ly.v_mean_d, ly.cb_k, ly.cb_v, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
+                           n_seq, seq_lens, ctx->cfg.n_kv_heads, 1, 1, 1, ctx->dev_status};
+    if (ctx->cfg.head_dim == 128)
+        return v_meta ? launch_prefill_t<128, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<128, 1>(ctx, a, stream) : launch_prefill_t<128, 0>(ctx, a, stream));
+    return v_meta ? launch_prefill_t<64, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<64, 1>(ctx, a, stream) : launch_prefill_t<64, 0>(ctx, a, stream));
+}
+
+// ------------------------------------------------------------------------------------------------
+// calibration images of this kernel (host)
+// ------------------------------------------------------------------------------------------------
+// One (KV head, side): the three bfloat16 slices of R as K-major operands (row = output column, 64-element panels of
+// 128-byte rows, 16-byte chunks swizzled by the row), the codebook images, and the constants of error bounds and scaling.
+void novakv_build_prefill_image(int d, const float* R /* [d][d] */, const float* mean /* [d] or null */, const float* cb /* [L][256][4] */,
+                                uint8_t* r_img, uint8_t* cb_img, float* consts) {
+    const int L = d / NOVAKV_G;
+    for (int k = 0; k < d; ++k)
+        for (int c = 0; c < d; ++c) {
+            float rem = R[(size_t)k * d + c];
+            for (int s = 0; s < 3; ++s) {
+                const __nv_bfloat16 h = __float2bfloat16_rn(rem);
+                rem -= __bfloat162float(h);
+                const size_t off = (size_t)s * d * d * 2 + (size_t)(k >> 6) * d * 128 + (size_t)c * 128 + ((((k & 63) >> 3) ^ (c & 7)) * 16) + (k & 7) * 2;
+                *reinterpret_cast<__nv_bfloat16*>(r_img + off) = h;
+            }
+        }
+    double mn2 = 0.0, fro2 = 0.0, colmax = 0.0;
+    for (int k = 0; k < d; ++k) mn2 += mean ? (double)mean[k] * mean[k] : 0.0;
+    for (int l = 0; l < L; ++l) {
+        double g2 = 0.0;
+        for (int c = 4 * l; c < 4 * l + 4; ++c) {
+            double m = 0.0, c2 = 0.0;
+            for (int k = 0; k < d; ++k) {
+                const double v = R[(size_t)k * d + c];
+                m += mean ? (double)mean[k] * v : 0.0;
+                c2 += v * v;
+            }
+            consts[c] = (float)m;
+            g2 += c2;
+            colmax = c2 > colmax ? c2 : colmax;
+        }
+        fro2 += g2;
+        consts[d + l] = (float)(sqrt(g2) * 1.000001);
+        // scale of the group: the longest codeword gets a length in [8, 16)
+        double cmax2 = 0.0;
+        for (int c = 0; c < NOVAKV_C; ++c) {
+            double n2 = 0.0;
+            for (int i = 0; i < 4; ++i) { const double v = cb[((size_t)l * NOVAKV_C + c) * 4 + i]; n2 += v * v; }
+            cmax2 = n2 > cmax2 ? n2 : cmax2;
+        }
+        int e = 0;
+        if (cmax2 > 0.0 && cmax2 < 1e300) { frexp(sqrt(cmax2), &e); e = 4 - e; }
+        e = e > 100 ? 100 : (e < -100 ? -100 : e);
+        consts[d + L + l] = (float)ldexp(1.0, e);
+        uint8_t* g = cb_img + (size_t)l * NOVAKV_PF_GROUP_BYTES;
+        for (int n = 0; n < NOVAKV_C; ++n) {
+            // column n of the product: packed minima over even / odd columns of 16 make the rows of 8 codewords
+            const int reg = n >> 4, half = n & 1, code = (reg * 2 + half) * 8 + ((n & 15) >> 1);
+            double pd = 0.0;
+            __half v[16];
+            for (int i = 0; i < 4; ++i) {
+                const float c = (float)ldexp((double)cb[((size_t)l * NOVAKV_C + code) * 4 + i], e);
+                pd += 0.5 * (double)c * (double)c;
+                const __half h = __float2half_rn(c);
+                v[i] = __float2half_rn(-__half2float(h));
+                v[8 + i] = v[i];
+                v[4 + i] = __float2half_rn(-(c - __half2float(h)));
+            }
+            v[12] = __float2half_rn((float)pd);
+            v[13] = __float2half_rn((float)(pd - (double)__half2float(v[12])));
+            v[14] = v[15] = __float2half_rn(1.f);
+            for (int kc = 0; kc < 2; ++kc) memcpy(g + kc * 4096 + (n >> 3) * 128 + (n & 7) * 16, v + 8 * kc, 16);
+        }
+        float* img = reinterpret_cast<float*>(g + 8192);
+        for (int code = 0; code < NOVAKV_C; ++code)
+            for (int i = 0; i < 4; ++i) img[codeword_offset(code, i)] = cb[((size_t)l * NOVAKV_C + code) * 4 + i];
+    }
+    consts[d + 2 * L] = (float)(sqrt(mn2) * 1.000001);
+    consts[d + 2 * L + 1] = (float)(sqrt(fro2) * 1.000001);
+    consts[d + 2 * L + 2] = (float)(sqrt(colmax) * 1.000001);
+    consts[d + 2 * L + 3] = 0.f;
+}

@@ -1,0 +1,84 @@
+"""Prompt encoder (more than 256 tokens per call) at the edges of its tiling: 256-token units of two 128-token halves,
+runs of units cut across (KV head, side, part of the groups) boundaries, and the exact re-search of close decisions.
+Indices, scales and (scale, zero) pairs must equal the oracle's; only float64 near-ties may differ (gpu_common)."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from gpu_common import Case, check_indices
+from paper_2608_04074_b200 import synth, workloads
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def _dev(a, dtype=None):
+    t = torch.from_numpy(np.ascontiguousarray(a))
+    return (t if dtype is None else t.to(dtype)).cuda()
+
+
+def _make(name, key_scale):
+    wl = (workloads.qwen3_8b(batch=1, seq_len=1024, calib_tokens=2048, lloyd_iters=4) if name == "qwen"
+          else workloads.gpt_oss_20b(batch=1, seq_len=1024, calib_tokens=2048, lloyd_iters=4))
+    return Case(dataclasses.replace(wl, calib_queries_for_values=256), key_scale=key_scale)
+
+
+@pytest.fixture(scope="module")
+def cases():
+    return {(n, s): _make(n, s) for n in ("qwen", "gptoss") for s in (False, True)}
+
+
+def _run(case, fmt, n, start, permute, holes, scale=1.0):
+    from paper_2608_04074_b200.runtime import PagedCache
+    k, v, _ = case.draw(4000 + n, n, 1)
+    k, v = (synth.to_bf16_representable(x * scale) for x in (k, v))
+    cache = PagedCache(case.ctx, np.array([0, 0], np.int32), capacity_tokens=np.array([start + n, 64], np.int32), seed=7,
+                       key_scale=fmt == "scaled", int2_values=fmt == "deployed")
+    pos = start + np.arange(n, dtype=np.int32)
+    seq = np.zeros(n, np.int32)
+    used = np.ones(n, bool)
+    if holes:
+        used[::7] = False
+        seq[~used] = -1
+    order = synth.rng(3).permutation(n) if permute else np.arange(n)
+    cache.append(0, _dev(k[order], torch.bfloat16), _dev(v[order], torch.bfloat16), _dev(seq[order]), _dev(pos[order]))
+    assert case.ctx.novakv_last_device_status() == 0
+    assert int(cache.seq_lens[0]) == start + int(np.flatnonzero(used)[-1]) + 1 and int(cache.seq_lens[1]) == 0
+    gk, gv = cache.load_logical(0, start, n)
+    assert not gk[~used].any() and not gv[~used].any()
+    k64, v64 = k[used].astype(np.float64), v[used].astype(np.float64)
+    if fmt == "plain":
+        e = case.oracle.encode(k64, v64)
+    else:
+        e = case.oracle.encode_scaled(k64, v64)
+        assert np.array_equal(cache.load_scales(0, start, n)[used], e["kscale"])
+    check_indices(gk[used], e, "k")
+    if fmt == "deployed":
+        from paper_2608_04074_b200 import cache_format
+        codes, meta = case.oracle.encode_values_int2(v64)
+        assert np.array_equal(gv[used], cache_format.pack_int2(codes))
+        assert np.array_equal(cache.load_value_meta(0, start, n)[used], meta)
+    else:
+        check_indices(gv[used], e, "v")
+
+
+@pytest.mark.parametrize("n,start,permute,holes", [
+    (257, 0, False, False),      # one unit and one token of a second; whole 16-token value blocks
+    (384, 64, False, False),     # the last half tile of a unit is empty
+    (511, 5, False, False),      # positions off the 16-token blocks
+    (512, 0, True, False),       # tokens of a warp scattered over pages
+    (513, 16, False, True),      # unused entries
+    (2049, 48, False, False),    # runs of units that cross head, side and group boundaries
+])
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "plain"), ("qwen", "scaled"), ("gptoss", "scaled"),
+                                      ("qwen", "deployed"), ("gptoss", "deployed")])
+def test_prefill_edges(cases, name, fmt, n, start, permute, holes):
+    _run(cases[name, fmt != "plain"], fmt, n, start, permute, holes)
+
+
+@pytest.mark.parametrize("name,scale", [("qwen", 0.0), ("qwen", 1e-3), ("qwen", 64.0), ("gptoss", 1e-3), ("gptoss", 64.0)])
+def test_prefill_far_from_the_codebook(cases, name, scale):
+    """Inputs a thousand times smaller and 64 times larger than the calibration's (and all zero): the binary16 ranking
+    is then dominated by rounding, or out of its range, and every decision rests on the exact re-search."""
+    _run(cases[name, False], "plain", 300, 0, False, False, scale)
