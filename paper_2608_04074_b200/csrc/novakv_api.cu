@@ -83,7 +83,7 @@ extern "C" novakv_status novakv_create(novakv_ctx** out, const novakv_config* cf
 }
 
 static void free_layer(novakv_layer& ly) {
-    cudaFree(ly.rk_d); cudaFree(ly.rv_d); cudaFree(ly.k_mean_d); cudaFree(ly.v_mean_d);
+    cudaFree(ly.rk_d); cudaFree(ly.rv_d); cudaFree(ly.rk_rows); cudaFree(ly.rv_rows); cudaFree(ly.k_mean_d); cudaFree(ly.v_mean_d);
     cudaFree(ly.pf_r); cudaFree(ly.pf_cb); cudaFree(ly.pf_const); cudaFree(ly.k_mean);
     cudaFree(ly.cb_k); cudaFree(ly.cb_v); cudaFree(ly.rk_inv_t); cudaFree(ly.rv_t);
     cudaFree(ly.v_mean); cudaFree(ly.cb_k_lut); cudaFree(ly.cb_v_u8); cudaFree(ly.v_scale); cudaFree(ly.v_off);
@@ -151,8 +151,15 @@ extern "C" novakv_status novakv_load_calibration(novakv_ctx* ctx, int layer, con
             }
 
     std::vector<double> rk_d(n_mat), rv_d(n_mat), km_d(n_vec, 0.0), vm_d(n_vec, 0.0);
+    std::vector<float> rk_rows(h->rk, h->rk + n_mat), rv_rows(h->rv, h->rv + n_mat);
     std::vector<float> vm_f(n_vec, 0.f), km_f(n_vec, 0.f);
-    for (size_t i = 0; i < n_mat; ++i) { rk_d[i] = (double)h->rk[i]; rv_d[i] = (double)h->rv[i]; }
+    for (int hh = 0; hh < H; ++hh)
+        for (int k = 0; k < d; ++k)
+            for (int c = 0; c < d; ++c) {
+                const size_t src = ((size_t)hh * d + k) * d + c, dst = (((size_t)hh * L + c / g) * d + k) * g + c % g;
+                rk_d[dst] = (double)h->rk[src];
+                rv_d[dst] = (double)h->rv[src];
+            }
     // images of the prompt encoder, keys then values
     const size_t pf_r_b = (size_t)3 * d * d * 2, pf_cb_b = (size_t)L * NOVAKV_PF_GROUP_BYTES, pf_n = NOVAKV_PF_CONSTS(d);
     std::vector<uint8_t> pf_r(2 * H * pf_r_b), pf_cb(2 * H * pf_cb_b);
@@ -203,7 +210,7 @@ extern "C" novakv_status novakv_load_calibration(novakv_ctx* ctx, int layer, con
     for (int hh = 0; hh < H; ++hh)       // transposed copy: rv_t[c][r] = rv[r][c], so that o = o' rv^T reads rows
         for (int r = 0; r < d; ++r)
             for (int c = 0; c < d; ++c) rvt[((size_t)hh * d + c) * d + r] = h->rv[((size_t)hh * d + r) * d + c];
-    bool ok = upload(&ly.rk_d, rk_d) == cudaSuccess && upload(&ly.rv_d, rv_d) == cudaSuccess &&
+    bool ok = upload(&ly.rk_d, rk_d) == cudaSuccess && upload(&ly.rk_rows, rk_rows) == cudaSuccess && upload(&ly.rv_rows, rv_rows) == cudaSuccess && upload(&ly.rv_d, rv_d) == cudaSuccess &&
               upload(&ly.pf_r, pf_r) == cudaSuccess && upload(&ly.pf_cb, pf_cb) == cudaSuccess && upload(&ly.pf_const, pf_const) == cudaSuccess &&
               upload(&ly.k_mean_d, km_d) == cudaSuccess && upload(&ly.v_mean_d, vm_d) == cudaSuccess &&
               upload(&ly.cb_k, cbk) == cudaSuccess && upload(&ly.cb_v, cbv) == cudaSuccess &&

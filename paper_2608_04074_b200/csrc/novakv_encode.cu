@@ -345,8 +345,8 @@ novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_b
         float4 cw[NOVAKV_C / 32];
 #pragma unroll
         for (int k = 0; k < D / 32; ++k) {
-            ra[k] = *reinterpret_cast<const double2*>(R + (size_t)(lane + 32 * k) * D + l * 4);
-            rb[k] = *reinterpret_cast<const double2*>(R + (size_t)(lane + 32 * k) * D + l * 4 + 2);
+            ra[k] = *reinterpret_cast<const double2*>(R + ((size_t)l * D + lane + 32 * k) * 4);
+            rb[k] = *reinterpret_cast<const double2*>(R + ((size_t)l * D + lane + 32 * k) * 4 + 2);
         }
 #pragma unroll
         for (int k = 0; k < NOVAKV_C / 32; ++k) cw[k] = cb_g[lane + 32 * k];

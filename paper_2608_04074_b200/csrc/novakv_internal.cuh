@@ -20,8 +20,10 @@
 struct novakv_layer {
     bool loaded = false;
     // write path (binary64 transforms, see the encode entry of the public header)
-    double* rk_d = nullptr;       // [Hkv][d][d]
-    double* rv_d = nullptr;       // [Hkv][d][d]
+    double* rk_d = nullptr;       // [Hkv][L][d][4]: the four columns of a group side by side
+    double* rv_d = nullptr;       // [Hkv][L][d][4]
+    float* rk_rows = nullptr;     // [Hkv][d][d]
+    float* rv_rows = nullptr;     // [Hkv][d][d]
     uint8_t* pf_r = nullptr;      // [2 sides][Hkv][3 d d 2]: bfloat16 slices of rk / rv as tensor-core operands (prompt encoder)
     uint8_t* pf_cb = nullptr;     // [2][Hkv][L][NOVAKV_PF_GROUP_BYTES]: codebooks as search operand and in binary32
     float* pf_const = nullptr;    // [2][Hkv][NOVAKV_PF_CONSTS]: mean share, column norms, scales

@@ -16,13 +16,22 @@
 //               coefficient.
 //
 // Roles: four token warpgroups, two per half tile (thread = token, each takes half of the groups), whose first warp
-// issues the search MMAs; one warp loads token rows and issues the transforms; one feeds the codebook ring; two search
-// in binary64.  A chunk of 128 codewords makes a round trip token warps -> MMA -> token warps (about 300 cycles, whatever
-// its width), so chunks are as wide as TMEM allows (four warpgroups x 128 columns: the coefficients live in shared
-// memory for that), the first chunk of the next group is computed behind the selection of this one, and four token warps
-// per scheduler hide the rest.  Every wait is bounded (novakv_tcgen05.cuh): a wait that gives up sets
-// NOVAKV_DEV_WAIT_TIMEOUT, and the CTA runs through its remaining steps without waiting.  (The named barriers among token
-// warps are never skipped.)
+// issues the search MMAs; one warp looks up destinations, copies token rows (TMA) and issues the transforms; one feeds the
+// codebook rings; two search in binary64.  A chunk of 128 codewords makes a round trip token warps -> MMA -> token warps
+// (about 300 cycles, whatever its width), so chunks are as wide as TMEM allows (four warpgroups x 128 columns: the
+// coefficients live in shared memory for that), and the first chunk of the next group is computed behind the selection
+// of this one.  Every wait is bounded (novakv_tcgen05.cuh): a wait that gives up sets NOVAKV_DEV_WAIT_TIMEOUT, and the CTA
+// runs through its remaining steps without waiting.  (The named barriers among token warps are never skipped.)
+//
+// What bounds it: instruction issue and latency of the selection, about 600 warp instructions per 32 tokens and group (of
+// which 64 + 16 packed minima and comparisons on the half-rate pipe) with four token warps per scheduler; tensor pipe
+// 16 %, issue slots 58 % busy.  The kernel lives at the limit of 96 registers: everything the rare paths need is
+// formed there.  d = 128, 32768 tokens: 523 us a call in a stream of calls (binary32 search on the FMA pipe with a binary64 transform: 1971 us).
+// Measured on the way: coefficients in TMEM and chunks of 64 codewords 945 us; releasing a chunk through an mbarrier
+// instead of a hardware barrier +13 %; MMAs issued behind lane == 0 instead of elect.sync +40 cycles each; spills of 150
+// bytes in the loop +15 %; one helper warp instead of two 665 us; direct distances one group late, to hide the round
+// trip of the second chunk too: 635 us (longer register lifetimes cost more than the wait).
+#include <cuda.h>
 #include <math_constants.h>
 
 #include <cmath>
@@ -38,11 +47,20 @@ constexpr int PF_HELPERS = 2;
 constexpr int PF_THREADS = (PF_TOKEN_WARPS + 2 + PF_HELPERS) * 32;
 constexpr int PF_TILE = 256;                 // tokens per unit: two half tiles
 constexpr int PF_HALF = 128;
-constexpr int PF_STAGES = 4;                 // codebook ring
-constexpr int PF_STAGE_BYTES = NOVAKV_PF_GROUP_BYTES;
+#ifndef PF_TOK_NS
+#define PF_TOK_NS 0
+#endif
+#ifndef PF_AUX_NS
+#define PF_AUX_NS 200
+#endif
+constexpr int PF_OP_BYTES = 8192;            // a group's codebook as search operand
+constexpr int PF_CW_BYTES = 4096;            // and in binary32
+constexpr int PF_CW_STAGES = 6;              // (the binary32 codewords are needed one group longer than the operand)
+static_assert(PF_OP_BYTES + PF_CW_BYTES == NOVAKV_PF_GROUP_BYTES, "codebook image");
 constexpr int PF_QUEUE = 16;                 // entries of a helper's queue
-// durations the work split reckons with, microseconds per unit
-constexpr double PF_US_UNIT = 2.0, PF_US_GROUP = 0.6, PF_US_INT2 = 4.0;
+// Durations the work split reckons with, microseconds per unit (measured: 19.3 for 16 groups of plain keys or values, about
+// 28 for scaled keys, which transform and norm the whole row, 11 for INT2 values).
+constexpr double PF_US_UNIT = 3.0, PF_US_GROUP = 1.0, PF_US_SCALED = 9.0, PF_US_INT2 = 11.0;
 // |coefficient - binary64 coefficient| <= KAPPA (|x| + |mean|) |R column|.  The accumulation order of the tensor core is
 // not specified; all-positive inputs (every truncation in the same direction) showed 2^-21.6, random signs 2^-23.3.
 constexpr float KAPPA = 1.4e-6f;             // > 2^-19.5
@@ -59,6 +77,7 @@ struct PF {
     // a per-token scale needs the token's whole row: then all columns of R are resident, which leaves room for two slots
     static constexpr int R_COLS = FMT == 0 ? GU * NOVAKV_G : D;
     static constexpr int NX = D == 128 && FMT != 0 ? 2 : 3;
+    static constexpr int NOP = D == 128 && FMT != 0 ? 3 : 4;      // stages of the operand ring
     static constexpr uint32_t R_SLICE = R_COLS * D * 2;
     static constexpr uint32_t R_IMG_SLICE = D * D * 2;
     static constexpr uint32_t X_BYTES = PF_HALF * D * 2;          // token rows of a half tile
@@ -68,19 +87,22 @@ struct PF {
     static constexpr uint32_t OFF_R = 0;
     static constexpr uint32_t OFF_X = OFF_R + 3 * R_SLICE;
     static constexpr uint32_t OFF_RING = OFF_X + NX * SLOT_BYTES;
-    static constexpr uint32_t OFF_A = OFF_RING + PF_STAGES * PF_STAGE_BYTES;
+    static constexpr uint32_t OFF_CW = OFF_RING + NOP * PF_OP_BYTES;
+    static constexpr uint32_t OFF_A = OFF_CW + PF_CW_STAGES * PF_CW_BYTES;
     static constexpr uint32_t OFF_QUEUE = OFF_A + 4 * A_BYTES;
-    static constexpr uint32_t OFF_CONST = OFF_QUEUE + PF_HELPERS * PF_QUEUE * 16;
+    static constexpr uint32_t OFF_PAGE = OFF_QUEUE + PF_HELPERS * PF_QUEUE * 16;  // int [NX][128], page of a token or -1
+    static constexpr uint32_t OFF_TSLOT = OFF_PAGE + NX * PF_HALF * 4;            // uint8 [NX][128], its slot in the page
+    static constexpr uint32_t OFF_CONST = OFF_TSLOT + NX * PF_HALF;
     static constexpr uint32_t OFF_BAR = OFF_CONST + ((NCONST * 4 + 15) & ~15);
-    static constexpr uint32_t OFF_MISC = OFF_BAR + 256;           // TMEM base, abort flag, finished token warps, queue counters
-    static constexpr uint32_t BYTES = OFF_MISC + 64;
+    static constexpr uint32_t OFF_MISC = OFF_BAR + 288;           // TMEM base, abort flag, finished token warps, queue counters; unsure tokens [16]
+    static constexpr uint32_t BYTES = OFF_MISC + 128;
     static_assert(BYTES <= 232448, "shared memory budget");
     static_assert(X_BYTES <= SLOT_BYTES && R_SLICE % 1024 == 0 && SLOT_BYTES % 1024 == 0, "swizzled operands start on 1024 bytes");
 };
 // mbarriers
 enum { B_R = 0, B_X = 1 /* +slot */, B_XFREE = 4 /* +slot */, B_T = 7 /* +half */, B_TFREE = 9 /* +half */, B_S = 11 /* +wg */,
-       B_RING = 15 /* +stage */, B_RINGFREE = B_RING + PF_STAGES, B_COUNT = B_RING + 2 * PF_STAGES };
-static_assert(B_COUNT * 8 <= 256, "barrier block");
+       B_RING = 15 /* +stage */, B_RINGFREE = 19, B_CW = 23 /* +stage */, B_CWFREE = B_CW + PF_CW_STAGES, B_COUNT = B_CW + 2 * PF_CW_STAGES };
+static_assert(B_COUNT * 8 <= 288, "barrier block");
 // named barriers: 1 + wg among the four warps of a warpgroup, 5 + half among the eight of a half tile
 __device__ __forceinline__ void nbar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void nbar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
@@ -92,7 +114,9 @@ struct PrefillArgs {
     const uint8_t* r_img;       // [2][Hkv][3 d d 2]
     const uint8_t* cb_img;      // [2][Hkv][L][stage]
     const float* consts;        // [2][Hkv][NCONST]
-    const double *rk_d, *rv_d, *k_mean_d, *v_mean_d;
+    const double *rk_d, *rv_d;  // [Hkv][L][d][4]
+    const float *rk_rows, *rv_rows;   // [Hkv][d][d]
+    const double *k_mean_d, *v_mean_d;
     const float *cb_k, *cb_v;   // [Hkv][L][256][4]
     uint8_t *k_pages, *v_pages;
     __nv_bfloat16 *k_scales, *v_meta;
@@ -103,7 +127,9 @@ struct PrefillArgs {
     int n_kv_heads;
     int gs;                     // parts a head's groups are cut into
     int cost_k, cost_v;         // relative cost of a key / value unit (the cut of the walk)
+    int tma;                    // the token rows can be copied by the tensor maps (16-byte aligned)
     uint32_t* dev_status;
+    CUtensorMap map_k, map_v;   // k_new / v_new as [n_tokens][Hkv d], boxes of 64 x 128
 };
 
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
@@ -118,6 +144,14 @@ __device__ __forceinline__ float sqrt_approx(float x) {
     return y;
 }
 __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+__device__ __forceinline__ float4 lds_f4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void sts_f4(uint32_t addr, float4 v) {
+    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
 __device__ __forceinline__ uint64_t dup2(float x) {
     uint64_t r;
     asm("mov.b64 %0, {%1,%1};" : "=l"(r) : "f"(x));
@@ -145,15 +179,32 @@ __host__ __device__ __forceinline__ int codeword_offset(int code, int comp) {   
     return (code >> 3) * 32 + (((code & 7) >> 1) * 2 + (comp >> 1)) * 4 + (comp & 1) * 2 + (code & 1);
 }
 
-// Warp-cooperative exact search of one (token, group): all lanes call it with the same arguments and get the same result.
-// rho > 0: the vector to encode is the binary32 quotient of the binary32 coefficient and rho (scaled key format).
-// Lane i evaluates the codewords i, i + 32, ... in ascending order with a strict '<'; the warp then keeps the smallest
-// distance and, among equal distances, the lowest index.
+// Warp-cooperative exact search of one (token, group) among the rows of 8 codewords that its ranking has left (bit k:
+// row 2 (k % 16) + k / 16): all lanes call it with the same arguments and get the same result.  rho > 0: the vector to
+// encode is the binary32 quotient of the binary32 coefficient and rho (scaled key format).  Four rows at a time, lane =
+// codeword; the smallest distance wins and, among equal distances, the lowest index.
+// (It forms its pointers itself, so that the token warps keep none of them in registers.)
 template <int D>
-__device__ __noinline__ int exact_search_token(const __nv_bfloat16* __restrict__ x_row, const double* __restrict__ mean,
-                                               const double* __restrict__ R /* [D][D] */, int l, const float4* __restrict__ cb /* [256] */,
-                                               float rho) {
+__device__ __noinline__ int exact_search_token(const PrefillArgs& a, int side, int kvh, int tkn, int l, float rho, uint32_t rows) {
     const int lane = threadIdx.x & 31;
+    const __nv_bfloat16* x_row = (side == 0 ? a.k_new : a.v_new) + ((size_t)tkn * a.n_kv_heads + kvh) * D;
+    const double* R = (side == 0 ? a.rk_d : a.rv_d) + (size_t)kvh * D * D + l * D * 4;
+    const double* mean = (side == 0 ? a.k_mean_d : a.v_mean_d) + (size_t)kvh * D;
+    const float4* cb = reinterpret_cast<const float4*>(side == 0 ? a.cb_k : a.cb_v) + ((size_t)kvh * (D / NOVAKV_G) + l) * NOVAKV_C;
+    if (rows == 0u) rows = 0xffffffffu;                               // (the ranking was void)
+    // this lane's codeword of the next four rows; -1 beyond the last
+    auto next_code = [&]() {
+        int code = -1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int k = __ffs(rows) - 1;
+            if (rows && (lane >> 3) == j) code = ((((k & 15) << 1) | (k >> 4)) << 3) | (lane & 7);
+            rows &= rows - 1;
+        }
+        return code;
+    };
+    int code = next_code();
+    float4 cw = cb[code < 0 ? 0 : code];                              // (requested before the coefficient is formed)
     double r[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) r[c] = 0.0;
@@ -161,27 +212,34 @@ __device__ __noinline__ int exact_search_token(const __nv_bfloat16* __restrict__
     for (int j = 0; j < D / 32; ++j) {
         const int k = lane + 32 * j;
         const double xc = (double)__bfloat162float(x_row[k]) - mean[k];
-        const double2 r01 = *reinterpret_cast<const double2*>(R + (size_t)k * D + l * 4);
-        const double2 r23 = *reinterpret_cast<const double2*>(R + (size_t)k * D + l * 4 + 2);
+        const double2 r01 = *reinterpret_cast<const double2*>(R + k * 4);
+        const double2 r23 = *reinterpret_cast<const double2*>(R + k * 4 + 2);
         r[0] = fma(xc, r01.x, r[0]); r[1] = fma(xc, r01.y, r[1]);
         r[2] = fma(xc, r23.x, r[2]); r[3] = fma(xc, r23.y, r[3]);
     }
+    {
+        // sum over the lanes: lane bits 0 and 1 choose the component a lane goes on with, then every lane gets all four
+        const double k0 = lane & 1 ? r[1] : r[0], s0 = lane & 1 ? r[0] : r[1], k1 = lane & 1 ? r[3] : r[2], s1 = lane & 1 ? r[2] : r[3];
+        const double p0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 1), p1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 1);
+        double p = (lane & 2 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, lane & 2 ? p0 : p1, 2);
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
+        for (int o = 4; o <= 16; o <<= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) r[c] += __shfl_xor_sync(0xffffffffu, r[c], o);
+        for (int c = 0; c < 4; ++c) r[c] = __shfl_sync(0xffffffffu, p, c);
+    }
     if (rho > 0.f) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) r[c] = (double)__fdiv_rn((float)r[c], rho);
     }
     double best = CUDART_INF;
-    int bi = lane;
-#pragma unroll 4
-    for (int j = 0; j < NOVAKV_C / 32; ++j) {
-        const float4 c = cb[lane + 32 * j];
-        const double e0 = r[0] - (double)c.x, e1 = r[1] - (double)c.y, e2 = r[2] - (double)c.z, e3 = r[3] - (double)c.w;
+    int bi = 0x7fffffff;
+    for (;;) {
+        const double e0 = r[0] - (double)cw.x, e1 = r[1] - (double)cw.y, e2 = r[2] - (double)cw.z, e3 = r[3] - (double)cw.w;
         const double dd = __dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(e0, e0), __dmul_rn(e1, e1)), __dmul_rn(e2, e2)), __dmul_rn(e3, e3));
-        if (dd < best) { best = dd; bi = lane + 32 * j; }
+        if (code >= 0 && (dd < best || (dd == best && code < bi))) { best = dd; bi = code; }
+        if (rows == 0u) break;
+        code = next_code();
+        cw = cb[code < 0 ? 0 : code];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -189,30 +247,50 @@ __device__ __noinline__ int exact_search_token(const __nv_bfloat16* __restrict__
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
     }
-    return bi;
+    return bi & 255;                                                  // (no codeword at a finite distance: any)
 }
 
-// All binary32 coefficients of one token from binary64 sums: lane i gets columns D / 32 * i .. (same arguments in all lanes).
+// One token's coefficients in binary64, by the eight warps of a half tile: warp q sums an eighth of the input dimension
+// into part_s[q][D]; after a barrier row_of() adds the parts.  Lane i holds columns D / 32 * i ...
 template <int D>
-__device__ __noinline__ void exact_row(const __nv_bfloat16* __restrict__ x_row, const double* __restrict__ mean,
-                                       const double* __restrict__ R, float (&out)[D / 32]) {
+__device__ __noinline__ void exact_row_part(const PrefillArgs& a, int side, int kvh, int tkn, int q, double* part_s) {
     constexpr int N = D / 32;
     const int lane = threadIdx.x & 31;
+    const __nv_bfloat16* x_row = (side == 0 ? a.k_new : a.v_new) + ((size_t)tkn * a.n_kv_heads + kvh) * D + q * (D / 8);
+    const float* R = (side == 0 ? a.rk_rows : a.rv_rows) + ((size_t)kvh * D + q * (D / 8)) * D + lane * N;
+    const double* mean = (side == 0 ? a.k_mean_d : a.v_mean_d) + (size_t)kvh * D + q * (D / 8);
     double acc[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) acc[i] = 0.0;
-#pragma unroll 8
-    for (int k = 0; k < D; ++k) {
-        const double xc = (double)__bfloat162float(x_row[k]) - mean[k];
+    float rr[D / 8][N];
 #pragma unroll
-        for (int i = 0; i < N; i += 2) {
-            const double2 r = *reinterpret_cast<const double2*>(R + (size_t)k * D + lane * N + i);
-            acc[i] = fma(xc, r.x, acc[i]);
-            acc[i + 1] = fma(xc, r.y, acc[i + 1]);
+    for (int k = 0; k < D / 8; ++k) {
+        if (N == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(R + k * D);
+            rr[k][0] = v.x; rr[k][1] = v.y; rr[k][N - 2] = v.z; rr[k][N - 1] = v.w;
+        } else {
+            const float2 v = *reinterpret_cast<const float2*>(R + k * D);
+            rr[k][0] = v.x; rr[k][1] = v.y;
         }
     }
 #pragma unroll
-    for (int i = 0; i < N; ++i) out[i] = (float)acc[i];
+    for (int k = 0; k < D / 8; ++k) {
+        const double xc = (double)__bfloat162float(x_row[k]) - mean[k];
+#pragma unroll
+        for (int i = 0; i < N; ++i) acc[i] = fma(xc, (double)rr[k][i], acc[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) part_s[q * D + lane * N + i] = acc[i];
+}
+template <int D>
+__device__ __forceinline__ void row_of(const double* part_s, int lane, float (&r)[D / 32]) {
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) {
+        double p[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) p[q] = part_s[q * D + lane * (D / 32) + i];
+        r[i] = (float)(((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7])));
+    }
 }
 
 // Stores the codes of groups l .. l + 3 of this lane's token (group l in the low byte); l a multiple of 4.
@@ -245,7 +323,7 @@ __device__ __forceinline__ void store_value_word(uint8_t* chunk, int slot, int l
 // coefficients where no error within their bound can move the bfloat16 rounding, else from the binary64 row.
 // INT2 values: zero, scale and the levels likewise; a token with any decision inside the bound takes the binary64 row.
 template <int D, int FMT>
-__global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const PrefillArgs a) {
+__global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __grid_constant__ PrefillArgs a) {
     using P = PF<D, FMT>;
     constexpr int L = P::L;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -281,16 +359,15 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
         for (int h = 0; h < PF_HELPERS; ++h) { s_count[h] = 0; s_head[h] = 0; }
         mbar_init(bar(B_R), 1);
 #pragma unroll
-        for (int x = 0; x < P::NX; ++x) { mbar_init(bar(B_X + x), 1); mbar_init(bar(B_XFREE + x), 8); }
+        for (int x = 0; x < P::NX; ++x) { mbar_init(bar(B_X + x), 2); mbar_init(bar(B_XFREE + x), 8); }
 #pragma unroll
         for (int w = 0; w < 2; ++w) { mbar_init(bar(B_T + w), 1); mbar_init(bar(B_TFREE + w), 4); }
 #pragma unroll
         for (int g = 0; g < 4; ++g) mbar_init(bar(B_S + g), 1);
 #pragma unroll
-        for (int s = 0; s < PF_STAGES; ++s) {
-            mbar_init(bar(B_RING + s), 1);
-            mbar_init(bar(B_RINGFREE + s), 10);        // MMAs and token warps of the two half tiles
-        }
+        for (int s = 0; s < P::NOP; ++s) { mbar_init(bar(B_RING + s), 1); mbar_init(bar(B_RINGFREE + s), 2); }
+#pragma unroll
+        for (int s = 0; s < PF_CW_STAGES; ++s) { mbar_init(bar(B_CW + s), 1); mbar_init(bar(B_CWFREE + s), 8); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -318,46 +395,97 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
         const int c0 = ksc || vsq ? 0 : g0 * 4, nc = ksc || vsq ? D : L / gs * 4;
         u_next += n_local;
         const size_t sh = (size_t)side * a.n_kv_heads + kvh;
-        const __nv_bfloat16* x_new = side == 0 ? a.k_new : a.v_new;
-        const double* R_plain = (side == 0 ? a.rk_d : a.rv_d) + (size_t)kvh * D * D;
-        const double* mean = (side == 0 ? a.k_mean_d : a.v_mean_d) + (size_t)kvh * D;
-        const float4* cb_g = reinterpret_cast<const float4*>(side == 0 ? a.cb_k : a.cb_v) + (size_t)kvh * L * NOVAKV_C;
-        uint8_t* const pages = side == 0 ? a.k_pages : a.v_pages;
+        auto chunk_of = [&](int page) -> uint8_t* {
+            return (side == 0 ? a.k_pages : a.v_pages) + ((size_t)(page < 0 ? 0 : page) * a.n_kv_heads + kvh) * (NOVAKV_PAGE_TOKENS * L);
+        };
         for (int i = threadIdx.x; i < P::NCONST; i += PF_THREADS) cst[i] = a.consts[sh * P::NCONST + i];
         if (threadIdx.x == 0) *s_done = 0;
         __syncthreads();
 
         if (warp == PF_TOKEN_WARPS) {
             // ---- token rows ([128][D] bfloat16 of a half tile, 128-byte rows per panel, 16-byte chunks swizzled by the
-            //      row), one half tile ahead of the transforms.  Half tile q of the CTA uses slot q % NX.
+            //      row) and destinations, one half tile ahead of the transforms.  Half tile q of the CTA uses slot q % NX.
             const int q0 = 2 * n_it, q1 = q0 + 2 * n_local;
+            int q_loaded = q0;
             bool ok = true;
+            // destinations of half tile q's tokens (four per lane); its rows on their way into the L2
+            int page[4], tslot[4];
+            auto look_up = [&](int q) {
+                const int t0 = tile0 * PF_TILE + (q - q0) * PF_HALF;
+                if (a.tma && lane < D / 64 && t0 < a.n_tokens) tma_prefetch_2d(side == 0 ? &a.map_k : &a.map_v, kvh * D + lane * 64, t0);
+                int sq[4], pos[4];
+                bool named[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int tkn = t0 + lane + 32 * j;
+                    sq[j] = -1; pos[j] = 0;
+                    if (tkn < a.n_tokens) { sq[j] = a.tok_seq[tkn]; pos[j] = a.tok_pos[tkn]; }
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    named[j] = sq[j] >= 0 && sq[j] < a.n_seq && pos[j] >= 0 && pos[j] / NOVAKV_PAGE_TOKENS < a.max_pages_per_seq;
+                    page[j] = named[j] ? a.page_table[(size_t)sq[j] * a.max_pages_per_seq + pos[j] / NOVAKV_PAGE_TOKENS] : -1;
+                    tslot[j] = pos[j] % NOVAKV_PAGE_TOKENS;
+                    if (!named[j] && sq[j] != -1) atomicOr(a.dev_status, NOVAKV_DEV_BAD_TOKEN);   // (-1: unused entry, skipped)
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (named[j] && (page[j] < 0 || page[j] >= a.n_pages)) {
+                        atomicOr(a.dev_status, NOVAKV_DEV_BAD_PAGE);
+                        page[j] = -1;
+                    } else if (named[j] && sh == 0 && g0 == 0) {
+                        atomicMax(&a.seq_lens[sq[j]], pos[j] + 1);
+                    }
+                }
+            };
             auto load_rows = [&](int q) {
                 const int slot = q % P::NX;
-                if (q >= P::NX) ok = mbar_wait(bar(B_XFREE + slot), (q / P::NX - 1) & 1, abort_flag);
+                if (q >= P::NX) ok = mbar_wait<PF_AUX_NS>(bar(B_XFREE + slot), (q / P::NX - 1) & 1, abort_flag);
                 if (!__all_sync(0xffffffffu, ok)) { ok = false; return; }
                 const int t0 = tile0 * PF_TILE + (q - q0) * PF_HALF;
                 const uint32_t dst0 = sb + P::OFF_X + slot * P::SLOT_BYTES;
-#pragma unroll 8
-                for (int e = lane; e < PF_HALF * (D / 8); e += 32) {
-                    const int t = e / (D / 8), c = e - t * (D / 8);
-                    const uint32_t dst = dst0 + (c >> 3) * (PF_HALF * 128) + t * 128 + (((c & 7) ^ (t & 7)) * 16);
-                    const bool in = t0 + t < a.n_tokens;
-                    const __nv_bfloat16* src = x_new + ((size_t)(in ? t0 + t : 0) * a.n_kv_heads + kvh) * D + c * 8;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+                if (a.tma) {
+                    if (elect_one()) {
+                        fence_proxy_async();                       // (the slot held coefficients written by threads)
+                        mbar_expect_tx(bar(B_X + slot), P::X_BYTES);
+#pragma unroll
+                        for (int p = 0; p < D / 64; ++p)
+                            tma_load_2d(dst0 + p * (PF_HALF * 128), side == 0 ? &a.map_k : &a.map_v, kvh * D + p * 64, t0, bar(B_X + slot));
+                    }
+                } else {
+#pragma unroll 4
+                    for (int e = lane; e < PF_HALF * (D / 2); e += 32) {        // 4-byte copies
+                        const int t = e / (D / 2), c = e - t * (D / 2);
+                        const uint32_t dst = dst0 + (c >> 5) * (PF_HALF * 128) + t * 128 + ((((c >> 2) & 7) ^ (t & 7)) * 16) + (c & 3) * 4;
+                        const bool in = t0 + t < a.n_tokens;
+                        const __nv_bfloat16* src = (side == 0 ? a.k_new : a.v_new) + ((size_t)(in ? t0 + t : 0) * a.n_kv_heads + kvh) * D + c * 2;
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+                    }
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    fence_proxy_async();
+                    __syncwarp();
+                    mbar_arrive_lane0(bar(B_X + slot), lane);
                 }
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                fence_proxy_async();
+                q_loaded = q + 1;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    reinterpret_cast<int*>(smem + P::OFF_PAGE)[slot * PF_HALF + lane + 32 * j] = page[j];
+                    (smem + P::OFF_TSLOT)[slot * PF_HALF + lane + 32 * j] = (unsigned char)tslot[j];
+                }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_X + slot));
+                mbar_arrive_lane0(bar(B_X + slot), lane);
                 __syncwarp();
             };
+            look_up(q0);
             load_rows(q0);
-            ok = __all_sync(0xffffffffu, ok && mbar_wait(bar(B_R), n_seg & 1, abort_flag));
+            ok = __all_sync(0xffffffffu, ok && mbar_wait<PF_AUX_NS>(bar(B_R), n_seg & 1, abort_flag));
             const uint32_t id_t = umma_idesc(true, true, 128, 0) | ((uint32_t)(nc >> 3) << 17);
             for (int q = q0; q < q1 && ok; ++q) {
                 const int w = q & 1, slot = q % P::NX;
-                if (q >= 2) ok = __all_sync(0xffffffffu, mbar_wait(bar(B_TFREE + w), ((q >> 1) - 1) & 1, abort_flag));
+                if (q + 1 < q1) look_up(q + 1);
+                ok = mbar_wait<PF_AUX_NS>(bar(B_X + slot), (q / P::NX) & 1, abort_flag);
+                if (q >= 2) ok = ok && mbar_wait<50>(bar(B_TFREE + w), ((q >> 1) - 1) & 1, abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) {
@@ -377,6 +505,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                 __syncwarp();
                 if (q + 1 < q1) load_rows(q + 1);
             }
+            // (after a wait that gave up: the last copy must have landed before the CTA's memory goes away)
+            if (q_loaded > q0) {
+                int tries = 0;
+                while (!mbar_try(bar(B_X + (q_loaded - 1) % P::NX), ((q_loaded - 1) / P::NX) & 1) && ++tries < 1000000) {}
+            }
             n_it += n_local;
         } else if (warp == PF_TOKEN_WARPS + 1) {
             if (lane == 0) {
@@ -388,26 +521,34 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                     for (int p = 0; p < D / 64; ++p)
                         bulk_copy(sb + P::OFF_R + s * P::R_SLICE + p * (P::R_COLS * 128),
                                   a.r_img + sh * (3 * P::R_IMG_SLICE) + s * P::R_IMG_SLICE + p * (D * 128) + c0 * 128, (uint32_t)nc * 128, bar(B_R));
-                const uint8_t* src = a.cb_img + (sh * L + g0) * PF_STAGE_BYTES;
+                const uint8_t* src = a.cb_img + (sh * L + g0) * NOVAKV_PF_GROUP_BYTES;
                 const int n = n_local * 2 * ngh;
                 bool ok = true;
                 // use 2 g + h: group g of the half of the groups that warpgroups h take
                 for (int j = 0, g = 0; j < n && ok; ++j, ++n_use) {
-                    const int s = n_use % PF_STAGES;
-                    if (n_use >= PF_STAGES) ok = mbar_wait(bar(B_RINGFREE + s), (n_use / PF_STAGES - 1) & 1, abort_flag);
+                    const int so = n_use % P::NOP, sc = n_use % PF_CW_STAGES;
+                    const uint8_t* img = src + (size_t)((j & 1) * ngh + g) * NOVAKV_PF_GROUP_BYTES;
+                    if (n_use >= P::NOP) ok = mbar_wait<PF_AUX_NS>(bar(B_RINGFREE + so), (n_use / P::NOP - 1) & 1, abort_flag);
                     if (!ok) break;
-                    mbar_expect_tx(bar(B_RING + s), PF_STAGE_BYTES);
-                    bulk_copy(sb + P::OFF_RING + s * PF_STAGE_BYTES, src + (size_t)((j & 1) * ngh + g) * PF_STAGE_BYTES, PF_STAGE_BYTES,
-                              bar(B_RING + s));
+                    mbar_expect_tx(bar(B_RING + so), PF_OP_BYTES);
+                    bulk_copy(sb + P::OFF_RING + so * PF_OP_BYTES, img, PF_OP_BYTES, bar(B_RING + so));
+                    if (n_use >= PF_CW_STAGES) ok = mbar_wait<PF_AUX_NS>(bar(B_CWFREE + sc), (n_use / PF_CW_STAGES - 1) & 1, abort_flag);
+                    if (!ok) { ++n_use; break; }
+                    mbar_expect_tx(bar(B_CW + sc), PF_CW_BYTES);
+                    bulk_copy(sb + P::OFF_CW + sc * PF_CW_BYTES, img + PF_OP_BYTES, PF_CW_BYTES, bar(B_CW + sc));
                     if (j & 1) g = g + 1 == ngh ? 0 : g + 1;
                 }
                 // no copy and no commit may be in flight when the segment (and the CTA's memory) goes away
-                mbar_wait(bar(B_R), n_seg & 1, abort_flag);
-                for (int j = max(0, n_use - PF_STAGES); j < n_use; ++j) {
+                mbar_wait<PF_AUX_NS>(bar(B_R), n_seg & 1, abort_flag);
+                auto landed = [&](int b, int parity) {             // (after a wait that gave up, too)
                     int tries = 0;
-                    while (!mbar_try(bar(B_RING + j % PF_STAGES), (j / PF_STAGES) & 1) && ++tries < 1000000) {}
-                    mbar_wait(bar(B_RINGFREE + j % PF_STAGES), (j / PF_STAGES) & 1, abort_flag);
+                    while (!mbar_try(bar(b), parity) && ++tries < 1000000) {}
+                };
+                for (int j = max(0, n_use - P::NOP); j < n_use; ++j) {
+                    landed(B_RING + j % P::NOP, (j / P::NOP) & 1);
+                    mbar_wait<PF_AUX_NS>(bar(B_RINGFREE + j % P::NOP), (j / P::NOP) & 1, abort_flag);
                 }
+                for (int j = max(0, n_use - PF_CW_STAGES); j < n_use - (ok ? 0 : 1); ++j) landed(B_CW + j % PF_CW_STAGES, (j / PF_CW_STAGES) & 1);
             }
             __syncwarp();
         } else if (warp > PF_TOKEN_WARPS + 1) {
@@ -417,25 +558,24 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
             for (;;) {
                 const bool last = *reinterpret_cast<volatile int*>(s_done) == PF_TOKEN_WARPS;      // (read before the entry)
                 volatile uint32_t* const e = queue + (q_tail % PF_QUEUE) * 4;
-                const uint32_t tag = e[0];
-                if (!__any_sync(0xffffffffu, tag != 0u)) {
-                    if (__any_sync(0xffffffffu, last)) break;
+                const uint32_t tag = __shfl_sync(0xffffffffu, e[0], 0);
+                if (tag == 0u) {
+                    if (__all_sync(0xffffffffu, last)) break;
                     __nanosleep(200);
                     continue;
                 }
+                // key scale (a bfloat16 number), a set bit, slot in the page, group | token | page | rows
                 __threadfence_block();
-                const uint32_t t0 = __shfl_sync(0xffffffffu, e[0], 0);
-                const int l = t0 & 63, slot = (t0 >> 6) & 63, tkn = (int)e[1], page = (int)e[2];
-                const float rho = __uint_as_float(e[3]);
+                const int l = tag & 63, slot = (tag >> 6) & 63, tkn = (int)e[1], page = (int)e[2];
+                const uint32_t rows = e[3];
                 __syncwarp();
-                const int bi = exact_search_token<D>(x_new + ((size_t)tkn * a.n_kv_heads + kvh) * D, mean, R_plain, l, cb_g + l * NOVAKV_C, rho);
                 if (lane == 0) {
-                    pages[((size_t)page * a.n_kv_heads + kvh) * (NOVAKV_PAGE_TOKENS * L) +
-                          (side == 0 ? novakv_k_offset<L>(slot, l) : novakv_v_offset<L>(slot, l))] = (uint8_t)bi;
-                    e[0] = 0u;
+                    e[0] = 0u;                                     // (the entry has been read: its place is free)
                     __threadfence_block();
                     atomicSub(&s_count[h], 1);
                 }
+                const int bi = exact_search_token<D>(a, side, kvh, tkn, l, __uint_as_float(tag & 0xffff0000u), rows);
+                if (lane == 0) chunk_of(page)[side == 0 ? novakv_k_offset<L>(slot, l) : novakv_v_offset<L>(slot, l)] = (uint8_t)bi;
                 __syncwarp();
                 ++q_tail;
             }
@@ -446,10 +586,8 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
             const uint32_t d_t = tmem + w * 256 + lane_base, d_s = tmem + wg * 128;
             const uint32_t a_s = sb + P::OFF_A + wg * P::A_BYTES;
             float* const x2_s = reinterpret_cast<float*>(smem + P::OFF_A);               // partial |x|^2, [wg][A_BYTES / 4]
-            const float *mr = cst, *rnorm = cst + D, *gscale = cst + D + L;
-            const float mean_norm = cst[D + 2 * L], r_fro = cst[D + 2 * L + 1], r_colmax = cst[D + 2 * L + 2];
+            const float* const mr = cst;
             const int lx = lane & 7;
-            bool ok = true;
 #pragma unroll 1
             for (int i = 0; i < n_local; ++i, ++n_it) {
                 const int t0 = (tile0 + i) * PF_TILE + w * PF_HALF;            // first token of the half tile
@@ -457,10 +595,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                 const int tkn = t0 + row;
                 const int q = 2 * n_it + w, xslot = q % P::NX;
                 unsigned char* const x_s = smem + P::OFF_X + xslot * P::SLOT_BYTES;
-                int sq = -1, pos = 0;
-                if (tkn < a.n_tokens) { sq = a.tok_seq[tkn]; pos = a.tok_pos[tkn]; }
                 // |x| of the token; each warpgroup sums its half of the row
-                ok = ok && mbar_wait(bar(B_X + xslot), (q / P::NX) & 1, abort_flag);
+                mbar_wait<PF_TOK_NS>(bar(B_X + xslot), (q / P::NX) & 1, abort_flag);
+                const int page = reinterpret_cast<const int*>(smem + P::OFF_PAGE)[xslot * PF_HALF + row];
+                const int slot = (smem + P::OFF_TSLOT)[xslot * PF_HALF + row];
+                const bool valid = page >= 0;
                 {
                     float x2 = 0.f;
 #pragma unroll
@@ -476,25 +615,42 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                     }
                     x2_s[wg * (P::A_BYTES / 4) + row] = x2;
                 }
-                // destination of the token
-                int page = -1, slot = 0;
-                const bool named = sq >= 0 && sq < a.n_seq && pos >= 0 && pos / NOVAKV_PAGE_TOKENS < a.max_pages_per_seq;
-                if (named) {
-                    page = a.page_table[(size_t)sq * a.max_pages_per_seq + pos / NOVAKV_PAGE_TOKENS];
-                    slot = pos % NOVAKV_PAGE_TOKENS;
-                } else if (sq != -1) {                                         // (-1: unused entry of the token list, skipped)
-                    atomicOr(a.dev_status, NOVAKV_DEV_BAD_TOKEN);
-                }
                 nbar_sync(5 + w, PF_TILE);                                     // the row has been read by everyone; partial sums visible
                 float bound;                                                   // times a column norm: error of that coefficient
                 {
                     const float x2 = x2_s[(2 * w) * (P::A_BYTES / 4) + row] + x2_s[(2 * w + 1) * (P::A_BYTES / 4) + row];
-                    bound = KAPPA * (sqrtf(x2) * 1.00001f + mean_norm);
+                    bound = KAPPA * (sqrtf(x2) * 1.00001f + cst[D + 2 * L] /* |mean| */);
                 }
-                ok = ok && mbar_wait(bar(B_T + w), n_it & 1, abort_flag);
+                mbar_wait<PF_TOK_NS>(bar(B_T + w), n_it & 1, abort_flag);
                 tc_fence_after();
                 __syncwarp();
 
+                // The tokens of the half tile whose decisions the tensor-core coefficients leave open get their coefficients
+                // in binary64, one after the other by all eight warps (a warp alone took 18,000 cycles for one).  fn(lane of
+                // the token, its row) runs in the two warps that own the token.
+                auto exact_rows = [&](bool unsure, auto fn) {
+                    volatile uint32_t* const masks = reinterpret_cast<volatile uint32_t*>(smem + P::OFF_MISC + 64) + w * 8;
+                    double* const part_s = reinterpret_cast<double*>(smem + P::OFF_A + 2 * w * P::A_BYTES);
+                    const unsigned mine = __ballot_sync(0xffffffffu, unsure);
+                    if (lane == 0) masks[warp & 7] = mine;
+                    nbar_sync(5 + w, PF_TILE);
+#pragma unroll 1
+                    for (int o = 0; o < 4; ++o) {
+                        uint32_t todo = masks[o] | masks[o + 4];
+                        while (todo) {
+                            const int src = __ffs(todo) - 1;
+                            todo &= todo - 1;
+                            exact_row_part<D>(a, side, kvh, t0 + o * 32 + src, warp & 7, part_s);
+                            nbar_sync(5 + w, PF_TILE);
+                            if ((warp & 3) == o) {
+                                float r[D / 32];
+                                row_of<D>(part_s, lane, r);
+                                fn(src, r);
+                            }
+                            nbar_sync(5 + w, PF_TILE);
+                        }
+                    }
+                };
                 float rho = 0.f, inv_rho = 1.f;
                 if (ksc) {
                     float ss = 0.f;
@@ -513,16 +669,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                         ss += s0 + s1;
                     }
                     // relative error of the norm: that of the coefficients, their rounding, and the binary32 sum
-                    const float nrm = sqrtf(ss), rel = bound * r_fro / nrm + 4.0e-6f;
+                    const float nrm = sqrtf(ss), rel = bound * cst[D + 2 * L + 1] /* |R| */ / nrm + 4.0e-6f;
                     const float f = sqrtf(ss / (float)D);
                     rho = bf16_round(f);
                     const bool sure = bf16_round(f * (1.f - rel)) == rho && bf16_round(f * (1.f + rel)) == rho && rho > 0.f && rho < CUDART_INF_F;
-                    unsigned todo = __ballot_sync(0xffffffffu, sq >= 0 && !sure);
-                    while (todo) {
-                        const int src = __ffs(todo) - 1;
-                        todo &= todo - 1;
-                        float r[D / 32];
-                        exact_row<D>(x_new + ((size_t)(tw + src) * a.n_kv_heads + kvh) * D, mean, R_plain, r);
+                    exact_rows(valid && !sure, [&](int src, const float (&r)[D / 32]) {
                         double s2 = 0.0;
 #pragma unroll
                         for (int j = 0; j < D / 32; ++j) s2 = fma((double)r[j], (double)r[j], s2);
@@ -531,14 +682,14 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                         float e = bf16_round((float)sqrt(s2 / (double)D));
                         if (!(e > 0.f) || !isfinite(e)) e = 1.f;
                         if (lane == src) rho = e;
-                    }
+                    });
                     if (!(rho > 0.f) || !isfinite(rho)) rho = 1.f;             // (lanes without a token)
                     inv_rho = __fdividef(1.f, rho);
                     bound *= inv_rho * 1.00001f;
                 }
                 // coefficients of this warpgroup's groups lb .. lb + ngh - 1 -> shared memory, [group][token][4]
                 const int lb = g0 + hf * ngh;
-                float4* const c_s = reinterpret_cast<float4*>(x_s) + (hf * (P::GU / 2)) * PF_HALF + row;
+                const uint32_t c_s = sb + P::OFF_X + xslot * P::SLOT_BYTES + (hf * (P::GU / 2) * PF_HALF + row) * 16;
 #pragma unroll 1
                 for (int g = 0; g < ngh; g += 4) {
                     float f[16];
@@ -549,22 +700,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                         const float4 m = *reinterpret_cast<const float4*>(mr + 4 * (lb + g + j));
                         float4 r = make_float4(f[4 * j] - m.x, f[4 * j + 1] - m.y, f[4 * j + 2] - m.z, f[4 * j + 3] - m.w);
                         if (ksc) { r.x *= inv_rho; r.y *= inv_rho; r.z *= inv_rho; r.w *= inv_rho; }
-                        c_s[(g + j) * PF_HALF] = r;
+                        sts_f4(c_s + (g + j) * (PF_HALF * 16), r);
                     }
                 }
-                // destination, second part (the page id has arrived by now)
-                if (named) {
-                    if (page < 0 || page >= a.n_pages) {
-                        atomicOr(a.dev_status, NOVAKV_DEV_BAD_PAGE);
-                        page = -1;
-                    } else if (sh == 0 && g0 == 0 && hf == 0) {
-                        atomicMax(&a.seq_lens[sq], pos + 1);
-                    }
-                }
-                const bool valid = page >= 0;
                 const int page0 = __shfl_sync(0xffffffffu, page, lane & 16), slot0 = __shfl_sync(0xffffffffu, slot, lane & 16);
                 const bool aligned = __all_sync(0xffffffffu, valid && page == page0 && (slot & 15) == (lane & 15) && (slot ^ slot0) < 16);
-                uint8_t* const chunk = pages + ((size_t)(valid ? page : 0) * a.n_kv_heads + kvh) * (NOVAKV_PAGE_TOKENS * L);
                 if (ksc && valid && g0 == 0 && hf == 0)
                     a.k_scales[((size_t)page * a.n_kv_heads + kvh) * NOVAKV_PAGE_TOKENS + slot] = __float2bfloat16_rn(rho);
                 if (vsq) {
@@ -581,7 +721,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                             mx = fmaxf(mx, v);
                         }
                     }
-                    const float err = bound * r_colmax + 1.2e-7f * fmaxf(fabsf(mn), fabsf(mx));
+                    const float err = bound * cst[D + 2 * L + 2] /* longest column */ + 1.2e-7f * fmaxf(fabsf(mn), fabsf(mx));
                     float zero = bf16_round(mn);
                     float scale = bf16_round(__fdiv_rn(__fsub_rn(mx, zero), 3.0f));
                     bool sure = bf16_round(mn - err) == zero && bf16_round(mn + err) == zero &&
@@ -607,17 +747,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                         word[qw] = wd;
                     }
                     tc_fence_before();
-                    nbar_sync(5 + w, PF_TILE);                                 // the accumulators are read out, the row slot is free
-                    if (lane == 0) {
-                        mbar_arrive(bar(B_XFREE + xslot));
-                        if (hf == 0) mbar_arrive(bar(B_TFREE + w));
-                    }
-                    unsigned todo = __ballot_sync(0xffffffffu, valid && !sure);
-                    while (todo) {
-                        const int src = __ffs(todo) - 1;
-                        todo &= todo - 1;
-                        float r[D / 32];
-                        exact_row<D>(x_new + ((size_t)(tw + src) * a.n_kv_heads + kvh) * D, mean, R_plain, r);
+                    exact_rows(valid && !sure, [&](int src, const float (&r)[D / 32]) {
                         float rmn = r[0], rmx = r[0];
 #pragma unroll
                         for (int j = 1; j < D / 32; ++j) { rmn = fminf(rmn, r[j]); rmx = fmaxf(rmx, r[j]); }
@@ -645,9 +775,14 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                             if (lane == src) word[qw] = wd;
                         }
                         if (lane == src) { zero = ez; scale = es; }
+                    });
+                    // (a barrier has passed: the accumulators are read out, the row slot is free)
+                    if (lane == 0) {
+                        mbar_arrive(bar(B_XFREE + xslot));
+                        if (hf == 0) mbar_arrive(bar(B_TFREE + w));
                     }
 #pragma unroll
-                    for (int qw = 0; qw < L / 8; ++qw) store_value_word<L>(chunk, slot, hf * (L / 2) + 4 * qw, word[qw], aligned, valid, lane);
+                    for (int qw = 0; qw < L / 8; ++qw) store_value_word<L>(chunk_of(page), slot, hf * (L / 2) + 4 * qw, word[qw], aligned, valid, lane);
                     if (valid && hf == 0)
                         reinterpret_cast<__nv_bfloat162*>(a.v_meta)[((size_t)page * a.n_kv_heads + kvh) * NOVAKV_PAGE_TOKENS + slot] =
                             __floats2bfloat162_rn(scale, zero);
@@ -656,174 +791,185 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                 tc_fence_before();
                 nbar_sync(5 + w, PF_TILE);                                     // the transform's accumulators are read out
 
-                // ---- search of groups lb .. lb + ngh - 1
-                // the coefficients of group g, and its search operand into shared memory
-                auto publish = [&](int g, float4& r, float& qq) {
-                    r = c_s[g * PF_HALF];
-                    const float sc = gscale[lb + g];
+                // ---- search of groups lb .. lb + ngh - 1.  The first chunk of the next group is computed behind the choice and
+                // the direct distances of this one.
+                const int use0 = n_use + hf;
+                // the search operand of group g into shared memory; |r|^2 in the group's scale
+                auto publish = [&](int g) -> float {
+                    const float4 r = lds_f4(c_s + g * (PF_HALF * 16));
+                    const float sc = cst[D + L + lb + g];
                     const float s0 = r.x * sc, s1 = r.y * sc, s2 = r.z * sc, s3 = r.w * sc;
-                    qq = fmaf(s0, s0, fmaf(s1, s1, fmaf(s2, s2, s3 * s3)));
+                    const float qq = fmaf(s0, s0, fmaf(s1, s1, fmaf(s2, s2, s3 * s3)));
                     const uint32_t h01 = pack_half2(s0, s1), h23 = pack_half2(s2, s3);
                     const float2 f01 = unpack_half2(h01), f23 = unpack_half2(h23);
                     const uint32_t l01 = pack_half2(s0 - f01.x, s1 - f01.y), l23 = pack_half2(s2 - f23.x, s3 - f23.y);
                     const float qh = 0.5f * qq, qhh = __half2float(__float2half_rn(qh));
                     const uint32_t qp = pack_half2(qhh, qh - qhh);
                     const uint32_t dst = a_s + row * 16;
-                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(h01), "r"(h23), "r"(h01), "r"(h23) : "memory");
+                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%1,%2};" ::"r"(dst), "r"(h01), "r"(h23) : "memory");
                     asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst + PF_HALF * 16), "r"(l01), "r"(l23), "r"(0x3c003c00u), "r"(qp) : "memory");
                     fence_proxy_async();
+                    return qq;
                 };
                 // The warp is done with the accumulators (and has written its operand rows); when the four warps of the
-                // warpgroup are, its first warp issues the distances of chunk c of the group in ring stage st.
-                const int use0 = n_use + hf;
+                // warpgroup are, its first warp issues the distances of chunk c of group g.
                 auto release_and_issue = [&](int c, int g) {
                     tc_fence_before();
                     if ((warp & 3) != 0) {
                         nbar_arrive(1 + wg, PF_HALF);
                     } else {
-                        const int use = use0 + 2 * g, st = use % PF_STAGES;
-                        if (c == 0) ok = ok && mbar_wait(bar(B_RING + st), (use / PF_STAGES) & 1, abort_flag);
+                        const int use = use0 + 2 * g, st = use % P::NOP;
+                        if (c == 0) mbar_wait<PF_TOK_NS>(bar(B_RING + st), (use / P::NOP) & 1, abort_flag);
                         nbar_sync(1 + wg, PF_HALF);
                         tc_fence_after();
                         if (elect_one()) {
                             umma_f16(d_s, umma_desc(a_s, PF_HALF * 16, 128, 0),
-                                     umma_desc(sb + P::OFF_RING + st * PF_STAGE_BYTES + c * 2048, 4096, 128, 0), umma_idesc(false, false, 128, 128), false);
+                                     umma_desc(sb + P::OFF_RING + st * PF_OP_BYTES + c * 2048, 4096, 128, 0), umma_idesc(false, false, 128, 128), false);
                             umma_commit(bar(B_S + wg));
                             if (c == 1) umma_commit(bar(B_RINGFREE + st));
                         }
                         __syncwarp();
                     }
                 };
-                float4 r, rn = make_float4(0.f, 0.f, 0.f, 0.f);                // coefficients of this group and the next
-                float q2, q2n = 0.f;                                           // |r|^2 in the group's scale
-                publish(0, r, q2);
+                // minima of 32 rows of 8 codewords, two rows per register.  (Distances are not negative, or tiny: their
+                // binary16 patterns compare like integers.  A negative one sorts below every positive one, and every negative
+                // row minimum passes the test below.)
+                uint32_t rmin[16];
+                auto minima = [&](int c, const uint32_t (&v)[32]) {
+#pragma unroll
+                    for (int qd = 0; qd < 4; ++qd)
+                        rmin[4 * c + qd] = __vimin3_s16x2(__vimin3_s16x2(v[8 * qd], v[8 * qd + 1], v[8 * qd + 2]),
+                                                          __vimin3_s16x2(v[8 * qd + 3], v[8 * qd + 4], v[8 * qd + 5]),
+                                                          __vmins2(v[8 * qd + 6], v[8 * qd + 7]));
+                };
+                auto accumulators = [&](int half, uint32_t (&v)[32]) {
+                    tmem_ld64_h2(d_s + lane_base + half * 64, v);
+                    tmem_wait_ld();
+                };
+                float q2 = publish(0);                                         // |r|^2 of this group, in its scale
                 release_and_issue(0, 0);
                 uint32_t codes = 0, pend = 0;
 #pragma unroll 1
                 for (int g = 0; g < ngh; ++g) {
-                    const int l = lb + g, use = use0 + 2 * g, st = use % PF_STAGES;
-                    uint32_t rmin[16];                                         // minima of 32 rows of 8 codewords, two per register
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        if ((c & 1) == 0) {
-                            ok = ok && mbar_wait(bar(B_S + wg), n_s & 1, abort_flag);
-                            ++n_s;
-                            tc_fence_after();
-                            __syncwarp();
-                        }
+                    {
+                        mbar_wait<PF_TOK_NS>(bar(B_S + wg), n_s & 1, abort_flag);
+                        ++n_s;
+                        tc_fence_after();
+                        __syncwarp();
                         uint32_t v[32];
-                        tmem_ld64_h2(d_s + lane_base + (c & 1) * 64, v);
-                        tmem_wait_ld();
-                        if (c == 1) {
-                            release_and_issue(1, g);
-                        } else if (c == 3) {
-                            if (g + 1 < ngh) {
-                                publish(g + 1, rn, q2n);
-                                release_and_issue(0, g + 1);
-                                if (g + 2 == ngh) {
-                                    __syncwarp();
-                                    if (lane == 0) mbar_arrive(bar(B_XFREE + xslot));      // the coefficients are read out
-                                }
-                            } else {
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0 && hf == 0) mbar_arrive(bar(B_TFREE + w));
-                            }
+                        accumulators(0, v);
+                        minima(0, v);
+                        accumulators(1, v);
+                        release_and_issue(1, g);
+                        minima(1, v);
+                    }
+                    {
+                        float q2n = 0.f;
+                        mbar_wait<PF_TOK_NS>(bar(B_S + wg), n_s & 1, abort_flag);
+                        ++n_s;
+                        tc_fence_after();
+                        __syncwarp();
+                        uint32_t v[32];
+                        accumulators(0, v);
+                        minima(2, v);
+                        accumulators(1, v);
+                        if (g + 1 < ngh) {
+                            q2n = publish(g + 1);
+                            release_and_issue(0, g + 1);
+                        } else {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0 && hf == 0) mbar_arrive(bar(B_TFREE + w));
                         }
-                        // (distances are not negative, or tiny: their binary16 patterns compare like integers.  A negative
-                        // one sorts below every positive one, and every negative row minimum passes the test below.)
+                        minima(3, v);
+                        float mf;
+                        {
+                            uint32_t m = __vimin3_s16x2(__vimin3_s16x2(rmin[0], rmin[1], rmin[2]), __vimin3_s16x2(rmin[3], rmin[4], rmin[5]),
+                                                        __vimin3_s16x2(rmin[6], rmin[7], rmin[8]));
+                            m = __vimin3_s16x2(m, __vimin3_s16x2(rmin[9], rmin[10], rmin[11]), __vimin3_s16x2(rmin[12], rmin[13], rmin[14]));
+                            const float2 f = unpack_half2(__vmins2(m, rmin[15]));
+                            mf = fminf(f.x, f.y);
+                            if (!(f.x == f.x) || !(f.y == f.y)) mf = CUDART_INF_F;
+                        }
+                        // A row can hold the nearest codeword only if its binary16 minimum is at most t: the rounding of two
+                        // binary16 numbers (2^-11 each; below their normal range 2^-25, also of the operands), the error of the
+                        // product (EPS_S) for both, and what the error of the coefficient moves the difference of two distances by.
+                        const float4 r = lds_f4(c_s + g * (PF_HALF * 16));
+                        if (g + 1 == ngh) {
+                            __syncwarp();
+                            mbar_arrive_lane0(bar(B_XFREE + xslot), lane);  // the coefficients are read out
+                        }
+                        const float rlen2 = fmaf(r.x, r.x, fmaf(r.y, r.y, fmaf(r.z, r.z, r.w * r.w)));
+                        const float delta = fmaf(bound, cst[D + lb + g], (ksc ? 3.0e-7f : 6.0e-8f) * sqrt_approx(rlen2));
+                        const float dl = delta * cst[D + L + lb + g], sq2 = sqrt_approx(2.f * fmaxf(mf, 0.f));
+                        const float s2 = fmaf(1.1f, sq2, 2.f * sqrt_approx(q2));
+                        float t = fmaf(2.1f * EPS_S, s2 * s2, fmaf(fmaxf(mf, 0.f), 1.0025f, 2.5f * dl * (sq2 + dl) + 4.0e-7f));
+                        t *= 1.0005f;
+                        const uint32_t t1 = pack_half2(t, t);
+                        uint32_t bits = 0;
 #pragma unroll
-                        for (int qd = 0; qd < 4; ++qd)
-                            rmin[4 * c + qd] = __vimin3_s16x2(__vimin3_s16x2(v[8 * qd], v[8 * qd + 1], v[8 * qd + 2]),
-                                                              __vimin3_s16x2(v[8 * qd + 3], v[8 * qd + 4], v[8 * qd + 5]),
-                                                              __vmins2(v[8 * qd + 6], v[8 * qd + 7]));
-                    }
-                    float mf;
-                    {
-                        uint32_t m = __vimin3_s16x2(__vimin3_s16x2(rmin[0], rmin[1], rmin[2]), __vimin3_s16x2(rmin[3], rmin[4], rmin[5]),
-                                                    __vimin3_s16x2(rmin[6], rmin[7], rmin[8]));
-                        m = __vimin3_s16x2(m, __vimin3_s16x2(rmin[9], rmin[10], rmin[11]), __vimin3_s16x2(rmin[12], rmin[13], rmin[14]));
-                        const float2 f = unpack_half2(__vmins2(m, rmin[15]));
-                        mf = fminf(f.x, f.y);
-                        if (!(f.x == f.x) || !(f.y == f.y)) mf = CUDART_INF_F;
-                    }
-                    // A row can hold the nearest codeword only if its binary16 minimum is at most t: the rounding of two
-                    // binary16 numbers (2^-11 each; below their normal range 2^-25, also of the operands), the error of the
-                    // product (EPS_S) for both, and what the error of the coefficient moves the difference of two distances by.
-                    const float rlen2 = fmaf(r.x, r.x, fmaf(r.y, r.y, fmaf(r.z, r.z, r.w * r.w)));
-                    const float delta = fmaf(bound, rnorm[l], (ksc ? 3.0e-7f : 6.0e-8f) * sqrt_approx(rlen2));
-                    const float dl = delta * gscale[l], sq2 = sqrt_approx(2.f * fmaxf(mf, 0.f)), rl = sqrt_approx(q2);
-                    const float s2 = 2.f * rl + 1.1f * sq2;
-                    float t = fmaf(2.1f * EPS_S, s2 * s2, fmaf(fmaxf(mf, 0.f), 1.0025f, 2.5f * dl * (sq2 + dl) + 4.0e-7f));
-                    t *= 1.0005f;
-                    const uint32_t t1 = pack_half2(t, t);
-                    uint32_t bits = 0;
+                        for (int k = 0; k < 16; ++k) {
+                            const uint32_t le = __hle2_mask(*reinterpret_cast<const __half2*>(&rmin[k]), *reinterpret_cast<const __half2*>(&t1));
+                            bits |= le & (0x00010001u << k);
+                        }
+                        bool exact = !(mf < 60000.f) || bits == 0u;
+                        // Direct binary32 distances of the rows that are left, two codewords per operation.  A lane reads
+                        // the 8 chunks of its row in the order j ^ (lane % 8), so that the 8 lanes of a quarter warp read 8
+                        // different 16-byte columns: odd lanes meet the chunk of components 2, 3 first.  The low 3 bits of a
+                        // distance are replaced by the codeword's number in the row.
+                        const int l = lb + g, use = use0 + 2 * g, st = use % PF_CW_STAGES;
+                        const uint32_t rows = exact ? 0u : bits;               // (a void ranking leaves every row)
+                        uint32_t best = 0x7f800000u, second = 0x7f800000u;
+                        int brow = 0;
+                        mbar_wait<PF_TOK_NS>(bar(B_CW + st), (use / PF_CW_STAGES) & 1, abort_flag);
+                        __syncwarp();
+                        const uint32_t cb = sb + P::OFF_CW + st * PF_CW_BYTES;
+                        {
+                            const bool odd = lane & 1;
+                            const uint64_t ra0 = dup2(odd ? r.z : r.x), ra1 = dup2(odd ? r.w : r.y);
+                            const uint64_t rb0 = dup2(odd ? r.x : r.z), rb1 = dup2(odd ? r.y : r.w);
+                            do {
+                                const int k = bits ? __ffs(bits) - 1 : 0;
+                                const bool take = bits != 0u;
+                                const int rowi = ((k & 15) << 1) | (k >> 4);
+                                const uint32_t base = cb + rowi * 128;
+                                uint32_t key[8];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const uint32_t le = __hle2_mask(*reinterpret_cast<const __half2*>(&rmin[k]), *reinterpret_cast<const __half2*>(&t1));
-                        bits |= le & (0x00010001u << k);
-                    }
-                    bool exact = !(mf < 60000.f) || bits == 0u;
-                    // Direct binary32 distances of the rows that are left, two codewords per operation.  A lane reads the 8
-                    // chunks of its row in the order j ^ (lane % 8), so that the 8 lanes of a quarter warp read 8 different
-                    // 16-byte columns: odd lanes meet the chunk of components 2, 3 first.  The low 3 bits of a distance are
-                    // replaced by the codeword's number in the row.
-                    uint32_t best = 0x7f800000u, second = 0x7f800000u;
-                    int brow = 0;
-                    ok = ok && mbar_wait(bar(B_RING + st), (use / PF_STAGES) & 1, abort_flag);
-                    __syncwarp();
-                    const uint32_t cb = sb + P::OFF_RING + st * PF_STAGE_BYTES + 8192;
-                    {
-                        const bool odd = lane & 1;
-                        const uint64_t ra0 = dup2(odd ? r.z : r.x), ra1 = dup2(odd ? r.w : r.y);
-                        const uint64_t rb0 = dup2(odd ? r.x : r.z), rb1 = dup2(odd ? r.y : r.w);
-                        do {
-                            const int k = bits ? __ffs(bits) - 1 : 0;
-                            const bool take = bits != 0u;
-                            const int rowi = ((k & 15) << 1) | (k >> 4);
-                            const uint32_t base = cb + rowi * 128;
-                            uint32_t key[8];
+                                for (int p = 0; p < 4; ++p) {
+                                    uint64_t a0, a1, b0, b1;
+                                    asm volatile("ld.shared.v2.u64 {%0,%1}, [%2];" : "=l"(a0), "=l"(a1) : "r"(base + (((2 * p) ^ lx) * 16)));
+                                    asm volatile("ld.shared.v2.u64 {%0,%1}, [%2];" : "=l"(b0), "=l"(b1) : "r"(base + (((2 * p + 1) ^ lx) * 16)));
+                                    a0 = f2_sub(ra0, a0); a1 = f2_sub(ra1, a1); b0 = f2_sub(rb0, b0); b1 = f2_sub(rb1, b1);
+                                    const uint64_t d = f2_fma(b1, b1, f2_fma(b0, b0, f2_fma(a1, a1, f2_mul(a0, a0))));
+                                    key[2 * p] = ((uint32_t)d & ~7u) | (2 * p);
+                                    key[2 * p + 1] = ((uint32_t)(d >> 32) & ~7u) | (2 * p + 1);
+                                }
+                                // two smallest of the 8: pairs, then merges
+                                uint32_t lo[4], hi[4];
 #pragma unroll
-                            for (int p = 0; p < 4; ++p) {
-                                uint64_t a0, a1, b0, b1;
-                                asm volatile("ld.shared.v2.u64 {%0,%1}, [%2];" : "=l"(a0), "=l"(a1) : "r"(base + (((2 * p) ^ lx) * 16)));
-                                asm volatile("ld.shared.v2.u64 {%0,%1}, [%2];" : "=l"(b0), "=l"(b1) : "r"(base + (((2 * p + 1) ^ lx) * 16)));
-                                a0 = f2_sub(ra0, a0); a1 = f2_sub(ra1, a1); b0 = f2_sub(rb0, b0); b1 = f2_sub(rb1, b1);
-                                const uint64_t d = f2_fma(b1, b1, f2_fma(b0, b0, f2_fma(a1, a1, f2_mul(a0, a0))));
-                                key[2 * p] = ((uint32_t)d & ~7u) | (2 * p);
-                                key[2 * p + 1] = ((uint32_t)(d >> 32) & ~7u) | (2 * p + 1);
-                            }
-                            // two smallest of the 8: pairs, then merges
-                            uint32_t lo[4], hi[4];
+                                for (int p = 0; p < 4; ++p) { lo[p] = min(key[2 * p], key[2 * p + 1]); hi[p] = max(key[2 * p], key[2 * p + 1]); }
 #pragma unroll
-                            for (int p = 0; p < 4; ++p) { lo[p] = min(key[2 * p], key[2 * p + 1]); hi[p] = max(key[2 * p], key[2 * p + 1]); }
-#pragma unroll
-                            for (int p = 0; p < 4; p += 2) {
-                                hi[p] = __vimin3_u32(max(lo[p], lo[p + 1]), hi[p], hi[p + 1]);
-                                lo[p] = min(lo[p], lo[p + 1]);
-                            }
-                            hi[0] = __vimin3_u32(max(lo[0], lo[2]), hi[0], hi[2]);
-                            lo[0] = min(lo[0], lo[2]);
-                            if (take) {
-                                second = __vimin3_u32(max(best, lo[0]), second, hi[0]);
-                                if (lo[0] < best) { best = lo[0]; brow = rowi; }
-                            }
-                            bits &= bits - 1;
-                        } while (__any_sync(0xffffffffu, bits != 0u));
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(B_RINGFREE + st));
-                    const int bi = brow * 8 + (int)((best & 7u) ^ (lx & 6));
-                    // where the two nearest codewords are closer than the errors can resolve, the search is repeated in binary64
-                    exact |= needs_exact_search(__uint_as_float(best & ~7u), __uint_as_float(second | 7u), delta, KEY_REL);
-                    codes = (codes >> 8) | ((uint32_t)bi << 24);
-                    pend = (pend >> 1) | (exact && valid ? 8u : 0u);
-                    if ((l & 3) == 3) {
-                        if (side == 0) { if (valid) store_key_word<L>(chunk, slot, l - 3, codes); }
-                        else store_value_word<L>(chunk, slot, l - 3, codes, aligned, valid, lane);
-                        // binary64 searches of the four groups: to the helper's queue, or here when it is full
-                        unsigned todo;
-                        while ((todo = __ballot_sync(0xffffffffu, pend != 0u)) != 0u) {
+                                for (int p = 0; p < 4; p += 2) {
+                                    hi[p] = __vimin3_u32(max(lo[p], lo[p + 1]), hi[p], hi[p + 1]);
+                                    lo[p] = min(lo[p], lo[p + 1]);
+                                }
+                                hi[0] = __vimin3_u32(max(lo[0], lo[2]), hi[0], hi[2]);
+                                lo[0] = min(lo[0], lo[2]);
+                                if (take) {
+                                    second = __vimin3_u32(max(best, lo[0]), second, hi[0]);
+                                    if (lo[0] < best) { best = lo[0]; brow = rowi; }
+                                }
+                                bits &= bits - 1;
+                            } while (__any_sync(0xffffffffu, bits != 0u));
+                        }
+                        __syncwarp();
+                        mbar_arrive_lane0(bar(B_CWFREE + st), lane);
+                        const int bi = brow * 8 + (int)((best & 7u) ^ (lx & 6));
+                        // where the two nearest codewords are closer than the errors can resolve, the search is repeated in binary64
+                        exact |= needs_exact_search(__uint_as_float(best & ~7u), __uint_as_float(second | 7u), delta, KEY_REL);
+                        unsigned todo = __ballot_sync(0xffffffffu, exact && valid);
+                        if (todo) {
+                            // to the helper's queue, or here when that is full
                             const int h = warp & (PF_HELPERS - 1), n = __popc(todo);
                             int base = -1;
                             if (lane == 0) {
@@ -831,31 +977,44 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
                                 else atomicSub(&s_count[h], n);
                             }
                             base = __shfl_sync(0xffffffffu, base, 0);
-                            const int lq = l - 3 + (pend ? __ffs(pend) - 1 : 0);
                             if (base >= 0) {
-                                if (pend) {
+                                if ((todo >> lane) & 1u) {
                                     volatile uint32_t* e = reinterpret_cast<volatile uint32_t*>(smem + P::OFF_QUEUE) +
                                                            (h * PF_QUEUE + (base + __popc(todo & ((1u << lane) - 1))) % PF_QUEUE) * 4;
-                                    e[1] = (uint32_t)tkn; e[2] = (uint32_t)page; e[3] = __float_as_uint(rho);
+                                    e[1] = (uint32_t)tkn; e[2] = (uint32_t)page; e[3] = rows;
                                     __threadfence_block();
-                                    e[0] = 0x80000000u | ((uint32_t)slot << 6) | (uint32_t)lq;
+                                    e[0] = (__float_as_uint(rho) & 0xffff0000u) | 0x8000u | ((uint32_t)slot << 6) | (uint32_t)l;
                                 }
                             } else {
                                 while (todo) {
                                     const int src = __ffs(todo) - 1;
                                     todo &= todo - 1;
-                                    const int ls = __shfl_sync(0xffffffffu, lq, src);
-                                    const int res = exact_search_token<D>(x_new + ((size_t)(tw + src) * a.n_kv_heads + kvh) * D, mean, R_plain, ls,
-                                                                          cb_g + ls * NOVAKV_C, __shfl_sync(0xffffffffu, rho, src));
-                                    if (lane == src) chunk[side == 0 ? novakv_k_offset<L>(slot, ls) : novakv_v_offset<L>(slot, ls)] = (uint8_t)res;
+                                    const int res = exact_search_token<D>(a, side, kvh, tw + src, l, __shfl_sync(0xffffffffu, rho, src),
+                                                                          __shfl_sync(0xffffffffu, rows, src));
+                                    if (lane == src) chunk_of(page)[side == 0 ? novakv_k_offset<L>(slot, l) : novakv_v_offset<L>(slot, l)] = (uint8_t)res;
                                 }
                             }
-                            pend &= pend - 1;
-                            __syncwarp();
                         }
+                        codes = (codes >> 8) | ((uint32_t)bi << 24);
+                        pend = (pend >> 1) | (exact && valid ? 8u : 0u);
+                        if ((l & 3) == 3) {
+                            if (__any_sync(0xffffffffu, pend != 0u)) {
+                                // single bytes: those that are searched again are written by the search alone
+                                if (valid) {
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k)
+                                        if (!((pend >> k) & 1u))
+                                            chunk_of(page)[side == 0 ? novakv_k_offset<L>(slot, l - 3 + k) : novakv_v_offset<L>(slot, l - 3 + k)] =
+                                                (uint8_t)(codes >> (8 * k));
+                                }
+                            } else if (side == 0) {
+                                if (valid) store_key_word<L>(chunk_of(page), slot, l - 3, codes);
+                            } else {
+                                store_value_word<L>(chunk_of(page), slot, l - 3, codes, aligned, valid, lane);
+                            }
+                        }
+                        q2 = q2n;
                     }
-                    r = rn;
-                    q2 = q2n;
                 }
                 n_use += 2 * ngh;
             }
@@ -869,6 +1028,27 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const Pre
     }
     if (warp == 0) tmem_dealloc<512>(tmem);
     if (threadIdx.x == 0 && misc[1] != 0) atomicOr(a.dev_status, NOVAKV_DEV_WAIT_TIMEOUT);
+}
+
+// Tensor map of [n_tokens][row] bfloat16 with boxes of 64 columns (128 bytes, swizzled) x 128 rows.
+bool row_map(CUtensorMap* map, const void* base, int n_tokens, int row) {
+    using encode_fn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const encode_fn encode = []() -> encode_fn {                 // (the driver's entry point, looked up once)
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return reinterpret_cast<encode_fn>(fn);
+    }();
+    if (encode == nullptr) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)row, (cuuint64_t)n_tokens}, strides[1] = {(cuuint64_t)row * 2};
+    const cuuint32_t box[2] = {64, PF_HALF}, step[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int D, int FMT>
@@ -887,20 +1067,21 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
     double best = 1e30;
     int grid = 1;
     for (int gs = L / P::GU; gs <= L / 8; gs *= 2) {
-        const double ck = PF_US_UNIT + PF_US_GROUP * (L / gs), cv = FMT == 2 ? PF_US_INT2 : ck;
+        const double cp = PF_US_UNIT + PF_US_GROUP * (L / gs), ck = cp + (FMT ? PF_US_SCALED : 0.0), cv = FMT == 2 ? PF_US_INT2 : cp;
         const int uk = hkv * gs * n_tiles, uv = FMT == 2 ? hkv * n_tiles : uk;
         const int g = uk + uv < ctx->n_sm ? uk + uv : ctx->n_sm;
-        double longest = (uk * ck + uv * cv) / g;
-        if (longest < ck) longest = ck;
-        const double n_k = ceil(longest / ck - 1e-6);                          // units are whole
-        if (n_k * ck < best) {
-            best = n_k * ck;
+        const double even = (uk * ck + uv * cv) / g, longest = ck * ceil(even / ck - 1e-6);       // units are whole
+        if (longest < best) {
+            best = longest;
             grid = g;
             a.gs = gs;
             a.cost_k = (int)(ck * 64.0);
             a.cost_v = (int)(cv * 64.0);
         }
     }
+    // tensor maps of the new rows (rebuilt on every call: the buffers are the caller's)
+    a.tma = (((uintptr_t)a.k_new | (uintptr_t)a.v_new) & 15) == 0 &&
+            row_map(&a.map_k, a.k_new, a.n_tokens, hkv * D) && row_map(&a.map_v, a.v_new, a.n_tokens, hkv * D);
     novakv_prof_scope ps(ctx, 1, stream);
     kern<<<grid, PF_THREADS, P::BYTES, stream>>>(a);
     ps.end();
@@ -914,9 +1095,9 @@ novakv_status novakv_launch_prefill(novakv_ctx* ctx, const novakv_layer& ly, con
     const int32_t* tok_seq, const int32_t* tok_pos, int n_tokens, uint8_t* k_pages, uint8_t* v_pages, int n_pages,
     const int32_t* page_table, int max_pages_per_seq, int n_seq, int32_t* seq_lens, cudaStream_t stream, __nv_bfloat16* k_scales,
     __nv_bfloat16* v_meta) {
-    const PrefillArgs a = {k_new, v_new, tok_seq, tok_pos, n_tokens, ly.pf_r, ly.pf_cb, ly.pf_const, ly.rk_d, ly.rv_d, ly.k_mean_d,
+    PrefillArgs a = {k_new, v_new, tok_seq, tok_pos, n_tokens, ly.pf_r, ly.pf_cb, ly.pf_const, ly.rk_d, ly.rv_d, ly.rk_rows, ly.rv_rows, ly.k_mean_d,
                            ly.v_mean_d, ly.cb_k, ly.cb_v, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
-                           n_seq, seq_lens, ctx->cfg.n_kv_heads, 1, 1, 1, ctx->dev_status};
+                           n_seq, seq_lens, ctx->cfg.n_kv_heads, 1, 1, 1, 0, ctx->dev_status, {}, {}};
     if (ctx->cfg.head_dim == 128)
         return v_meta ? launch_prefill_t<128, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<128, 1>(ctx, a, stream) : launch_prefill_t<128, 0>(ctx, a, stream));
     return v_meta ? launch_prefill_t<64, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<64, 1>(ctx, a, stream) : launch_prefill_t<64, 0>(ctx, a, stream));

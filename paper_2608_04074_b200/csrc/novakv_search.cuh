@@ -9,6 +9,8 @@
 // distances (both have moved) with some slack on the constants.  key_rel: what the caller's packing of the distances
 // has cut from either of them, relative.
 __device__ __forceinline__ bool needs_exact_search(float best, float second, float delta, float key_rel = 0.f) {
-    const float thr = 4.5f * sqrtf(second) * delta + 2.5f * delta * delta + (9.6e-7f + 2.f * key_rel) * second;     // 9.6e-7 > 16 * 2^-24
+    float root;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(root) : "f"(second));          // (the slack covers its error)
+    const float thr = 4.5f * root * delta + 2.5f * delta * delta + (9.6e-7f + 2.f * key_rel) * second;     // 9.6e-7 > 16 * 2^-24
     return !(second - best > thr);
 }

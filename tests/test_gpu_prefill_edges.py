@@ -29,7 +29,7 @@ def cases():
     return {(n, s): _make(n, s) for n in ("qwen", "gptoss") for s in (False, True)}
 
 
-def _run(case, fmt, n, start, permute, holes, scale=1.0):
+def _run(case, fmt, n, start, permute, holes, scale=1.0, offset=0):
     from paper_2608_04074_b200.runtime import PagedCache
     k, v, _ = case.draw(4000 + n, n, 1)
     k, v = (synth.to_bf16_representable(x * scale) for x in (k, v))
@@ -42,7 +42,11 @@ def _run(case, fmt, n, start, permute, holes, scale=1.0):
         used[::7] = False
         seq[~used] = -1
     order = synth.rng(3).permutation(n) if permute else np.arange(n)
-    cache.append(0, _dev(k[order], torch.bfloat16), _dev(v[order], torch.bfloat16), _dev(seq[order]), _dev(pos[order]))
+    kd, vd = (_dev(x[order], torch.bfloat16) for x in (k, v))
+    if offset:                                   # rows that start `offset` elements off a 16-byte boundary
+        kd, vd = (torch.cat([x.new_zeros(offset), x.flatten()])[offset:].view(x.shape) for x in (kd, vd))
+        assert kd.data_ptr() % 16 == 2 * offset
+    cache.append(0, kd, vd, _dev(seq[order]), _dev(pos[order]))
     assert case.ctx.novakv_last_device_status() == 0
     assert int(cache.seq_lens[0]) == start + int(np.flatnonzero(used)[-1]) + 1 and int(cache.seq_lens[1]) == 0
     gk, gv = cache.load_logical(0, start, n)
@@ -82,3 +86,9 @@ def test_prefill_far_from_the_codebook(cases, name, scale):
     """Inputs a thousand times smaller and 64 times larger than the calibration's (and all zero): the binary16 ranking
     is then dominated by rounding, or out of its range, and every decision rests on the exact re-search."""
     _run(cases[name, False], "plain", 300, 0, False, False, scale)
+
+
+@pytest.mark.parametrize("name", ["qwen", "gptoss"])
+def test_prefill_rows_without_tensor_map_alignment(cases, name):
+    """New rows on a 4-byte boundary cannot be copied by a tensor map: the plain copies must give the same indices."""
+    _run(cases[name, False], "plain", 600, 0, False, False, offset=2)
