@@ -263,8 +263,10 @@ __device__ __forceinline__ void search_tile(const float* r_s, const float4* cb_s
 // Append-sized batches (a decode step appends one token per sequence): the prompt encoder would
 // pad every (head, side) to a 256-token tile.  Here one warp owns one
 // group of one (head, side) and stages only its 4 columns of the transform (4 KB of binary64) and its
-// group's codebook (4 KB), so the work spreads over L/4 * Hkv * 2 CTAs.  A pass covers tp tokens
-// (tp = 1, 2, ... 32, the smallest power of two that holds the batch, at most 32): lane = grp * tp + token.
+// group's codebook (4 KB), so the work spreads over L/4 * Hkv * 2 CTAs per chunk of the token list.  A pass covers tp
+// tokens (tp = 1, 2, 4, 8, the smallest power of two that holds the batch, at most 8): lane = grp * tp + token.
+// Chunk c of n takes the passes c, c + n, ...: batches of more than 8 tokens get as many chunks as CTAs fit on the
+// machine at once (128 tokens, d = 128: 30.5 us with one CTA per four groups and four passes of 32 tokens).
 // The 32 / tp lane groups of a token share its transform (each takes one block of the input dimension, at most 8
 // blocks; a butterfly adds the partial sums, so every lane holds the same coefficients) and search disjoint
 // ranges of the codebook; their minima are merged with the lowest index winning ties.
@@ -301,8 +303,10 @@ __device__ __forceinline__ int exact_search_warp(const double (&rd)[4], const fl
     return bi;
 }
 
+constexpr int SMALL_CTAS_PER_SM = 5;             // (shared memory allows six at d = 128; five leave a thread 96 registers)
+constexpr int SMALL_TP_LOG2 = 3;
 template <int D, int FMT>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, SMALL_CTAS_PER_SM)
 novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
                            const int32_t* __restrict__ tok_seq, const int32_t* __restrict__ tok_pos, int n_tokens,
                            int tp_log2,
@@ -325,7 +329,8 @@ novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_b
     __shared__ double ss_s[4][32];                  // KSC: sum of squares of a warp's 4 coefficients, per token of the pass
     __shared__ float mx_s[4][32];                   // VSQ: maximum of a warp's 4 value coefficients (the minimum rides in ss_s)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int l = blockIdx.x * 4 + warp, kvh = blockIdx.y, side = blockIdx.z;
+    const int l = blockIdx.x * 4 + warp, kvh = blockIdx.y, side = blockIdx.z & 1;
+    const int chunk = blockIdx.z >> 1, n_chunks = gridDim.z >> 1;
     const __nv_bfloat16* x_new = side == 0 ? k_new : v_new;
     const double* R = (side == 0 ? rk_d : rv_d) + (size_t)kvh * D * D;
     const double* mean = (side == 0 ? k_mean_d : v_mean_d) + (size_t)kvh * D;
@@ -374,18 +379,19 @@ novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_b
     // (at most 8 blocks), and a butterfly over the lane groups adds the partial sums
     const int ts_log2 = min(5 - tp_log2, 3);
     const int part = grp & ((1 << ts_log2) - 1);
-    const int per = (D / 8) >> ts_log2;             // 16-byte chunks of the token row per lane (>= 1)
+    constexpr int PER_MAX = (D / 8) >> (5 - SMALL_TP_LOG2);
+    const int per = (D / 8) >> ts_log2;             // 16-byte chunks of the token row per lane (1 .. PER_MAX)
 
-    for (int t0 = 0; t0 < n_tokens; t0 += tp) {
+    for (int t0 = chunk * tp; t0 < n_tokens; t0 += n_chunks * tp) {
         const int tkn = t0 + tok_in_pass;
         const bool in_range = tkn < n_tokens;
         int s = -1, pos = 0;
         if (in_range) { s = tok_seq[tkn]; pos = tok_pos[tkn]; }
         // this lane's block of its token's row (the loads are in flight together with the token list's)
-        uint4 xr[D / 8];
+        uint4 xr[PER_MAX];
         const uint4* xrow = reinterpret_cast<const uint4*>(x_new + ((size_t)(in_range ? tkn : 0) * n_kv_heads + kvh) * D) + part * per;
 #pragma unroll
-        for (int c = 0; c < D / 8; ++c)
+        for (int c = 0; c < PER_MAX; ++c)
             if (c < per) xr[c] = xrow[c];
         // a pass whose entries are all unused does nothing (the same decision in every warp and CTA: it depends
         // on the token list alone)
@@ -401,7 +407,7 @@ novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_b
         // pairwise (neighbours first); all lanes of a token end with the same bits
         double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0, acc3 = 0.0;
 #pragma unroll
-        for (int c = 0; c < D / 8; ++c) {
+        for (int c = 0; c < PER_MAX; ++c) {
             if (c < per) {
                 const __nv_bfloat16* xb = reinterpret_cast<const __nv_bfloat16*>(&xr[c]);
 #pragma unroll
@@ -577,7 +583,7 @@ novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_b
 #ifdef NOVAKV_TIMING
     NOVAKV_ETICK(5)
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_a1));
-    if (threadIdx.x == 0 && blockIdx.y == 0 && (blockIdx.x == 0 || blockIdx.x == gridDim.x - 1))
+    if (threadIdx.x == 0 && blockIdx.y == 0 && blockIdx.z < 2 && (blockIdx.x == 0 || blockIdx.x == gridDim.x - 1))
         printf("append cta (%d,%d,%d) clocks: constants %lld dependency wait %lld rows+lookup %lld transform %lld ranking %lld merge %lld certificate+re-search %lld (%lld re-searches) store %lld | ns start %llu end %llu\n",
                blockIdx.x, blockIdx.y, blockIdx.z, tm[0], tm[1], tm[2], tm[3], tm[6], tm[7], tm[4], tm[8], tm[5], g_a0, g_a1);
 #endif
@@ -623,10 +629,13 @@ novakv_status launch_encode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
                               const int32_t* page_table, int max_pages_per_seq, int n_seq, int32_t* seq_lens,
                               cudaStream_t stream, __nv_bfloat16* k_scales, __nv_bfloat16* v_meta) {
     if (n_tokens <= NOVAKV_SMALL_APPEND_TOKENS) {
-        dim3 grid(D / NOVAKV_G / 4, ctx->cfg.n_kv_heads, 2);
-        novakv_prof_scope ps(ctx, 1, stream);
         int tp_log2 = 0;
-        while ((1 << tp_log2) < n_tokens && tp_log2 < 5) ++tp_log2;
+        while ((1 << tp_log2) < n_tokens && tp_log2 < SMALL_TP_LOG2) ++tp_log2;
+        // chunks of the token list: as many as there are passes, while all CTAs are resident together
+        const int passes = (n_tokens + (1 << tp_log2) - 1) >> tp_log2, per_chunk = D / NOVAKV_G / 4 * ctx->cfg.n_kv_heads * 2;
+        const int chunks = max(1, min(passes, SMALL_CTAS_PER_SM * ctx->n_sm / per_chunk));
+        dim3 grid(D / NOVAKV_G / 4, ctx->cfg.n_kv_heads, 2 * chunks);
+        novakv_prof_scope ps(ctx, 1, stream);
         auto small = v_meta ? novakv_encode_small_kernel<D, 2>
                             : (k_scales ? novakv_encode_small_kernel<D, 1> : novakv_encode_small_kernel<D, 0>);
         if (k_scales == nullptr) {

@@ -92,3 +92,10 @@ def test_prefill_far_from_the_codebook(cases, name, scale):
 def test_prefill_rows_without_tensor_map_alignment(cases, name):
     """New rows on a 4-byte boundary cannot be copied by a tensor map: the plain copies must give the same indices."""
     _run(cases[name, False], "plain", 600, 0, False, False, offset=2)
+
+
+@pytest.mark.parametrize("n", [24, 41, 100, 256])
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "plain"), ("qwen", "scaled"), ("gptoss", "deployed")])
+def test_append_batches_of_several_chunks(cases, name, fmt, n):
+    """Batches that still take the append kernel but span several of its passes and chunks of the token list."""
+    _run(cases[name, fmt != "plain"], fmt, n, 40, True, n == 100)
