@@ -127,8 +127,11 @@ __device__ __forceinline__ int clamp_len(int len, int max_pages) {
 // ------------------------------------------------------------------------------------------------
 // prepare: query transform + page prefix
 // ------------------------------------------------------------------------------------------------
-// One block per (sequence, KV head): the Hg queries of the head share every load of rk_inv_t.
-// 512 threads = D columns x (512/D) row parts; each thread's loads are independent and all in flight.
+// One block per KV head and run of `seqs_per_block` sequences: its share of rk_inv_t is read once into registers, and the
+// Hg queries of a (sequence, head) share it.  512 threads = D columns x (512/D) row parts; each thread's loads are
+// independent and all in flight.  Small batches take one sequence per block (latency); once there are more pairs than the
+// machine holds blocks, runs save the 64 KB per pair that re-reading the transform costs: 128 sequences x 8 heads,
+// d = 128: 13.5 -> 8.2 us.
 template <int D, int HG>
 __global__ void __launch_bounds__(512)
 novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict__ rk_inv_t,
@@ -139,14 +142,15 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
                       int32_t* __restrict__ cost_prefix /* [batch + 1] */, int seg_weight,
                       const float* __restrict__ k_center /* [Hkv][D], transform domain */, float* __restrict__ qc /* [batch][Hq] or null */,
                       int32_t* __restrict__ pair_count /* [Hkv * batch] arrival counters of the fused merge, or null */,
-                      void* __restrict__ out_fused /* outputs, when the scan kernel itself merges */, int out_is_fp32) {
+                      void* __restrict__ out_fused /* outputs, when the scan kernel itself merges */, int out_is_fp32,
+                      int seqs_per_block) {
     const int blk = blockIdx.x;
 #ifdef NOVAKV_TIMING
     unsigned long long g_p0, g_p1;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_p0));
 #endif
     constexpr int PARTS = 512 / D, ROWS = D / PARTS;
-    const int b = blk / n_kv_heads, kvh = blk - b * n_kv_heads;
+    const int run = blk / n_kv_heads, kvh = blk - run * n_kv_heads;
     const int c = threadIdx.x % D, part = threadIdx.x / D;
     // The query transform depends on nothing the preceding kernel of the stream (normally the append of this
     // step's tokens) writes: queries are produced before that kernel started, the transform is a constant.  So
@@ -154,12 +158,12 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
     // kernel.  Only the block that forms the page prefix (it reads seq_lens, which an append updates) waits;
     // since a grid completes only when all its blocks have, the scan kernel's own wait still covers both.
     float rv[ROWS];
-    if (blk < batch * n_kv_heads) {
+    if (blk < (int)gridDim.x - 1) {
         const float* R = rk_inv_t + (size_t)kvh * D * D + (size_t)part * ROWS * D + c;
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) rv[r] = R[(size_t)r * D];
     }
-    if (blk == batch * n_kv_heads) {
+    if (blk == (int)gridDim.x - 1) {
         novakv_grid_dependency_wait();
         // exclusive prefix over sequences of their page counts; small, done by one warp.  Beside it the same
         // prefix in "cost" units, in which every non-empty sequence weighs seg_weight pages more: the scan
@@ -211,57 +215,61 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
         return;
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (pair_count != nullptr && threadIdx.x == 0) pair_count[kvh * batch + b] = 0;
     __shared__ float q_s[HG][D];
     __shared__ float red_s[PARTS][HG][D];
-    for (int i = threadIdx.x; i < HG * D; i += 512)
-        q_s[i / D][i % D] = __bfloat162float(q[((size_t)b * n_q_heads + kvh * HG) * D + i]);
-    __syncthreads();
-    float acc[HG];
-#pragma unroll
-    for (int h = 0; h < HG; ++h) acc[h] = 0.f;
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r)
-#pragma unroll
-        for (int h = 0; h < HG; ++h) acc[h] = fmaf(q_s[h][part * ROWS + r], rv[r], acc[h]);
-#pragma unroll
-    for (int h = 0; h < HG; ++h) red_s[part][h][c] = acc[h];
-    __syncthreads();
-    for (int i = threadIdx.x; i < HG * D; i += 512) {
-        const int h = i / D, cc = i % D;
-        float v = 0.f;
-#pragma unroll
-        for (int p = 0; p < PARTS; ++p) v += red_s[p][h][cc];
-        v *= scale_log2;
-        qp[((size_t)b * n_q_heads + kvh * HG + h) * D + cc] = v;
-        if (qc != nullptr) red_s[0][h][cc] = v * k_center[(size_t)kvh * D + cc];       // (each thread rewrites only what it read)
-    }
-    // the constant the read path drops from every logit of a query, q . k_mean * sm_scale (base-2 units):
-    // only a learned sink logit and the BF16 band need it (they must be shifted by the same amount)
-    if (qk_off != nullptr && (threadIdx.x >> 5) < HG) {
-        const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        float acc = 0.f;
-        for (int i = lane; i < D; i += 32) acc = fmaf(q_s[h][i], k_mean[(size_t)kvh * D + i], acc);
-        acc = warp_sum_f(acc);
-        // (the merge kernel of a preceding decode call on this workspace reads qk_off: its grid must have completed)
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (lane == 0) qk_off[(size_t)b * n_q_heads + kvh * HG + h] = acc * scale_log2;
-    }
-    // scaled key format: the table is built from centred codewords, and the centre's share <q', centre> of
-    // every logit is added back before the per-token scale multiplies it
-    if (qc != nullptr) {
+    const int b_end = min(batch, (run + 1) * seqs_per_block);
+    for (int b = run * seqs_per_block; b < b_end; ++b) {
+        if (b != run * seqs_per_block) __syncthreads();        // the shared arrays are free
+        if (pair_count != nullptr && threadIdx.x == 0) pair_count[kvh * batch + b] = 0;
+        for (int i = threadIdx.x; i < HG * D; i += 512)
+            q_s[i / D][i % D] = __bfloat162float(q[((size_t)b * n_q_heads + kvh * HG) * D + i]);
         __syncthreads();
-        if ((threadIdx.x >> 5) < HG) {
+        float acc[HG];
+#pragma unroll
+        for (int h = 0; h < HG; ++h) acc[h] = 0.f;
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+            for (int h = 0; h < HG; ++h) acc[h] = fmaf(q_s[h][part * ROWS + r], rv[r], acc[h]);
+#pragma unroll
+        for (int h = 0; h < HG; ++h) red_s[part][h][c] = acc[h];
+        __syncthreads();
+        for (int i = threadIdx.x; i < HG * D; i += 512) {
+            const int h = i / D, cc = i % D;
+            float v = 0.f;
+#pragma unroll
+            for (int p = 0; p < PARTS; ++p) v += red_s[p][h][cc];
+            v *= scale_log2;
+            qp[((size_t)b * n_q_heads + kvh * HG + h) * D + cc] = v;
+            if (qc != nullptr) red_s[0][h][cc] = v * k_center[(size_t)kvh * D + cc];       // (each thread rewrites only what it read)
+        }
+        // the constant the read path drops from every logit of a query, q . k_mean * sm_scale (base-2 units):
+        // only a learned sink logit and the BF16 band need it (they must be shifted by the same amount)
+        if (qk_off != nullptr && (threadIdx.x >> 5) < HG) {
             const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
             float acc = 0.f;
-            for (int i = lane; i < D; i += 32) acc += red_s[0][h][i];
+            for (int i = lane; i < D; i += 32) acc = fmaf(q_s[h][i], k_mean[(size_t)kvh * D + i], acc);
             acc = warp_sum_f(acc);
-            if (lane == 0) qc[(size_t)b * n_q_heads + kvh * HG + h] = acc;
+            // (the merge kernel of a preceding decode call on this workspace reads qk_off: its grid must have completed)
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            if (lane == 0) qk_off[(size_t)b * n_q_heads + kvh * HG + h] = acc * scale_log2;
+        }
+        // scaled key format: the table is built from centred codewords, and the centre's share <q', centre> of
+        // every logit is added back before the per-token scale multiplies it
+        if (qc != nullptr) {
+            __syncthreads();
+            if ((threadIdx.x >> 5) < HG) {
+                const int h = threadIdx.x >> 5, lane = threadIdx.x & 31;
+                float acc = 0.f;
+                for (int i = lane; i < D; i += 32) acc += red_s[0][h][i];
+                acc = warp_sum_f(acc);
+                if (lane == 0) qc[(size_t)b * n_q_heads + kvh * HG + h] = acc;
+            }
         }
     }
 #ifdef NOVAKV_TIMING
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_p1));
-    if (threadIdx.x == 0 && (blk == 0 || blk == batch * n_kv_heads - 1))
+    if (threadIdx.x == 0 && (blk == 0 || blk == (int)gridDim.x - 2))
         printf("prepare block %d | ns start %llu end %llu\n", blk, g_p0, g_p1);
 #endif
 }
@@ -1260,11 +1268,15 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 // ------------------------------------------------------------------------------------------------
 // merge + inverse value transform
 // ------------------------------------------------------------------------------------------------
-// MINB = resident blocks per SM the register budget allows for: 1 keeps the prefetched constants in
-// registers (lowest latency, small batches), 2 trades a few spills for occupancy (many pairs).
+// One block per KV head and run of sequences, NP sequences at a time; it keeps its slice of the inverse transform in
+// registers.  A warp finds the pieces of one sequence (the CTAs whose recorded ranges meet it), their common maximum and
+// their scales; then every thread sums its coordinate over the pieces, all loads independent.  Bound by that chain of
+// memory latencies (lengths and prefixes, ranges, (max, sum) pairs, accumulators: about 3 us), which the sequences of a
+// block share: 256 pairs 11.5 -> 9.0 us, 1024 pairs 22.4 -> 19.3 us (cold caches).
 // EXT = the call carries a learned sink logit and/or a BF16 band partial; without it that code is compiled out.
-template <int D, int HG, int MINB, bool EXT>
-__global__ void __launch_bounds__(HG * D > 512 ? 512 : HG * D, MINB)
+
+template <int D, int HG, bool EXT>
+__global__ void __launch_bounds__(HG * D > 512 ? 512 : HG * D, 1)
 novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __restrict__ part_acc,
                            const int32_t* __restrict__ page_prefix, const int32_t* __restrict__ seq_lens,
                            int batch, int n_q_heads, int n_kv_heads, int max_pages_per_seq, int grid_s1,
@@ -1274,14 +1286,20 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
                            const float* __restrict__ qk_off /* [batch][Hq], base-2 units */,
                            const float* __restrict__ band_ml /* [batch][Hq][2] (max, sum) of the BF16 band, or null */,
                            const float* __restrict__ band_acc /* [batch][Hq][D] sum p v of the band, original value domain */,
-                           const int32_t* __restrict__ cost_prefix, int seg_weight, const long* __restrict__ cta_range) {
-    __shared__ float o_s[HG * D];
-    __shared__ float frac_s[HG];      // share of the softmax mass on quantised tokens (1 without sink and band)
-    __shared__ float bsc_s[HG];       // multiplier of the band accumulator (0 without a band)
-    constexpr int NT = HG * D > 512 ? 512 : HG * D;
-    constexpr int PARTS = NT / D, COLS = D / PARTS;
-    const int pair = blockIdx.x;
-    const int b = pair / n_kv_heads, kvh = pair - b * n_kv_heads;
+                           const int32_t* __restrict__ cost_prefix, int seg_weight, const long* __restrict__ cta_range,
+                           int seqs_per_block) {
+    constexpr int NP = HG <= 4 ? 4 : 2 /* as shared memory allows */, NT = HG * D > 512 ? 512 : HG * D, NW = NT / 32;
+    constexpr int PARTS = NT / D, COLS = D / PARTS, PER = (HG * D + NT - 1) / NT;
+    __shared__ float o_s[NP][HG * D];
+    __shared__ float red_s[PARTS][HG][D];
+    __shared__ short piece_s[NP][MAX_SCAN_CTAS + 1];          // scan CTAs that hold a piece of the sequence
+    __shared__ float scale_s[NP][MAX_SCAN_CTAS + 1][HG];      // 2^(max of the piece - common max)
+    __shared__ float m_s[NP][HG], l_s[NP][HG];                // common maximum and sum
+    __shared__ float frac_s[NP][HG];                          // share of the softmax mass on quantised tokens (1 without sink and band)
+    __shared__ float bsc_s[NP][HG];                           // multiplier of the band accumulator (0 without a band)
+    __shared__ int n_s[NP];                                   // pieces; -1 = empty sequence
+    const int run = blockIdx.x / n_kv_heads, kvh = blockIdx.x - run * n_kv_heads;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // constants of the inverse transform are fetched before the grid-dependency wait (they overlap the
     // tail of the scan kernel): this thread's slice of rv_t and the mean of its output coordinates
     float rv[COLS];
@@ -1290,9 +1308,9 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
 #pragma unroll
         for (int c = 0; c < COLS; ++c) rv[c] = R[(size_t)c * D];
     }
-    float vm[(HG * D + NT - 1) / NT];
+    float vm[PER];
 #pragma unroll
-    for (int k = 0; k < (HG * D + NT - 1) / NT; ++k) vm[k] = v_mean[(size_t)kvh * D + (threadIdx.x + k * NT) % D];
+    for (int k = 0; k < PER; ++k) vm[k] = v_mean[(size_t)kvh * D + (threadIdx.x + k * NT) % D];
 #ifdef NOVAKV_TIMING
     unsigned long long g_m0, g_m1, g_m2;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_m0));
@@ -1301,113 +1319,156 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
 #ifdef NOVAKV_TIMING
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_m1));
 #endif
-    const int len = clamp_len(seq_lens[b], max_pages_per_seq);
-    const int pages_b = (len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
-    const long P = page_prefix[batch];
-    const int slot0 = kvh * batch + b;                     // the scan kernel's pair index (walk order)
-    // CTAs that may hold a piece of this pair: those whose cost range meets the pair's (the largest c with
-    // floor(c*T/G) <= x for its first and last cost unit), widened by one on each side; the ranges the scan
-    // CTAs recorded decide.  Their ranges, then their (max, sum) pairs, are fetched into shared memory by
-    // parallel threads (two memory latencies, whatever the number of pieces), so that the loop below only issues
-    // independent loads of the accumulators.
-    __shared__ int cand_s[MAX_SCAN_CTAS + 1];              // 1 = this CTA holds a piece of the pair
-    __shared__ float2 ml_s[MAX_SCAN_CTAS + 1][HG];
-    int c_first = 0, n_cand = 0;
-    if (pages_b > 0) {
-        const long u0 = (long)kvh * P + page_prefix[b], u1 = u0 + pages_b;
-        const long T = (long)cost_prefix[batch] * n_kv_heads;
-        const long x0 = (long)kvh * cost_prefix[batch] + cost_prefix[b] + seg_weight, x1 = x0 + pages_b - 1;
-        c_first = max((int)(((x0 + 1) * grid_s1 - 1) / T) - 1, 0);
-        const int c_last = min((int)(((x1 + 1) * grid_s1 - 1) / T) + 1, grid_s1 - 1);
-        n_cand = min(c_last - c_first + 1, MAX_SCAN_CTAS + 1);
-        for (int t = threadIdx.x; t < n_cand; t += blockDim.x) {
-            const long r0 = cta_range[(c_first + t) * 2], r1 = cta_range[(c_first + t) * 2 + 1];
-            cand_s[t] = (r0 < r1 && r1 > u0 && r0 < u1) ? 1 : 0;
+    const int b_end = min(batch, (run + 1) * seqs_per_block);
+    for (int b0 = run * seqs_per_block; b0 < b_end; b0 += NP) {
+        const int np = min(NP, b_end - b0);
+        for (int p = warp; p < np; p += NW) {
+            const int b = b0 + p;
+            const int len = clamp_len(seq_lens[b], max_pages_per_seq);
+            const int pages_b = (len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
+            const size_t slot0 = (size_t)kvh * batch + b;          // the scan kernel's pair index (walk order)
+            int n = pages_b > 0 ? 0 : -1;
+            if (pages_b > 0) {
+                // CTAs that may hold a piece: those whose cost range meets the pair's (the largest c with
+                // floor(c*T/G) <= x for its first and last cost unit), widened by one on each side; the ranges the scan
+                // CTAs recorded decide
+                const long P = page_prefix[batch], cost_all = cost_prefix[batch];
+                const long u0 = (long)kvh * P + page_prefix[b], u1 = u0 + pages_b;
+                const long T = cost_all * n_kv_heads;
+                const long x0 = (long)kvh * cost_all + cost_prefix[b] + seg_weight, x1 = x0 + pages_b - 1;
+                const int c_first = max((int)(((x0 + 1) * grid_s1 - 1) / T) - 1, 0);
+                const int c_last = min((int)(((x1 + 1) * grid_s1 - 1) / T) + 1, grid_s1 - 1);
+                for (int c0 = c_first; c0 <= c_last; c0 += 32) {
+                    bool has = false;
+                    if (c0 + lane <= c_last) {
+                        const long r0 = cta_range[(c0 + lane) * 2], r1 = cta_range[(c0 + lane) * 2 + 1];
+                        has = r0 < r1 && r1 > u0 && r0 < u1;
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, has);
+                    if (has) piece_s[p][n + __popc(m & ((1u << lane) - 1))] = (short)(c0 + lane);
+                    n += __popc(m);
+                }
+                __syncwarp();
+                // exact log-sum-exp combination: lane = (piece, head)
+                float M[HG], l[HG];
+#pragma unroll
+                for (int h = 0; h < HG; ++h) { M[h] = M_INIT; l[h] = 0.f; }
+                for (int k0 = 0; k0 < n; k0 += 32) {
+#pragma unroll
+                    for (int h = 0; h < HG; ++h) {
+                        float2 ml = make_float2(M_INIT, 0.f);
+                        if (k0 + lane < n) ml = *reinterpret_cast<const float2*>(part_ml + ((slot0 + piece_s[p][k0 + lane]) * HG + h) * 2);
+                        float mx = ml.x;
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                        const float m_new = fmaxf(M[h], mx);
+                        float sum = ex2(ml.x - m_new) * ml.y;
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                        l[h] = fmaf(l[h], ex2(M[h] - m_new), sum);
+                        M[h] = m_new;
+                        if (k0 + lane < n) scale_s[p][k0 + lane][h] = ml.x;
+                    }
+                }
+                __syncwarp();
+                for (int k = lane; k < n; k += 32)
+#pragma unroll
+                    for (int h = 0; h < HG; ++h) scale_s[p][k][h] = ex2(scale_s[p][k][h] - M[h]);
+                if (lane == 0) {
+#pragma unroll
+                    for (int h = 0; h < HG; ++h) { m_s[p][h] = M[h]; l_s[p][h] = l[h]; }
+                }
+            } else if (lane < HG) {
+                m_s[p][lane] = M_INIT; l_s[p][lane] = 0.f;
+            }
+            if (lane == 0) n_s[p] = n;
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < n_cand * HG; t += blockDim.x) {
-            const int ci = t / HG, h = t - ci * HG;
-            if (cand_s[ci]) ml_s[ci][h] = *reinterpret_cast<const float2*>(part_ml + (((size_t)slot0 + c_first + ci) * HG + h) * 2);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            if (p >= np) break;
+            const int b = b0 + p, n = n_s[p];
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const int i = threadIdx.x + k * NT;
+                if (i >= HG * D) break;
+                const int h = i / D, c = i - h * D;
+                float a = 0.f;
+#pragma unroll 4
+                for (int j = 0; j < n; ++j)
+                    a = fmaf(scale_s[p][j][h], part_acc[(((size_t)kvh * batch + b + piece_s[p][j]) * HG + h) * D + c], a);
+                float M = m_s[p][h], lsum = l_s[p][h];
+                float lq = lsum;          // mass of the quantised tokens at the running scale
+                float wb = 0.f;           // weight of the band accumulator at the running scale
+                const int hq = kvh * HG + h;
+                if (EXT && band_ml != nullptr) {
+                    // BF16 sink-plus-recent band: one more partial, accumulated in the original value domain
+                    const float mb = band_ml[((size_t)b * n_q_heads + hq) * 2], lb = band_ml[((size_t)b * n_q_heads + hq) * 2 + 1];
+                    const float M2 = fmaxf(M, mb);
+                    const float wq = ex2(M - M2);
+                    wb = ex2(mb - M2);
+                    a *= wq;
+                    lq *= wq;
+                    lsum = fmaf(lb, wb, lq);
+                    M = M2;
+                }
+                if (EXT && sink_logits != nullptr) {
+                    // learned sink: an extra logit in the normaliser, added exactly once, after the cross-split
+                    // combine; it is shifted by the per-query constant the token logits dropped (q . k_mean)
+                    const float s2 = sink_logits[hq] * 1.4426950408889634f - qk_off[(size_t)b * n_q_heads + hq];
+                    const float M2 = fmaxf(M, s2);
+                    const float w = ex2(M - M2);
+                    a *= w;
+                    lq *= w;
+                    wb *= w;
+                    lsum = fmaf(lsum, w, ex2(s2 - M2));
+                }
+                float val = 0.f, frac = 0.f, bsc = 0.f;
+                if (lsum > 0.f) {
+                    val = a / lsum;
+                    if (EXT) { frac = lq / lsum; bsc = wb / lsum; }
+                }
+                if (EXT && c == 0) { frac_s[p][h] = frac; bsc_s[p][h] = bsc; }
+                o_s[p][i] = val;
+            }
         }
         __syncthreads();
-    }
-    for (int i = threadIdx.x; i < HG * D; i += blockDim.x) {
-        const int h = i / D, c = i - h * D;
-        float M = M_INIT, a = 0.f, lsum = 0.f;
-        for (int ci = 0; ci < n_cand; ++ci)
-            if (cand_s[ci]) M = fmaxf(M, ml_s[ci][h].x);
-        for (int ci = 0; ci < n_cand; ++ci) {
-            if (!cand_s[ci]) continue;
-            const float sc = ex2(ml_s[ci][h].x - M);
-            a = fmaf(sc, part_acc[(((size_t)slot0 + c_first + ci) * HG + h) * D + c], a);
-            lsum = fmaf(sc, ml_s[ci][h].y, lsum);
+        // o_h = o'_h rv^T + v_mean: threads = D outputs x PARTS column parts, all HG heads share each load
+        for (int p = 0; p < np; ++p) {
+            const int b = b0 + p;
+            {
+                const int r = threadIdx.x % D, part = threadIdx.x / D;
+                float acc[HG];
+#pragma unroll
+                for (int h = 0; h < HG; ++h) acc[h] = 0.f;
+                if (n_s[p] >= 0) {
+#pragma unroll
+                    for (int c = 0; c < COLS; ++c)
+#pragma unroll
+                        for (int h = 0; h < HG; ++h) acc[h] = fmaf(o_s[p][h * D + part * COLS + c], rv[c], acc[h]);
+                }
+#pragma unroll
+                for (int h = 0; h < HG; ++h) red_s[part][h][r] = acc[h];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                const int i = threadIdx.x + k * NT;
+                if (i >= HG * D) break;
+                const int h = i / D, r = i - h * D;
+                float o = 0.f;
+#pragma unroll
+                for (int q = 0; q < PARTS; ++q) o += red_s[q][h][r];
+                // sum_j p_j (s^_j R_V^T + v_mean): the mean carries the quantised-token mass (all of it without sink and band)
+                if (EXT) o = fmaf(vm[k], frac_s[p][h], o);
+                else if (n_s[p] >= 0) o += vm[k];
+                const size_t oi = ((size_t)b * n_q_heads + kvh * HG + h) * D + r;
+                if (EXT && band_acc != nullptr) o = fmaf(band_acc[oi], bsc_s[p][h], o);
+                if (out_is_fp32) reinterpret_cast<float*>(out)[oi] = o;
+                else reinterpret_cast<__nv_bfloat16*>(out)[oi] = __float2bfloat16_rn(o);
+            }
+            __syncthreads();
         }
-        float lq = lsum;          // mass of the quantised tokens at the running scale
-        float wb = 0.f;           // weight of the band accumulator at the running scale
-        const int hq = kvh * HG + h;
-        if (EXT && band_ml != nullptr) {
-            // BF16 sink-plus-recent band: one more partial, accumulated in the original value domain
-            const float mb = band_ml[((size_t)b * n_q_heads + hq) * 2], lb = band_ml[((size_t)b * n_q_heads + hq) * 2 + 1];
-            const float M2 = fmaxf(M, mb);
-            const float wq = ex2(M - M2);
-            wb = ex2(mb - M2);
-            a *= wq;
-            lq *= wq;
-            lsum = fmaf(lb, wb, lq);
-            M = M2;
-        }
-        if (EXT && sink_logits != nullptr) {
-            // learned sink: an extra logit in the normaliser, added exactly once, after the cross-split
-            // combine; it is shifted by the per-query constant the token logits dropped (q . k_mean)
-            const float s2 = sink_logits[hq] * 1.4426950408889634f - qk_off[(size_t)b * n_q_heads + hq];
-            const float M2 = fmaxf(M, s2);
-            const float w = ex2(M - M2);
-            a *= w;
-            lq *= w;
-            wb *= w;
-            lsum = fmaf(lsum, w, ex2(s2 - M2));
-        }
-        float val = 0.f, frac = 0.f, bsc = 0.f;
-        if (lsum > 0.f) {
-            val = a / lsum;
-            if (EXT) { frac = lq / lsum; bsc = wb / lsum; }
-        }
-        if (EXT && c == 0) { frac_s[h] = frac; bsc_s[h] = bsc; }
-        o_s[i] = val;
-    }
-    __syncthreads();
-    // o_h = o'_h rv^T + v_mean: threads = D outputs x PARTS column parts, all HG heads share each load
-    __shared__ float red_s[PARTS][HG][D];
-    {
-        const int r = threadIdx.x % D, part = threadIdx.x / D;
-        float acc[HG];
-#pragma unroll
-        for (int h = 0; h < HG; ++h) acc[h] = 0.f;
-        if (pages_b > 0) {
-#pragma unroll
-            for (int c = 0; c < COLS; ++c)
-#pragma unroll
-                for (int h = 0; h < HG; ++h) acc[h] = fmaf(o_s[h * D + part * COLS + c], rv[c], acc[h]);
-        }
-#pragma unroll
-        for (int h = 0; h < HG; ++h) red_s[part][h][r] = acc[h];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < (HG * D + NT - 1) / NT; ++k) {
-        const int i = threadIdx.x + k * NT;
-        if (i >= HG * D) break;
-        const int h = i / D, r = i - h * D;
-        float o = 0.f;
-#pragma unroll
-        for (int p = 0; p < PARTS; ++p) o += red_s[p][h][r];
-        // sum_j p_j (s^_j R_V^T + v_mean): the mean carries the quantised-token mass (all of it without sink and band)
-        if (EXT) o = fmaf(vm[k], frac_s[h], o);
-        else if (pages_b > 0) o += vm[k];
-        const size_t oi = ((size_t)b * n_q_heads + kvh * HG + h) * D + r;
-        if (EXT && band_acc != nullptr) o = fmaf(band_acc[oi], bsc_s[h], o);
-        if (out_is_fp32) reinterpret_cast<float*>(out)[oi] = o;
-        else reinterpret_cast<__nv_bfloat16*>(out)[oi] = __float2bfloat16_rn(o);
     }
 #ifdef NOVAKV_TIMING
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_m2));
@@ -1589,10 +1650,12 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     // kernel follows.
     const bool fuse = sink_logits == nullptr && band == nullptr && ctx->fused_merge;
 
-    novakv_launch_pdl(novakv_prepare_kernel<D, HG>, dim3(batch * hkv + 1), dim3(512), 0, stream, q, ly.rk_inv_t, seq_lens,
+    // sequences per prepare block: one while all pairs fit on the machine twice over, then enough to make that so
+    const int seqs_per_block = max(1, min(8, (batch * hkv + 2 * ctx->n_sm - 1) / (2 * ctx->n_sm)));
+    novakv_launch_pdl(novakv_prepare_kernel<D, HG>, dim3((batch + seqs_per_block - 1) / seqs_per_block * hkv + 1), dim3(512), 0, stream, q, ly.rk_inv_t, seq_lens,
                       batch, hq, hkv, max_pages_per_seq, sm_scale * 1.4426950408889634f, qp, prefix, ctx->dev_status,
                       k_off_vec, qk_off, cost_prefix, ctx->seg_weight, (const float*)ly.k_center, qc,
-                      fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32);
+                      fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32, seqs_per_block);
     ctx->launches++;
 
     auto kern = novakv_decode_stage1_kernel<D, HG, VM, KSC, VSQ>;
@@ -1622,13 +1685,14 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     }
     if (fuse) return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
     const bool ext = sink_logits != nullptr || band != nullptr;
-    auto merge = batch * hkv > 2 * ctx->n_sm
-                     ? (ext ? novakv_decode_merge_kernel<D, HG, 2, true> : novakv_decode_merge_kernel<D, HG, 2, false>)
-                     : (ext ? novakv_decode_merge_kernel<D, HG, 1, true> : novakv_decode_merge_kernel<D, HG, 1, false>);
-    novakv_launch_pdl(merge, dim3(batch * hkv), dim3(HG * D > 512 ? 512 : HG * D), 0, stream,
+    auto merge = ext ? novakv_decode_merge_kernel<D, HG, true> : novakv_decode_merge_kernel<D, HG, false>;
+    // (one block per SM, so that the slice of the transform stays in registers, and one wave of blocks where at most 8
+    // sequences a block make that possible)
+    const int merge_run = max(1, min(8, (batch + max(1, ctx->n_sm / hkv) - 1) / max(1, ctx->n_sm / hkv)));
+    novakv_launch_pdl(merge, dim3((batch + merge_run - 1) / merge_run * hkv), dim3(HG * D > 512 ? 512 : HG * D), 0, stream,
                       part_ml, part_acc, prefix, seq_lens, batch, hq, hkv, max_pages_per_seq, grid, ly.rv_t, ly.v_mean, out,
                       out_is_fp32, sink_logits, qk_off, (const float*)band_ml, (const float*)band_acc,
-                      (const int32_t*)cost_prefix, ctx->seg_weight, (const long*)cta_range);
+                      (const int32_t*)cost_prefix, ctx->seg_weight, (const long*)cta_range, merge_run);
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
 }
