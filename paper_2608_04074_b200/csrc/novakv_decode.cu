@@ -1480,27 +1480,45 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
 // ------------------------------------------------------------------------------------------------
 // BF16 sink-plus-recent band: exact attention partial over the tokens that are not quantised
 // ------------------------------------------------------------------------------------------------
-// One CTA per (sequence, KV head), 16 warps; a warp takes 4 band tokens at a time (their 8 row loads in
-// flight together), lanes hold D/32 dimensions, logits by warp reduction, online softmax per warp, then a
-// merge of the warps.  Output: (max, sum) and sum_j p_j v_j per query head, base-2 domain, unnormalised.
+// One CTA per (sequence, KV head), 8 warps.  A warp takes groups of 32 / Hg (at least 8) band tokens, one row per warp
+// instruction, lanes hold D/32 dimensions, the next group's rows in flight; the group's Hg logits per token are reduced
+// across the lanes by one transposing butterfly (31 shuffles for 32 logits; five per logit before), online softmax per
+// warp, then a merge of the warps.  Output: (max, sum) and sum_j p_j v_j per query head, base-2 domain, unnormalised.
+// Bound by memory latency: 64 sequences x 8 heads x 320 tokens, d = 128 (84 MB): 63 -> 30 us; two blocks an SM
+// (128 registers) against one: 39 us.
 // Band buffers: bf16 [batch][band_cap][Hkv][D]; of sequence b, slots 0 .. sink_cnt-1 hold the sink tokens
 // and slots n_sink + (ring_start + i) % (band_cap - n_sink), i < ring_len, the recent tokens.
-constexpr int BAND_WARPS = 16, BAND_U = 4;
+// The kernel reads nothing the scan writes: its blocks start as scan CTAs leave, and the dependency wait comes before the
+// outputs (it is what orders the merge kernel behind the scan).
+constexpr int BAND_WARPS = 8;
+template <int N>
+__device__ __forceinline__ void butterfly_halves(float (&v)[N], int s, int lane) {
+    // lanes with bit s set keep the upper half, the others the lower half; the kept half receives the partner's share
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+        const bool up = (lane & s) != 0;
+        const float send = up ? v[i] : v[i + N / 2];
+        const float keep = up ? v[i + N / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+}
 template <int D, int HG>
-__global__ void __launch_bounds__(BAND_WARPS * 32)
+__global__ void __launch_bounds__(BAND_WARPS * 32, HG >= 4 ? 2 : 1)
 novakv_band_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ band_k,
                    const __nv_bfloat16* __restrict__ band_v, int band_cap, int n_sink,
                    const int32_t* __restrict__ band_meta, int n_q_heads, int n_kv_heads, float scale_log2,
                    const float* __restrict__ k_mean, float* __restrict__ band_ml, float* __restrict__ band_acc) {
-    constexpr int DPL = D / 32;
+    constexpr int DPL = D / 32, WPL = DPL / 2;              // dimensions / 32-bit words of a row per lane
+    constexpr int TG = HG >= 4 ? 8 : 32 / HG;               // tokens per group
+    constexpr int NV = TG * HG, VPL = NV / 32;              // logits per group, of which a lane finishes VPL
     __shared__ float m_s[BAND_WARPS][HG], l_s[BAND_WARPS][HG];
     __shared__ float acc_s[BAND_WARPS][HG][D];
-    novakv_grid_dependency_wait();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.x / n_kv_heads, kvh = blockIdx.x - b * n_kv_heads;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int ring_cap = band_cap - n_sink;
     const int sink_cnt = min(max(band_meta[b * 3 + 0], 0), n_sink);
-    const int ring_start = max(band_meta[b * 3 + 1], 0);
+    const int ring_start = ring_cap > 0 ? max(band_meta[b * 3 + 1], 0) % ring_cap : 0;
     const int ring_len = ring_cap > 0 ? min(max(band_meta[b * 3 + 2], 0), ring_cap) : 0;
     const int n = sink_cnt + ring_len;
     float qr[HG][DPL];
@@ -1509,64 +1527,129 @@ novakv_band_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __r
 #pragma unroll
         for (int i = 0; i < DPL; ++i)
             qr[h][i] = __bfloat162float(q[((size_t)b * n_q_heads + kvh * HG + h) * D + lane * DPL + i]) * scale_log2;
-    // the quantised tokens' logits omit the constant q . k_mean * sm_scale (Lemma S1): the band's logits must
-    // sit on the same scale, so the same constant is subtracted here
-    float zoff[HG];
+    // the quantised tokens' logits omit the constant q . k_mean (Lemma S1): the band's logits must sit on the same scale,
+    // so the same constant is subtracted; the lane finishes the logits with flat index lane * VPL + j = token * HG + head
+    float zoff[VPL];
+    {
+        float z[HG];
 #pragma unroll
-    for (int h = 0; h < HG; ++h) {
-        float t = 0.f;
+        for (int h = 0; h < HG; ++h) {
+            float t = 0.f;
 #pragma unroll
-        for (int i = 0; i < DPL; ++i) t = fmaf(qr[h][i], k_mean[(size_t)kvh * D + lane * DPL + i], t);
-        zoff[h] = warp_sum_f(t);
+            for (int i = 0; i < DPL; ++i) t = fmaf(qr[h][i], k_mean[(size_t)kvh * D + lane * DPL + i], t);
+            z[h] = warp_sum_f(t);
+        }
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            float v = z[0];
+#pragma unroll
+            for (int h = 1; h < HG; ++h) v = (lane * VPL + j) % HG == h ? z[h] : v;
+            zoff[j] = v;
+        }
     }
-    float m[HG], l[HG], acc[HG][DPL];
+    const uint32_t* const kb = reinterpret_cast<const uint32_t*>(band_k) + (((size_t)b * band_cap * n_kv_heads + kvh) * D + lane * DPL) / 2;
+    const uint32_t* const vb = reinterpret_cast<const uint32_t*>(band_v) + (((size_t)b * band_cap * n_kv_heads + kvh) * D + lane * DPL) / 2;
+    const bool by8 = ((reinterpret_cast<uintptr_t>(band_k) | reinterpret_cast<uintptr_t>(band_v)) & 7) == 0;    // (4 is guaranteed)
+    auto load_row = [&](const uint32_t* p, uint32_t (&w)[WPL]) {
+        if (WPL == 2 && by8) {
+            const uint2 x = *reinterpret_cast<const uint2*>(p);
+            w[0] = x.x; w[WPL - 1] = x.y;
+        } else {
+            w[0] = p[0];
+            if (WPL == 2) w[WPL - 1] = p[1];
+        }
+    };
+    uint32_t kn[TG][WPL], vn[TG][WPL];
+    auto load_group = [&](int i0) {
 #pragma unroll
-    for (int h = 0; h < HG; ++h) {
-        m[h] = M_INIT; l[h] = 0.f;
+        for (int t = 0; t < TG; ++t) {
+            const int i = min(i0 + t, n - 1);                // (a valid row; its weight is zeroed below)
+            int r = ring_start + (i - sink_cnt);
+            r = r >= ring_cap ? r - ring_cap : r;
+            const size_t off = (size_t)(i < sink_cnt ? i : n_sink + r) * n_kv_heads * (D / 2);
+            load_row(kb + off, kn[t]);
+            load_row(vb + off, vn[t]);
+        }
+    };
+    float m_run[VPL], l_run[VPL], acc[HG][DPL];
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) { m_run[j] = M_INIT; l_run[j] = 0.f; }
+#pragma unroll
+    for (int h = 0; h < HG; ++h)
 #pragma unroll
         for (int i = 0; i < DPL; ++i) acc[h][i] = 0.f;
-    }
-    for (int base = warp * BAND_U; base < n; base += BAND_WARPS * BAND_U) {
-        float kf[BAND_U][DPL], vf[BAND_U][DPL];
+    if (warp * TG < n) load_group(warp * TG);
+    for (int i0 = warp * TG; i0 < n; i0 += BAND_WARPS * TG) {
+        uint32_t kc[TG][WPL], vc[TG][WPL];
 #pragma unroll
-        for (int u = 0; u < BAND_U; ++u) {
-            const int i = base + u;
-            const int ii = i < n ? i : base;               // a valid row; its weight is zeroed below
-            const int slot = ii < sink_cnt ? ii : n_sink + (ring_start + (ii - sink_cnt)) % ring_cap;
-            const size_t off = (((size_t)b * band_cap + slot) * n_kv_heads + kvh) * D + lane * DPL;
+        for (int t = 0; t < TG; ++t)
 #pragma unroll
-            for (int j = 0; j < DPL; j += 2) {
-                const __nv_bfloat162 k2 = *reinterpret_cast<const __nv_bfloat162*>(band_k + off + j);
-                const __nv_bfloat162 v2 = *reinterpret_cast<const __nv_bfloat162*>(band_v + off + j);
-                kf[u][j] = __bfloat162float(k2.x); kf[u][j + 1] = __bfloat162float(k2.y);
-                vf[u][j] = __bfloat162float(v2.x); vf[u][j + 1] = __bfloat162float(v2.y);
-            }
-        }
+            for (int w = 0; w < WPL; ++w) { kc[t][w] = kn[t][w]; vc[t][w] = vn[t][w]; }
+        if (i0 + BAND_WARPS * TG < n) load_group(i0 + BAND_WARPS * TG);
+        float z[NV];
 #pragma unroll
-        for (int u = 0; u < BAND_U; ++u) {
-            const bool valid = base + u < n;
+        for (int t = 0; t < TG; ++t)
 #pragma unroll
             for (int h = 0; h < HG; ++h) {
-                float z = 0.f;
+                float s = 0.f;
 #pragma unroll
-                for (int i = 0; i < DPL; ++i) z = fmaf(qr[h][i], kf[u][i], z);
-                z = warp_sum_f(z) - zoff[h];
-                if (!valid) z = -CUDART_INF_F;
-                const float m_new = fmaxf(m[h], z);
-                const float alpha = ex2(m[h] - m_new), p = ex2(z - m_new);
-                l[h] = fmaf(l[h], alpha, p);
-#pragma unroll
-                for (int i = 0; i < DPL; ++i) acc[h][i] = fmaf(acc[h][i], alpha, p * vf[u][i]);
-                m[h] = m_new;
+                for (int w = 0; w < WPL; ++w) {
+                    s = fmaf(qr[h][2 * w], __uint_as_float(kc[t][w] << 16), s);
+                    s = fmaf(qr[h][2 * w + 1], __uint_as_float(kc[t][w] & 0xffff0000u), s);
+                }
+                z[t * HG + h] = s;
             }
+        butterfly_halves<NV>(z, 16, lane);
+        butterfly_halves<NV / 2>(reinterpret_cast<float (&)[NV / 2]>(z), 8, lane);
+        butterfly_halves<NV / 4>(reinterpret_cast<float (&)[NV / 4]>(z), 4, lane);
+        butterfly_halves<NV / 8>(reinterpret_cast<float (&)[NV / 8]>(z), 2, lane);
+        butterfly_halves<NV / 16>(reinterpret_cast<float (&)[NV / 16]>(z), 1, lane);
+        // online softmax; the lanes that share a head differ in the lane bits above log2(HG / VPL)
+        float p[VPL], alpha[VPL];
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            const float zz = i0 + (lane * VPL + j) / HG < n ? z[j] - zoff[j] : -CUDART_INF_F;
+            float mx = zz;
+#pragma unroll
+            for (int s = HG / VPL; s < 32; s <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+            const float m_new = fmaxf(m_run[j], mx);
+            alpha[j] = ex2(m_run[j] - m_new);
+            m_run[j] = m_new;
+            p[j] = ex2(zz - m_new);
+            l_run[j] = fmaf(l_run[j], alpha[j], p[j]);
         }
+#pragma unroll
+        for (int h = 0; h < HG; ++h) {
+            const float al = __shfl_sync(0xffffffffu, alpha[h % VPL], h / VPL);     // head h lives at flat index h (token 0)
+#pragma unroll
+            for (int i = 0; i < DPL; ++i) acc[h][i] *= al;
+        }
+#pragma unroll
+        for (int t = 0; t < TG; ++t)
+#pragma unroll
+            for (int h = 0; h < HG; ++h) {
+                const int flat = t * HG + h;
+                const float ph = __shfl_sync(0xffffffffu, p[flat % VPL], flat / VPL);
+#pragma unroll
+                for (int w = 0; w < WPL; ++w) {
+                    acc[h][2 * w] = fmaf(ph, __uint_as_float(vc[t][w] << 16), acc[h][2 * w]);
+                    acc[h][2 * w + 1] = fmaf(ph, __uint_as_float(vc[t][w] & 0xffff0000u), acc[h][2 * w + 1]);
+                }
+            }
     }
 #pragma unroll
-    for (int h = 0; h < HG; ++h) {
-        if (lane == 0) { m_s[warp][h] = m[h]; l_s[warp][h] = l[h]; }
+    for (int j = 0; j < VPL; ++j) {
+        float l = l_run[j];
+#pragma unroll
+        for (int s = HG / VPL; s < 32; s <<= 1) l += __shfl_xor_sync(0xffffffffu, l, s);
+        const int flat = lane * VPL + j;
+        if (flat < HG) { m_s[warp][flat] = m_run[j]; l_s[warp][flat] = l; }
+    }
+#pragma unroll
+    for (int h = 0; h < HG; ++h)
 #pragma unroll
         for (int i = 0; i < DPL; ++i) acc_s[warp][h][lane * DPL + i] = acc[h][i];
-    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
     for (int idx = threadIdx.x; idx < HG * D; idx += BAND_WARPS * 32) {
         const int h = idx / D, c = idx - h * D;
