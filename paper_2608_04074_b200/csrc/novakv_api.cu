@@ -87,7 +87,7 @@ static void free_layer(novakv_layer& ly) {
     cudaFree(ly.pf_r); cudaFree(ly.pf_cb); cudaFree(ly.pf_const); cudaFree(ly.k_mean);
     cudaFree(ly.cb_k); cudaFree(ly.cb_v); cudaFree(ly.rk_inv_t); cudaFree(ly.rv_t);
     cudaFree(ly.v_mean); cudaFree(ly.cb_k_lut); cudaFree(ly.cb_v_u8); cudaFree(ly.v_scale); cudaFree(ly.v_off);
-    cudaFree(ly.k_mean_eff); cudaFree(ly.k_center);
+    cudaFree(ly.cb_k_mma); cudaFree(ly.k_mma_scale); cudaFree(ly.k_mean_eff); cudaFree(ly.k_center);
     ly = novakv_layer();
 }
 
@@ -194,6 +194,30 @@ extern "C" novakv_status novakv_load_calibration(novakv_ctx* ctx, int layer, con
                     cbk_lut[(((size_t)hh * C + c) * L + l) * g + i] =
                         (float)((double)h->cb_k[(((size_t)hh * L + l) * C + c) * g + i] - (double)cen);
             }
+    // d = 64: the centred codewords as binary16 numbers and their binary16 remainders, every coordinate scaled by a power
+    // of two to at most 1 (the query takes the scale)
+    std::vector<uint16_t> cbk_mma;
+    std::vector<float> mma_scale;
+    if (d == 64) {
+        cbk_mma.resize((size_t)H * C * L * 8);
+        mma_scale.assign((size_t)H * d, 1.f);
+        for (int hh = 0; hh < H; ++hh)
+            for (int l = 0; l < L; ++l)
+                for (int i = 0; i < g; ++i) {
+                    float mx = 0.f;
+                    for (int c = 0; c < C; ++c) mx = fmaxf(mx, fabsf(cbk_lut[(((size_t)hh * C + c) * L + l) * g + i]));
+                    int e = 0;
+                    if (mx > 0.f && mx < 1e30f) frexp((double)mx, &e);
+                    mma_scale[(size_t)hh * d + l * g + i] = (float)ldexp(1.0, e);
+                    for (int c = 0; c < C; ++c) {
+                        const float x = (float)ldexp((double)cbk_lut[(((size_t)hh * C + c) * L + l) * g + i], -e);
+                        const __half hi = __float2half_rn(x), lo = __float2half_rn(x - __half2float(hi));
+                        uint16_t* dst = &cbk_mma[(((size_t)hh * C + c) * L + l) * 8];
+                        memcpy(dst + i, &hi, 2);
+                        memcpy(dst + 4 + i, &lo, 2);
+                    }
+                }
+    }
     // what the centred table drops from a logit, <q rk_inv_t, centre> = q . (rk_inv_t centre^T), joins q . k_mean
     for (int hh = 0; hh < H; ++hh)
         for (int r = 0; r < d; ++r) {
@@ -219,6 +243,7 @@ extern "C" novakv_status novakv_load_calibration(novakv_ctx* ctx, int layer, con
               upload(&ly.cb_v_u8, cbv_u8) == cudaSuccess && upload(&ly.v_scale, v_scale) == cudaSuccess &&
               upload(&ly.v_off, v_off) == cudaSuccess && upload(&ly.k_mean_eff, km_eff) == cudaSuccess &&
               upload(&ly.k_center, kcen) == cudaSuccess;
+    if (d == 64) ok = ok && upload(&ly.cb_k_mma, cbk_mma) == cudaSuccess && upload(&ly.k_mma_scale, mma_scale) == cudaSuccess;
     if (!ok) { free_layer(ly); return NOVAKV_ECUDA; }
     ly.loaded = true;
     return NOVAKV_OK;

@@ -294,6 +294,19 @@ __device__ __forceinline__ uint32_t prmt_rep(uint32_t a, uint32_t b, uint32_t se
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
     return d;
 }
+// reads at an address plus a constant of the instruction
+template <int OFF>
+__device__ __forceinline__ uint4 lds_u128_at(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4+%5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ uint32_t lds_u32_at(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(OFF));
+    return v;
+}
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
@@ -350,6 +363,11 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+// the same with a zero accumulator
+__device__ __forceinline__ void mma_f16_zero(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
 __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
@@ -393,6 +411,11 @@ __device__ __forceinline__ uint4 ldg_stream_128(const void* p) {
     uint4 v;
     asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ldg_stream_32(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ uint2 ldg_stream_64(const void* p) {
@@ -1266,6 +1289,353 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 }
 
 // ------------------------------------------------------------------------------------------------
+// stage 1 for d = 64 and eight query heads per KV head: logits on tensor cores too
+// ------------------------------------------------------------------------------------------------
+// A score table costs 32 bytes of shared-memory reads and eight additions per (token, group) here.  A key codeword costs 16
+// bytes - four binary16 coordinates and their binary16 remainders, about 22 bits - and the additions are matrix products
+// over all eight heads at once, binary32 accumulators (against binary64: rel 3e-7 of the logits, as the binary32 table).
+// The codewords belong to the KV head, so a segment has no table to build: its set-up is 16 numbers of q' per lane.
+//   mma m16n8k16: rows 0-7 = q_hi and rows 8-15 = q_lo of the eight heads, columns = 8 tokens, K = 4 groups; one product
+//   takes the codewords' hi halves and one their remainders, and a logit is the sum of its two rows.  Lane
+//   (fr, fc) = (lane / 4, lane % 4) supplies groups 4 fc .. 4 fc + 3 (one per k-step) of the token in column fr: the two
+//   64-bit halves of a 128-bit gather are the two B operands as they stand.  (Codewords as A, tokens as rows, need three
+//   products for 16 tokens instead of four, but the operand then mixes two gathers: 64 register moves per 32 tokens.)
+//   Column c of a block of 8 tokens is token c / 2 + 4 (c % 2): the weights of a lane then are the B operand of the value
+//   product in the order in which the cache keeps the value bytes of a lane (tokens fc, 4 + fc, 8 + fc, 12 + fc).
+//   value product: rows = (group 8 gb + fr, coordinate 2 cp) and, at fr + 8, coordinate 2 cp + 1; K = 16 tokens.  One byte
+//   permutation takes the same coordinate of two codewords and widens it (bytes with a clear top bit pair with their
+//   replicated top bit).
+// Rows of 256 bytes, so that one byte permutation puts a code into an address.  Bank conflicts: the eight lanes of a quarter
+// warp read four groups of two tokens; two copies of the key codewords, their columns 64 bytes apart, serve even and odd fr.
+// Four copies of the value codewords, 32 bytes apart, serve the four fc.
+// MMA_FIGURES
+struct S1M {
+    static constexpr int D = 64, HG = 8, L = 16;
+    static constexpr int KEY_COPY = 65536, VAL_BYTES = 65536;
+    static constexpr int TILE_BYTES = 32 * L, PAGE_BYTES = 2 * TILE_BYTES;
+    static constexpr int MROW = D + 4, MHEADS = 4;                         // merge buffer: four heads at a time
+    // Shared-window addresses, fixed so that they are immediates of the gathers: 32 additions per 32 tokens otherwise.
+    // (The window's first KB and the static words lie below; checked at run time.)
+    static constexpr int KEY = 4096;                                       // [2 copies][256 codes][16 columns][16 B]
+    static constexpr int VAL = KEY + 2 * KEY_COPY;                         // [256 codes][2 group blocks][4 copies][8 groups][4 B]
+    static constexpr int MACC = VAL + VAL_BYTES;
+    static constexpr int ML = MACC + NCW * MHEADS * MROW * 4;
+    static constexpr int BND = ML + NCW * HG * 8;
+    static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;
+    static constexpr int SMEM = PFX + 2 * (PFX_CAP + 1) * 4;
+    static_assert(SMEM <= S1_SMEM_BYTES, "shared memory budget");
+};
+__global__ void __launch_bounds__(S1_THREADS, 1)
+novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__ cb_k_mma /* [Hkv][256][16] (hi, lo) */,
+                         const float* __restrict__ k_mma_scale /* [Hkv][64] */, const uint8_t* __restrict__ cb_v_img,
+                         const float* __restrict__ v_scale, const float* __restrict__ v_off, const uint8_t* __restrict__ k_pages,
+                         const uint8_t* __restrict__ v_pages, int n_pages, const int32_t* __restrict__ page_table,
+                         int max_pages_per_seq, const int32_t* __restrict__ seq_lens, const int32_t* __restrict__ page_prefix,
+                         int batch, int n_q_heads, int n_kv_heads, float* __restrict__ part_ml, float* __restrict__ part_acc,
+                         uint32_t* __restrict__ dev_status, int pt_stride, const int32_t* __restrict__ cost_prefix,
+                         int seg_weight, long* __restrict__ cta_range) {
+    using C = S1M;
+    constexpr int D = C::D, HG = C::HG, L = C::L;
+    constexpr float SH = 15.f;                                // weights are scaled by 2^SH before the binary16 rounding
+    constexpr float CEN = 64.f * 5.9604644775390625e-08f;     // what one unit of weight adds beyond u - 64, in units of 2^-24
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ int s_found[4];
+    const uint32_t s_base = smem_u32(smem);
+    if (s_base > C::KEY || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
+        // cannot happen with the shared address window of this architecture; reported, never trapped
+        if (threadIdx.x == 0) {
+            atomicOr(dev_status, NOVAKV_DEV_SMEM_LAYOUT);
+            cta_range[blockIdx.x * 2] = 0; cta_range[blockIdx.x * 2 + 1] = 0;
+        }
+        return;
+    }
+    unsigned char* const s_abs = smem - s_base;               // s_abs + a: the byte at shared-window address a
+
+    // codewords of a KV head -> shared memory
+    auto stage_head = [&](int kvh) {
+        const uint4* src = cb_k_mma + (size_t)kvh * 256 * L;
+        for (int i = threadIdx.x; i < 256 * L; i += S1_THREADS) {
+            const uint32_t dst = C::KEY + (i >> 4) * 256, col = (i & 3) * 4 + ((i >> 2) & 3);     // k-step, fc
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst + col * 16), "l"(src + i) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst + C::KEY_COPY + (col ^ 4) * 16), "l"(src + i) : "memory");
+        }
+        const uint8_t* vsrc = cb_v_img + (size_t)kvh * VCB_COPY_BYTES;
+        for (int i = threadIdx.x; i < 256 * (L / 4); i += S1_THREADS) {
+            const int code = i >> 2, ch = i & 3;              // four groups of a codeword row
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(C::VAL + code * 256 + (ch >> 1) * 128 + c * 32 + (ch & 1) * 16),
+                             "l"(vsrc + code * VCB_ROW + ch * 16) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int head = (int)(((long)blockIdx.x * n_kv_heads) / gridDim.x);   // KV head whose codewords are resident (see the other kernel)
+    stage_head(head);
+    novakv_grid_dependency_wait();
+
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    if (batch <= PFX_CAP) {
+        int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
+        for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix[i]; pfx[PFX_CAP + 1 + i] = cost_prefix[i]; }
+        __syncthreads();
+        page_prefix = pfx;
+        cost_prefix = pfx + PFX_CAP + 1;
+    }
+    long* const s_bnd = reinterpret_cast<long*>(s_abs + C::BND);
+    for (int c = threadIdx.x; c <= (int)gridDim.x; c += S1_THREADS)
+        s_bnd[c] = scan_boundary(c, gridDim.x, page_prefix, cost_prefix, batch, n_kv_heads, seg_weight);
+    __syncthreads();
+    const long u_begin = s_bnd[blockIdx.x], u_end = s_bnd[blockIdx.x + 1];
+    if (threadIdx.x == 0) { cta_range[blockIdx.x * 2] = u_begin; cta_range[blockIdx.x * 2 + 1] = u_end; }
+    if (u_begin >= u_end) { async_copies_wait(); return; }
+
+    // ---- lane roles and constants
+    const int fr = lane >> 2, fc = lane & 3;
+    const int tau = (fr >> 1) + 4 * (fr & 1);                 // this lane's token in a block of 8 (rows fr, fr + 8 of an operand)
+    // byte j of a token holds group j ^ tau: the codes of groups 4 fc + ks lie in word fc ^ (tau / 4), byte ks ^ (tau % 4)
+    const uint32_t key_word = (uint32_t)(fc ^ (tau >> 2)) * 4;
+    uint32_t ksel[4], kcol[4];                                // gather offset = byte permutation of (codes, kcol[ks]) by ksel[ks]
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        ksel[ks] = 0x7604u | ((uint32_t)(ks ^ (tau & 3)) << 4);
+        kcol[ks] = (fr & 1) * C::KEY_COPY + ((4 * ks + fc) ^ (4 * (fr & 1))) * 16;
+    }
+    const uint32_t vcol = fc * 32 + fr * 4;
+
+    float m_run = M_INIT, l_run = 0.f, wsum[2] = {0.f, 0.f};  // head fr (wsum: even and odd columns)
+    float macc[2][2][4];                                      // [gb][cp]: coordinate 2 cp of heads 2 fc, + 1, then 2 cp + 1
+#pragma unroll
+    for (int i = 0; i < 16; ++i) macc[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
+    // remove the centre of the value grid from the sums of the tiles since the last call
+    auto flush_window = [&]() {
+        float ws = wsum[0] + wsum[1];
+        ws += __shfl_xor_sync(0xffffffffu, ws, 1);
+        ws += __shfl_xor_sync(0xffffffffu, ws, 2);
+        l_run += ws;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float w = __shfl_sync(0xffffffffu, ws, 8 * fc + 4 * j);
+#pragma unroll
+            for (int gb = 0; gb < 2; ++gb)
+#pragma unroll
+                for (int cp = 0; cp < 2; ++cp) {
+                    macc[gb][cp][j] = fmaf(-CEN, w, macc[gb][cp][j]);
+                    macc[gb][cp][2 + j] = fmaf(-CEN, w, macc[gb][cp][2 + j]);
+                }
+        }
+        wsum[0] = wsum[1] = 0.f;
+    };
+
+    long u = u_begin;
+    while (u < u_end) {
+        const Segment sg = locate(page_prefix, seq_lens, batch, max_pages_per_seq, u, u_end, s_found);
+        const int pair = sg.kvh * batch + sg.b;
+        if (head != sg.kvh) { stage_head(sg.kvh); head = sg.kvh; }       // (every warp is past the last segment's scan)
+
+        // q' of head fr, groups 4 fc + ks, in the key codewords' scale; per head a power of two brings the largest to
+        // [2^9, 2^10), so that binary16 halves neither overflow nor lose small coordinates
+        uint32_t qa[4][4];                                    // A operand of a k-step: hi, lo of coordinates 0, 1, then of 2, 3
+        float us;
+        {
+            const float4* q4 = reinterpret_cast<const float4*>(qp + ((size_t)sg.b * n_q_heads + sg.kvh * HG + fr) * D) + 4 * fc;
+            const float4* s4 = reinterpret_cast<const float4*>(k_mma_scale + (size_t)sg.kvh * D) + 4 * fc;
+            float4 qv[4];
+            float mx = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                const float4 a = q4[ks], s = s4[ks];
+                qv[ks] = make_float4(a.x * s.x, a.y * s.y, a.z * s.z, a.w * s.w);
+                mx = fmaxf(fmaxf(mx, fmaxf(fabsf(qv[ks].x), fabsf(qv[ks].y))), fmaxf(fabsf(qv[ks].z), fabsf(qv[ks].w)));
+            }
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            int e = (int)(__float_as_uint(mx) >> 23) - 127 - 9;
+            e = max(-100, min(e, 110));
+            const float down = __uint_as_float((uint32_t)(127 - e) << 23);
+            us = __uint_as_float((uint32_t)(127 + e) << 23);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                const float v[4] = {qv[ks].x * down, qv[ks].y * down, qv[ks].z * down, qv[ks].w * down};
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const uint32_t hi = pack_h2(v[2 * i], v[2 * i + 1]);
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+                    qa[ks][2 * i] = hi;
+                    qa[ks][2 * i + 1] = pack_h2(v[2 * i] - f.x, v[2 * i + 1] - f.y);
+                }
+            }
+        }
+
+        // this warp's tiles of the segment: half pages hp = warp, warp + NCW, ...
+        const int n_half = min(2 * sg.npg, (sg.len - sg.pg0 * NOVAKV_PAGE_TOKENS + 31) / 32);
+        const int n_it = n_half > warp ? (n_half - warp + NCW - 1) / NCW : 0;
+        const int32_t* pt = page_table + (size_t)sg.b * pt_stride + sg.pg0;
+        auto load_ids = [&](int batch_i) {
+            const int it = batch_i * 32 + lane;
+            int page = 0;
+            if (it < n_it) {
+                page = pt[(warp + NCW * it) >> 1];
+                if (page < 0 || page >= n_pages) { atomicOr(dev_status, NOVAKV_DEV_BAD_PAGE); page = 0; }
+            }
+            return page;
+        };
+        int ids_cur = load_ids(0), ids_next = load_ids(1);
+        uint32_t kn[4];                                       // key codes of tokens tau, + 8, + 16, + 24
+        uint2 vn[2];                                          // value codes of a 16-token block: group blocks fc % 2, 1 - fc % 2
+        auto load_tile = [&](int it) {
+            if ((it & 31) == 0 && it > 0) { ids_cur = ids_next; ids_next = load_ids((it >> 5) + 1); }
+            const int page = __shfl_sync(0xffffffffu, ids_cur, it & 31);
+            const int half = (warp + NCW * it) & 1;
+            const size_t off = ((size_t)page * n_kv_heads + sg.kvh) * C::PAGE_BYTES + half * C::TILE_BYTES;
+            const uint8_t* kp = k_pages + off + tau * 16 + key_word;
+            const uint8_t* vp = v_pages + off + lane * 8;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) kn[i] = ldg_stream_32(kp + 128 * i);
+#pragma unroll
+            for (int blk = 0; blk < 2; ++blk) vn[blk] = ldg_stream_64(vp + blk * (L * 16));
+        };
+        if (n_it > 0) load_tile(0);
+        async_copies_wait();
+        __syncthreads();                                      // codewords complete (and the last segment's merge is read out)
+
+#pragma unroll 1
+        for (int it = 0; it < n_it; ++it) {
+            uint32_t kc[4];
+            uint2 vc[2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) kc[i] = kn[i];
+            vc[0] = vn[0]; vc[1] = vn[1];
+            if (it + 1 < n_it) load_tile(it + 1);
+            const int hp = warp + NCW * it;
+            const int nvalid = min(32, sg.len - ((sg.pg0 + (hp >> 1)) * NOVAKV_PAGE_TOKENS + (hp & 1) * 32));
+
+            // ---- logits of head fr, tokens 8 i + fc and 8 i + 4 + fc, over us
+            float z[4][2];
+            {
+                float acc[4][4];
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {
+                    uint4 c[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) c[i] = lds_u128_at<C::KEY>(prmt_rep(kc[i], kcol[ks], ksel[ks]));
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (ks == 0) mma_f16_zero(acc[i], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], c[i].x, c[i].y);
+                        else mma_f16(acc[i], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], c[i].x, c[i].y);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) mma_f16(acc[i], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], c[i].z, c[i].w);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { z[i][0] = acc[i][0] + acc[i][2]; z[i][1] = acc[i][1] + acc[i][3]; }
+            }
+            if (nvalid < 32) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (8 * (i >> 1) + 4 * (i & 1) + fc >= nvalid) z[i >> 1][i & 1] = -CUDART_INF_F;
+            }
+            // ---- online softmax (base 2), as in the other kernel; the four lanes of a quad share a head
+            {
+                float t = fmaxf(fmaxf(fmaxf(z[0][0], z[0][1]), fmaxf(z[1][0], z[1][1])), fmaxf(fmaxf(z[2][0], z[2][1]), fmaxf(z[3][0], z[3][1]))) * us;
+                if (__any_sync(0xffffffffu, t > m_run)) {
+                    t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, 1));
+                    t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, 2));
+                    const float m_new = t > m_run ? t + M_SLACK : m_run;
+                    const float al = ex2(m_run - m_new);
+                    m_run = m_new;
+                    l_run *= al;
+                    wsum[0] *= al;
+                    wsum[1] *= al;
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float a = __shfl_sync(0xffffffffu, al, 8 * fc + 4 * j);
+#pragma unroll
+                        for (int gb = 0; gb < 2; ++gb)
+#pragma unroll
+                            for (int cp = 0; cp < 2; ++cp) { macc[gb][cp][j] *= a; macc[gb][cp][2 + j] *= a; }
+                    }
+                }
+            }
+            // ---- weights: as they stand the B operand of the value product
+            uint32_t bw[4];
+            {
+                const float o = SH - m_run;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    bw[i] = pack_h2(ex2(fmaf(z[i][0], us, o)), ex2(fmaf(z[i][1], us, o)));
+                    flush_h2(bw[i], wsum[0], wsum[1]);        // the rounded weights are what the normaliser sums
+                }
+            }
+            // ---- values
+#pragma unroll
+            for (int blk = 0; blk < 2; ++blk) {
+                const uint32_t codes[2] = {fc & 1 ? vc[blk].y : vc[blk].x, fc & 1 ? vc[blk].x : vc[blk].y};
+#pragma unroll
+                for (int gb = 0; gb < 2; ++gb) {
+                    uint32_t X[4];                            // codewords of tokens fc, 4 + fc, 8 + fc, 12 + fc
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        X[t] = gb ? lds_u32_at<C::VAL + 128>(__byte_perm(codes[gb], vcol, 0x7604u | (t << 4))) : lds_u32_at<C::VAL>(__byte_perm(codes[gb], vcol, 0x7604u | (t << 4)));
+#pragma unroll
+                    for (int cp = 0; cp < 2; ++cp) {
+                        constexpr uint32_t SEL0 = 0xC480u;     // bytes (u0, 0, u4, 0): the same coordinate of two codewords
+                        const uint32_t sa = SEL0 + 0x1111u * (2 * cp), sb = SEL0 + 0x1111u * (2 * cp + 1);
+                        mma_f16(macc[gb][cp], prmt_rep(X[0], X[1], sa), prmt_rep(X[0], X[1], sb), prmt_rep(X[2], X[3], sa), prmt_rep(X[2], X[3], sb),
+                                bw[2 * blk], bw[2 * blk + 1]);
+                    }
+                }
+            }
+            if ((it & (NOVAKV_WINDOW - 1)) == NOVAKV_WINDOW - 1) flush_window();
+        }
+
+        // ---- segment epilogue: merge the warps' partials, four heads at a time, and write one partial
+        flush_window();
+        float* const m_acc = reinterpret_cast<float*>(s_abs + C::MACC);             // [NCW][MHEADS][MROW]
+        float2* const m_ml = reinterpret_cast<float2*>(s_abs + C::ML);              // [NCW][HG]
+        if (fc == 0) m_ml[warp * HG + fr] = make_float2(m_run, l_run);
+        const size_t pidx = (size_t)pair + blockIdx.x;          // unique: pair and CTA index both grow along the walk
+#pragma unroll 1
+        for (int hp = 0; hp < HG / C::MHEADS; ++hp) {
+            if ((fc >> 1) == hp) {
+#pragma unroll
+                for (int gb = 0; gb < 2; ++gb)
+#pragma unroll
+                    for (int cp = 0; cp < 2; ++cp)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            *reinterpret_cast<float2*>(m_acc + (warp * C::MHEADS + 2 * (fc & 1) + j) * C::MROW + (8 * gb + fr) * 4 + 2 * cp) =
+                                make_float2(macc[gb][cp][j], macc[gb][cp][2 + j]);
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < C::MHEADS * D; i += S1_THREADS) {
+                const int hl = i / D, c = i - hl * D, h = hp * C::MHEADS + hl;
+                float M = M_INIT;
+#pragma unroll
+                for (int w = 0; w < NCW; ++w) M = fmaxf(M, m_ml[w * HG + h].x);
+                float a = 0.f, lsum = 0.f;
+#pragma unroll
+                for (int w = 0; w < NCW; ++w) {
+                    const float2 ml = m_ml[w * HG + h];
+                    const float sc = ex2(ml.x - M);
+                    a = fmaf(sc, m_acc[(w * C::MHEADS + hl) * C::MROW + c], a);
+                    lsum = fmaf(sc, ml.y, lsum);
+                }
+                // grid index sums -> value-transform coefficients: s (u - 64) + (lo + 64 s) per unit of weight
+                const float val = (v_scale[(size_t)sg.kvh * D + c] * (a * 16777216.f) + v_off[(size_t)sg.kvh * D + c] * lsum) * 3.0517578125e-05f;
+                part_acc[(pidx * HG + h) * D + c] = val;
+                if (c == 0) { part_ml[(pidx * HG + h) * 2] = M; part_ml[(pidx * HG + h) * 2 + 1] = lsum * 3.0517578125e-05f; }
+            }
+            __syncthreads();
+        }
+        m_run = M_INIT;
+        l_run = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) macc[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
+        u += sg.npg;
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
 // merge + inverse value transform
 // ------------------------------------------------------------------------------------------------
 // One block per KV head and run of sequences, NP sequences at a time; it keeps its slice of the inverse transform in
@@ -1741,24 +2111,42 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
                       fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32, seqs_per_block);
     ctx->launches++;
 
-    auto kern = novakv_decode_stage1_kernel<D, HG, VM, KSC, VSQ>;
-    // the opt-in is per device and per kernel instantiation: remembered in the context (one device each)
-    constexpr unsigned inst_bit = 1u << ((VM ? 1 : 0) + (KSC ? 2 : 0) + (VSQ ? 4 : 0));
-    if (!(ctx->smem_opt_in & inst_bit)) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_BYTES) != cudaSuccess) return NOVAKV_ECUDA;
-        ctx->smem_opt_in |= inst_bit;
-    }
-    {
+    // d = 64 with eight query heads per KV head, plain format: the kernel that takes the logits from tensor cores.  (At
+    // d = 128 its two copies of the key codewords do not fit; with four heads the table reads no more than they do.)
+    constexpr bool MMA = D == 64 && HG == 8 && VM && !KSC && !VSQ;
+    if (MMA && !fuse) {
+        constexpr unsigned mma_bit = 1u << 8;
+        if (!(ctx->smem_opt_in & mma_bit)) {
+            if (cudaFuncSetAttribute(novakv_decode_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_BYTES) != cudaSuccess) return NOVAKV_ECUDA;
+            ctx->smem_opt_in |= mma_bit;
+        }
         novakv_prof_scope ps(ctx, 0, stream);
-        novakv_launch_pdl(kern, dim3(grid), dim3(S1_THREADS), S1_SMEM_BYTES, stream, qp, ly.cb_k_lut,
-                          VSQ ? (const uint8_t*)ctx->int2_img : (const uint8_t*)ly.cb_v_u8, (const float*)ly.v_scale,
-                          (const float*)ly.v_off, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
-                          seq_lens, prefix, batch, hq, hkv, part_ml, part_acc, ctx->dev_status, pt_stride,
-                          (const int32_t*)cost_prefix, ctx->seg_weight, cta_range, (const float*)qc,
-                          VSQ ? 0 : VCB_COPY_BYTES, pair_count, (const float*)ly.rv_t, (const float*)ly.v_mean,
-                          fuse ? out : (void*)nullptr, out_is_fp32);
+        novakv_launch_pdl(novakv_decode_mma_kernel, dim3(grid), dim3(S1_THREADS), S1_SMEM_BYTES, stream, qp, (const uint4*)ly.cb_k_mma,
+                          (const float*)ly.k_mma_scale, (const uint8_t*)ly.cb_v_u8, (const float*)ly.v_scale, (const float*)ly.v_off,
+                          k_pages, v_pages, n_pages, page_table, max_pages_per_seq, seq_lens, prefix, batch, hq, hkv, part_ml, part_acc,
+                          ctx->dev_status, pt_stride, (const int32_t*)cost_prefix, ctx->seg_weight, cta_range);
         ps.end();
         ctx->launches++;
+    } else {
+        auto kern = novakv_decode_stage1_kernel<D, HG, VM, KSC, VSQ>;
+        // the opt-in is per device and per kernel instantiation: remembered in the context (one device each)
+        constexpr unsigned inst_bit = 1u << ((VM ? 1 : 0) + (KSC ? 2 : 0) + (VSQ ? 4 : 0));
+        if (!(ctx->smem_opt_in & inst_bit)) {
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_BYTES) != cudaSuccess) return NOVAKV_ECUDA;
+            ctx->smem_opt_in |= inst_bit;
+        }
+        {
+            novakv_prof_scope ps(ctx, 0, stream);
+            novakv_launch_pdl(kern, dim3(grid), dim3(S1_THREADS), S1_SMEM_BYTES, stream, qp, ly.cb_k_lut,
+                              VSQ ? (const uint8_t*)ctx->int2_img : (const uint8_t*)ly.cb_v_u8, (const float*)ly.v_scale,
+                              (const float*)ly.v_off, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
+                              seq_lens, prefix, batch, hq, hkv, part_ml, part_acc, ctx->dev_status, pt_stride,
+                              (const int32_t*)cost_prefix, ctx->seg_weight, cta_range, (const float*)qc,
+                              VSQ ? 0 : VCB_COPY_BYTES, pair_count, (const float*)ly.rv_t, (const float*)ly.v_mean,
+                              fuse ? out : (void*)nullptr, out_is_fp32);
+            ps.end();
+            ctx->launches++;
+        }
     }
     if (band != nullptr) {
         novakv_launch_pdl(novakv_band_kernel<D, HG>, dim3(batch * hkv), dim3(BAND_WARPS * 32), 0, stream, q, band->k, band->v,

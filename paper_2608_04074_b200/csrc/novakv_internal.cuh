@@ -39,6 +39,8 @@ struct novakv_layer {
     float* rv_t = nullptr;        // [Hkv][d][d]  transposed R_V: rv_t[c][r] = R_V[r][c]
     float* v_mean = nullptr;      // [Hkv][d]
     float* cb_k_lut = nullptr;    // [Hkv][256][L][4]   key codewords minus k_center, the order the score table is built in
+    uint16_t* cb_k_mma = nullptr; // d = 64: [Hkv][256][16][8] the same as binary16 numbers and their remainders, in units of k_mma_scale
+    float* k_mma_scale = nullptr; // d = 64: [Hkv][d] powers of two
     uint8_t* cb_v_u8 = nullptr;   // [Hkv][256][32][4]  value codewords as indices (0..127) of their 7-bit grid, slot = group
     float* v_scale = nullptr;     // [Hkv][d]  grid step s of each value coefficient: codeword = lo + s u
     float* v_off = nullptr;       // [Hkv][d]  lo + 128 s
