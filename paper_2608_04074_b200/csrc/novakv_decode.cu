@@ -1288,6 +1288,29 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 #endif
 }
 
+// locate() in two parts with the barrier between them left to the caller: the look-up of a CTA's next segment hides in the
+// scan of the present one.
+__device__ __forceinline__ void find_segment(const int32_t* __restrict__ page_prefix, const int32_t* __restrict__ seq_lens,
+                                             int batch, int max_pages, long u, int kvh, int* found) {
+    const long r = u - (long)kvh * page_prefix[batch];
+    for (int t = threadIdx.x; t < batch; t += S1_THREADS) {
+        const int lo = page_prefix[t], hi = page_prefix[t + 1];
+        if ((long)lo <= r && r < (long)hi) { found[0] = t; found[1] = clamp_len(seq_lens[t], max_pages); found[2] = lo; found[3] = kvh; }
+    }
+}
+__device__ __forceinline__ Segment segment_at(const int32_t* __restrict__ page_prefix, int batch, long u, long u_end, const int* found) {
+    Segment s;
+    s.b = found[0];
+    s.len = found[1];
+    s.kvh = found[3];
+    const long r = u - (long)s.kvh * page_prefix[batch];
+    const int pages_b = (s.len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
+    s.pg0 = (int)(r - found[2]);
+    const long left = u_end - u;
+    s.npg = (int)(left < (long)(pages_b - s.pg0) ? left : (long)(pages_b - s.pg0));
+    return s;
+}
+
 // ------------------------------------------------------------------------------------------------
 // stage 1 for d = 64 and eight query heads per KV head: logits on tensor cores too
 // ------------------------------------------------------------------------------------------------
@@ -1308,7 +1331,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 // Rows of 256 bytes, so that one byte permutation puts a code into an address.  Bank conflicts: the eight lanes of a quarter
 // warp read four groups of two tokens; two copies of the key codewords, their columns 64 bytes apart, serve even and odd fr.
 // Four copies of the value codewords, 32 bytes apart, serve the four fc.
-// Measured (16 sequences of 65536 tokens, 8 KV heads, sink, whole call): score table 193 us, this kernel 153 us.  No single
+// Measured (16 sequences of 65536 tokens, 8 KV heads, sink, whole call): score table 193 us, this kernel 149 us.  No single
 // bound: HMMA pipe 54 %, issue slots 50 %, shared-memory pipe 60 %.  Taken out one at a time, the gathers give nothing, the
 // remainder products 18 us, the value product 26 us, all key products 32 us; loads alone take 99 us.
 struct S1M {
@@ -1341,7 +1364,7 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
     constexpr float SH = 15.f;                                // weights are scaled by 2^SH before the binary16 rounding
     constexpr float CEN = 64.f * 5.9604644775390625e-08f;     // what one unit of weight adds beyond u - 64, in units of 2^-24
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ int s_found[4];
+    __shared__ int s_found[2][4];
     const uint32_t s_base = smem_u32(smem);
     if (s_base > C::KEY || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
         // cannot happen with the shared address window of this architecture; reported, never trapped
@@ -1433,24 +1456,74 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
         wsum[0] = wsum[1] = 0.f;
     };
 
+    // What a segment needs from global memory before its first tile - query, page ids - is asked for while the partials of
+    // the segment before are merged, and its place in the batch is looked up during the scan before that: 16 sequences of
+    // 65536 tokens 151 -> 149 us, 5 of 5001 52.9 -> 52.4.  (The table kernel does not gain: its table build needs the SM
+    // for twice the time of these loads, and the registers slow its scan by 0-2 %.)
     long u = u_begin;
+    Segment sg;
+    int n_it = 0, ids_cur = 0, ids_next = 0;
+    const int32_t* pt = nullptr;
+    float4 qv[4];                                             // q' of head fr, groups 4 fc + ks
+    auto load_ids = [&](int batch_i) {
+        const int it = batch_i * 32 + lane;
+        int page = 0;
+        if (it < n_it) {
+            page = pt[(warp + NCW * it) >> 1];
+            if (page < 0 || page >= n_pages) { atomicOr(dev_status, NOVAKV_DEV_BAD_PAGE); page = 0; }
+        }
+        return page;
+    };
+    auto fetch_segment = [&]() {
+        // this warp's tiles of the segment: half pages hp = warp, warp + NCW, ...
+        const int n_half = min(2 * sg.npg, (sg.len - sg.pg0 * NOVAKV_PAGE_TOKENS + 31) / 32);
+        n_it = n_half > warp ? (n_half - warp + NCW - 1) / NCW : 0;
+        pt = page_table + (size_t)sg.b * pt_stride + sg.pg0;
+        const float4* q4 = reinterpret_cast<const float4*>(qp + ((size_t)sg.b * n_q_heads + sg.kvh * HG + fr) * D) + 4 * fc;
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) qv[ks] = q4[ks];
+        ids_cur = load_ids(0);
+        ids_next = load_ids(1);
+    };
+    uint32_t kn[4];                                       // key codes of tokens tau, + 8, + 16, + 24
+    uint2 vn[2];                                          // value codes of a 16-token block: group blocks fc % 2, 1 - fc % 2
+    auto load_tile = [&](int it) {
+        if ((it & 31) == 0 && it > 0) { ids_cur = ids_next; ids_next = load_ids((it >> 5) + 1); }
+        const int page = __shfl_sync(0xffffffffu, ids_cur, it & 31);
+        const int half = (warp + NCW * it) & 1;
+        const size_t off = ((size_t)page * n_kv_heads + sg.kvh) * C::PAGE_BYTES + half * C::TILE_BYTES;
+        const uint8_t* kp = k_pages + off + tau * 16 + key_word;
+        const uint8_t* vp = v_pages + off + lane * 8;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) kn[i] = ldg_stream_32(kp + 128 * i);
+#pragma unroll
+        for (int blk = 0; blk < 2; ++blk) vn[blk] = ldg_stream_64(vp + blk * (L * 16));
+    };
+
+    int found = 0;                                            // the half of s_found that holds the current segment
+    find_segment(page_prefix, seq_lens, batch, max_pages_per_seq, u, (int)(u / page_prefix[batch]), s_found[0]);
+    __syncthreads();
+    sg = segment_at(page_prefix, batch, u, u_end, s_found[0]);
+    fetch_segment();
     while (u < u_end) {
-        const Segment sg = locate(page_prefix, seq_lens, batch, max_pages_per_seq, u, u_end, s_found);
         const int pair = sg.kvh * batch + sg.b;
+        if (n_it > 0) load_tile(0);
         if (head != sg.kvh) { stage_head(sg.kvh); head = sg.kvh; }       // (every warp is past the last segment's scan)
+        const long u_next = u + sg.npg;
+        if (u_next < u_end)
+            find_segment(page_prefix, seq_lens, batch, max_pages_per_seq, u_next,
+                         sg.kvh + (u_next >= (long)(sg.kvh + 1) * page_prefix[batch]), s_found[found ^ 1]);
 
         // q' of head fr, groups 4 fc + ks, in the key codewords' scale; per head a power of two brings the largest to
         // [2^9, 2^10), so that binary16 halves neither overflow nor lose small coordinates
         uint32_t qa[4][4];                                    // A operand of a k-step: hi, lo of coordinates 0, 1, then of 2, 3
         float us;
         {
-            const float4* q4 = reinterpret_cast<const float4*>(qp + ((size_t)sg.b * n_q_heads + sg.kvh * HG + fr) * D) + 4 * fc;
             const float4* s4 = reinterpret_cast<const float4*>(k_mma_scale + (size_t)sg.kvh * D) + 4 * fc;
-            float4 qv[4];
             float mx = 0.f;
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {
-                const float4 a = q4[ks], s = s4[ks];
+                const float4 a = qv[ks], s = s4[ks];
                 qv[ks] = make_float4(a.x * s.x, a.y * s.y, a.z * s.z, a.w * s.w);
                 mx = fmaxf(fmaxf(mx, fmaxf(fabsf(qv[ks].x), fabsf(qv[ks].y))), fmaxf(fabsf(qv[ks].z), fabsf(qv[ks].w)));
             }
@@ -1473,35 +1546,6 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
             }
         }
 
-        // this warp's tiles of the segment: half pages hp = warp, warp + NCW, ...
-        const int n_half = min(2 * sg.npg, (sg.len - sg.pg0 * NOVAKV_PAGE_TOKENS + 31) / 32);
-        const int n_it = n_half > warp ? (n_half - warp + NCW - 1) / NCW : 0;
-        const int32_t* pt = page_table + (size_t)sg.b * pt_stride + sg.pg0;
-        auto load_ids = [&](int batch_i) {
-            const int it = batch_i * 32 + lane;
-            int page = 0;
-            if (it < n_it) {
-                page = pt[(warp + NCW * it) >> 1];
-                if (page < 0 || page >= n_pages) { atomicOr(dev_status, NOVAKV_DEV_BAD_PAGE); page = 0; }
-            }
-            return page;
-        };
-        int ids_cur = load_ids(0), ids_next = load_ids(1);
-        uint32_t kn[4];                                       // key codes of tokens tau, + 8, + 16, + 24
-        uint2 vn[2];                                          // value codes of a 16-token block: group blocks fc % 2, 1 - fc % 2
-        auto load_tile = [&](int it) {
-            if ((it & 31) == 0 && it > 0) { ids_cur = ids_next; ids_next = load_ids((it >> 5) + 1); }
-            const int page = __shfl_sync(0xffffffffu, ids_cur, it & 31);
-            const int half = (warp + NCW * it) & 1;
-            const size_t off = ((size_t)page * n_kv_heads + sg.kvh) * C::PAGE_BYTES + half * C::TILE_BYTES;
-            const uint8_t* kp = k_pages + off + tau * 16 + key_word;
-            const uint8_t* vp = v_pages + off + lane * 8;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) kn[i] = ldg_stream_32(kp + 128 * i);
-#pragma unroll
-            for (int blk = 0; blk < 2; ++blk) vn[blk] = ldg_stream_64(vp + blk * (L * 16));
-        };
-        if (n_it > 0) load_tile(0);
         async_copies_wait();
         __syncthreads();                                      // codewords complete (and the last segment's merge is read out)
 
@@ -1598,11 +1642,17 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
         }
 
         // ---- segment epilogue: merge the warps' partials, four heads at a time, and write one partial
+        const float vs = v_scale[(size_t)sg.kvh * D + threadIdx.x % D], vo = v_off[(size_t)sg.kvh * D + threadIdx.x % D];
         flush_window();
         float* const m_acc = reinterpret_cast<float*>(s_abs + C::MACC);             // [NCW][MHEADS][MROW]
         float2* const m_ml = reinterpret_cast<float2*>(s_abs + C::ML);              // [NCW][HG]
         if (fc == 0) m_ml[warp * HG + fr] = make_float2(m_run, l_run);
         const size_t pidx = (size_t)pair + blockIdx.x;          // unique: pair and CTA index both grow along the walk
+        if (u_next < u_end) {
+            found ^= 1;
+            sg = segment_at(page_prefix, batch, u_next, u_end, s_found[found]);
+            fetch_segment();                                  // flies during the merge
+        }
 #pragma unroll 1
         for (int hp = 0; hp < HG / C::MHEADS; ++hp) {
             if ((fc >> 1) == hp) {
@@ -1630,7 +1680,7 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
                     lsum = fmaf(sc, ml.y, lsum);
                 }
                 // grid index sums -> value-transform coefficients: s (u - 64) + (lo + 64 s) per unit of weight
-                const float val = (v_scale[(size_t)sg.kvh * D + c] * (a * 16777216.f) + v_off[(size_t)sg.kvh * D + c] * lsum) * 3.0517578125e-05f;
+                const float val = (vs * (a * 16777216.f) + vo * lsum) * 3.0517578125e-05f;
                 part_acc[(pidx * HG + h) * D + c] = val;
                 if (c == 0) { part_ml[(pidx * HG + h) * 2] = M; part_ml[(pidx * HG + h) * 2 + 1] = lsum * 3.0517578125e-05f; }
             }
@@ -1640,7 +1690,7 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
         l_run = 0.f;
 #pragma unroll
         for (int i = 0; i < 16; ++i) macc[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
-        u += sg.npg;
+        u = u_next;
     }
 }
 
