@@ -14,7 +14,8 @@
 namespace {
 
 constexpr int BF16_SPLIT_PAGES = 16;     // 1024 tokens per CTA
-constexpr int BF16_WARPS = 4;
+constexpr int BF16_WARPS = 4;            // per CTA of several splits
+constexpr int BF16_WARPS_ONE = 8;        // per CTA that has its sequence (or window) to itself
 constexpr int TG = 8;                    // tokens per warp iteration
 constexpr float M_INIT = -1.0e30f;
 
@@ -56,13 +57,18 @@ __device__ __forceinline__ RowChunk<DPL> load_chunk(const __nv_bfloat16* p) {
 __device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
-template <int D, int HG>
-__global__ void __launch_bounds__(BF16_WARPS * 32)
+// ONE: a single split covers whatever a sequence can have (the host knows: window or capacity of at most BF16_SPLIT_PAGES
+// pages), so the CTA writes the output itself.  Bound by latency then (length -> page id -> rows -> merge): eight warps, so
+// that a window of 128 tokens is two or three groups each (16 would spill at d = 64, Hg = 8), no second kernel.  Window of 128, 16 sequences, 8 KV heads of
+// d = 64: 13.5 us with four warps and the merge kernel, 10.9 us so.
+template <int D, int HG, int WARPS, bool ONE>
+__global__ void __launch_bounds__(WARPS * 32)
 novakv_bf16_stage1_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k_pages,
                           const __nv_bfloat16* __restrict__ v_pages, int n_pages,
                           const int32_t* __restrict__ page_table, int max_pages_per_seq,
                           const int32_t* __restrict__ seq_lens, int n_q_heads, int n_kv_heads, float scale_log2,
-                          int window, int max_splits, float* __restrict__ part_ml, float* __restrict__ part_acc) {
+                          int window, int max_splits, float* __restrict__ part_ml, float* __restrict__ part_acc,
+                          void* __restrict__ out, int out_is_fp32) {
     constexpr int DPL = D / 32;
     constexpr int NV = TG * HG;              // logits per warp iteration
     constexpr int VPL = NV / 32;             // of which each lane finishes VPL (1 at Hg = 4, 2 at Hg = 8)
@@ -73,9 +79,19 @@ novakv_bf16_stage1_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat
     len = len < 0 ? 0 : min(len, max_pages_per_seq * NOVAKV_PAGE_TOKENS);
     const int start = window > 0 ? max(0, len - window) : 0;
     const int first_page = start / NOVAKV_PAGE_TOKENS;
-    const int t_begin = (first_page + split * BF16_SPLIT_PAGES) * NOVAKV_PAGE_TOKENS;
-    const int t_end = min(len, t_begin + BF16_SPLIT_PAGES * NOVAKV_PAGE_TOKENS);
-    if (t_begin >= t_end) return;
+    const int t_split = (first_page + split * BF16_SPLIT_PAGES) * NOVAKV_PAGE_TOKENS;
+    const int t_begin = max(t_split, start & ~(TG - 1));       // whole groups before the window are not read
+    const int t_end = min(len, t_split + BF16_SPLIT_PAGES * NOVAKV_PAGE_TOKENS);
+    auto write_out = [&](int i, float o) {                     // i = head, coordinate of the KV head's group
+        const size_t oi = ((size_t)b * n_q_heads + kvh * HG) * D + i;
+        if (out_is_fp32) reinterpret_cast<float*>(out)[oi] = o;
+        else reinterpret_cast<__nv_bfloat16*>(out)[oi] = __float2bfloat16_rn(o);
+    };
+    if (t_begin >= t_end) {
+        if (ONE)
+            for (int i = threadIdx.x; i < HG * D; i += WARPS * 32) write_out(i, 0.f);
+        return;
+    }
 
     // q of the Hg heads, this lane's dims, pre-scaled into the base-2 domain
     float qr[HG][DPL];
@@ -110,11 +126,11 @@ novakv_bf16_stage1_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat
         for (int t = 0; t < TG; ++t) { kn[t] = load_chunk<DPL>(kp + (size_t)t * D); vn[t] = load_chunk<DPL>(vp + (size_t)t * D); }
     };
     if (warp < n_groups) load_group(warp);
-    for (int g = warp; g < n_groups; g += BF16_WARPS) {
+    for (int g = warp; g < n_groups; g += WARPS) {
         RowChunk<DPL> kc[TG], vc[TG];
 #pragma unroll
         for (int t = 0; t < TG; ++t) { kc[t] = kn[t]; vc[t] = vn[t]; }
-        if (g + BF16_WARPS < n_groups) load_group(g + BF16_WARPS);
+        if (g + WARPS < n_groups) load_group(g + WARPS);
         const int tok0 = t_begin + g * TG;
         // partial dot products of this lane's dims: z[token*HG + head]
         float z[NV];
@@ -185,9 +201,9 @@ novakv_bf16_stage1_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat
         }
     }
 
-    // ---- merge the 4 warps and write the split's partial ---------------------------------------
-    __shared__ float s_acc[BF16_WARPS][HG][D];
-    __shared__ float s_ml[BF16_WARPS][HG][2];
+    // ---- merge the warps and write the split's partial (or the output) ---------------------------------------
+    __shared__ float s_acc[WARPS][HG][D];
+    __shared__ float s_ml[WARPS][HG][2];
 #pragma unroll
     for (int j = 0; j < VPL; ++j) {
         float l = l_run[j];
@@ -202,17 +218,21 @@ novakv_bf16_stage1_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat
         for (int i = 0; i < DPL; ++i) s_acc[warp][h][lane * DPL + i] = acc[h][i];
     __syncthreads();
     const size_t pidx = ((size_t)(b * n_kv_heads + kvh) * max_splits + split);
-    for (int i = threadIdx.x; i < HG * D; i += BF16_WARPS * 32) {
+    for (int i = threadIdx.x; i < HG * D; i += WARPS * 32) {
         const int h = i / D, c = i % D;
         float M = M_INIT;
 #pragma unroll
-        for (int w = 0; w < BF16_WARPS; ++w) M = fmaxf(M, s_ml[w][h][0]);
+        for (int w = 0; w < WARPS; ++w) M = fmaxf(M, s_ml[w][h][0]);
         float a = 0.f, l = 0.f;
 #pragma unroll
-        for (int w = 0; w < BF16_WARPS; ++w) {
+        for (int w = 0; w < WARPS; ++w) {
             const float sc = ex2f(s_ml[w][h][0] - M);
             a = fmaf(sc, s_acc[w][h][c], a);
             l = fmaf(sc, s_ml[w][h][1], l);
+        }
+        if (ONE) {
+            write_out(i, a / l);
+            continue;
         }
         part_acc[(pidx * HG + h) * D + c] = a;
         if (c == 0) { part_ml[(pidx * HG + h) * 2] = M; part_ml[(pidx * HG + h) * 2 + 1] = l; }
@@ -270,11 +290,16 @@ novakv_status launch_bf16_t(novakv_ctx* ctx, const __nv_bfloat16* q, const __nv_
     dim3 grid(grid_x, hkv, batch);
     {
         novakv_prof_scope ps(ctx, 2, stream);
-        novakv_bf16_stage1_kernel<D, HG><<<grid, BF16_WARPS * 32, 0, stream>>>(q, k_pages, v_pages, n_pages, page_table,
-            max_pages_per_seq, seq_lens, hq, hkv, sm_scale * 1.4426950408889634f, window, ms, part_ml, part_acc);
+        auto stage1 = [&](auto* kern, int warps) {
+            kern<<<grid, warps * 32, 0, stream>>>(q, k_pages, v_pages, n_pages, page_table, max_pages_per_seq, seq_lens, hq, hkv,
+                                                  sm_scale * 1.4426950408889634f, window, ms, part_ml, part_acc, out, out_is_fp32);
+        };
+        if (grid_x == 1) stage1(novakv_bf16_stage1_kernel<D, HG, BF16_WARPS_ONE, true>, BF16_WARPS_ONE);
+        else stage1(novakv_bf16_stage1_kernel<D, HG, BF16_WARPS, false>, BF16_WARPS);
         ps.end();
         ctx->launches++;
     }
+    if (grid_x == 1) return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
     novakv_bf16_merge_kernel<D, HG><<<batch * hkv, 256, 0, stream>>>(part_ml, part_acc, seq_lens, max_pages_per_seq, hq, hkv,
                                                                      window, ms, out, out_is_fp32);
     ctx->launches++;
