@@ -1,8 +1,6 @@
-// Write path: forward transforms (binary64) + brute-force nearest-codeword search + paged store.
-// One CTA handles a tile of tokens for one (KV head, side); side 0 = keys, 1 = values.
-//
-// The search is ALU-bound (256 distance evaluations per group, per token, per side); the codebook
-// of the CTA's head and side stays in shared memory and every warp reads codewords as broadcasts.
+// Write path of append-sized batches: forward transforms (binary64) + brute-force nearest-codeword search + paged store; the
+// search of given coefficients; the staging kernels of the BF16 band.  (Prompt-sized batches: novakv_prefill.cu.)
+// Side 0 = keys, 1 = values.  The search is ALU-bound (256 distance evaluations per group, per token, per side).
 //
 // The index the write path stores is the exact Euclidean nearest codeword of the binary64 coefficient
 // (lowest index on a tie).  The 256 distances are evaluated in binary32; beside the minimum the search
@@ -103,35 +101,14 @@ __device__ __forceinline__ float fmin3(float a, float b, float c) {
 }
 
 // Warp-cooperative exact search of one (token, group) in binary64: all 32 lanes call it with the same
-// arguments and get the same result.  The coefficient is either taken from shared memory (EXACT_IN_SMEM:
-// the binary32 values there ARE the vector to encode: given coefficients, normalised keys) or recomputed in
-// binary64 from the token's bfloat16 input row and the transform's columns 4l .. 4l+3.  Lane i evaluates the
-// codewords i, i+32, ... in ascending order with a strict '<'; the warp then keeps the smallest distance
-// and, among equal distances, the lowest index.
-template <int D, bool EXACT_IN_SMEM>
-__device__ __noinline__ int exact_search_group(const float* r_row_s, const __nv_bfloat16* __restrict__ x_row_g,
-                                               const double* mean_s, const double* __restrict__ R_plain /* [D][D] */,
-                                               int l, const float* cb_pairs_s /* [L][128][4][2] */) {
+// arguments and get the same result.  The binary32 coefficients in shared memory ARE the vector to encode.
+// Lane i evaluates the codewords i, i+32, ... in ascending order with a strict '<'; the warp then keeps the
+// smallest distance and, among equal distances, the lowest index.
+__device__ __noinline__ int exact_search_group(const float* r_row_s, int l, const float* cb_pairs_s /* [L][128][4][2] */) {
     const int lane = threadIdx.x & 31;
     double r[4];
-    if (EXACT_IN_SMEM) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) r[c] = (double)r_row_s[l * 4 + c];
-    } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) r[c] = 0.0;
-        for (int k = lane; k < D; k += 32) {
-            const double xc = (double)__bfloat162float(x_row_g[k]) - mean_s[k];
-            const double2 r01 = *reinterpret_cast<const double2*>(R_plain + (size_t)k * D + l * 4);
-            const double2 r23 = *reinterpret_cast<const double2*>(R_plain + (size_t)k * D + l * 4 + 2);
-            r[0] = fma(xc, r01.x, r[0]); r[1] = fma(xc, r01.y, r[1]);
-            r[2] = fma(xc, r23.x, r[2]); r[3] = fma(xc, r23.y, r[3]);
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) r[c] += __shfl_xor_sync(0xffffffffu, r[c], o);
-    }
+    for (int c = 0; c < 4; ++c) r[c] = (double)r_row_s[l * 4 + c];
     double best = CUDART_INF;
     int bi = lane;
     const float* cb = cb_pairs_s + (size_t)l * NOVAKV_C * 4;
@@ -167,14 +144,8 @@ __device__ __noinline__ int exact_search_group(const float* r_row_s, const __nv_
 //      the minimum gives the index and the others enter the second smallest distance.
 // Then the certification: a group whose two smallest distances are too close to tell apart in binary32 is
 // searched again in binary64 by the whole warp (exact_search_group).
-// EXACT_IN_SMEM: the binary32 coefficients in r_s are the vector to encode (delta = 0); otherwise they are
-// roundings of binary64 coefficients that exact_search_group recomputes from the inputs x_tile_g
-// (bfloat16 rows of the tile's tokens, row stride x_stride elements).
-template <int D, bool EXACT_IN_SMEM>
-__device__ __forceinline__ void search_tile(const float* r_s, const float4* cb_s, uint8_t* idx_s, int n_valid,
-                                            int warp, int n_warps, const __nv_bfloat16* __restrict__ x_tile_g,
-                                            size_t x_stride, const double* mean_s,
-                                            const double* __restrict__ R_plain) {
+template <int D>
+__device__ __forceinline__ void search_tile(const float* r_s, const float4* cb_s, uint8_t* idx_s, int n_valid, int warp, int n_warps) {
     constexpr int L = D / NOVAKV_G;
     constexpr int RS = EncSmem<D>::RSTRIDE;
     const int lane = threadIdx.x & 31;
@@ -231,28 +202,19 @@ __device__ __forceinline__ void search_tile(const float* r_s, const float4* cb_s
             ia += ka; ib += kb;
         }
         // certification
-        float del_a = 0.f, del_b = 0.f;
-        if (!EXACT_IN_SMEM) {
-            // |coefficient - its binary32 rounding| <= 2^-24 |coefficient| per component
-            del_a = 5.97e-8f * sqrtf(fmaf(ra.x, ra.x, fmaf(ra.y, ra.y, fmaf(ra.z, ra.z, ra.w * ra.w)))) * 1.0001f;
-            del_b = 5.97e-8f * sqrtf(fmaf(rb.x, rb.x, fmaf(rb.y, rb.y, fmaf(rb.z, rb.z, rb.w * rb.w)))) * 1.0001f;
-        }
-        const bool ta = lane < n_valid && needs_exact_search(best_a, sec_a, del_a);
-        const bool tb = lane + 32 < n_valid && needs_exact_search(best_b, sec_b, del_b);
+        const bool ta = lane < n_valid && needs_exact_search(best_a, sec_a, 0.f);
+        const bool tb = lane + 32 < n_valid && needs_exact_search(best_b, sec_b, 0.f);
         unsigned todo_a = __ballot_sync(0xffffffffu, ta), todo_b = __ballot_sync(0xffffffffu, tb);
         while (todo_a) {
             const int src = __ffs(todo_a) - 1;
             todo_a &= todo_a - 1;
-            const int res = exact_search_group<D, EXACT_IN_SMEM>(r_s + (size_t)src * RS, x_tile_g + (size_t)src * x_stride,
-                                                                 mean_s, R_plain, l, reinterpret_cast<const float*>(cb_s));
+            const int res = exact_search_group(r_s + (size_t)src * RS, l, reinterpret_cast<const float*>(cb_s));
             if (lane == src) ia = res;
         }
         while (todo_b) {
             const int src = __ffs(todo_b) - 1;
             todo_b &= todo_b - 1;
-            const int res = exact_search_group<D, EXACT_IN_SMEM>(r_s + (size_t)(src + 32) * RS,
-                                                                 x_tile_g + (size_t)(src + 32) * x_stride, mean_s, R_plain, l,
-                                                                 reinterpret_cast<const float*>(cb_s));
+            const int res = exact_search_group(r_s + (size_t)(src + 32) * RS, l, reinterpret_cast<const float*>(cb_s));
             if (lane == src) ib = res;
         }
         if (lane < n_valid) idx_s[lane * L + l] = (uint8_t)ia;
@@ -273,7 +235,7 @@ __device__ __forceinline__ void search_tile(const float* r_s, const float4* cb_s
 // Everything that depends only on the calibration is staged before the grid-dependency wait, so it
 // overlaps the tail of the preceding kernel in the stream.
 // The coefficients are accumulated in binary64 (index order inside a block, then the blocks pairwise).  The
-// search is the certified one of the tiled kernel: binary32 ranking, and a binary64 search by the whole warp
+// search is certified like search_tile: binary32 ranking, and a binary64 search by the whole warp
 // wherever the two nearest codewords are closer than binary32 rounding can resolve (the binary64 pipe is the
 // slowest unit of the SM: a binary64 search of every token was 60 % of this kernel's time after the launch).
 // KSC (key format with a per-token scale): the L/4 CTAs of a (head, side) form a thread-block cluster;
@@ -501,7 +463,7 @@ novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_b
         // The vector to encode is the binary64 coefficient; for normalised keys it is the binary32 quotient.
         double rd[4] = {acc0, acc1, acc2, acc3};
         if (KSC && side == 0) { rd[0] = (double)r.x; rd[1] = (double)r.y; rd[2] = (double)r.z; rd[3] = (double)r.w; }
-        // Certified search, as in the tiled kernel: this lane group's range of the codebook is ranked in binary32
+        // Certified search, as in search_tile: this lane group's range of the codebook is ranked in binary32
         // from the coefficient rounded to binary32 (first minimum in ascending order), with the second-smallest
         // distance tracked beside the smallest (equal distances count as two: their gap is zero).
         // The range is a whole number of blocks of 8 codewords.  Per block the 8 distances are independent; the block
@@ -613,7 +575,7 @@ novakv_search_kernel(const float* __restrict__ coef, int n, const float* __restr
             r_s[(size_t)t * RS + c] = t < n_valid ? coef[((size_t)(t0 + t) * n_kv_heads + kvh) * D + c] : 0.f;
         }
         __syncthreads();
-        search_tile<D, true>(r_s, cb_s, idx_s, n_valid, threadIdx.x >> 5, ENC_THREADS / 32, nullptr, 0, nullptr, nullptr);
+        search_tile<D>(r_s, cb_s, idx_s, n_valid, threadIdx.x >> 5, ENC_THREADS / 32);
         __syncthreads();
         for (int i = threadIdx.x; i < n_valid * L; i += ENC_THREADS) {
             const int t = i / L, l = i - t * L;
