@@ -1331,7 +1331,7 @@ __device__ __forceinline__ Segment segment_at(const int32_t* __restrict__ page_p
 // Rows of 256 bytes, so that one byte permutation puts a code into an address.  Bank conflicts: the eight lanes of a quarter
 // warp read four groups of two tokens; two copies of the key codewords, their columns 64 bytes apart, serve even and odd fr.
 // Four copies of the value codewords, 32 bytes apart, serve the four fc.
-// Measured (16 sequences of 65536 tokens, 8 KV heads, sink, whole call): score table 193 us, this kernel 149 us.  No single
+// Measured (16 sequences of 65536 tokens, 8 KV heads, sink, whole call): score table 193 us, this kernel 147-151 us.  No single
 // bound: HMMA pipe 54 %, issue slots 50 %, shared-memory pipe 60 %.  Taken out one at a time, the gathers give nothing, the
 // remainder products 18 us, the value product 26 us, all key products 32 us; loads alone take 99 us.
 struct S1M {
