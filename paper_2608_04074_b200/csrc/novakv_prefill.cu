@@ -247,7 +247,8 @@ __device__ __noinline__ int exact_search_token(const PrefillArgs& a, int side, i
         const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob < best || (ob == best && oi < bi)) { best = ob; bi = oi; }
     }
-    return bi & 255;                                                  // (no codeword at a finite distance: any)
+    return bi == 0x7fffffff ? 0 : bi;                                 // (a coefficient that is not a number is nearest to none: index 0, as in
+                                                                      // a scan with a strict '<')
 }
 
 // One token's coefficients in binary64, by the eight warps of a half tile: warp q sums an eighth of the input dimension

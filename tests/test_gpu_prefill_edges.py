@@ -99,3 +99,34 @@ def test_prefill_rows_without_tensor_map_alignment(cases, name):
 def test_append_batches_of_several_chunks(cases, name, fmt, n):
     """Batches that still take the append kernel but span several of its passes and chunks of the token list."""
     _run(cases[name, fmt != "plain"], fmt, n, 40, True, n == 100)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "plain"), ("qwen", "scaled"), ("gptoss", "deployed")])
+def test_prefill_token_that_is_not_finite(cases, name, fmt, bad):
+    """One element of one token is not a number: its distances are not either, and a scan that keeps a smaller distance
+    keeps index 0 - what the append kernel stores.  (INT2 values: the same bytes as the append kernel's.)  The other tokens
+    do not notice."""
+    from paper_2608_04074_b200.runtime import PagedCache
+    case, n, t = cases[name, fmt != "plain"], 300, 130
+    k, v, _ = case.draw(4300, n, 1)
+
+    def stored(bad_value, step):
+        kb, vb = k.copy(), v.copy()
+        if bad_value is not None:
+            kb[t, :, 5] = vb[t, :, 5] = bad_value
+        cache = PagedCache(case.ctx, np.array([0], np.int32), capacity_tokens=np.array([n], np.int32), seed=7,
+                           key_scale=fmt == "scaled", int2_values=fmt == "deployed")
+        for i in range(0, n, step):
+            j = min(i + step, n)
+            cache.append(0, _dev(kb[i:j], torch.bfloat16), _dev(vb[i:j], torch.bfloat16), _dev(np.zeros(j - i, np.int32)),
+                         _dev(np.arange(i, j, dtype=np.int32)))
+        assert case.ctx.novakv_last_device_status() == 0
+        return [*cache.load_logical(0, 0, n), *([cache.load_scales(0, 0, n)] if fmt != "plain" else [])]
+
+    clean, prompt, small = stored(None, n), stored(bad, n), stored(bad, 150)
+    for c, p, s in zip(clean, prompt, small):
+        assert np.array_equal(p[t], s[t])
+        assert np.array_equal(np.delete(p, t, 0), np.delete(c, t, 0))
+    if np.isnan(bad):
+        assert not prompt[0][t].any() and (fmt == "deployed" or not prompt[1][t].any())
