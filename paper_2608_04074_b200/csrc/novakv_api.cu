@@ -545,6 +545,7 @@ extern "C" novakv_status novakv_step_host_async(novakv_ctx* ctx, int layer, cons
     };
     novakv_stage_args sa;
     sa.n = 0;
+    sa.release = n_tokens > 0;
     auto stage_in = [&](const void* host_ptr, char* dev_buf, size_t bytes) -> cudaError_t {
         const void* view = device_view(host_ptr);
         if (view != nullptr && ((uintptr_t)view & 3) == 0 && (bytes & 3) == 0) {

@@ -668,9 +668,9 @@ novakv_status novakv_launch_encode(novakv_ctx* ctx, const novakv_layer& ly, cons
 // Gather of up to 5 page-locked host buffers into device staging: every 32-bit word crosses the bus
 // once, consecutive threads take consecutive words (128-byte requests per warp).
 __global__ void __launch_bounds__(256) novakv_stage_kernel(const novakv_stage_args a) {
-    // the kernels behind this one in the stream may start their own prologues (calibration constants) now; they
-    // wait for this grid's completion before they touch the staged inputs
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // an append behind this kernel may start its prologue (calibration constants) now; it waits for this grid's completion
+    // before it touches the staged inputs.  (The query blocks of a decode call do not wait: see novakv_prepare_kernel.)
+    if (a.release) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const unsigned stride = gridDim.x * blockDim.x;
 #pragma unroll 1
     for (int sgm = 0; sgm < a.n; ++sgm) {

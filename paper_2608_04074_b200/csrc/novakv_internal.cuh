@@ -119,6 +119,7 @@ struct novakv_stage_args {
     uint32_t* dst[5];
     unsigned words[5];
     int n;
+    int release;                // the next kernel of the stream waits before it reads what is staged: it may start early
 };
 novakv_status novakv_launch_stage(novakv_ctx* ctx, const novakv_stage_args& a, cudaStream_t stream);
 novakv_status novakv_launch_band_insert(novakv_ctx* ctx, const void* k_new, const void* v_new, int batch, void* band_k,
