@@ -421,6 +421,13 @@ novakv_status novakv_debug_set_segment_weight(novakv_ctx* ctx, int pages);
  */
 novakv_status novakv_debug_set_fused_merge(novakv_ctx* ctx, int on);
 
+/*
+ * Test knob: SM clocks after which a wait inside the prompt encoder gives up (default 2000000000, about a second; 0 = at
+ * once).  A call in which one does sets NOVAKV_DEV_WAIT_TIMEOUT; what it has stored for its own tokens is unspecified,
+ * nothing else is touched.
+ */
+novakv_status novakv_debug_set_wait_limit(novakv_ctx* ctx, long clocks);
+
 /* Kernels this library launched since the context was created (all kinds). */
 long novakv_launch_count(const novakv_ctx* ctx);
 

@@ -25,7 +25,7 @@ EXPORTED = [
     "novakv_decode_attention_sink", "novakv_decode_attention_banded",
     "novakv_value_meta_page_bytes", "novakv_encode_append_deployed", "novakv_decode_attention_deployed",
     "novakv_debug_set_segment_weight", "novakv_debug_set_fused_merge",
-    "novakv_band_append_staging_bytes", "novakv_band_append",
+    "novakv_band_append_staging_bytes", "novakv_band_append", "novakv_debug_set_wait_limit",
 ]
 
 
@@ -123,6 +123,7 @@ def load_library(path=None):
     lib.novakv_debug_set_value_path.argtypes = [c_void_p, c_int]
     lib.novakv_debug_set_segment_weight.argtypes = [c_void_p, c_int]
     lib.novakv_debug_set_fused_merge.argtypes = [c_void_p, c_int]
+    lib.novakv_debug_set_wait_limit.argtypes = [c_void_p, c_long]
     lib.novakv_launch_count.restype = c_long
     if path is None:
         _lib = lib
@@ -368,6 +369,9 @@ class Context:
 
     def novakv_debug_set_fused_merge(self, on):
         _check(self.lib, self.lib.novakv_debug_set_fused_merge(self.handle, int(bool(on))), "novakv_debug_set_fused_merge")
+
+    def novakv_debug_set_wait_limit(self, clocks):
+        _check(self.lib, self.lib.novakv_debug_set_wait_limit(self.handle, int(clocks)), "novakv_debug_set_wait_limit")
 
     def novakv_launch_count(self):
         return int(self.lib.novakv_launch_count(self.handle))

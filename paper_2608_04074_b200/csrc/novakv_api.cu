@@ -695,6 +695,12 @@ extern "C" novakv_status novakv_debug_set_fused_merge(novakv_ctx* ctx, int on) {
     return NOVAKV_OK;
 }
 
+extern "C" novakv_status novakv_debug_set_wait_limit(novakv_ctx* ctx, long clocks) {
+    if (!ctx || clocks < 0) return NOVAKV_EINVAL;
+    ctx->wait_clocks = clocks;
+    return NOVAKV_OK;
+}
+
 extern "C" novakv_status novakv_debug_set_value_path(novakv_ctx* ctx, int path) {
     if (!ctx || (path != 0 && path != 1)) return NOVAKV_EINVAL;
     ctx->value_path = path;

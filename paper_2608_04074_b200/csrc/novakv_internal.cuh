@@ -66,6 +66,7 @@ struct novakv_ctx {
     bool fused_merge = false;     // true: the scan kernel merges the partials itself where it can (no sink, no band)
     unsigned smem_opt_in = 0;     // scan-kernel instantiations whose shared-memory opt-in was set on this device
     unsigned prefill_opt_in = 0;  // the same for the prompt encoder's formats
+    long wait_clocks = 2000000000;   // limit of a wait inside the prompt encoder: about a second
 };
 
 // RAII-free helper: brackets a launch with events when profiling is on.

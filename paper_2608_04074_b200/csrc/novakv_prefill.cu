@@ -21,7 +21,10 @@
 // (about 300 cycles, whatever its width), so chunks are as wide as TMEM allows (four warpgroups x 128 columns: the
 // coefficients live in shared memory for that), and the first chunk of the next group is computed behind the selection
 // of this one.  Every wait is bounded (novakv_tcgen05.cuh): a wait that gives up sets NOVAKV_DEV_WAIT_TIMEOUT, and the CTA
-// runs through its remaining steps without waiting.  (The named barriers among token warps are never skipped.)
+// runs through the rest of its segment without waiting and leaves.  Three things hold on that way: the token warps take
+// no destination that the flag has overtaken (tokens without one are neither stored nor looked at again), the named
+// barriers among token warps are never skipped and never run ahead (hold() below), and the tensor core and the copies are
+// given time to finish before the CTA's memory goes away.
 //
 // What bounds it: instruction issue and latency of the selection, about 600 warp instructions per 32 tokens and group (of
 // which 64 + 16 packed minima and comparisons on the half-rate pipe) with four token warps per scheduler; tensor pipe
@@ -94,14 +97,16 @@ struct PF {
     static constexpr uint32_t OFF_TSLOT = OFF_PAGE + NX * PF_HALF * 4;            // uint8 [NX][128], its slot in the page
     static constexpr uint32_t OFF_CONST = OFF_TSLOT + NX * PF_HALF;
     static constexpr uint32_t OFF_BAR = OFF_CONST + ((NCONST * 4 + 15) & ~15);
-    static constexpr uint32_t OFF_MISC = OFF_BAR + 288;           // TMEM base, abort flag, finished token warps, queue counters; unsure tokens [16]
+    // ints: TMEM base, abort flag, finished token warps, -, queue counters [4], wait limit [2], releases [4], -, -; unsure tokens [16]
+    static constexpr uint32_t OFF_MISC = OFF_BAR + 288;
     static constexpr uint32_t BYTES = OFF_MISC + 128;
     static_assert(BYTES <= 232448, "shared memory budget");
     static_assert(X_BYTES <= SLOT_BYTES && R_SLICE % 1024 == 0 && SLOT_BYTES % 1024 == 0, "swizzled operands start on 1024 bytes");
 };
 // mbarriers
 enum { B_R = 0, B_X = 1 /* +slot */, B_XFREE = 4 /* +slot */, B_T = 7 /* +half */, B_TFREE = 9 /* +half */, B_S = 11 /* +wg */,
-       B_RING = 15 /* +stage */, B_RINGFREE = 19, B_CW = 23 /* +stage */, B_CWFREE = B_CW + PF_CW_STAGES, B_COUNT = B_CW + 2 * PF_CW_STAGES };
+       B_RING = 15 /* +stage */, B_RINGFREE = 19, B_CW = 23 /* +stage */, B_CWFREE = B_CW + PF_CW_STAGES,
+       B_DRAIN = B_CW + 2 * PF_CW_STAGES, B_COUNT };
 static_assert(B_COUNT * 8 <= 288, "barrier block");
 // named barriers: 1 + wg among the four warps of a warpgroup, 5 + half among the eight of a half tile
 __device__ __forceinline__ void nbar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
@@ -128,6 +133,7 @@ struct PrefillArgs {
     int gs;                     // parts a head's groups are cut into
     int cost_k, cost_v;         // relative cost of a key / value unit (the cut of the walk)
     int tma;                    // the token rows can be copied by the tensor maps (16-byte aligned)
+    long wait_clocks;           // limit of a wait
     uint32_t* dev_status;
     CUtensorMap map_k, map_v;   // k_new / v_new as [n_tokens][Hkv d], boxes of 64 x 128
 };
@@ -339,6 +345,8 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
     int* const s_done = reinterpret_cast<int*>(smem + P::OFF_MISC) + 2;               // token warps that have finished the segment
     int* const s_count = reinterpret_cast<int*>(smem + P::OFF_MISC) + 4;              // [helper] entries in the queue
     int* const s_head = reinterpret_cast<int*>(smem + P::OFF_MISC) + 4 + PF_HELPERS;  // [helper] entries ever queued
+    volatile uint32_t* const s_rel = reinterpret_cast<volatile uint32_t*>(smem + P::OFF_MISC) + 10;   // [wg] releases its first warp has passed
+    static_assert(4 + 2 * PF_HELPERS == 1 + MBAR_LIMIT, "the wait limit follows the queue counters");
     float* const cst = reinterpret_cast<float*>(smem + P::OFF_CONST);
     auto bar = [&](int i) -> uint32_t { return sb + P::OFF_BAR + i * 8; };
 
@@ -356,6 +364,9 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
     if (warp == 0) tmem_alloc<512>(sb + P::OFF_MISC);
     if (threadIdx.x == 0) {
         misc[1] = 0;
+        *reinterpret_cast<volatile long long*>(abort_flag + MBAR_LIMIT) = a.wait_clocks;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) s_rel[g] = 0;
 #pragma unroll
         for (int h = 0; h < PF_HELPERS; ++h) { s_count[h] = 0; s_head[h] = 0; }
         mbar_init(bar(B_R), 1);
@@ -369,6 +380,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
         for (int s = 0; s < P::NOP; ++s) { mbar_init(bar(B_RING + s), 1); mbar_init(bar(B_RINGFREE + s), 2); }
 #pragma unroll
         for (int s = 0; s < PF_CW_STAGES; ++s) { mbar_init(bar(B_CW + s), 1); mbar_init(bar(B_CWFREE + s), 8); }
+        mbar_init(bar(B_DRAIN), 5);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -540,11 +552,11 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                     if (j & 1) g = g + 1 == ngh ? 0 : g + 1;
                 }
                 // no copy and no commit may be in flight when the segment (and the CTA's memory) goes away
-                mbar_wait<PF_AUX_NS>(bar(B_R), n_seg & 1, abort_flag);
                 auto landed = [&](int b, int parity) {             // (after a wait that gave up, too)
                     int tries = 0;
                     while (!mbar_try(bar(b), parity) && ++tries < 1000000) {}
                 };
+                landed(B_R, n_seg & 1);
                 for (int j = max(0, n_use - P::NOP); j < n_use; ++j) {
                     landed(B_RING + j % P::NOP, (j / P::NOP) & 1);
                     mbar_wait<PF_AUX_NS>(bar(B_RINGFREE + j % P::NOP), (j / P::NOP) & 1, abort_flag);
@@ -561,7 +573,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                 volatile uint32_t* const e = queue + (q_tail % PF_QUEUE) * 4;
                 const uint32_t tag = __shfl_sync(0xffffffffu, e[0], 0);
                 if (tag == 0u) {
-                    if (__all_sync(0xffffffffu, last)) break;
+                    if (__all_sync(0xffffffffu, last || *abort_flag)) break;
                     __nanosleep(200);
                     continue;
                 }
@@ -598,7 +610,9 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                 unsigned char* const x_s = smem + P::OFF_X + xslot * P::SLOT_BYTES;
                 // |x| of the token; each warpgroup sums its half of the row
                 mbar_wait<PF_TOK_NS>(bar(B_X + xslot), (q / P::NX) & 1, abort_flag);
-                const int page = reinterpret_cast<const int*>(smem + P::OFF_PAGE)[xslot * PF_HALF + row];
+                __syncwarp();
+                // (the flag is read after the wait: while it is clear no wait of this thread was skipped, so this one counts)
+                const int page = *abort_flag ? -1 : reinterpret_cast<const int*>(smem + P::OFF_PAGE)[xslot * PF_HALF + row];
                 const int slot = (smem + P::OFF_TSLOT)[xslot * PF_HALF + row];
                 const bool valid = page >= 0;
                 {
@@ -824,6 +838,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                         nbar_sync(1 + wg, PF_HALF);
                         tc_fence_after();
                         if (elect_one()) {
+                            s_rel[wg] = n_s + 1;
                             umma_f16(d_s, umma_desc(a_s, PF_HALF * 16, 128, 0),
                                      umma_desc(sb + P::OFF_RING + st * PF_OP_BYTES + c * 2048, 4096, 128, 0), umma_idesc(false, false, 128, 128), false);
                             umma_commit(bar(B_S + wg));
@@ -847,16 +862,28 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                     tmem_ld64_h2(d_s + lane_base + half * 64, v);
                     tmem_wait_ld();
                 };
+                // The other three warps arrive at the barrier of a release without waiting there; what keeps them from arriving
+                // at the next one before the first warp has come to this one is the wait for its MMA.  Where that wait was
+                // given up, they wait for the first warp itself.  (It comes: everything it meets on its way is either
+                // bounded or a barrier at which these warps have arrived.)
+                bool gone = *abort_flag != 0;
+                auto wait_chunk = [&]() {
+                    const bool ok = mbar_wait<PF_TOK_NS>(bar(B_S + wg), n_s & 1, abort_flag);
+                    if (__any_sync(0xffffffffu, !ok || gone)) {
+                        gone = true;
+                        for (int tries = 0; (int)(s_rel[wg] - n_s) <= 0 && tries < 10000000; ++tries) __nanosleep(100);
+                        __syncwarp();
+                    }
+                    ++n_s;
+                    tc_fence_after();
+                };
                 float q2 = publish(0);                                         // |r|^2 of this group, in its scale
                 release_and_issue(0, 0);
                 uint32_t codes = 0, pend = 0;
 #pragma unroll 1
                 for (int g = 0; g < ngh; ++g) {
                     {
-                        mbar_wait<PF_TOK_NS>(bar(B_S + wg), n_s & 1, abort_flag);
-                        ++n_s;
-                        tc_fence_after();
-                        __syncwarp();
+                        wait_chunk();
                         uint32_t v[32];
                         accumulators(0, v);
                         minima(0, v);
@@ -866,10 +893,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                     }
                     {
                         float q2n = 0.f;
-                        mbar_wait<PF_TOK_NS>(bar(B_S + wg), n_s & 1, abort_flag);
-                        ++n_s;
-                        tc_fence_after();
-                        __syncwarp();
+                        wait_chunk();
                         uint32_t v[32];
                         accumulators(0, v);
                         minima(2, v);
@@ -1026,6 +1050,17 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
         tc_fence_before();
         __syncthreads();                               // constants, matrix slices and TMEM are free for the next segment
         tc_fence_after();
+        if (*abort_flag) break;                        // (the same in every warp: nobody waits before the next barrier)
+    }
+    if (*abort_flag) {
+        // the MMAs of the five issuing warps have to end before TMEM is handed back
+        if (warp == PF_TOKEN_WARPS || (warp < PF_TOKEN_WARPS && (warp & 3) == 0)) {
+            if (elect_one()) umma_commit(bar(B_DRAIN));
+            __syncwarp();
+        }
+        int tries = 0;
+        while (!mbar_try(bar(B_DRAIN), 0) && ++tries < 1000000) {}
+        __syncthreads();
     }
     if (warp == 0) tmem_dealloc<512>(tmem);
     if (threadIdx.x == 0 && misc[1] != 0) atomicOr(a.dev_status, NOVAKV_DEV_WAIT_TIMEOUT);
@@ -1098,7 +1133,7 @@ novakv_status novakv_launch_prefill(novakv_ctx* ctx, const novakv_layer& ly, con
     __nv_bfloat16* v_meta) {
     PrefillArgs a = {k_new, v_new, tok_seq, tok_pos, n_tokens, ly.pf_r, ly.pf_cb, ly.pf_const, ly.rk_d, ly.rv_d, ly.rk_rows, ly.rv_rows, ly.k_mean_d,
                            ly.v_mean_d, ly.cb_k, ly.cb_v, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
-                           n_seq, seq_lens, ctx->cfg.n_kv_heads, 1, 1, 1, 0, ctx->dev_status, {}, {}};
+                           n_seq, seq_lens, ctx->cfg.n_kv_heads, 1, 1, 1, 0, ctx->wait_clocks, ctx->dev_status, {}, {}};
     if (ctx->cfg.head_dim == 128)
         return v_meta ? launch_prefill_t<128, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<128, 1>(ctx, a, stream) : launch_prefill_t<128, 0>(ctx, a, stream));
     return v_meta ? launch_prefill_t<64, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<64, 1>(ctx, a, stream) : launch_prefill_t<64, 0>(ctx, a, stream));

@@ -4,7 +4,10 @@
 #include <stdint.h>
 
 // Bounded wait on an mbarrier phase.  Returns false when the wait has given up (or another warp of the CTA has, which
-// *abort_flag in shared memory tells); the caller then stops issuing work and goes to the teardown.
+// *abort_flag in shared memory tells); the caller then stops issuing work and goes to the teardown.  The limit in clocks is
+// the 64-bit number at abort_flag + MBAR_LIMIT.  Once a wait has given up the parities of this thread's later waits mean
+// nothing: one may succeed on the phase before the one it wants, so what it guards has to be checked by other means.
+constexpr int MBAR_LIMIT = 7;
 // A try returns after a few dozen cycles whether or not the phase is over, so a polling warp takes issue slots from the
 // warps it waits for: NS nanoseconds are slept between tries.
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
@@ -15,15 +18,16 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
 }
 template <int NS>
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-    const long long t0 = clock64();
+    const long long t0 = clock64(), limit = *reinterpret_cast<volatile const long long*>(abort_flag + MBAR_LIMIT);
+    const int tries = limit < 64 ? (int)limit : 64;               // (a limit of 0 gives up at once)
     for (;;) {
 #pragma unroll 1
-        for (int i = 0; i < 64; ++i) {
+        for (int i = 0; i < tries; ++i) {
             if (NS > 0) __nanosleep(NS);
             if (mbar_try(bar, parity)) return true;
         }
         if (*abort_flag) return false;
-        if (clock64() - t0 > 2000000000ll) { *abort_flag = 1; return false; }        // about a second
+        if (clock64() - t0 > limit) { *abort_flag = 1; return false; }
     }
 }
 template <int NS = 0>
