@@ -133,6 +133,7 @@ struct PrefillArgs {
     int gs;                     // parts a head's groups are cut into
     int cost_k, cost_v;         // relative cost of a key / value unit (the cut of the walk)
     int tma;                    // the token rows can be copied by the tensor maps (16-byte aligned)
+    int words;                  // the pools can be written in words (4-byte aligned; single bytes otherwise)
     long wait_clocks;           // limit of a wait
     uint32_t* dev_status;
     CUtensorMap map_k, map_v;   // k_new / v_new as [n_tokens][Hkv d], boxes of 64 x 128
@@ -719,7 +720,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                     }
                 }
                 const int page0 = __shfl_sync(0xffffffffu, page, lane & 16), slot0 = __shfl_sync(0xffffffffu, slot, lane & 16);
-                const bool aligned = __all_sync(0xffffffffu, valid && page == page0 && (slot & 15) == (lane & 15) && (slot ^ slot0) < 16);
+                const bool aligned = a.words && __all_sync(0xffffffffu, valid && page == page0 && (slot & 15) == (lane & 15) && (slot ^ slot0) < 16);
                 if (ksc && valid && g0 == 0 && hf == 0)
                     a.k_scales[((size_t)page * a.n_kv_heads + kvh) * NOVAKV_PAGE_TOKENS + slot] = __float2bfloat16_rn(rho);
                 if (vsq) {
@@ -1023,7 +1024,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                         codes = (codes >> 8) | ((uint32_t)bi << 24);
                         pend = (pend >> 1) | (exact && valid ? 8u : 0u);
                         if ((l & 3) == 3) {
-                            if (__any_sync(0xffffffffu, pend != 0u)) {
+                            if (__any_sync(0xffffffffu, pend != 0u) || !a.words) {
                                 // single bytes: those that are searched again are written by the search alone
                                 if (valid) {
 #pragma unroll
@@ -1118,6 +1119,7 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
     // tensor maps of the new rows (rebuilt on every call: the buffers are the caller's)
     a.tma = (((uintptr_t)a.k_new | (uintptr_t)a.v_new) & 15) == 0 &&
             row_map(&a.map_k, a.k_new, a.n_tokens, hkv * D) && row_map(&a.map_v, a.v_new, a.n_tokens, hkv * D);
+    a.words = (((uintptr_t)a.k_pages | (uintptr_t)a.v_pages) & 3) == 0;
     novakv_prof_scope ps(ctx, 1, stream);
     kern<<<grid, PF_THREADS, P::BYTES, stream>>>(a);
     ps.end();
@@ -1133,7 +1135,7 @@ novakv_status novakv_launch_prefill(novakv_ctx* ctx, const novakv_layer& ly, con
     __nv_bfloat16* v_meta) {
     PrefillArgs a = {k_new, v_new, tok_seq, tok_pos, n_tokens, ly.pf_r, ly.pf_cb, ly.pf_const, ly.rk_d, ly.rv_d, ly.rk_rows, ly.rv_rows, ly.k_mean_d,
                            ly.v_mean_d, ly.cb_k, ly.cb_v, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
-                           n_seq, seq_lens, ctx->cfg.n_kv_heads, 1, 1, 1, 0, ctx->wait_clocks, ctx->dev_status, {}, {}};
+                           n_seq, seq_lens, ctx->cfg.n_kv_heads, 1, 1, 1, 0, 0, ctx->wait_clocks, ctx->dev_status, {}, {}};
     if (ctx->cfg.head_dim == 128)
         return v_meta ? launch_prefill_t<128, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<128, 1>(ctx, a, stream) : launch_prefill_t<128, 0>(ctx, a, stream));
     return v_meta ? launch_prefill_t<64, 2>(ctx, a, stream) : (k_scales ? launch_prefill_t<64, 1>(ctx, a, stream) : launch_prefill_t<64, 0>(ctx, a, stream));

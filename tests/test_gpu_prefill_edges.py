@@ -94,6 +94,27 @@ def test_prefill_rows_without_tensor_map_alignment(cases, name):
     _run(cases[name, False], "plain", 600, 0, False, False, offset=2)
 
 
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "scaled"), ("qwen", "deployed")])
+@pytest.mark.parametrize("shift", [1, 2])
+def test_prefill_pools_off_a_word_boundary(cases, name, fmt, shift):
+    """The append entries take pools on any address (decode wants 16 bytes): same bytes, written one by one."""
+    from paper_2608_04074_b200.runtime import PagedCache
+    case, n = cases[name, fmt != "plain"], 333
+    k, v, _ = case.draw(4400, n, 1)
+    args = (_dev(k, torch.bfloat16), _dev(v, torch.bfloat16), _dev(np.zeros(n, np.int32)), _dev(np.arange(n, dtype=np.int32)))
+    stored = []
+    for off in (0, shift):
+        cache = PagedCache(case.ctx, np.array([0], np.int32), capacity_tokens=np.array([n], np.int32), seed=7,
+                           key_scale=fmt == "scaled", int2_values=fmt == "deployed")
+        shifted = lambda x: torch.zeros(x.numel() + off, dtype=torch.uint8, device="cuda")[off:].view(x.shape)
+        cache.k_pages, cache.v_pages = shifted(cache.k_pages), shifted(cache.v_pages)
+        assert cache.k_pages.data_ptr() % 4 == off
+        cache.append(0, *args)
+        assert case.ctx.novakv_last_device_status() == 0
+        stored.append((cache.k_pages.clone(), cache.v_pages.clone()))
+    assert all(torch.equal(a, b) for a, b in zip(*stored))
+
+
 @pytest.mark.parametrize("n", [24, 41, 100, 256])
 @pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "plain"), ("qwen", "scaled"), ("gptoss", "deployed")])
 def test_append_batches_of_several_chunks(cases, name, fmt, n):
