@@ -132,7 +132,7 @@ size_t novakv_decode_workspace_bytes(const novakv_ctx* ctx, int batch);
  * can differ from a binary64 reference only where the two nearest codewords are within ~1e-12 relative.)
  * The 2L index bytes go to page page_table[tok_seq[t]][tok_pos[t]/64] at slot tok_pos[t]%64, and
  * seq_lens[tok_seq[t]] becomes max(seq_lens[tok_seq[t]], tok_pos[t]+1).
- *   k_new, v_new  bf16 [n_tokens][Hkv][d]
+ *   k_new, v_new  bf16 [n_tokens][Hkv][d], 4-byte aligned (NOVAKV_EINVAL otherwise; 16-byte aligned rows are faster)
  *   tok_seq, tok_pos  int32 [n_tokens]; two tokens of one call must not share (seq, pos);
  *                     tok_seq[t] = -1 marks an unused entry of the list: it is skipped, no status bit
  *   n_tokens = 0 is a no-op.  Out-of-range tokens/pages set device status bits and are skipped.

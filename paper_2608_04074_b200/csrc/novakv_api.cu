@@ -276,6 +276,7 @@ extern "C" novakv_status novakv_encode_append(novakv_ctx* ctx, int layer, const 
     if (n_tokens == 0) return NOVAKV_OK;
     if (!k_new || !v_new || !tok_seq || !tok_pos || !k_pages || !v_pages || !page_table || !seq_lens) return NOVAKV_EINVAL;
     if (n_pages <= 0 || max_pages_per_seq <= 0 || n_seq <= 0) return NOVAKV_EPAGE;
+    if (((uintptr_t)k_new | (uintptr_t)v_new) & 3) return NOVAKV_EINVAL;
     if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return NOVAKV_ECUDA;
     return novakv_launch_encode(ctx, ctx->layers[layer], (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
                                 tok_seq, tok_pos, n_tokens, k_pages, v_pages, n_pages, page_table,
@@ -316,6 +317,7 @@ extern "C" novakv_status novakv_encode_append_scaled(novakv_ctx* ctx, int layer,
     if (!k_new || !v_new || !tok_seq || !tok_pos || !k_pages || !v_pages || !k_scales || !page_table || !seq_lens) return NOVAKV_EINVAL;
     if (n_pages <= 0 || max_pages_per_seq <= 0 || n_seq <= 0) return NOVAKV_EPAGE;
     if ((uintptr_t)k_scales & 1) return NOVAKV_EINVAL;
+    if (((uintptr_t)k_new | (uintptr_t)v_new) & 3) return NOVAKV_EINVAL;
     if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return NOVAKV_ECUDA;
     return novakv_launch_encode(ctx, ctx->layers[layer], (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
                                 tok_seq, tok_pos, n_tokens, k_pages, v_pages, n_pages, page_table,
@@ -406,6 +408,7 @@ extern "C" novakv_status novakv_encode_append_deployed(novakv_ctx* ctx, int laye
         return NOVAKV_EINVAL;
     if (n_pages <= 0 || max_pages_per_seq <= 0 || n_seq <= 0) return NOVAKV_EPAGE;
     if (((uintptr_t)k_scales & 1) || ((uintptr_t)v_meta & 3)) return NOVAKV_EINVAL;
+    if (((uintptr_t)k_new | (uintptr_t)v_new) & 3) return NOVAKV_EINVAL;
     if (cudaSetDevice(ctx->cfg.device) != cudaSuccess) return NOVAKV_ECUDA;
     return novakv_launch_encode(ctx, ctx->layers[layer], (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new,
                                 tok_seq, tok_pos, n_tokens, k_pages, v_pages, n_pages, page_table,

@@ -590,7 +590,10 @@ novakv_status launch_encode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
                               int n_tokens, uint8_t* k_pages, uint8_t* v_pages, int n_pages,
                               const int32_t* page_table, int max_pages_per_seq, int n_seq, int32_t* seq_lens,
                               cudaStream_t stream, __nv_bfloat16* k_scales, __nv_bfloat16* v_meta) {
-    if (n_tokens <= NOVAKV_SMALL_APPEND_TOKENS) {
+    // (the append kernel reads the new rows in 16-byte pieces; rows on a 4-byte boundary take the prompt encoder, which can
+    // copy them in words, whatever their number)
+    const bool rows16 = (((uintptr_t)k_new | (uintptr_t)v_new) & 15) == 0;
+    if (n_tokens <= NOVAKV_SMALL_APPEND_TOKENS && rows16) {
         int tp_log2 = 0;
         while ((1 << tp_log2) < n_tokens && tp_log2 < SMALL_TP_LOG2) ++tp_log2;
         // chunks of the token list: as many as there are passes, while all CTAs are resident together

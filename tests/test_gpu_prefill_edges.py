@@ -94,6 +94,20 @@ def test_prefill_rows_without_tensor_map_alignment(cases, name):
     _run(cases[name, False], "plain", 600, 0, False, False, offset=2)
 
 
+@pytest.mark.parametrize("n", [1, 8, 130, 256])
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "scaled"), ("qwen", "deployed")])
+def test_append_rows_on_a_word_boundary(cases, name, fmt, n):
+    """Batches of the append kernel's size whose rows it cannot read (16-byte loads): the same indices, at any number."""
+    _run(cases[name, fmt != "plain"], fmt, n, 40, False, False, offset=2)
+
+
+@pytest.mark.parametrize("n", [8, 600])
+def test_append_rows_off_a_word_boundary_are_refused(cases, n):
+    from paper_2608_04074_b200.binding import NovaKVError
+    with pytest.raises(NovaKVError, match="invalid argument"):
+        _run(cases["qwen", False], "plain", n, 0, False, False, offset=1)
+
+
 @pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "scaled"), ("qwen", "deployed")])
 @pytest.mark.parametrize("shift", [1, 2])
 def test_prefill_pools_off_a_word_boundary(cases, name, fmt, shift):
