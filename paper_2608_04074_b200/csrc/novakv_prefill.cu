@@ -635,7 +635,8 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                 float bound;                                                   // times a column norm: error of that coefficient
                 {
                     const float x2 = x2_s[(2 * w) * (P::A_BYTES / 4) + row] + x2_s[(2 * w + 1) * (P::A_BYTES / 4) + row];
-                    bound = KAPPA * (sqrtf(x2) * 1.00001f + cst[D + 2 * L] /* |mean| */);
+                    // (a sum of squares below 1e-30 may have lost terms to underflow: 1e-15 bounds |x| then)
+                    bound = KAPPA * (sqrtf(fmaxf(x2, 1e-30f)) * 1.00001f + cst[D + 2 * L] /* |mean| */);
                 }
                 mbar_wait<PF_TOK_NS>(bar(B_T + w), n_it & 1, abort_flag);
                 tc_fence_after();

@@ -108,6 +108,30 @@ def test_append_rows_off_a_word_boundary_are_refused(cases, n):
         _run(cases["qwen", False], "plain", n, 0, False, False, offset=1)
 
 
+@pytest.mark.parametrize("factor", [1e-17, 1e-22, 1e-30])
+@pytest.mark.parametrize("name,fmt", [("qwen", "scaled"), ("gptoss", "scaled"), ("qwen", "deployed")])
+def test_prefill_squares_that_underflow(cases, name, fmt, factor):
+    """Per-token scales make the format indifferent to the size of the inputs, so the error bound of the coefficients must not
+    vanish with the squares of the row: the same bytes as the append kernel's, which searches binary64 coefficients."""
+    from paper_2608_04074_b200.runtime import PagedCache
+    case, n = cases[name, True], 16384
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    k, v = ((torch.randn((n, case.ctx.n_kv_heads, case.ctx.head_dim), generator=gen, device="cuda") * factor).to(torch.bfloat16)
+            for _ in range(2))
+    k[:, :, ::16] *= 40.0                                  # a few large elements: small coefficients with large errors beside them
+    seq, pos = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.arange(n, dtype=torch.int32, device="cuda")
+    stored = []
+    for step in (n, 256):
+        cache = PagedCache(case.ctx, np.array([0], np.int32), capacity_tokens=np.array([n], np.int32), seed=7,
+                           key_scale=fmt == "scaled", int2_values=fmt == "deployed")
+        for i in range(0, n, step):
+            cache.append(0, k[i:i + step], v[i:i + step], seq[i:i + step], pos[i:i + step])
+        assert case.ctx.novakv_last_device_status() == 0
+        stored.append([x for x in (cache.k_pages, cache.v_pages, cache.k_scales, cache.v_meta) if x is not None])
+    for prompt, small in zip(*stored):
+        assert torch.equal(prompt, small), int((prompt != small).sum())
+
+
 @pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "scaled"), ("qwen", "deployed")])
 @pytest.mark.parametrize("shift", [1, 2])
 def test_prefill_pools_off_a_word_boundary(cases, name, fmt, shift):
