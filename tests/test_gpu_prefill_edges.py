@@ -108,6 +108,28 @@ def test_append_rows_off_a_word_boundary_are_refused(cases, n):
         _run(cases["qwen", False], "plain", n, 0, False, False, offset=1)
 
 
+@pytest.mark.parametrize("first,n", [(0, 600), (299, 300), (640, 700), (1279, 2048), (2047, 2048), (3000, 3000)])
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "scaled"), ("qwen", "deployed")])
+def test_prefill_leading_entries_unused(cases, name, fmt, first, n):
+    """Lists that begin with `first` unused entries (first = n: nothing else): the CTAs that meet none leave, the
+    others store what they always store."""
+    from paper_2608_04074_b200.runtime import PagedCache
+    case = cases[name, fmt != "plain"]
+    k, v, _ = case.draw(4500, n, 1)
+    kd, vd, pos = _dev(k, torch.bfloat16), _dev(v, torch.bfloat16), np.arange(n, dtype=np.int32)
+    stored = []
+    for seq in (np.where(pos < first, -1, 0), np.zeros(n)):
+        cache = PagedCache(case.ctx, np.array([0], np.int32), capacity_tokens=np.array([n], np.int32), seed=7,
+                           key_scale=fmt == "scaled", int2_values=fmt == "deployed")
+        cache.append(0, kd, vd, _dev(seq.astype(np.int32)), _dev(pos))
+        assert case.ctx.novakv_last_device_status() == 0
+        stored.append([*cache.load_logical(0, 0, n), *([cache.load_scales(0, 0, n)] if fmt != "plain" else []), cache.seq_lens.cpu()])
+    part, full = stored
+    assert int(part[-1][0]) == (n if first < n else 0)
+    for i, (p, f) in enumerate(zip(part[:-1], full[:-1])):
+        assert np.array_equal(p[first:], f[first:]) and (p[:first] == (1 if i == 2 else 0)).all()
+
+
 @pytest.mark.parametrize("factor", [1e-17, 1e-22, 1e-30])
 @pytest.mark.parametrize("name,fmt", [("qwen", "scaled"), ("gptoss", "scaled"), ("qwen", "deployed")])
 def test_prefill_squares_that_underflow(cases, name, fmt, factor):
