@@ -1127,8 +1127,9 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
             best = longest;
             grid = g;
             a.gs = gs;
-            a.cost_k = (int)(ck * 64.0);
-            a.cost_v = (int)(cv * 64.0);
+            // one unit per CTA where there are no more than SMs: a cut in cost would hand some a key and a value unit
+            a.cost_k = uk + uv <= ctx->n_sm ? 1 : (int)(ck * 64.0);
+            a.cost_v = uk + uv <= ctx->n_sm ? 1 : (int)(cv * 64.0);
         }
     }
     // tensor maps of the new rows (rebuilt on every call: the buffers are the caller's)
