@@ -129,10 +129,11 @@ __device__ __forceinline__ int clamp_len(int len, int max_pages) {
 // ------------------------------------------------------------------------------------------------
 // One block per KV head and run of `seqs_per_block` sequences: its share of rk_inv_t is read once into registers, and the
 // Hg queries of a (sequence, head) share it.  512 threads = D columns x (512/D) row parts; each thread's loads are
-// independent and all in flight.  Small batches take one sequence per block (latency); once there are more pairs than the
+// independent and all in flight.  Small batches take one sequence per block, in an instantiation without the loop (RUNS =
+// false: the loop's registers cost 0.7 us of 4.1, cold, at 8 sequences x 8 heads); once there are more pairs than the
 // machine holds blocks, runs save the 64 KB per pair that re-reading the transform costs: 128 sequences x 8 heads,
 // d = 128: 13.5 -> 8.2 us.
-template <int D, int HG>
+template <int D, int HG, bool RUNS>
 __global__ void __launch_bounds__(512)
 novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict__ rk_inv_t,
                       const int32_t* __restrict__ seq_lens, int batch, int n_q_heads, int n_kv_heads,
@@ -217,9 +218,9 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ float q_s[HG][D];
     __shared__ float red_s[PARTS][HG][D];
-    const int b_end = min(batch, (run + 1) * seqs_per_block);
-    for (int b = run * seqs_per_block; b < b_end; ++b) {
-        if (b != run * seqs_per_block) __syncthreads();        // the shared arrays are free
+    const int b0 = RUNS ? run * seqs_per_block : run, b_end = RUNS ? min(batch, b0 + seqs_per_block) : run + 1;
+    for (int b = b0; b < b_end; ++b) {
+        if (RUNS && b != b0) __syncthreads();                  // the shared arrays are free
         if (pair_count != nullptr && threadIdx.x == 0) pair_count[kvh * batch + b] = 0;
         for (int i = threadIdx.x; i < HG * D; i += 512)
             q_s[i / D][i % D] = __bfloat162float(q[((size_t)b * n_q_heads + kvh * HG) * D + i]);
@@ -2164,7 +2165,8 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
 
     // sequences per prepare block: one while all pairs fit on the machine twice over, then enough to make that so
     const int seqs_per_block = max(1, min(8, (batch * hkv + 2 * ctx->n_sm - 1) / (2 * ctx->n_sm)));
-    novakv_launch_pdl(novakv_prepare_kernel<D, HG>, dim3((batch + seqs_per_block - 1) / seqs_per_block * hkv + 1), dim3(512), 0, stream, q, ly.rk_inv_t, seq_lens,
+    auto prepare = seqs_per_block > 1 ? novakv_prepare_kernel<D, HG, true> : novakv_prepare_kernel<D, HG, false>;
+    novakv_launch_pdl(prepare, dim3((batch + seqs_per_block - 1) / seqs_per_block * hkv + 1), dim3(512), 0, stream, q, ly.rk_inv_t, seq_lens,
                       batch, hq, hkv, max_pages_per_seq, sm_scale * 1.4426950408889634f, qp, prefix, ctx->dev_status,
                       k_off_vec, qk_off, cost_prefix, ctx->seg_weight, (const float*)ly.k_center, qc,
                       fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32, seqs_per_block);
