@@ -284,8 +284,9 @@ novakv_status launch_bf16_t(novakv_ctx* ctx, const __nv_bfloat16* q, const __nv_
     float* part_ml = (float*)workspace;
     const size_t ml_bytes = (((size_t)batch * hkv * ms * HG * 2 * 4) + 255) & ~(size_t)255;
     float* part_acc = (float*)((char*)workspace + ml_bytes);
-    // with a window only the pages it touches are scanned
-    const int scan_pages = window > 0 ? (window + 2 * NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS : max_pages_per_seq;
+    // with a window only the pages it can touch are scanned: w tokens that end anywhere lie on at most (w - 2) / 64 + 2 pages
+    const bool windowed = window > 0 && window / NOVAKV_PAGE_TOKENS < max_pages_per_seq;
+    const int scan_pages = windowed ? (window + 2 * NOVAKV_PAGE_TOKENS - 2) / NOVAKV_PAGE_TOKENS : max_pages_per_seq;
     const int grid_x = (min(scan_pages, max_pages_per_seq) + BF16_SPLIT_PAGES - 1) / BF16_SPLIT_PAGES;
     dim3 grid(grid_x, hkv, batch);
     {

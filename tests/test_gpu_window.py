@@ -20,7 +20,8 @@ def cases():
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("window,lens", [(1, [1, 64, 65]), (127, [5, 128, 191, 0, 700]), (130, [1023, 131]), (961, [1000, 1088]),
-                                         (962, [1000, 1088]), (0, [1024, 3, 0]), (0, [1025, 9])])
+                                         (962, [1000, 1088]), (960, [1087, 1023]), (961, [1026, 1087]), (962, [1026, 1087]),
+                                         (0x7fffffff, [1088, 7]), (0, [1024, 3, 0]), (0, [1025, 9])])
 @pytest.mark.parametrize("name", ["qwen", "gptoss"])
 def test_one_cta_per_sequence(cases, name, window, lens, dtype):
     case, lens = cases[name], np.array(lens, np.int32)
@@ -38,8 +39,11 @@ def test_one_cta_per_sequence(cases, name, window, lens, dtype):
     _, _, q = case.draw(1550, 1, len(lens))
     ws = torch.empty(ctx.novakv_bf16_workspace_bytes(len(lens), table.shape[1]), dtype=torch.uint8, device="cuda")
     out = torch.full((len(lens), ctx.n_q_heads, ctx.head_dim), float("nan"), dtype=dtype, device="cuda")
+    before = ctx.novakv_launch_count()
     ctx.novakv_bf16_decode_attention(dev(q).to(torch.bfloat16), dev(kp).to(torch.bfloat16), dev(vp).to(torch.bfloat16),
                                      dev(np.where(table < 0, 0, table).astype(np.int32)), dev(lens), out, ws, window=window)
+    # one kernel while 16 pages hold the capacity, or the window wherever it ends; else a merge kernel follows
+    assert ctx.novakv_launch_count() - before == (1 if table.shape[1] <= 16 or 0 < window <= 961 else 2)
     got = out.float().cpu().numpy()
     for b, n in enumerate(lens):
         if n == 0:
