@@ -1703,9 +1703,12 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
 // their scales; then every thread sums its coordinate over the pieces, all loads independent.  Bound by that chain of
 // memory latencies (lengths and prefixes, ranges, (max, sum) pairs, accumulators: about 3 us), which the sequences of a
 // block share: 256 pairs 11.5 -> 9.0 us, 1024 pairs 22.4 -> 19.3 us (cold caches).
+// RUNS = false: one sequence per block (batches that give every SM at most one block).  Nothing is shared then, and the
+// warp's 10 shuffles per head would only lengthen the chain: all threads fetch the candidates and their (max, sum) pairs, and
+// every thread combines them itself.  16 sequences of the d = 64 shape with eight heads: 7.7 us with the shuffles, 6.5
+// without (cold); d = 128, 8 sequences: 7.9 us where one warp searches, 7.1 so.
 // EXT = the call carries a learned sink logit and/or a BF16 band partial; without it that code is compiled out.
-
-template <int D, int HG, bool EXT>
+template <int D, int HG, bool EXT, bool RUNS>
 __global__ void __launch_bounds__(HG * D > 512 ? 512 : HG * D, 1)
 novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __restrict__ part_acc,
                            const int32_t* __restrict__ page_prefix, const int32_t* __restrict__ seq_lens,
@@ -1718,12 +1721,14 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
                            const float* __restrict__ band_acc /* [batch][Hq][D] sum p v of the band, original value domain */,
                            const int32_t* __restrict__ cost_prefix, int seg_weight, const long* __restrict__ cta_range,
                            int seqs_per_block) {
-    constexpr int NP = HG <= 4 ? 4 : 2 /* as shared memory allows */, NT = HG * D > 512 ? 512 : HG * D, NW = NT / 32;
+    constexpr int NP = !RUNS ? 1 : HG <= 4 ? 4 : 2 /* as shared memory allows */, NT = HG * D > 512 ? 512 : HG * D, NW = NT / 32;
     constexpr int PARTS = NT / D, COLS = D / PARTS, PER = (HG * D + NT - 1) / NT;
     __shared__ float o_s[NP][HG * D];
     __shared__ float red_s[PARTS][HG][D];
-    __shared__ short piece_s[NP][MAX_SCAN_CTAS + 1];          // scan CTAs that hold a piece of the sequence
-    __shared__ float scale_s[NP][MAX_SCAN_CTAS + 1][HG];      // 2^(max of the piece - common max)
+    __shared__ short piece_s[RUNS ? NP : 1][RUNS ? MAX_SCAN_CTAS + 1 : 1];          // scan CTAs that hold a piece of the sequence
+    __shared__ float scale_s[RUNS ? NP : 1][RUNS ? MAX_SCAN_CTAS + 1 : 1][HG];      // 2^(max of the piece - common max)
+    __shared__ float2 ml_s[RUNS ? 1 : MAX_SCAN_CTAS + 1][HG];                       // (max, sum) of a candidate's piece
+    __shared__ int cand_s[RUNS ? 1 : MAX_SCAN_CTAS + 1];                            // 1 = this candidate holds a piece
     __shared__ float m_s[NP][HG], l_s[NP][HG];                // common maximum and sum
     __shared__ float frac_s[NP][HG];                          // share of the softmax mass on quantised tokens (1 without sink and band)
     __shared__ float bsc_s[NP][HG];                           // multiplier of the band accumulator (0 without a band)
@@ -1749,10 +1754,31 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
 #ifdef NOVAKV_TIMING
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_m1));
 #endif
-    const int b_end = min(batch, (run + 1) * seqs_per_block);
-    for (int b0 = run * seqs_per_block; b0 < b_end; b0 += NP) {
-        const int np = min(NP, b_end - b0);
-        for (int p = warp; p < np; p += NW) {
+    const int b_end = RUNS ? min(batch, (run + 1) * seqs_per_block) : run + 1;
+    for (int b0 = RUNS ? run * seqs_per_block : run; b0 < b_end; b0 += NP) {
+        const int np = RUNS ? min(NP, b_end - b0) : 1;
+        int c_first = 0, n_cand = 0;
+        if (!RUNS) {
+            // the same search, candidates and their (max, sum) pairs each fetched by as many threads
+            const int pages_b = (clamp_len(seq_lens[b0], max_pages_per_seq) + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
+            if (pages_b > 0) {
+                const long P = page_prefix[batch], cost_all = cost_prefix[batch];
+                const long u0 = (long)kvh * P + page_prefix[b0], u1 = u0 + pages_b, T = cost_all * n_kv_heads;
+                const long x0 = (long)kvh * cost_all + cost_prefix[b0] + seg_weight, x1 = x0 + pages_b - 1;
+                c_first = max((int)(((x0 + 1) * grid_s1 - 1) / T) - 1, 0);
+                n_cand = min((int)(((x1 + 1) * grid_s1 - 1) / T) + 1, grid_s1 - 1) - c_first + 1;
+                for (int t = threadIdx.x; t < n_cand; t += NT) {
+                    const long r0 = cta_range[(c_first + t) * 2], r1 = cta_range[(c_first + t) * 2 + 1];
+                    cand_s[t] = r0 < r1 && r1 > u0 && r0 < u1;
+                }
+            }
+            if (threadIdx.x == 0) n_s[0] = pages_b > 0 ? 0 : -1;
+            __syncthreads();
+            for (int i = threadIdx.x; i < n_cand * HG; i += NT)
+                if (cand_s[i / HG])
+                    ml_s[i / HG][i % HG] = *reinterpret_cast<const float2*>(part_ml + (((size_t)kvh * batch + b0 + c_first + i / HG) * HG + i % HG) * 2);
+        }
+        for (int p = RUNS ? warp : np; p < np; p += NW) {
             const int b = b0 + p;
             const int len = clamp_len(seq_lens[b], max_pages_per_seq);
             const int pages_b = (len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
@@ -1823,11 +1849,25 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
                 const int i = threadIdx.x + k * NT;
                 if (i >= HG * D) break;
                 const int h = i / D, c = i - h * D;
-                float a = 0.f;
+                float a = 0.f, M, lsum;
+                if (RUNS) {
 #pragma unroll 4
-                for (int j = 0; j < n; ++j)
-                    a = fmaf(scale_s[p][j][h], part_acc[(((size_t)kvh * batch + b + piece_s[p][j]) * HG + h) * D + c], a);
-                float M = m_s[p][h], lsum = l_s[p][h];
+                    for (int j = 0; j < n; ++j)
+                        a = fmaf(scale_s[p][j][h], part_acc[(((size_t)kvh * batch + b + piece_s[p][j]) * HG + h) * D + c], a);
+                    M = m_s[p][h];
+                    lsum = l_s[p][h];
+                } else {
+                    M = M_INIT;
+                    lsum = 0.f;
+                    for (int j = 0; j < n_cand; ++j)
+                        if (cand_s[j]) M = fmaxf(M, ml_s[j][h].x);
+                    for (int j = 0; j < n_cand; ++j) {
+                        if (!cand_s[j]) continue;
+                        const float sc = ex2(ml_s[j][h].x - M);
+                        a = fmaf(sc, part_acc[(((size_t)kvh * batch + b + c_first + j) * HG + h) * D + c], a);
+                        lsum = fmaf(sc, ml_s[j][h].y, lsum);
+                    }
+                }
                 float lq = lsum;          // mass of the quantised tokens at the running scale
                 float wb = 0.f;           // weight of the band accumulator at the running scale
                 const int hq = kvh * HG + h;
@@ -2217,10 +2257,11 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     }
     if (fuse) return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
     const bool ext = sink_logits != nullptr || band != nullptr;
-    auto merge = ext ? novakv_decode_merge_kernel<D, HG, true> : novakv_decode_merge_kernel<D, HG, false>;
     // (one block per SM, so that the slice of the transform stays in registers, and one wave of blocks where at most 8
     // sequences a block make that possible)
     const int merge_run = max(1, min(8, (batch + max(1, ctx->n_sm / hkv) - 1) / max(1, ctx->n_sm / hkv)));
+    auto merge = merge_run > 1 ? (ext ? novakv_decode_merge_kernel<D, HG, true, true> : novakv_decode_merge_kernel<D, HG, false, true>)
+                               : (ext ? novakv_decode_merge_kernel<D, HG, true, false> : novakv_decode_merge_kernel<D, HG, false, false>);
     novakv_launch_pdl(merge, dim3((batch + merge_run - 1) / merge_run * hkv), dim3(HG * D > 512 ? 512 : HG * D), 0, stream,
                       part_ml, part_acc, prefix, seq_lens, batch, hq, hkv, max_pages_per_seq, grid, ly.rv_t, ly.v_mean, out,
                       out_is_fp32, sink_logits, qk_off, (const float*)band_ml, (const float*)band_acc,
