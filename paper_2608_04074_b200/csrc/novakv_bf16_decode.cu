@@ -15,7 +15,7 @@ namespace {
 
 constexpr int BF16_SPLIT_PAGES = 16;     // 1024 tokens per CTA
 constexpr int BF16_WARPS = 4;            // per CTA of several splits
-constexpr int BF16_WARPS_ONE = 8;        // per CTA that has its sequence (or window) to itself
+constexpr int BF16_WARPS_ONE = 8;        // per CTA that has its sequence (or window) and an SM to itself
 constexpr int TG = 8;                    // tokens per warp iteration
 constexpr float M_INIT = -1.0e30f;
 
@@ -58,8 +58,9 @@ __device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w <
 __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
 // ONE: a single split covers whatever a sequence can have (the host knows: window or capacity of at most BF16_SPLIT_PAGES
-// pages), so the CTA writes the output itself.  Bound by latency then (length -> page id -> rows -> merge): eight warps, so
-// that a window of 128 tokens is two or three groups each (16 would spill at d = 64, Hg = 8), no second kernel.  Window of 128, 16 sequences, 8 KV heads of
+// pages), so the CTA writes the output itself.  Bound by latency then (length -> page id -> rows -> merge): eight warps while
+// there is an SM for each CTA, so that a window of 128 tokens is two or three groups each (16 would spill at d = 64, Hg = 8),
+// no second kernel.  Window of 128, 16 sequences, 8 KV heads of
 // d = 64: 13.5 us with four warps and the merge kernel, 10.9 us so.
 template <int D, int HG, int WARPS, bool ONE>
 __global__ void __launch_bounds__(WARPS * 32)
@@ -295,7 +296,12 @@ novakv_status launch_bf16_t(novakv_ctx* ctx, const __nv_bfloat16* q, const __nv_
             kern<<<grid, warps * 32, 0, stream>>>(q, k_pages, v_pages, n_pages, page_table, max_pages_per_seq, seq_lens, hq, hkv,
                                                   sm_scale * 1.4426950408889634f, window, ms, part_ml, part_acc, out, out_is_fp32);
         };
-        if (grid_x == 1) stage1(novakv_bf16_stage1_kernel<D, HG, BF16_WARPS_ONE, true>, BF16_WARPS_ONE);
+        // Eight warps where every CTA has an SM to itself; more CTAs than SMs hide one another's latencies, and two of four
+        // warps get further than one of eight.  8 KV heads of d = 64, 8 / 4 warps: 16 sequences, window 128 5.1 / 5.7 us,
+        // window 512 11.9 / 14.5; 24 sequences 8.8 / 7.6 and 21.9 / 20.3; 128 sequences 28.0 / 20.9 and 77 / 62 (four warps
+        // and the merge kernel: 25.4 and 67).
+        if (grid_x == 1 && batch * hkv <= ctx->n_sm) stage1(novakv_bf16_stage1_kernel<D, HG, BF16_WARPS_ONE, true>, BF16_WARPS_ONE);
+        else if (grid_x == 1) stage1(novakv_bf16_stage1_kernel<D, HG, BF16_WARPS, true>, BF16_WARPS);
         else stage1(novakv_bf16_stage1_kernel<D, HG, BF16_WARPS, false>, BF16_WARPS);
         ps.end();
         ctx->launches++;

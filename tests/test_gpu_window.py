@@ -21,7 +21,8 @@ def cases():
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("window,lens", [(1, [1, 64, 65]), (127, [5, 128, 191, 0, 700]), (130, [1023, 131]), (961, [1000, 1088]),
                                          (962, [1000, 1088]), (960, [1087, 1023]), (961, [1026, 1087]), (962, [1026, 1087]),
-                                         (0x7fffffff, [1088, 7]), (0, [1024, 3, 0]), (0, [1025, 9])])
+                                         (0x7fffffff, [1088, 7]), (0, [1024, 3, 0]), (0, [1025, 9]),
+                                         (127, [5, 128, 191, 0, 700, *range(120, 140)])])     # more CTAs than SMs: four warps each
 @pytest.mark.parametrize("name", ["qwen", "gptoss"])
 def test_one_cta_per_sequence(cases, name, window, lens, dtype):
     case, lens = cases[name], np.array(lens, np.int32)
