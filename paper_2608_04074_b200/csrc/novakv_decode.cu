@@ -364,6 +364,12 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+// two grid indices u 2^-24 -> (u - 64) 2^-10, exact
+__device__ __forceinline__ uint32_t grid_steps(uint32_t u) {
+    uint32_t d;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(u), "r"(0x74007400u), "r"(0xac00ac00u));
+    return d;
+}
 // the same with a zero accumulator
 __device__ __forceinline__ void mma_f16_zero(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
@@ -1317,10 +1323,13 @@ __device__ __forceinline__ Segment segment_at(const int32_t* __restrict__ page_p
 // ------------------------------------------------------------------------------------------------
 // A score table costs 32 bytes of shared-memory reads and eight additions per (token, group) here.  A key codeword costs 16
 // bytes - four binary16 coordinates and their binary16 remainders, about 22 bits - and the additions are matrix products
-// over all eight heads at once, binary32 accumulators (against binary64: rel 3e-7 of the logits, as the binary32 table).
+// over all eight heads at once, binary32 accumulators.
 // The codewords belong to the KV head, so a segment has no table to build: its set-up is 16 numbers of q' per lane.
 //   mma m16n8k16: rows 0-7 = q_hi and rows 8-15 = q_lo of the eight heads, columns = 8 tokens, K = 4 groups; one product
-//   takes the codewords' hi halves and one their remainders, and a logit is the sum of its two rows.  Lane
+//   takes the codewords' hi halves and one their remainders, and a logit is the sum of its two rows.  The tensor core
+//   truncates: the remainders have accumulators of their own, so that four truncations at the size of the logit are left
+//   instead of eight, and what those lose on average (half an ulp each at a size that grows: 1.0e-7, measured) is given back
+//   by the addition that the remainders need anyway.  Lane
 //   (fr, fc) = (lane / 4, lane % 4) supplies groups 4 fc .. 4 fc + 3 (one per k-step) of the token in column fr: the two
 //   64-bit halves of a 128-bit gather are the two B operands as they stand.  (Codewords as A, tokens as rows, need three
 //   products for 16 tokens instead of four, but the operand then mixes two gathers: 64 register moves per 32 tokens.)
@@ -1328,13 +1337,16 @@ __device__ __forceinline__ Segment segment_at(const int32_t* __restrict__ page_p
 //   product in the order in which the cache keeps the value bytes of a lane (tokens fc, 4 + fc, 8 + fc, 12 + fc).
 //   value product: rows = (group 8 gb + fr, coordinate 2 cp) and, at fr + 8, coordinate 2 cp + 1; K = 16 tokens.  One byte
 //   permutation takes the same coordinate of two codewords and widens it (bytes with a clear top bit pair with their
-//   replicated top bit).
+//   replicated top bit), and one multiply-add centres the grid.  (Sixteen products of one sign, truncated at the size of
+//   their sum before its centre is removed, cost 0.4 % of the output error at 32 tokens and 5 % at 512.)
+// Error against binary64, 96 sequences: outputs (rel) 6.47e-5 / 5.09e-5 / 5.89e-5 at 60 / 700 / 4000 tokens, the table kernel
+// 6.49e-5 / 5.17e-5 / 6.23e-5; log-sum-exp at 512 tokens 1.357e-5 against 1.356e-5 (binary16 weights are what both show).
 // Rows of 256 bytes, so that one byte permutation puts a code into an address.  Bank conflicts: the eight lanes of a quarter
 // warp read four groups of two tokens; two copies of the key codewords, their columns 64 bytes apart, serve even and odd fr.
 // Four copies of the value codewords, 32 bytes apart, serve the four fc.
-// Measured (16 sequences of 65536 tokens, 8 KV heads, sink, whole call): score table 193 us, this kernel 147-151 us.  No single
-// bound: HMMA pipe 54 %, issue slots 50 %, shared-memory pipe 60 %.  Taken out one at a time, the gathers give nothing, the
-// remainder products 18 us, the value product 26 us, all key products 32 us; loads alone take 99 us.
+// Measured (16 sequences of 65536 tokens, 8 KV heads, sink, whole call): score table 193 us, this kernel 161 us (145 us with one
+// chain of products and the centre removed afterwards, 4 us of it the accumulators of the remainders and 12 us the
+// multiply-adds, two chains of hi products 165 us).  No single bound.
 struct S1M {
     static constexpr int D = 64, HG = 8, L = 16;
     static constexpr int KEY_COPY = 65536, VAL_BYTES = 65536;
@@ -1363,7 +1375,7 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
     using C = S1M;
     constexpr int D = C::D, HG = C::HG, L = C::L;
     constexpr float SH = 15.f;                                // weights are scaled by 2^SH before the binary16 rounding
-    constexpr float CEN = 64.f * 5.9604644775390625e-08f;     // what one unit of weight adds beyond u - 64, in units of 2^-24
+    constexpr float LOST = 1.0e-7f;                           // share of a logit that four truncated accumulations lose on average
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ int s_found[2][4];
     const uint32_t s_base = smem_u32(smem);
@@ -1437,23 +1449,8 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
     float macc[2][2][4];                                      // [gb][cp]: coordinate 2 cp of heads 2 fc, + 1, then 2 cp + 1
 #pragma unroll
     for (int i = 0; i < 16; ++i) macc[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
-    // remove the centre of the value grid from the sums of the tiles since the last call
     auto flush_window = [&]() {
-        float ws = wsum[0] + wsum[1];
-        ws += __shfl_xor_sync(0xffffffffu, ws, 1);
-        ws += __shfl_xor_sync(0xffffffffu, ws, 2);
-        l_run += ws;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const float w = __shfl_sync(0xffffffffu, ws, 8 * fc + 4 * j);
-#pragma unroll
-            for (int gb = 0; gb < 2; ++gb)
-#pragma unroll
-                for (int cp = 0; cp < 2; ++cp) {
-                    macc[gb][cp][j] = fmaf(-CEN, w, macc[gb][cp][j]);
-                    macc[gb][cp][2 + j] = fmaf(-CEN, w, macc[gb][cp][2 + j]);
-                }
-        }
+        l_run += wsum[0] + wsum[1];
         wsum[0] = wsum[1] = 0.f;
     };
 
@@ -1564,12 +1561,12 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
             // ---- logits of head fr, tokens 8 i + fc and 8 i + 4 + fc, over us
             float z[4][2];
             {
-                float acc[4][4];
+                float acc[4][4], rem[4][4];                       // products of the codewords' hi halves; of their remainders
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks) {
                     uint4 c[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) 
+                    for (int i = 0; i < 4; ++i)
                         c[i] = ks < 2 ? lds_u128_at<C::KEY>(prmt_rep(kc[i], kcol[ks & 1], ksel[ks]))
                                       : lds_u128_at<C::KEY + 128>(prmt_rep(kc[i], kcol[ks & 1], ksel[ks]));
 #pragma unroll
@@ -1578,10 +1575,15 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
                         else mma_f16(acc[i], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], c[i].x, c[i].y);
                     }
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) mma_f16(acc[i], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], c[i].z, c[i].w);
+                    for (int i = 0; i < 4; ++i) {
+                        if (ks == 0) mma_f16_zero(rem[i], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], c[i].z, c[i].w);
+                        else mma_f16(rem[i], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], c[i].z, c[i].w);
+                    }
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) { z[i][0] = acc[i][0] + acc[i][2]; z[i][1] = acc[i][1] + acc[i][3]; }
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) z[i][j] = acc[i][j] + fmaf(acc[i][j], LOST, (rem[i][j] + rem[i][2 + j]) + acc[i][2 + j]);
             }
             if (nvalid < 32) {
 #pragma unroll
@@ -1634,8 +1636,8 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
                     for (int cp = 0; cp < 2; ++cp) {
                         constexpr uint32_t SEL0 = 0xC480u;     // bytes (u0, 0, u4, 0): the same coordinate of two codewords
                         const uint32_t sa = SEL0 + 0x1111u * (2 * cp), sb = SEL0 + 0x1111u * (2 * cp + 1);
-                        mma_f16(macc[gb][cp], prmt_rep(X[0], X[1], sa), prmt_rep(X[0], X[1], sb), prmt_rep(X[2], X[3], sa), prmt_rep(X[2], X[3], sb),
-                                bw[2 * blk], bw[2 * blk + 1]);
+                        mma_f16(macc[gb][cp], grid_steps(prmt_rep(X[0], X[1], sa)), grid_steps(prmt_rep(X[0], X[1], sb)),
+                                grid_steps(prmt_rep(X[2], X[3], sa)), grid_steps(prmt_rep(X[2], X[3], sb)), bw[2 * blk], bw[2 * blk + 1]);
                     }
                 }
             }
@@ -1645,6 +1647,8 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
         // ---- segment epilogue: merge the warps' partials, four heads at a time, and write one partial
         const float vs = v_scale[(size_t)sg.kvh * D + threadIdx.x % D], vo = v_off[(size_t)sg.kvh * D + threadIdx.x % D];
         flush_window();
+        l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+        l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
         float* const m_acc = reinterpret_cast<float*>(s_abs + C::MACC);             // [NCW][MHEADS][MROW]
         float2* const m_ml = reinterpret_cast<float2*>(s_abs + C::ML);              // [NCW][HG]
         if (fc == 0) m_ml[warp * HG + fr] = make_float2(m_run, l_run);
@@ -1681,7 +1685,7 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
                     lsum = fmaf(sc, ml.y, lsum);
                 }
                 // grid index sums -> value-transform coefficients: s (u - 64) + (lo + 64 s) per unit of weight
-                const float val = (vs * (a * 16777216.f) + vo * lsum) * 3.0517578125e-05f;
+                const float val = (vs * (a * 1024.f) + vo * lsum) * 3.0517578125e-05f;
                 part_acc[(pidx * HG + h) * D + c] = val;
                 if (c == 0) { part_ml[(pidx * HG + h) * 2] = M; part_ml[(pidx * HG + h) * 2 + 1] = lsum * 3.0517578125e-05f; }
             }

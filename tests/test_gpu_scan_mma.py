@@ -43,3 +43,26 @@ def test_logits_on_tensor_cores(case, lens, factor):
             assert not out[b].any()
         else:
             check_output(out[b], case.oracle.decode(q[b].astype(np.float64), encs[b]["kidx"], encs[b]["vidx"], sm_scale=scale))
+
+
+def test_no_further_from_binary64_than_the_table_kernel(case):
+    """The halves of query and codewords and the tensor core's truncation must not cost what the binary32 score table had: the
+    output error against binary64 stays within that of the table kernel (reached by the fused merge) on the same cache.  The
+    weights are binary16 numbers in both, and round alike: the two errors are equal to a percent (1.03 with eight chained
+    products per logit and the grid's centre removed afterwards)."""
+    from paper_2608_04074_b200.runtime import PagedCache
+    lens = np.full(24, 700, np.int32)
+    cache = PagedCache(case.ctx, lens, seed=5)
+    encs = [case.oracle.encode(*(x.astype(np.float64) for x in case.draw(900 + b, 700, 1)[:2]), with_gaps=False) for b in range(24)]
+    cache.store_logical_batch([(b, 0, e["kidx"], e["vidx"]) for b, e in enumerate(encs)])
+    _, _, q = case.draw(901, 1, 24)
+    scale = case.ctx.head_dim ** -0.5
+    refs = np.stack([case.oracle.decode(q[b].astype(np.float64), e["kidx"], e["vidx"], sm_scale=scale) for b, e in enumerate(encs)])
+    err = {}
+    try:
+        for fused in (False, True):
+            case.ctx.novakv_debug_set_fused_merge(fused)
+            err[fused] = np.linalg.norm(cache.decode(0, torch.from_numpy(q).to(torch.bfloat16).cuda(), sm_scale=scale).cpu().numpy() - refs)
+    finally:
+        case.ctx.novakv_debug_set_fused_merge(False)
+    assert err[False] <= 1.01 * err[True], err[False] / err[True]
