@@ -69,6 +69,7 @@ constexpr float M_INIT = -1.0e30f;
 #endif
 constexpr float M_SLACK = (float)NOVAKV_M_SLACK;   // headroom (bits) a running maximum gets when it moves
 constexpr int MAX_SCAN_CTAS = 255;            // scan CTAs (one per SM) the boundary table has room for
+constexpr int MMA_MIN_PAGES = 5;              // pages per SM from which on the d = 64 kernel with tensor-core logits is taken
 constexpr int PFX_CAP = 511;                  // batches up to this size keep their page / cost prefixes in shared memory
 
 // VM selects the value side: true = tensor cores (mma.sync m16n8k16, fp16 weights and codewords,
@@ -2217,9 +2218,13 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     ctx->launches++;
 
     // d = 64 with eight query heads per KV head, plain format: the kernel that takes the logits from tensor cores.  (At
-    // d = 128 its two copies of the key codewords do not fit; with four heads the table reads no more than they do.)
+    // d = 128 its two copies of the key codewords do not fit; with four heads a look-up in the table reads no more bytes than
+    // a gather of a codeword; the scaled format has not been built with it.)  Not for short calls: its CTAs stage 192 KB of
+    // codewords, which only pages pay back - 18 sequences of 100 tokens (2 pages an SM) 12.9 us with the table, 13.9 with
+    // products; 1 of 5000 and 48 of 100 (4 and 5) within 3 % of each other; 8 of 2000 (14) 18.4 and 17.6.  The capacity stands
+    // in for the lengths, which only the device knows.
     constexpr bool MMA = D == 64 && HG == 8 && VM && !KSC && !VSQ;
-    if (MMA && !fuse) {
+    if (MMA && !fuse && (long)batch * hkv * max_pages_per_seq >= (long)MMA_MIN_PAGES * ctx->n_sm) {
         constexpr unsigned mma_bit = 1u << 8;
         if (!(ctx->smem_opt_in & mma_bit)) {
             if (cudaFuncSetAttribute(novakv_decode_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_BYTES) != cudaSuccess) return NOVAKV_ECUDA;

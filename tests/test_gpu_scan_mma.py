@@ -19,12 +19,23 @@ def case():
     return Case(workloads.gpt_oss_20b(batch=2, seq_len=2048, calib_tokens=4096, lloyd_iters=6))
 
 
+# The tensor-core kernel is taken from a capacity of 5 pages (of 64 tokens) per SM on; the calls below it take the score table.
+# `wide`: the smallest page table that reaches the first, and the largest that stays with the second.
+@pytest.mark.parametrize("wide", [True, False], ids=["products", "table"])
 @pytest.mark.parametrize("factor", [1.0, 16.0, 1e-3, 1e-30])
 @pytest.mark.parametrize("lens", [[1], [31, 32, 33, 0, 63, 64, 65], [511, 512, 513, 1025], [3000], list(range(1, 160, 4))],
                          ids=lambda x: f"{len(x)}x{max(x)}")
-def test_logits_on_tensor_cores(case, lens, factor):
+def test_logits_on_tensor_cores(case, lens, factor, wide):
     from paper_2608_04074_b200.runtime import PagedCache
-    cache = PagedCache(case.ctx, np.array(lens, np.int32), seed=5)
+    need, per_page = 5 * torch.cuda.get_device_properties(0).multi_processor_count, len(lens) * case.ctx.n_kv_heads
+    pages = -(-need // per_page) - (0 if wide else 1)
+    assert wide == (pages * per_page >= need)
+    if 64 * pages < max(lens):
+        pytest.skip("so many sequences of this length are past the line whatever the capacity")
+    cap = np.array(lens, np.int32)
+    cap[0] = 64 * pages                                       # (the table is as wide as its longest row)
+    cache = PagedCache(case.ctx, np.array(lens, np.int32), capacity_tokens=cap, seed=5)
+    assert cache.page_table.shape[1] == pages
     encs, items = [], []
     for b, n in enumerate(lens):
         k, v, _ = case.draw(700 + b, max(n, 1), 1)
