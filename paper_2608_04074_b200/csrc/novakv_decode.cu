@@ -1713,8 +1713,12 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
 // every thread combines them itself.  16 sequences of the d = 64 shape with eight heads: 7.7 us with the shuffles, 6.5
 // without (cold); d = 128, 8 sequences: 7.9 us where one warp searches, 7.1 so.
 // EXT = the call carries a learned sink logit and/or a BF16 band partial; without it that code is compiled out.
-template <int D, int HG, bool EXT, bool RUNS>
-__global__ void __launch_bounds__(HG * D > 512 ? 512 : HG * D, 1)
+// With eight heads per KV head runs do not pay: a block then has 512 threads and 126 registers, one an SM, and two sequences
+// at a time.  One sequence per block in 64 registers (MINB = 2 blocks an SM) beyond one block per SM: whole calls of 100
+// tokens, 37 / 64 / 192 sequences 23.0 / 35.4 / 77.0 us in runs, 19.8 / 33.6 / 72.5 so (with up to four heads and d = 128,
+// 64 / 192: 38.1 / 96.5 and 40.6 / 103).
+template <int D, int HG, bool EXT, bool RUNS, int MINB>
+__global__ void __launch_bounds__(HG * D > 512 ? 512 : HG * D, MINB)
 novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __restrict__ part_acc,
                            const int32_t* __restrict__ page_prefix, const int32_t* __restrict__ seq_lens,
                            int batch, int n_q_heads, int n_kv_heads, int max_pages_per_seq, int grid_s1,
@@ -1726,7 +1730,7 @@ novakv_decode_merge_kernel(const float* __restrict__ part_ml, const float* __res
                            const float* __restrict__ band_acc /* [batch][Hq][D] sum p v of the band, original value domain */,
                            const int32_t* __restrict__ cost_prefix, int seg_weight, const long* __restrict__ cta_range,
                            int seqs_per_block) {
-    constexpr int NP = !RUNS ? 1 : HG <= 4 ? 4 : 2 /* as shared memory allows */, NT = HG * D > 512 ? 512 : HG * D, NW = NT / 32;
+    constexpr int NP = RUNS ? 4 : 1, NT = HG * D > 512 ? 512 : HG * D, NW = NT / 32;
     constexpr int PARTS = NT / D, COLS = D / PARTS, PER = (HG * D + NT - 1) / NT;
     __shared__ float o_s[NP][HG * D];
     __shared__ float red_s[PARTS][HG][D];
@@ -2268,9 +2272,11 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     const bool ext = sink_logits != nullptr || band != nullptr;
     // (one block per SM, so that the slice of the transform stays in registers, and one wave of blocks where at most 8
     // sequences a block make that possible)
-    const int merge_run = max(1, min(8, (batch + max(1, ctx->n_sm / hkv) - 1) / max(1, ctx->n_sm / hkv)));
-    auto merge = merge_run > 1 ? (ext ? novakv_decode_merge_kernel<D, HG, true, true> : novakv_decode_merge_kernel<D, HG, false, true>)
-                               : (ext ? novakv_decode_merge_kernel<D, HG, true, false> : novakv_decode_merge_kernel<D, HG, false, false>);
+    constexpr bool NO_RUNS = HG == 8;
+    const int one_wave = max(1, ctx->n_sm / hkv), merge_run = NO_RUNS ? 1 : max(1, min(8, (batch + one_wave - 1) / one_wave));
+    auto merge = ext ? novakv_decode_merge_kernel<D, HG, true, false, 1> : novakv_decode_merge_kernel<D, HG, false, false, 1>;
+    if (batch > one_wave)
+        merge = ext ? novakv_decode_merge_kernel<D, HG, true, !NO_RUNS, NO_RUNS ? 2 : 1> : novakv_decode_merge_kernel<D, HG, false, !NO_RUNS, NO_RUNS ? 2 : 1>;
     novakv_launch_pdl(merge, dim3((batch + merge_run - 1) / merge_run * hkv), dim3(HG * D > 512 ? 512 : HG * D), 0, stream,
                       part_ml, part_acc, prefix, seq_lens, batch, hq, hkv, max_pages_per_seq, grid, ly.rv_t, ly.v_mean, out,
                       out_is_fp32, sink_logits, qk_off, (const float*)band_ml, (const float*)band_acc,
