@@ -50,12 +50,7 @@ constexpr int PF_HELPERS = 2;
 constexpr int PF_THREADS = (PF_TOKEN_WARPS + 2 + PF_HELPERS) * 32;
 constexpr int PF_TILE = 256;                 // tokens per unit: two half tiles
 constexpr int PF_HALF = 128;
-#ifndef PF_TOK_NS
-#define PF_TOK_NS 0
-#endif
-#ifndef PF_AUX_NS
-#define PF_AUX_NS 200
-#endif
+constexpr int PF_TOK_NS = 0, PF_AUX_NS = 200; // nanoseconds slept between tries of a wait: token warps, the others
 constexpr int PF_OP_BYTES = 8192;            // a group's codebook as search operand
 constexpr int PF_CW_BYTES = 4096;            // and in binary32
 constexpr int PF_CW_STAGES = 6;              // (the binary32 codewords are needed one group longer than the operand)
