@@ -128,7 +128,9 @@ size_t novakv_decode_workspace_bytes(const novakv_ctx* ctx, int batch);
  * sum_i (coef_i - codeword_i)^2 of the binary64 coefficient.  (The kernels rank
  * the 256 distances first - append-sized batches in binary32, larger ones on the tensor cores from coefficients of
  * about 22 bits - and keep that result only where the two smallest distances are further apart than the errors of
- * coefficient and distance can have moved them; every other group is searched again in binary64.  The result
+ * coefficient and distance can have moved them; every other group is searched again in binary64.  The bound of these
+ * errors is derived for the binary32 ranking.  For the tensor cores, whose accumulation order and rounding are not
+ * specified, it is the largest error measured over random and all-positive operands times about four.  The result
  * can differ from a binary64 reference only where the two nearest codewords are within ~1e-12 relative.)
  * The 2L index bytes go to page page_table[tok_seq[t]][tok_pos[t]/64] at slot tok_pos[t]%64, and
  * seq_lens[tok_seq[t]] becomes max(seq_lens[tok_seq[t]], tok_pos[t]+1).
@@ -150,7 +152,13 @@ novakv_status novakv_encode_append(novakv_ctx* ctx, int layer,
  *     z_hj = sm_scale * sum_l < q'_h[4l..4l+3], cb_k[l][kidx_j[l]] >     (k_mean dropped: Lemma S1)
  *     p_h  = softmax_j(z_hj)  over positions 0 .. seq_lens[b]-1
  *     o_h  = ( sum_j p_hj concat_l cb_v[l][vidx_j[l]] ) rv^T + v_mean    (Remark after Corollary 1)
- * computed split over the sequence with an exact log-sum-exp merge, binary32 accumulation.
+ * computed split over the sequence with an exact log-sum-exp merge, binary32 accumulation.  The softmax weights
+ * that meet the value codewords are binary16 numbers (the normaliser sums the same rounded numbers).  At d = 64 with
+ * Hq/Hkv = 8 calls of more than a few pages per SM form the logits from binary16 pairs of query and codeword (about 22 bits)
+ * on tensor cores, others from a binary32 table; against binary64 neither output is further off than the other by more than
+ * the weights' rounding.
+ * q is read as soon as the kernel before this call in `stream` lets its dependents start: it must not be the output of the
+ * library call directly before this one.
  *   q    bf16 [batch][Hq][d]
  *   out  [batch][Hq][d], float32 if out_is_fp32 else bf16; a sequence of length 0 yields zeros
  *   workspace  at least novakv_decode_workspace_bytes(ctx, batch) bytes; contents are scratch

@@ -108,6 +108,36 @@ def test_append_rows_off_a_word_boundary_are_refused(cases, n):
         _run(cases["qwen", False], "plain", n, 0, False, False, offset=1)
 
 
+@pytest.mark.parametrize("kind", ["positive", "cancelling", "wide"])
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "plain"), ("qwen", "scaled"), ("gptoss", "scaled")])
+def test_prefill_bounds_hold_on_hard_inputs(cases, name, fmt, kind):
+    """The bounds of the tensor core's errors are measured, not derived: inputs that strain them - all positive (every
+    truncation in one direction), pairs of opposite sign (small coefficients of large rows), elements over three decades -
+    must leave no index that the append kernel, whose bound is derived, decides differently."""
+    from paper_2608_04074_b200.runtime import PagedCache
+    case, n = cases[name, fmt != "plain"], 16384
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    shape = (n, case.ctx.n_kv_heads, case.ctx.head_dim)
+    x = torch.randn((2, *shape), generator=gen, device="cuda")
+    if kind == "positive":
+        x = x.abs()
+    elif kind == "cancelling":
+        x = torch.stack([x[..., ::2] * 4, -x[..., ::2] * 4 + x[..., 1::2] * 0.25], dim=-1).flatten(-2)
+    else:
+        x = x * 10.0 ** (torch.rand(x.shape, generator=gen, device="cuda") * 3 - 2)
+    k, v = x.to(torch.bfloat16)
+    seq, pos = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.arange(n, dtype=torch.int32, device="cuda")
+    stored = []
+    for step in (n, 256):
+        cache = PagedCache(case.ctx, np.array([0], np.int32), capacity_tokens=np.array([n], np.int32), seed=7, key_scale=fmt == "scaled")
+        for i in range(0, n, step):
+            cache.append(0, k[i:i + step], v[i:i + step], seq[i:i + step], pos[i:i + step])
+        assert case.ctx.novakv_last_device_status() == 0
+        stored.append([y for y in (cache.k_pages, cache.v_pages, cache.k_scales) if y is not None])
+    for prompt, small in zip(*stored):
+        assert torch.equal(prompt, small), int((prompt != small).sum())
+
+
 @pytest.mark.parametrize("first,n", [(0, 600), (299, 300), (640, 700), (1279, 2048), (2047, 2048), (3000, 3000)])
 @pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "scaled"), ("qwen", "deployed")])
 def test_prefill_leading_entries_unused(cases, name, fmt, first, n):
