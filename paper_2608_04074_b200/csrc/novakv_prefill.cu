@@ -23,8 +23,9 @@
 // of this one.  Every wait is bounded (novakv_tcgen05.cuh): a wait that gives up sets NOVAKV_DEV_WAIT_TIMEOUT, and the CTA
 // runs through the rest of its segment without waiting and leaves.  Three things hold on that way: the token warps take
 // no destination that the flag has overtaken (tokens without one are neither stored nor looked at again), the named
-// barriers among token warps are never skipped and never run ahead (hold() below), and the tensor core and the copies are
-// given time to finish before the CTA's memory goes away.
+// barriers among token warps and the waits for the search MMAs between them are never skipped (each of these MMAs is issued
+// whatever has happened, so that they end; skipping one would let a warp overtake its warpgroup's barrier), and the
+// tensor core and the copies are given time to finish before the CTA's memory goes away.
 //
 // What bounds it: instruction issue and latency of the selection, about 600 warp instructions per 32 tokens and group (of
 // which 64 + 16 packed minima and comparisons on the half-rate pipe) with four token warps per scheduler; tensor pipe
@@ -92,7 +93,7 @@ struct PF {
     static constexpr uint32_t OFF_TSLOT = OFF_PAGE + NX * PF_HALF * 4;            // uint8 [NX][128], its slot in the page
     static constexpr uint32_t OFF_CONST = OFF_TSLOT + NX * PF_HALF;
     static constexpr uint32_t OFF_BAR = OFF_CONST + ((NCONST * 4 + 15) & ~15);
-    // ints: TMEM base, abort flag, finished token warps, -, queue counters [4], wait limit [2], releases [4], -, -; unsure tokens [16]
+    // ints: TMEM base, abort flag, finished token warps, -, queue counters [4], wait limit [2], -; unsure tokens [16]
     static constexpr uint32_t OFF_MISC = OFF_BAR + 288;
     static constexpr uint32_t BYTES = OFF_MISC + 128;
     static_assert(BYTES <= 232448, "shared memory budget");
@@ -348,7 +349,6 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
     int* const s_done = reinterpret_cast<int*>(smem + P::OFF_MISC) + 2;               // token warps that have finished the segment
     int* const s_count = reinterpret_cast<int*>(smem + P::OFF_MISC) + 4;              // [helper] entries in the queue
     int* const s_head = reinterpret_cast<int*>(smem + P::OFF_MISC) + 4 + PF_HELPERS;  // [helper] entries ever queued
-    volatile uint32_t* const s_rel = reinterpret_cast<volatile uint32_t*>(smem + P::OFF_MISC) + 10;   // [wg] releases its first warp has passed
     static_assert(4 + 2 * PF_HELPERS == 1 + MBAR_LIMIT, "the wait limit follows the queue counters");
     float* const cst = reinterpret_cast<float*>(smem + P::OFF_CONST);
     auto bar = [&](int i) -> uint32_t { return sb + P::OFF_BAR + i * 8; };
@@ -376,8 +376,6 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
         misc[1] = 0;
         *reinterpret_cast<volatile long long*>(abort_flag + MBAR_LIMIT) = a.wait_clocks;
 #pragma unroll
-        for (int g = 0; g < 4; ++g) s_rel[g] = 0;
-#pragma unroll
         for (int h = 0; h < PF_HELPERS; ++h) { s_count[h] = 0; s_head[h] = 0; }
         mbar_init(bar(B_R), 1);
 #pragma unroll
@@ -390,7 +388,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
         for (int s = 0; s < P::NOP; ++s) { mbar_init(bar(B_RING + s), 1); mbar_init(bar(B_RINGFREE + s), 2); }
 #pragma unroll
         for (int s = 0; s < PF_CW_STAGES; ++s) { mbar_init(bar(B_CW + s), 1); mbar_init(bar(B_CWFREE + s), 8); }
-        mbar_init(bar(B_DRAIN), 5);
+        mbar_init(bar(B_DRAIN), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
@@ -849,7 +847,6 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                         nbar_sync(1 + wg, PF_HALF);
                         tc_fence_after();
                         if (elect_one()) {
-                            s_rel[wg] = n_s + 1;
                             umma_f16(d_s, umma_desc(a_s, PF_HALF * 16, 128, 0),
                                      umma_desc(sb + P::OFF_RING + st * PF_OP_BYTES + c * 2048, 4096, 128, 0), umma_idesc(false, false, 128, 128), false);
                             umma_commit(bar(B_S + wg));
@@ -873,28 +870,16 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                     tmem_ld64_h2(d_s + lane_base + half * 64, v);
                     tmem_wait_ld();
                 };
-                // The other three warps arrive at the barrier of a release without waiting there; what keeps them from arriving
-                // at the next one before the first warp has come to this one is the wait for its MMA.  Where that wait was
-                // given up, they wait for the first warp itself.  (It comes: everything it meets on its way is either
-                // bounded or a barrier at which these warps have arrived.)
-                bool gone = *abort_flag != 0;
-                auto wait_chunk = [&]() {
-                    const bool ok = mbar_wait<PF_TOK_NS>(bar(B_S + wg), n_s & 1, abort_flag);
-                    if (__any_sync(0xffffffffu, !ok || gone)) {
-                        gone = true;
-                        for (int tries = 0; (int)(s_rel[wg] - n_s) <= 0 && tries < 10000000; ++tries) __nanosleep(100);
-                        __syncwarp();
-                    }
-                    ++n_s;
-                    tc_fence_after();
-                };
                 float q2 = publish(0);                                         // |r|^2 of this group, in its scale
                 release_and_issue(0, 0);
                 uint32_t codes = 0, pend = 0;
 #pragma unroll 1
                 for (int g = 0; g < ngh; ++g) {
                     {
-                        wait_chunk();
+                        mbar_wait_mma(bar(B_S + wg), n_s & 1, abort_flag);
+                        ++n_s;
+                        tc_fence_after();
+                        __syncwarp();
                         uint32_t v[32];
                         accumulators(0, v);
                         minima(0, v);
@@ -904,7 +889,10 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                     }
                     {
                         float q2n = 0.f;
-                        wait_chunk();
+                        mbar_wait_mma(bar(B_S + wg), n_s & 1, abort_flag);
+                        ++n_s;
+                        tc_fence_after();
+                        __syncwarp();
                         uint32_t v[32];
                         accumulators(0, v);
                         minima(2, v);
@@ -1064,8 +1052,8 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
         if (*abort_flag) break;                        // (the same in every warp: nobody waits before the next barrier)
     }
     if (*abort_flag) {
-        // the MMAs of the five issuing warps have to end before TMEM is handed back
-        if (warp == PF_TOKEN_WARPS || (warp < PF_TOKEN_WARPS && (warp & 3) == 0)) {
+        // transforms may be under way: they have to end before TMEM is handed back
+        if (warp == PF_TOKEN_WARPS) {
             if (elect_one()) umma_commit(bar(B_DRAIN));
             __syncwarp();
         }

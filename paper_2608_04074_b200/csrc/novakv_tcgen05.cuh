@@ -35,6 +35,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try(bar, parity)) return true;
     return mbar_wait_slow<NS>(bar, parity, abort_flag);
 }
+// Wait for an MMA that has been or will be issued by this CTA whatever happens: the flag does not end it.  (After a second
+// it raises the flag, after ten the MMA is given up for lost.)
+__device__ __noinline__ void mbar_wait_mma_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i)
+            if (mbar_try(bar, parity)) return;
+        const long long t = clock64() - t0;
+        if (t > 2000000000ll) *abort_flag = 1;
+        if (t > 20000000000ll) return;
+    }
+}
+__device__ __forceinline__ void mbar_wait_mma(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    if (!mbar_try(bar, parity)) mbar_wait_mma_slow(bar, parity, abort_flag);
+}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
