@@ -88,7 +88,7 @@ struct S1 {
     static constexpr int K32 = D == 128 ? 8 : L;
     static constexpr bool HAS16 = K32 < L;
     static_assert(!HAS16 || HSETS == 1, "binary16 entries hold one head set");
-    static constexpr int ROW32 = K32 * 16;
+    static constexpr int ROW32 = 256;
     static constexpr int PLANE32 = 256 * ROW32;
     static constexpr int T32_BYTES = HSETS * PLANE32;
     static constexpr int TILE_BYTES = 32 * L;                 // index bytes of a 32-token tile, K or V
@@ -96,22 +96,22 @@ struct S1 {
     //   VM: fp16 [HPAD][4 k-slot pairs][8 tokens]        otherwise: fp32 [32 tokens][HPAD]
     static constexpr int P_WARP_BYTES = VM ? HPAD * 64 : 32 * HPAD * 4;
     static constexpr int P_BYTES = NCW * P_WARP_BYTES;
-    // Shared-memory map.  Below the binary16 table: T32, the weight staging, q' of the pair.  The binary16 table
-    // sits at the first 64 KB boundary of the shared address window that leaves that much room (a row then
-    // starts at an address whose low 16 bits are code * 256, so that one byte permutation builds a gather
-    // address); without a binary16 table nothing needs aligning.  The two copies of the value codebook follow.
-    static constexpr int OFFB_T32 = 0;
-    static constexpr int OFFB_P = OFFB_T32 + T32_BYTES;
-    static constexpr int OFFB_Q = OFFB_P + P_BYTES;                     // fp32 [HPAD][D]
-    static constexpr int OFFB_BND = OFFB_Q + HPAD * D * 4;              // long [MAX_SCAN_CTAS + 1]: first unit of every CTA
-    static constexpr int OFFB_PFX = OFFB_BND + (MAX_SCAN_CTAS + 1) * 8; // int [2][PFX_CAP + 1]: page and cost prefix of small batches
-    static constexpr int BELOW_BYTES = OFFB_PFX + 2 * (PFX_CAP + 1) * 4;
+    // Shared-window addresses, fixed so that they are immediates of the gathers.  Rows of 256 bytes: one byte permutation
+    // puts a code above a column byte.  (The window's first KB and the static words lie below; checked at run time.)
+    static constexpr int T16 = 4096;
+    static constexpr int T32 = T16 + (HAS16 ? T16_BYTES : 0);
+    static constexpr int VCB = T32 + T32_BYTES;                         // two copies of the value codebook
+    static constexpr int P = VCB + 2 * VCB_COPY_BYTES;
+    static constexpr int Q = P + P_BYTES;                               // fp32 [HPAD][D]
+    static constexpr int BND = Q + HPAD * D * 4;                        // long [MAX_SCAN_CTAS + 1]: first unit of every CTA
+    static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;           // int [2][PFX_CAP + 1]: page and cost prefix of small batches
+    static constexpr int SMEM = PFX + 2 * (PFX_CAP + 1) * 4;
     // merge buffer (aliases the larger table once a segment's scan is done)
     static constexpr int MROW = D + 4;                                  // floats per (warp, head) row of the merge buffer: 16 bytes of padding
                                                                         // keep the four head rows a warp writes at once on different banks
     static constexpr int MERGE_ACC_BYTES = NCW * HPAD * MROW * 4;
     static_assert(MERGE_ACC_BYTES + NCW * HPAD * 16 <= (HAS16 ? T16_BYTES : T32_BYTES), "merge buffer must fit in a table");
-    static_assert(BELOW_BYTES + (HAS16 ? T16_BYTES : 0) + 2 * VCB_COPY_BYTES <= S1_SMEM_BYTES, "shared memory budget (before alignment)");
+    static_assert(SMEM <= S1_SMEM_BYTES, "shared memory budget");
     static_assert(S1_THREADS % L == 0, "table build mapping");
 };
 
@@ -279,11 +279,6 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
 // ------------------------------------------------------------------------------------------------
 // stage 1 helpers
 // ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint2 lds_u64(uint32_t addr) {
-    uint2 v;
-    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
-    return v;
-}
 __device__ __forceinline__ uint4 lds_u128(uint32_t addr) {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
@@ -304,14 +299,15 @@ __device__ __forceinline__ uint4 lds_u128_at(uint32_t addr) {
     return v;
 }
 template <int OFF>
+__device__ __forceinline__ uint2 lds_u64_at(uint32_t addr) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2+%3];" : "=r"(v.x), "=r"(v.y) : "r"(addr), "n"(OFF));
+    return v;
+}
+template <int OFF>
 __device__ __forceinline__ uint32_t lds_u32_at(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(OFF));
-    return v;
-}
-__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
 }
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
@@ -426,6 +422,11 @@ __device__ __forceinline__ uint32_t ldg_stream_32(const void* p) {
     asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
+__device__ __forceinline__ uint32_t ldg_stream_16(const void* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.u16 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ uint2 ldg_stream_64(const void* p) {
     uint2 v;
     asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
@@ -436,20 +437,14 @@ __device__ __forceinline__ uint2 ldg_stream_64(const void* p) {
 // shared memory, copy c holding group g in slot (g + 16 c) % 32, without registers: asynchronous 16-byte
 // copies that land while the caller does other work (segment lookup, page ids, table build);
 // async_copies_wait() before the barrier that publishes the copies.  A 16-byte chunk holds 4 slots, so the
-// rotation by 16 slots moves whole chunks.  INTERLEAVED: the two copies share 256-byte rows
-// [code][copy][32 slots] (a row then starts at code * 256 of a 64 KB block); otherwise copy 1 follows copy 0.
-template <bool INTERLEAVED>
-__device__ __forceinline__ void stage_value_codebook_async(unsigned char* vcb, const uint8_t* __restrict__ src_g) {
-    const uint32_t d0 = smem_u32(vcb);
+// rotation by 16 slots moves whole chunks.
+__device__ __forceinline__ void stage_value_codebook_async(uint32_t d0, const uint8_t* __restrict__ src_g) {
     for (int i = threadIdx.x; i < VCB_COPY_BYTES / 16; i += S1_THREADS) {
         const int row = i >> 3, ch = i & 7;
         const uint8_t* src = src_g + (size_t)i * 16;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const uint32_t dst = d0 + (INTERLEAVED ? row * (2 * VCB_ROW) + c * VCB_ROW : c * VCB_COPY_BYTES + row * VCB_ROW) +
-                                 ((ch + 4 * c) & 7) * 16;
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-        }
+        for (int c = 0; c < 2; ++c)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d0 + c * VCB_COPY_BYTES + row * VCB_ROW + ((ch + 4 * c) & 7) * 16), "l"(src) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -558,7 +553,7 @@ template <int L>
 struct TileRegs {
     uint32_t kw[L / 4];
     uint32_t vw[2][L / 8];
-    uint32_t ks;          // this lane's token: bfloat16 key scale in the high half (a binary32 bit pattern), if used
+    uint32_t ks;          // this lane's token: bfloat16 key scale in the low half, if used
     uint32_t vm;          // this lane's token: bfloat16 value scale (low half) and zero-point (high half), if used
 };
 
@@ -688,11 +683,8 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ int s_found[4];
     __shared__ int s_arrived, s_first, s_last;
-    // ---- shared-memory map (see S1)
     const uint32_t s_base = smem_u32(smem);
-    const uint32_t t16_abs = HAS16 ? ((s_base + C::BELOW_BYTES + 65535u) & ~65535u) : s_base + C::BELOW_BYTES;
-    const uint32_t pad = t16_abs - s_base;
-    if (pad + (HAS16 ? T16_BYTES : 0) + 2 * VCB_COPY_BYTES > (uint32_t)S1_SMEM_BYTES || (s_base & 255u) != 0u) {
+    if (s_base > C::T16 || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
         // cannot happen with the shared address window of this architecture; reported, never trapped
         if (threadIdx.x == 0) {
             atomicOr(dev_status, NOVAKV_DEV_SMEM_LAYOUT);
@@ -700,18 +692,16 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         }
         return;
     }
-    unsigned char* const t32_p = smem + C::OFFB_T32;
-    unsigned char* const t16_p = smem + pad;
-    unsigned char* const vcb_p = t16_p + (HAS16 ? T16_BYTES : 0);
-    const uint32_t vcb_abs = t16_abs + (HAS16 ? T16_BYTES : 0);
-    float* const q_s = reinterpret_cast<float*>(smem + C::OFFB_Q);
-    const uint32_t s_p = s_base + C::OFFB_P;
+    unsigned char* const s_abs = smem - s_base;               // s_abs + a: the byte at shared-window address a
+    unsigned char* const t32_p = s_abs + C::T32;
+    unsigned char* const t16_p = s_abs + C::T16;
+    float* const q_s = reinterpret_cast<float*>(s_abs + C::Q);
 
     // With the KV-head-major walk the first KV head of CTA c is floor(c * Hkv / G) whatever the lengths are:
     // its (constant) value codebook starts flowing into shared memory before the grid-dependency wait and
     // lands behind the segment lookup and the first table build.
     int vcb_head = (int)(((long)blockIdx.x * n_kv_heads) / gridDim.x);   // KV head whose value codebook is resident
-    stage_value_codebook_async<HAS16>(vcb_p, cb_v_img + (size_t)vcb_head * vcb_per_head);
+    stage_value_codebook_async(C::VCB, cb_v_img + (size_t)vcb_head * vcb_per_head);
     // With the merge fused in, the kernels that follow (the query transform of the next call writes the same
     // workspace) must not start before this grid is done: no early release of the dependents.
     if (out_fused != nullptr) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -720,14 +710,14 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // The two prefixes are read many times (boundaries, segment look-ups): small batches keep them in shared memory.
     if (batch <= PFX_CAP) {
-        int32_t* pfx = reinterpret_cast<int32_t*>(smem + C::OFFB_PFX);
+        int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
         for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix[i]; pfx[PFX_CAP + 1 + i] = cost_prefix[i]; }
         __syncthreads();
         page_prefix = pfx;
         cost_prefix = pfx + PFX_CAP + 1;
     }
     // First unit of every CTA (see scan_boundary): one thread per boundary.  This CTA owns [s_bnd[c], s_bnd[c + 1]).
-    long* const s_bnd = reinterpret_cast<long*>(smem + C::OFFB_BND);
+    long* const s_bnd = reinterpret_cast<long*>(s_abs + C::BND);
     for (int c = threadIdx.x; c <= (int)gridDim.x; c += S1_THREADS)
         s_bnd[c] = scan_boundary(c, gridDim.x, page_prefix, cost_prefix, batch, n_kv_heads, seg_weight);
     __syncthreads();
@@ -737,35 +727,34 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 
     // ---- lane roles and constants
     const int fr = lane >> 2, fc = lane & 3;          // value side: MMA fragment coordinates
-    // key side: token = lane; its byte j holds group j ^ (lane & 7) (j < 16) or j ^ (lane & 15) (j >= 16).
-    //   binary32 entries (steps j < K32): address = T32 + code * ROW32 + ((j ^ lane%8) * 16): the column part is
-    //     one xor with a constant away from a per-lane word, the row part one multiply-add;
-    //   binary16 entries: address = T16 + code * 256 + ((j ^ mask) * 8) = a byte permutation of (index word,
-    //     column word): the column word holds the column bytes of an even / odd step in bytes 0 / 1 and the
-    //     table's upper address half in bytes 2, 3; stepping to another pair of j is one xor with a constant.
-    const uint32_t col32 = s_base + C::OFFB_T32 + (lane & 7) * 16;
-    const uint32_t colword15 = t16_abs | (uint32_t)((lane & 15) * 8) * 0x0101u;
+    // key side: token = lane; its byte j holds group j ^ (lane & 7) (j < 16) or j ^ (lane & 15) (j >= 16).  The column of
+    // step j is one byte below 128 (columns from 128 on come as an immediate), four steps to a word; a byte permutation of
+    // (index word, column word) makes a gather address: column, code, and twice the column's replicated top bit, a zero.
+    uint32_t col32[2], col16[HAS16 ? 4 : 1];
+#pragma unroll
+    for (int w = 0; w < 2; ++w) col32[w] = (0x30201000u ^ ((uint32_t)(lane & 7) * 0x10101010u)) ^ (w * 0x40404040u);
+#pragma unroll
+    for (int w = 0; w < (HAS16 ? 4 : 1); ++w) col16[w] = (0x18100800u ^ ((uint32_t)(lane & 15) * 0x08080808u)) ^ (w * 0x20202020u);
+#pragma unroll
+    for (int w = 0; w < 2; ++w) asm volatile("" : "+r"(col32[w]));               // (kept in registers: formed again in every tile otherwise)
+#pragma unroll
+    for (int w = 0; w < (HAS16 ? 4 : 1); ++w) asm volatile("" : "+r"(col16[w]));
     // value side: lane column fc reads copy fc / 2 of the value codebook; odd columns take the group blocks in
-    // swapped order (x ^ 1), so that the 32 lanes of a gather hit 32 different slots.  With the binary16 table
-    // (d = 128) the codebook block is 64 KB aligned too and its two copies share 256-byte rows, so that a gather
-    // address is one byte permutation of (code word, pos); otherwise address = pos + code * 128.
+    // swapped order (x ^ 1), so that the 32 lanes of a gather hit 32 different slots.  Address = pos + code * 128, a byte
+    // dot product: the permutations above and those that widen a codeword fill the integer pipe (55 % busy), dot products run
+    // on the one of the multiply-adds.  With the columns above 55 -> 45 %; 64 sequences of 65536 tokens 655 -> 639 us a call.
     uint32_t pos[NGB];
 #pragma unroll
-    for (int x = 0; x < NGB; ++x) {
-        const uint32_t slot4 = ((8 * (x ^ (fc & 1)) + fr + 16 * (fc >> 1)) & 31) * 4;
-        pos[x] = HAS16 ? (vcb_abs | ((fc >> 1) * VCB_ROW + slot4)) : vcb_abs + (fc >> 1) * VCB_COPY_BYTES + slot4;
-    }
-    // address of the codeword whose code is byte b of word w, for load x
-    auto vaddr = [&](uint32_t w, int b, int x) -> uint32_t {
-        return HAS16 ? __byte_perm(w, pos[x], 0x7604u | (b << 4)) : pos[x] + __byte_perm(w, 0u, 0x4440u | b) * VCB_ROW;
-    };
+    for (int x = 0; x < NGB; ++x) pos[x] = (fc >> 1) * VCB_COPY_BYTES + ((8 * (x ^ (fc & 1)) + fr + 16 * (fc >> 1)) & 31) * 4;
+    // codeword whose code is byte b of word w, for load x
+    auto vgather = [&](uint32_t w, int b, int x) -> uint32_t { return lds_u32_at<C::VCB>(__dp4a(w, (uint32_t)VCB_ROW << (8 * b), pos[x])); };
     const bool odd_col = fc & 1;
     // widening selectors: byte pairs (u, replicated top bit of u = 0) of the low / high half of a codeword, taken
     // from the first operand in even columns and from the second in odd columns
     const uint32_t sel_lo = odd_col ? 0xD5C4u : 0x9180u, sel_hi = odd_col ? 0xF7E6u : 0xB3A2u;
     // B fragments carry a weight in the low or high half depending on the column parity (fr & 1)
     const uint32_t sel_b0 = (fr & 1) ? 0x1044u : 0x4410u, sel_b1 = (fr & 1) ? 0x3244u : 0x4432u;
-    const uint32_t s_pw = s_p + warp * C::P_WARP_BYTES;
+    const uint32_t s_pw = C::P + warp * C::P_WARP_BYTES;
 
     // ---- per-warp running state
     float m_run[HPAD];                           // running maximum of the logits (base 2), the same in every lane
@@ -835,7 +824,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 
         // ---- segment prologue -----------------------------------------------------------------
         if (vcb_head != sg.kvh) {
-            stage_value_codebook_async<HAS16>(vcb_p, cb_v_img + (size_t)sg.kvh * vcb_per_head);
+            stage_value_codebook_async(C::VCB, cb_v_img + (size_t)sg.kvh * vcb_per_head);
             vcb_head = sg.kvh;
         }
         // q' of the pair's heads -> shared memory (rows beyond HG are zero)
@@ -852,7 +841,8 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         }
 
         // this warp's tiles of the segment: half pages hp = warp, warp + NCW, ...
-        const int n_it = (2 * sg.npg > warp) ? (2 * sg.npg - warp + NCW - 1) / NCW : 0;
+        const int n_half = min(2 * sg.npg, (sg.len - sg.pg0 * NOVAKV_PAGE_TOKENS + 31) / 32);
+        const int n_it = n_half > warp ? (n_half - warp + NCW - 1) / NCW : 0;
         const int32_t* pt = page_table + (size_t)sg.b * pt_stride + sg.pg0;
         // page ids of 32 consecutive tiles of this warp, one per lane (coalesced gather, loaded a batch ahead)
         auto load_ids = [&](int batch_i) {
@@ -865,22 +855,23 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
             return page;
         };
         int ids_cur = load_ids(0), ids_next = load_ids(1);
+        // a warp's tiles are all first or all second halves of their pages (an even number of warps)
+        static_assert(NCW % 2 == 0, "half of a page is a constant of the warp");
+        const uint32_t k_step = (uint32_t)n_kv_heads * PAGE_BYTES;                       // bytes of a page
+        const uint8_t* const kb = k_pages + (size_t)sg.kvh * PAGE_BYTES + (warp & 1) * TILE_BYTES + lane * 16;
+        const uint8_t* const vb = v_pages + (size_t)sg.kvh * PAGE_BYTES + (warp & 1) * TILE_BYTES + lane * (NGB * 4);
+        const size_t m0 = (size_t)sg.kvh * NOVAKV_PAGE_TOKENS + (warp & 1) * 32 + lane;  // this lane's token in the pools of scales
         // tiles are loaded in ascending order, one ahead of the tile being consumed
         auto load_tile = [&](int it, TileRegs<L>& t) {
             if ((it & 31) == 0 && it > 0) { ids_cur = ids_next; ids_next = load_ids((it >> 5) + 1); }
             const int page = __shfl_sync(0xffffffffu, ids_cur, it & 31);
-            const int half = (warp + NCW * it) & 1;
-            const size_t off = ((size_t)page * n_kv_heads + sg.kvh) * PAGE_BYTES + half * TILE_BYTES;
-            if (KSC) {
-                const unsigned short raw = __ldg(reinterpret_cast<const unsigned short*>(k_scales) +
-                                                 ((size_t)page * n_kv_heads + sg.kvh) * NOVAKV_PAGE_TOKENS + half * 32 + lane);
-                t.ks = (uint32_t)raw << 16;
-            }
-            if (VSQ)
-                t.vm = __ldg(reinterpret_cast<const uint32_t*>(v_meta) +
-                             ((size_t)page * n_kv_heads + sg.kvh) * NOVAKV_PAGE_TOKENS + half * 32 + lane);
-            const uint8_t* kp = k_pages + off + lane * 16;
-            const uint8_t* vp = v_pages + off + lane * (NGB * 4);
+            const uint8_t* const kp = kb + (size_t)(uint32_t)page * k_step;
+            const uint8_t* const vp = vb + (size_t)(uint32_t)page * k_step;
+            const size_t mi = m0 + (size_t)(uint32_t)page * (uint32_t)(n_kv_heads * NOVAKV_PAGE_TOKENS);
+            // (kept as loaded: a shift here waits for the load, a tile ahead of its use; 64 scaled sequences of 32768 tokens
+            // 431 -> 368 us a call without it)
+            if (KSC) t.ks = ldg_stream_16(reinterpret_cast<const unsigned short*>(k_scales) + mi);
+            if (VSQ) t.vm = ldg_stream_32(reinterpret_cast<const uint32_t*>(v_meta) + mi);
 #pragma unroll
             for (int p = 0; p < KPL; ++p) {
                 const uint4 w = ldg_stream_128(kp + p * 512);
@@ -899,11 +890,9 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         };
 
         // ---- one 32-token tile -------------------------------------------------------------------
+        const int left = sg.len - sg.pg0 * NOVAKV_PAGE_TOKENS - warp * 32;     // tokens from this warp's first tile on
         auto process = [&](const TileRegs<L>& cur, int it) {
-            const int hp = warp + NCW * it;
-            const int tok0 = (sg.pg0 + (hp >> 1)) * NOVAKV_PAGE_TOKENS + (hp & 1) * 32;
-            const int nvalid = min(32, sg.len - tok0);
-            if (nvalid <= 0) return;
+            const int nvalid = left - it * (NCW * 32);
 
             // ---- key side: lane <-> token; step j gathers the entry of (code_j, group j ^ lane bits) ------
             float zf[HPAD];
@@ -913,11 +902,11 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
                 for (int k = 0; k < HPAD / 2; ++k) z2[k] = 0ull;
 #pragma unroll
                 for (int j = 0; j < K32; ++j) {
-                    const uint32_t code = __byte_perm(cur.kw[j >> 2], 0u, 0x4440u | (j & 3));
-                    const uint32_t a = (col32 ^ (uint32_t)(j * 16)) + code * C::ROW32;
+                    const uint32_t a = prmt_rep(cur.kw[j >> 2], col32[(j >> 2) & 1], 0xcc04u + (j & 3) * 0x1111u);
 #pragma unroll
                     for (int hs = 0; hs < HSETS; ++hs) {
-                        const uint4 v = lds_u128(a + hs * C::PLANE32);
+                        const uint4 v = j < 8 ? (hs ? lds_u128_at<C::T32 + C::PLANE32>(a) : lds_u128_at<C::T32>(a))
+                                              : (hs ? lds_u128_at<C::T32 + C::PLANE32 + 128>(a) : lds_u128_at<C::T32 + 128>(a));
                         fadd2(z2[2 * hs], (uint64_t)v.x | ((uint64_t)v.y << 32));
                         fadd2(z2[2 * hs + 1], (uint64_t)v.z | ((uint64_t)v.w << 32));
                     }
@@ -932,8 +921,8 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
                 uint32_t ch[2];
 #pragma unroll
                 for (int j = K32; j < L; ++j) {
-                    const uint32_t cw2 = colword15 ^ (uint32_t)(((j & ~1) * 8) | (((j | 1) * 8) << 8));
-                    const uint2 v = lds_u64(__byte_perm(cur.kw[j >> 2], cw2, 0x7600u | ((j & 3) << 4) | (4 + (j & 1))));
+                    const uint32_t a = prmt_rep(cur.kw[j >> 2], col16[HAS16 ? (j >> 2) & 3 : 0], 0xcc04u + (j & 3) * 0x1111u);
+                    const uint2 v = j < 16 ? lds_u64_at<C::T16>(a) : lds_u64_at<C::T16 + 128>(a);
                     if ((j - K32) % CHAIN == 0) { ch[0] = v.x; ch[1] = v.y; }
                     else { ch[0] = hadd2(ch[0], v.x); ch[1] = hadd2(ch[1], v.y); }
                     if ((j - K32) % CHAIN == CHAIN - 1 || j == L - 1) {
@@ -944,7 +933,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
             }
             float vscale = 1.f, vzero = 0.f, vsmax = 0.f;     // vsmax: this lane's scale as it enters the running bound (0 beyond the length)
             if (KSC) {
-                const float rho = __uint_as_float(cur.ks);
+                const float rho = __uint_as_float(cur.ks << 16);
 #pragma unroll
                 for (int h = 0; h < HPAD; ++h) zf[h] = (zf[h] + qcen[h]) * rho;
             }
@@ -1083,8 +1072,8 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 #pragma unroll
                         for (int x = 0; x < NGB; ++x) {
                             const uint32_t vwd = cur.vw[blk][x];      // codes of the group block this load fetches (x ^ 1 in odd columns)
-                            X[x][0] = lds_u32(vaddr(vwd, 2 * ts, x));
-                            X[x][1] = lds_u32(vaddr(vwd, 2 * ts + 1, x));
+                            X[x][0] = vgather(vwd, 2 * ts, x);
+                            X[x][1] = vgather(vwd, 2 * ts + 1, x);
                         }
 #pragma unroll
                         for (int gb = 0; gb < NGB; ++gb) {
@@ -1118,7 +1107,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 #pragma unroll
                         for (int x = 0; x < NGB; ++x) {
                             // (odd lane columns fetch group block x ^ 1 with load x; their accumulator x holds that block)
-                            const uint32_t cwd = lds_u32(vaddr(cur.vw[blk][x], tq, x));
+                            const uint32_t cwd = vgather(cur.vw[blk][x], tq, x);
                             // grid indices -> binary32, centred: bytes (u, 0) are the binary16 subnormals u 2^-24
                             const __half2 c64 = __halves2half2(__ushort_as_half((unsigned short)64), __ushort_as_half((unsigned short)64));
                             const uint32_t h01 = __byte_perm(cwd, 0u, 0x4140u), h23 = __byte_perm(cwd, 0u, 0x4342u);
