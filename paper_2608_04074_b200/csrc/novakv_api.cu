@@ -60,24 +60,6 @@ extern "C" novakv_status novakv_create(novakv_ctx** out, const novakv_config* cf
         delete ctx;
         return NOVAKV_ECUDA;
     }
-    {
-        // product codebook of the scalar INT2 value codec: byte c decodes to the levels (c & 3, (c >> 2) & 3,
-        // (c >> 4) & 3, c >> 6), the same for every group and head, in the layout the value gather reads
-        // (uint8 [256 codes][32 slots][4])
-        const size_t n = (size_t)NOVAKV_C * 32 * NOVAKV_G;
-        std::vector<uint8_t> img(n);
-        for (size_t i = 0; i < n; ++i) {
-            const int comp = (int)(i % NOVAKV_G), code = (int)(i / (32 * NOVAKV_G));
-            img[i] = (uint8_t)((code >> (2 * comp)) & 3);
-        }
-        if (cudaMalloc(&ctx->int2_img, n) != cudaSuccess ||
-            cudaMemcpy(ctx->int2_img, img.data(), n, cudaMemcpyHostToDevice) != cudaSuccess) {
-            cudaFree(ctx->dev_status);
-            cudaFree(ctx->int2_img);
-            delete ctx;
-            return NOVAKV_ECUDA;
-        }
-    }
     *out = ctx;
     return NOVAKV_OK;
 }
@@ -100,7 +82,6 @@ extern "C" novakv_status novakv_destroy(novakv_ctx* ctx) {
         for (auto& e : ctx->prof[k]) { cudaEventDestroy(e.start); cudaEventDestroy(e.stop); }
     for (auto& e : ctx->prof_free) { cudaEventDestroy(e.start); cudaEventDestroy(e.stop); }
     cudaFree(ctx->dev_status);
-    cudaFree(ctx->int2_img);
     delete ctx;
     return NOVAKV_OK;
 }

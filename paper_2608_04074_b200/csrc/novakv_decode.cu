@@ -636,10 +636,14 @@ __device__ __noinline__ void fused_merge(float* scratch, const float* part_ml, c
 // KSC: the key format carries a per-token bfloat16 scale (k_scales [n_pages][Hkv][64]); the logits of a
 // token are multiplied by it once, after the table lookups are summed (and the centre's share added back).
 // VSQ: scalar INT2 values with a per-token bfloat16 scale and zero-point (v_meta [n_pages][Hkv][64][2]).
-// A byte of four 2-bit codes indexes the product codebook {0,1,2,3}^4, so the value side is the same gather
-// with that fixed table as the value-codebook image; the weight of a token's codes is p * scale and the
-// zero-points enter through one extra running sum per head, sum_j p_j zero_j, added to every coefficient
-// in the epilogue.
+// A byte holds four 2-bit codes (levels 0 .. 3) of a group.  Both halves of a word get the byte, and a mask leaves two levels
+// where they stand, as the binary16 subnormals l 4^i 2^-24: no gather, and the accumulators of level i are divided by 4^i in
+// the epilogue.  64 sequences of 32768 tokens with band: 441 -> 418 us a call against a gather from the 256 products
+// {0,1,2,3}^4 in shared memory; error against binary64 at 700 / 6000 tokens 3.2e-4 / 4.4e-4 -> 2.4e-4 / 3.1e-4, because the
+// tensor core aligns subnormals without normalising them, so larger ones lose less.  (Both levels of a word from two
+// tokens, 16 tokens a product, saves 32 instructions per 32 tokens but doubles the accumulators: 421 us, and 4.0e-4.)
+// The weight of a token's codes is p * scale and the zero-points enter through one extra running sum per head,
+// sum_j p_j zero_j, added to every coefficient in the epilogue.
 //
 // Numerics of the tensor-core value side.  A softmax weight enters the product as the binary16 number
 // w = fp16(2^15 p) (p <= 1 relative to the running maximum, so w <= 2^15; weights down to 2^-39 stay
@@ -665,7 +669,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
                             int batch, int n_q_heads, int n_kv_heads, float* __restrict__ part_ml,
                             float* __restrict__ part_acc, uint32_t* __restrict__ dev_status, int pt_stride,
                             const int32_t* __restrict__ cost_prefix, int seg_weight, long* __restrict__ cta_range,
-                            const float* __restrict__ qc, int vcb_per_head,
+                            const float* __restrict__ qc,
                             int32_t* __restrict__ pair_count, const float* __restrict__ rv_t,
                             const float* __restrict__ v_mean, void* __restrict__ out_fused, int out_is_fp32) {
     // out_fused != null: the CTA that writes the last partial of a (sequence, KV head) pair also merges the pair's
@@ -701,7 +705,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     // its (constant) value codebook starts flowing into shared memory before the grid-dependency wait and
     // lands behind the segment lookup and the first table build.
     int vcb_head = (int)(((long)blockIdx.x * n_kv_heads) / gridDim.x);   // KV head whose value codebook is resident
-    stage_value_codebook_async(C::VCB, cb_v_img + (size_t)vcb_head * vcb_per_head);
+    if (!VSQ) stage_value_codebook_async(C::VCB, cb_v_img + (size_t)vcb_head * VCB_COPY_BYTES);
     // With the merge fused in, the kernels that follow (the query transform of the next call writes the same
     // workspace) must not start before this grid is done: no early release of the dependents.
     if (out_fused != nullptr) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -751,6 +755,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     const bool odd_col = fc & 1;
     // widening selectors: byte pairs (u, replicated top bit of u = 0) of the low / high half of a codeword, taken
     // from the first operand in even columns and from the second in odd columns
+    const uint32_t sel_lv = odd_col ? 0x4444u : 0u;
     const uint32_t sel_lo = odd_col ? 0xD5C4u : 0x9180u, sel_hi = odd_col ? 0xF7E6u : 0xB3A2u;
     // B fragments carry a weight in the low or high half depending on the column parity (fr & 1)
     const uint32_t sel_b0 = (fr & 1) ? 0x1044u : 0x4410u, sel_b1 = (fr & 1) ? 0x3244u : 0x4432u;
@@ -823,8 +828,8 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         const int pair = sg.kvh * batch + sg.b;            // grows along the walk
 
         // ---- segment prologue -----------------------------------------------------------------
-        if (vcb_head != sg.kvh) {
-            stage_value_codebook_async(C::VCB, cb_v_img + (size_t)sg.kvh * vcb_per_head);
+        if (!VSQ && vcb_head != sg.kvh) {
+            stage_value_codebook_async(C::VCB, cb_v_img + (size_t)sg.kvh * VCB_COPY_BYTES);
             vcb_head = sg.kvh;
         }
         // q' of the pair's heads -> shared memory (rows beyond HG are zero)
@@ -1070,16 +1075,26 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
                         // gather: X[x][u] = codeword of token 8ts + 4u + fc of the block, group block x ^ (fc & 1), row fr
                         uint32_t X[NGB][2];
 #pragma unroll
-                        for (int x = 0; x < NGB; ++x) {
+                        for (int x = 0; x < (VSQ ? 0 : NGB); ++x) {
                             const uint32_t vwd = cur.vw[blk][x];      // codes of the group block this load fetches (x ^ 1 in odd columns)
                             X[x][0] = vgather(vwd, 2 * ts, x);
                             X[x][1] = vgather(vwd, 2 * ts + 1, x);
                         }
 #pragma unroll
                         for (int gb = 0; gb < NGB; ++gb) {
-                            // bytes (u, 0) pairs from X[gb] (even columns) or X[gb ^ 1] (odd columns)
-                            const uint32_t a0 = prmt_rep(X[gb][0], X[gb ^ 1][0], sel_lo), a1 = prmt_rep(X[gb][0], X[gb ^ 1][0], sel_hi);
-                            const uint32_t a2 = prmt_rep(X[gb][1], X[gb ^ 1][1], sel_lo), a3 = prmt_rep(X[gb][1], X[gb ^ 1][1], sel_hi);
+                            uint32_t a0, a1, a2, a3;
+                            if (VSQ) {
+                                // the token's byte of four levels into both halves of a word, from the even or odd columns' word,
+                                // and two levels kept in place: the accumulators of level i carry 4^i
+                                const uint32_t d0 = __byte_perm(cur.vw[blk][gb], cur.vw[blk][gb ^ 1], sel_lv + 0x1111u * (2 * ts));
+                                const uint32_t d1 = __byte_perm(cur.vw[blk][gb], cur.vw[blk][gb ^ 1], sel_lv + 0x1111u * (2 * ts + 1));
+                                a0 = d0 & 0x000c0003u; a1 = d0 & 0x00c00030u;
+                                a2 = d1 & 0x000c0003u; a3 = d1 & 0x00c00030u;
+                            } else {
+                                // bytes (u, 0) pairs from X[gb] (even columns) or X[gb ^ 1] (odd columns)
+                                a0 = prmt_rep(X[gb][0], X[gb ^ 1][0], sel_lo); a1 = prmt_rep(X[gb][0], X[gb ^ 1][0], sel_hi);
+                                a2 = prmt_rep(X[gb][1], X[gb ^ 1][1], sel_lo); a3 = prmt_rep(X[gb][1], X[gb ^ 1][1], sel_hi);
+                            }
 #pragma unroll
                             for (int hs = 0; hs < HSETS; ++hs) mma_f16(macc[hs][gb], a0, a1, a2, a3, b0[hs], b1[hs]);
                         }
@@ -1185,7 +1200,8 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 #pragma unroll
                 for (int gb = 0; gb < NGB; ++gb) {
                     *reinterpret_cast<float4*>(m_acc + ((size_t)warp * HPAD + hs * 4 + fc) * C::MROW + (8 * gb + fr) * 4) =
-                        make_float4(macc[hs][gb][0] * unsh, macc[hs][gb][1] * unsh, macc[hs][gb][2] * unsh, macc[hs][gb][3] * unsh);
+                        VSQ ? make_float4(macc[hs][gb][0] * unsh, macc[hs][gb][1] * (unsh * 0.25f), macc[hs][gb][2] * (unsh * 0.0625f), macc[hs][gb][3] * (unsh * 0.015625f))
+                            : make_float4(macc[hs][gb][0], macc[hs][gb][1], macc[hs][gb][2], macc[hs][gb][3]);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) macc[hs][gb][i] = 0.f;
                 }
@@ -2241,11 +2257,11 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
         {
             novakv_prof_scope ps(ctx, 0, stream);
             novakv_launch_pdl(kern, dim3(grid), dim3(S1_THREADS), S1_SMEM_BYTES, stream, qp, ly.cb_k_lut,
-                              VSQ ? (const uint8_t*)ctx->int2_img : (const uint8_t*)ly.cb_v_u8, (const float*)ly.v_scale,
+                              (const uint8_t*)ly.cb_v_u8, (const float*)ly.v_scale,
                               (const float*)ly.v_off, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
                               seq_lens, prefix, batch, hq, hkv, part_ml, part_acc, ctx->dev_status, pt_stride,
                               (const int32_t*)cost_prefix, ctx->seg_weight, cta_range, (const float*)qc,
-                              VSQ ? 0 : VCB_COPY_BYTES, pair_count, (const float*)ly.rv_t, (const float*)ly.v_mean,
+                              pair_count, (const float*)ly.rv_t, (const float*)ly.v_mean,
                               fuse ? out : (void*)nullptr, out_is_fp32);
             ps.end();
             ctx->launches++;

@@ -55,7 +55,6 @@ struct novakv_ctx {
     int hg = 0, n_groups = 0, n_sm = 0;
     std::vector<novakv_layer> layers;
     uint32_t* dev_status = nullptr;
-    void* int2_img = nullptr;     // uint8 [256][32][4]: the product codebook {0,1,2,3}^4 in the value-gather layout
     bool profile = false;
     std::vector<novakv_event_pair> prof[3];
     std::vector<novakv_event_pair> prof_free;
