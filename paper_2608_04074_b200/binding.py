@@ -1,7 +1,8 @@
 """Thin ctypes binding of libnovakv.so: argument marshalling only.
 
 Every function mirrors the entry point of the same name in ``include/novakv.h`` and passes
-``torch`` tensors as raw device pointers plus the current CUDA stream.  There is no CPU or
+``torch`` tensors as raw device pointers plus the current CUDA stream; the calls of a step go through the
+``_novakv_calls`` extension, the others through ctypes.  There is no CPU or
 PyTorch fallback: if the shared library is missing or a call returns an error status, a
 ``NovaKVError`` is raised.
 """
@@ -144,6 +145,18 @@ def _stream():
     return c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
+def _bind_calls(lib):
+    """The per-step entries of the library, as callables that take tensors."""
+    import torch
+    try:
+        from . import _novakv_calls
+    except ImportError as e:
+        raise NovaKVError(f"cannot load {_build.LIB_CALLS}: build it with paper_2608_04074_b200.build.build_calls() ({e})")
+    torch.cuda.init()
+    _novakv_calls.setup(torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, torch.float32)
+    return _novakv_calls.bind(lib._handle)
+
+
 class Context:
     """Owns a ``novakv_ctx``; methods carry the names of the C entry points."""
 
@@ -154,6 +167,13 @@ class Context:
         _check(self.lib, self.lib.novakv_create(ctypes.byref(self.handle), ctypes.byref(self.cfg)), "novakv_create")
         self.n_q_heads, self.n_kv_heads, self.head_dim = n_q_heads, n_kv_heads, head_dim
         self.n_groups = head_dim // 4
+        self._scale = float(head_dim) ** -0.5
+        self._calls = _bind_calls(self.lib)
+
+    def _call(self, name, *args):
+        status = self._calls[name](self.handle.value, *args)
+        if status != 0:
+            _check(self.lib, status, name)
 
     def close(self):
         if self.handle:
@@ -190,83 +210,53 @@ class Context:
 
     # -- hot path ---------------------------------------------------------------------------
     def novakv_encode_append(self, layer, k_new, v_new, tok_seq, tok_pos, k_pages, v_pages, page_table, seq_lens):
-        n_tokens = int(k_new.shape[0]) if k_new is not None else 0
-        _check(self.lib, self.lib.novakv_encode_append(
-            self.handle, layer, _ptr(k_new), _ptr(v_new), _ptr(tok_seq), _ptr(tok_pos), n_tokens,
-            _ptr(k_pages), _ptr(v_pages), int(k_pages.shape[0]), _ptr(page_table), int(page_table.shape[1]),
-            int(page_table.shape[0]), _ptr(seq_lens), _stream()), "novakv_encode_append")
+        self._call("novakv_encode_append", layer, k_new, v_new, tok_seq, tok_pos, k_pages, v_pages, page_table, seq_lens)
+
 
     def novakv_decode_attention(self, layer, q, k_pages, v_pages, page_table, seq_lens, out, workspace,
                                 sm_scale=None):
-        import torch
-        batch = int(q.shape[0])
-        scale = float(self.head_dim) ** -0.5 if sm_scale is None else float(sm_scale)
-        _check(self.lib, self.lib.novakv_decode_attention(
-            self.handle, layer, _ptr(q), _ptr(k_pages), _ptr(v_pages), int(k_pages.shape[0]), _ptr(page_table),
-            int(page_table.shape[1]), _ptr(seq_lens), batch, scale, _ptr(out),
-            1 if out.dtype == torch.float32 else 0, _ptr(workspace),
-            int(workspace.numel() * workspace.element_size()), _stream()), "novakv_decode_attention")
+        self._call("novakv_decode_attention", layer, q, k_pages, v_pages, page_table, seq_lens, out, workspace,
+                   self._scale if sm_scale is None else sm_scale)
+
 
     def novakv_scale_page_bytes(self):
         return int(self.lib.novakv_scale_page_bytes(self.handle))
 
     def novakv_encode_append_scaled(self, layer, k_new, v_new, tok_seq, tok_pos, k_pages, v_pages, k_scales,
                                     page_table, seq_lens):
-        n_tokens = int(k_new.shape[0]) if k_new is not None else 0
-        _check(self.lib, self.lib.novakv_encode_append_scaled(
-            self.handle, layer, _ptr(k_new), _ptr(v_new), _ptr(tok_seq), _ptr(tok_pos), n_tokens,
-            _ptr(k_pages), _ptr(v_pages), _ptr(k_scales), int(k_pages.shape[0]), _ptr(page_table),
-            int(page_table.shape[1]), int(page_table.shape[0]), _ptr(seq_lens), _stream()),
-            "novakv_encode_append_scaled")
+        self._call("novakv_encode_append_scaled", layer, k_new, v_new, tok_seq, tok_pos, k_pages, v_pages, k_scales,
+                   page_table, seq_lens)
+
 
     def novakv_decode_attention_scaled(self, layer, q, k_pages, v_pages, k_scales, page_table, seq_lens, out,
                                        workspace, sm_scale=None):
-        import torch
-        batch = int(q.shape[0])
-        scale = float(self.head_dim) ** -0.5 if sm_scale is None else float(sm_scale)
-        _check(self.lib, self.lib.novakv_decode_attention_scaled(
-            self.handle, layer, _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(k_scales), int(k_pages.shape[0]),
-            _ptr(page_table), int(page_table.shape[1]), _ptr(seq_lens), batch, scale, _ptr(out),
-            1 if out.dtype == torch.float32 else 0, _ptr(workspace),
-            int(workspace.numel() * workspace.element_size()), _stream()), "novakv_decode_attention_scaled")
+        self._call("novakv_decode_attention_scaled", layer, q, k_pages, v_pages, k_scales, page_table, seq_lens, out,
+                   workspace, self._scale if sm_scale is None else sm_scale)
+
 
     def novakv_decode_attention_sink(self, layer, q, k_pages, v_pages, k_scales, sink_logits, page_table, seq_lens,
                                      out, workspace, sm_scale=None):
         """Decode step with a learned sink logit per query head (k_scales may be None)."""
-        import torch
-        batch = int(q.shape[0])
-        scale = float(self.head_dim) ** -0.5 if sm_scale is None else float(sm_scale)
-        _check(self.lib, self.lib.novakv_decode_attention_sink(
-            self.handle, layer, _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(k_scales) if k_scales is not None else None,
-            _ptr(sink_logits), int(k_pages.shape[0]), _ptr(page_table), int(page_table.shape[1]), _ptr(seq_lens),
-            batch, scale, _ptr(out), 1 if out.dtype == torch.float32 else 0, _ptr(workspace),
-            int(workspace.numel() * workspace.element_size()), _stream()), "novakv_decode_attention_sink")
+        self._call("novakv_decode_attention_sink", layer, q, k_pages, v_pages, k_scales, sink_logits, page_table, seq_lens,
+                   out, workspace, self._scale if sm_scale is None else sm_scale)
+
 
     def novakv_decode_attention_banded(self, layer, q, k_pages, v_pages, k_scales, sink_logits, page_table,
                                        quant_lens, band_k, band_v, n_sink, band_meta, out, workspace, sm_scale=None):
         """Decode step on a cache with a BF16 sink-plus-recent band (band_k/band_v [batch][cap][Hkv][d])."""
-        import torch
-        batch = int(q.shape[0])
-        scale = float(self.head_dim) ** -0.5 if sm_scale is None else float(sm_scale)
-        _check(self.lib, self.lib.novakv_decode_attention_banded(
-            self.handle, layer, _ptr(q), _ptr(k_pages), _ptr(v_pages),
-            _ptr(k_scales) if k_scales is not None else None, _ptr(sink_logits) if sink_logits is not None else None,
-            int(k_pages.shape[0]), _ptr(page_table), int(page_table.shape[1]), _ptr(quant_lens), _ptr(band_k),
-            _ptr(band_v), int(band_k.shape[1]), int(n_sink), _ptr(band_meta), batch, scale, _ptr(out),
-            1 if out.dtype == torch.float32 else 0, _ptr(workspace),
-            int(workspace.numel() * workspace.element_size()), _stream()), "novakv_decode_attention_banded")
+        self._call("novakv_decode_attention_banded", layer, q, k_pages, v_pages, k_scales, sink_logits, page_table,
+                   quant_lens, band_k, band_v, n_sink, band_meta, out, workspace,
+                   self._scale if sm_scale is None else sm_scale)
+
 
     def novakv_value_meta_page_bytes(self):
         return int(self.lib.novakv_value_meta_page_bytes(self.handle))
 
     def novakv_encode_append_deployed(self, layer, k_new, v_new, tok_seq, tok_pos, k_pages, v_pages, k_scales, v_meta,
                                       page_table, seq_lens):
-        n_tokens = int(k_new.shape[0]) if k_new is not None else 0
-        _check(self.lib, self.lib.novakv_encode_append_deployed(
-            self.handle, layer, _ptr(k_new), _ptr(v_new), _ptr(tok_seq), _ptr(tok_pos), n_tokens,
-            _ptr(k_pages), _ptr(v_pages), _ptr(k_scales), _ptr(v_meta), int(k_pages.shape[0]), _ptr(page_table),
-            int(page_table.shape[1]), int(page_table.shape[0]), _ptr(seq_lens), _stream()),
-            "novakv_encode_append_deployed")
+        self._call("novakv_encode_append_deployed", layer, k_new, v_new, tok_seq, tok_pos, k_pages, v_pages, k_scales, v_meta,
+                   page_table, seq_lens)
+
 
     def novakv_band_append_staging_bytes(self, batch, block):
         return int(self.lib.novakv_band_append_staging_bytes(self.handle, int(batch), int(block)))
@@ -274,27 +264,17 @@ class Context:
     def novakv_band_append(self, layer, k_new, v_new, band_k, band_v, n_sink, n_rec, block, band_meta, quant_lens,
                            k_pages, v_pages, k_scales, v_meta, page_table, seq_lens, staging):
         """One new token per sequence into the BF16 band; blocks that leave it are encoded (all on the device)."""
-        opt = lambda t: _ptr(t) if t is not None else None
-        _check(self.lib, self.lib.novakv_band_append(
-            self.handle, layer, _ptr(k_new), _ptr(v_new), int(k_new.shape[0]), _ptr(band_k), _ptr(band_v),
-            int(band_k.shape[1]), int(n_sink), int(n_rec), int(block), _ptr(band_meta), _ptr(quant_lens),
-            _ptr(k_pages), _ptr(v_pages), opt(k_scales), opt(v_meta), int(k_pages.shape[0]), _ptr(page_table),
-            int(page_table.shape[1]), _ptr(seq_lens), _ptr(staging), int(staging.numel() * staging.element_size()),
-            _stream()), "novakv_band_append")
+        self._call("novakv_band_append", layer, k_new, v_new, band_k, band_v, n_sink, n_rec, block, band_meta, quant_lens,
+                   k_pages, v_pages, k_scales, v_meta, page_table, seq_lens, staging)
+
 
     def novakv_decode_attention_deployed(self, layer, q, k_pages, v_pages, k_scales, v_meta, sink_logits, page_table,
                                          quant_lens, band_k, band_v, n_sink, band_meta, out, workspace, sm_scale=None):
         """Decode on the deployed format; band_k = band_v = band_meta = None: no BF16 band."""
-        import torch
-        batch = int(q.shape[0])
-        scale = float(self.head_dim) ** -0.5 if sm_scale is None else float(sm_scale)
-        opt = lambda t: _ptr(t) if t is not None else None
-        _check(self.lib, self.lib.novakv_decode_attention_deployed(
-            self.handle, layer, _ptr(q), _ptr(k_pages), _ptr(v_pages), _ptr(k_scales), _ptr(v_meta), opt(sink_logits),
-            int(k_pages.shape[0]), _ptr(page_table), int(page_table.shape[1]), _ptr(quant_lens), opt(band_k),
-            opt(band_v), int(band_k.shape[1]) if band_k is not None else 0, int(n_sink), opt(band_meta), batch, scale,
-            _ptr(out), 1 if out.dtype == torch.float32 else 0, _ptr(workspace),
-            int(workspace.numel() * workspace.element_size()), _stream()), "novakv_decode_attention_deployed")
+        self._call("novakv_decode_attention_deployed", layer, q, k_pages, v_pages, k_scales, v_meta, sink_logits, page_table,
+                   quant_lens, band_k, band_v, n_sink, band_meta, out, workspace,
+                   self._scale if sm_scale is None else sm_scale)
+
 
     def novakv_decode_attention_noalloc(self, layer, q, k_pages, v_pages, page_table, seq_lens, out, sm_scale=None):
         """Decode step whose scratch is the library's fixed device array (no workspace argument)."""
@@ -318,16 +298,10 @@ class Context:
                          v_pages, page_table, seq_lens, out_host, staging, workspace, sm_scale=None, wait=True):
         """Host tensors (ideally pinned) in, host tensor out; the cache stays on the device.  wait=False enqueues
         the step without waiting for it (``novakv_step_host_async``): read ``out_host`` after a stream sync."""
-        n_tokens = int(k_new_host.shape[0]) if k_new_host is not None else 0
-        batch = int(q_host.shape[0])
-        scale = float(self.head_dim) ** -0.5 if sm_scale is None else float(sm_scale)
-        fn = self.lib.novakv_step_host if wait else self.lib.novakv_step_host_async
-        _check(self.lib, fn(
-            self.handle, layer, _ptr(k_new_host), _ptr(v_new_host), _ptr(tok_seq_host), _ptr(tok_pos_host),
-            n_tokens, _ptr(q_host), _ptr(k_pages), _ptr(v_pages), int(k_pages.shape[0]), _ptr(page_table),
-            int(page_table.shape[1]), _ptr(seq_lens), batch, scale, _ptr(out_host), _ptr(staging),
-            int(staging.numel() * staging.element_size()), _ptr(workspace),
-            int(workspace.numel() * workspace.element_size()), _stream()), "novakv_step_host")
+        self._call("novakv_step_host" if wait else "novakv_step_host_async", layer, k_new_host, v_new_host, tok_seq_host,
+                   tok_pos_host, q_host, k_pages, v_pages, page_table, seq_lens, out_host, staging, workspace,
+                   self._scale if sm_scale is None else sm_scale)
+
 
     # -- helpers ----------------------------------------------------------------------------
     def novakv_search_coefficients(self, layer, which, coef, idx_out):
@@ -340,13 +314,9 @@ class Context:
 
     def novakv_bf16_decode_attention(self, q, k_pages_bf16, v_pages_bf16, page_table, seq_lens, out, workspace,
                                      sm_scale=None, window=0):
-        import torch
-        scale = float(self.head_dim) ** -0.5 if sm_scale is None else float(sm_scale)
-        _check(self.lib, self.lib.novakv_bf16_decode_attention(
-            self.handle, _ptr(q), _ptr(k_pages_bf16), _ptr(v_pages_bf16), int(k_pages_bf16.shape[0]),
-            _ptr(page_table), int(page_table.shape[1]), _ptr(seq_lens), int(q.shape[0]), scale, int(window),
-            _ptr(out), 1 if out.dtype == torch.float32 else 0, _ptr(workspace),
-            int(workspace.numel() * workspace.element_size()), _stream()), "novakv_bf16_decode_attention")
+        self._call("novakv_bf16_decode_attention", q, k_pages_bf16, v_pages_bf16, page_table, seq_lens, out, workspace,
+                   self._scale if sm_scale is None else sm_scale, window)
+
 
     def novakv_profile_enable(self, on=True):
         _check(self.lib, self.lib.novakv_profile_enable(self.handle, 1 if on else 0), "novakv_profile_enable")

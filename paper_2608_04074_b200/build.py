@@ -1,4 +1,4 @@
-"""In-tree builds: the CUDA C-ABI library (nvcc, sm_100a) and the host calibration helper (gcc).
+"""In-tree builds: the CUDA C-ABI library (nvcc, sm_100a), its Python entry and the host calibration helper (gcc).
 
 Artefacts are written next to this file so that they travel with a snapshot of the tree.
 """
@@ -7,6 +7,7 @@ from __future__ import annotations
 import os
 import shutil
 import subprocess
+import sysconfig
 from pathlib import Path
 
 PKG_DIR = Path(__file__).resolve().parent
@@ -14,6 +15,7 @@ CSRC = PKG_DIR / "csrc"
 INCLUDE = PKG_DIR.parent / "include"
 LIB_CUDA = PKG_DIR / "libnovakv.so"
 LIB_CALIB = PKG_DIR / "libnovakv_calib.so"
+LIB_CALLS = PKG_DIR / "_novakv_calls.so"
 
 CUDA_SOURCES = ["novakv_api.cu", "novakv_encode.cu", "novakv_prefill.cu", "novakv_decode.cu", "novakv_bf16_decode.cu",
                 "novakv_noalloc.cu"]
@@ -35,6 +37,7 @@ def _nvcc() -> str:
 
 def build_cuda(force: bool = False, verbose: bool = False) -> Path:
     srcs = [CSRC / s for s in CUDA_SOURCES if (CSRC / s).exists()]
+    build_calls(force)
     deps = srcs + sorted(CSRC.glob("*.cuh")) + sorted(INCLUDE.glob("*.h"))
     if not force and _newer(LIB_CUDA, deps):
         return LIB_CUDA
@@ -49,6 +52,17 @@ def build_cuda(force: bool = False, verbose: bool = False) -> Path:
     if verbose:
         print(res.stderr)
     return LIB_CUDA
+
+
+def build_calls(force: bool = False) -> Path:
+    src = CSRC / "novakv_calls.c"
+    if not force and _newer(LIB_CALLS, [src] + sorted(INCLUDE.glob("*.h"))):
+        return LIB_CALLS
+    cmd = ["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", str(INCLUDE), str(src), "-o", str(LIB_CALLS), "-ldl"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("gcc failed:\n" + res.stdout + res.stderr)
+    return LIB_CALLS
 
 
 def build_calib_host(force: bool = False) -> Path:
