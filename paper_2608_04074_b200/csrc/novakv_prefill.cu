@@ -17,10 +17,11 @@
 //
 // Roles: four token warpgroups, two per half tile (thread = token, each takes half of the groups), whose first warp
 // issues the search MMAs; one warp looks up destinations, copies token rows (TMA) and issues the transforms; one feeds the
-// codebook rings; two search in binary64.  A chunk of 128 codewords makes a round trip token warps -> MMA -> token warps
-// (about 300 cycles, whatever its width), so chunks are as wide as TMEM allows (four warpgroups x 128 columns: the
-// coefficients live in shared memory for that), and the first chunk of the next group is computed behind the selection
-// of this one.  Every wait is bounded (novakv_tcgen05.cuh): a wait that gives up sets NOVAKV_DEV_WAIT_TIMEOUT, and the CTA
+// codebook rings; two search in binary64.  The round trip token warps -> MMA -> token warps takes some 400 cycles and more
+// until the last warp is there, so the two warpgroups of a half tile take turns on its 256 columns: one reads all 256
+// distances of a group in one go (the next 32 columns on their way while 32 are looked at) and then ranks, evaluates and
+// stores while the other reads; each issues the other's MMA when it is done reading.  (One chunk of 128 columns for each
+// warpgroup, two round trips a group: 522 us where this takes 505.)  Every wait is bounded (novakv_tcgen05.cuh): a wait that gives up sets NOVAKV_DEV_WAIT_TIMEOUT, and the CTA
 // runs through the rest of its segment without waiting and leaves.  Three things hold on that way: the token warps take
 // no destination that the flag has overtaken (tokens without one are neither stored nor looked at again), the named
 // barriers among token warps and the waits for the search MMAs between them are never skipped (each of these MMAs is issued
@@ -30,8 +31,9 @@
 // What bounds it: instruction issue and latency of the selection, about 600 warp instructions per 32 tokens and group (of
 // which 64 + 16 packed minima and comparisons on the half-rate pipe) with four token warps per scheduler; tensor pipe
 // 16 %, issue slots 58 % busy.  The kernel lives at the limit of 96 registers: everything the rare paths need is
-// formed there.  d = 128, 32768 tokens: 523 us a call in a stream of calls (binary32 search on the FMA pipe with a binary64 transform: 1971 us).
-// Measured on the way: coefficients in TMEM and chunks of 64 codewords 945 us; releasing a chunk through an mbarrier
+// formed there.  d = 128, 32768 tokens: 493 us a call in a stream of calls (binary32 search on the FMA pipe with a binary64 transform: 1971 us).
+// Norms of the rows by the loading warp instead of the token warps: 528 us against 505 (the rows' way to the transform got longer).
+// Measured on the way, with chunks: coefficients in TMEM and chunks of 64 codewords 945 us; releasing a chunk through an mbarrier
 // instead of a hardware barrier +13 %; MMAs issued behind lane == 0 instead of elect.sync +40 cycles each; spills of 150
 // bytes in the loop +15 %; one helper warp instead of two 665 us; direct distances one group late, to hide the round
 // trip of the second chunk too: 635 us (longer register lifetimes cost more than the wait).
@@ -57,8 +59,13 @@ constexpr int PF_CW_BYTES = 4096;            // and in binary32
 constexpr int PF_CW_STAGES = 6;              // (the binary32 codewords are needed one group longer than the operand)
 static_assert(PF_OP_BYTES + PF_CW_BYTES == NOVAKV_PF_GROUP_BYTES, "codebook image");
 constexpr int PF_QUEUE = 16;                 // entries of a helper's queue
+constexpr int PF_QUEUE_LAST = 4;             // of which a segment's last tile fills so many (the CTA waits for what is queued at its end)
 // Durations the work split reckons with, microseconds per unit (measured: 19.3 for 16 groups of plain keys or values, about
 // 28 for scaled keys, which transform and norm the whole row, 11 for INT2 values).
+// Keys leave more to the helpers than values and take 7 % longer; the cut reckons with that where a CTA has enough units for
+// it to matter (32768 tokens, 28 units a CTA: 505 -> 490 us; 8191 of the d = 64 shape, 3.5 units: 73.4 -> 76).
+constexpr double PF_KEYS = 1.07;
+constexpr int PF_KEYS_UNITS = 8;
 constexpr double PF_US_UNIT = 3.0, PF_US_GROUP = 1.0, PF_US_SCALED = 9.0, PF_US_INT2 = 11.0;
 // |coefficient - binary64 coefficient| <= KAPPA (|x| + |mean|) |R column|.  The accumulation order of the tensor core is
 // not specified; all-positive inputs (every truncation in the same direction) showed 2^-21.6, random signs 2^-23.3.
@@ -400,7 +407,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
 
     // running phase counts of the barriers, over all segments
     int n_it = 0, n_use = 0, n_seg = 0;               // tiles; ring uses; segments
-    uint32_t n_s = 0;                                 // token warps: chunks seen
+    uint32_t n_s = 0;                                 // token warps: groups seen
     int q_tail = 0;                                   // helpers: entries taken
 
     // ---- segments: units of one (KV head, side, part of the groups)
@@ -604,7 +611,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
             // ---- token warps: thread = token; warpgroup wg = 2 * half tile + half of the groups
             const int wg = warp >> 2, w = wg >> 1, hf = wg & 1, row = threadIdx.x & (PF_HALF - 1);
             const uint32_t lane_base = (uint32_t)(warp & 3) << 21;
-            const uint32_t d_t = tmem + w * 256 + lane_base, d_s = tmem + wg * 128;
+            const uint32_t d_t = tmem + w * 256 + lane_base, d_s = tmem + w * 256;
             const uint32_t a_s = sb + P::OFF_A + wg * P::A_BYTES;
             float* const x2_s = reinterpret_cast<float*>(smem + P::OFF_A);               // partial |x|^2, [wg][A_BYTES / 4]
             const float* const mr = cst;
@@ -815,11 +822,10 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                 tc_fence_before();
                 nbar_sync(5 + w, PF_TILE);                                     // the transform's accumulators are read out
 
-                // ---- search of groups lb .. lb + ngh - 1.  The first chunk of the next group is computed behind the choice and
-                // the direct distances of this one.
+                // ---- search of groups lb .. lb + ngh - 1
                 const int use0 = n_use + hf;
-                // the search operand of group g into shared memory; |r|^2 in the group's scale
-                auto publish = [&](int g) -> float {
+                // the search operand of group g into shared memory
+                auto publish = [&](int g) {
                     const float4 r = lds_f4(c_s + g * (PF_HALF * 16));
                     const float sc = cst[D + L + lb + g];
                     const float s0 = r.x * sc, s1 = r.y * sc, s2 = r.z * sc, s3 = r.w * sc;
@@ -833,45 +839,59 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                     asm volatile("st.shared.v4.b32 [%0], {%1,%2,%1,%2};" ::"r"(dst), "r"(h01), "r"(h23) : "memory");
                     asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst + PF_HALF * 16), "r"(l01), "r"(l23), "r"(0x3c003c00u), "r"(qp) : "memory");
                     fence_proxy_async();
-                    return qq;
                 };
-                // The warp is done with the accumulators (and has written its operand rows); when the four warps of the
-                // warpgroup are, its first warp issues the distances of chunk c of group g.
-                auto release_and_issue = [&](int c, int g) {
+                // The two warpgroups of a half tile take turns on its 256 columns.  Group g of warpgroup x (distances to all
+                // 256 codewords, one MMA) is issued by x's partner, when the partner's four warps have read their own
+                // distances out of the columns and x's four warps have written the operand: x works on its previous group
+                // meanwhile, so that neither waits for the round trip.
+                auto issue = [&](int x, int g) {
+                    const int use = n_use + (x & 1) + 2 * g, st = use % P::NOP;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        umma_f16(d_s, umma_desc(sb + P::OFF_A + x * P::A_BYTES, PF_HALF * 16, 128, 0),
+                                 umma_desc(sb + P::OFF_RING + st * PF_OP_BYTES, 4096, 128, 0), umma_idesc(false, false, 128, 256), false);
+                        umma_commit(bar(B_S + x));
+                        umma_commit(bar(B_RINGFREE + st));
+                    }
+                    __syncwarp();
+                };
+                auto ring_wait = [&](int x, int g) {
+                    const int use = n_use + (x & 1) + 2 * g;
+                    mbar_wait<PF_TOK_NS>(bar(B_RING + use % P::NOP), (use / P::NOP) & 1, abort_flag);
+                };
+                // this warpgroup has read the columns: the partner's group g is next
+                auto hand_over = [&](int g) {
                     tc_fence_before();
                     if ((warp & 3) != 0) {
-                        nbar_arrive(1 + wg, PF_HALF);
+                        nbar_arrive(7 + (wg ^ 1), PF_TILE);
                     } else {
-                        const int use = use0 + 2 * g, st = use % P::NOP;
-                        if (c == 0) mbar_wait<PF_TOK_NS>(bar(B_RING + st), (use / P::NOP) & 1, abort_flag);
-                        nbar_sync(1 + wg, PF_HALF);
-                        tc_fence_after();
-                        if (elect_one()) {
-                            umma_f16(d_s, umma_desc(a_s, PF_HALF * 16, 128, 0),
-                                     umma_desc(sb + P::OFF_RING + st * PF_OP_BYTES + c * 2048, 4096, 128, 0), umma_idesc(false, false, 128, 128), false);
-                            umma_commit(bar(B_S + wg));
-                            if (c == 1) umma_commit(bar(B_RINGFREE + st));
-                        }
-                        __syncwarp();
+                        ring_wait(wg ^ 1, g);
+                        nbar_sync(7 + (wg ^ 1), PF_TILE);
+                        issue(wg ^ 1, g);
                     }
                 };
                 // minima of 32 rows of 8 codewords, two rows per register.  (Distances are not negative, or tiny: their
                 // binary16 patterns compare like integers.  A negative one sorts below every positive one, and every negative
                 // row minimum passes the test below.)
                 uint32_t rmin[16];
-                auto minima = [&](int c, const uint32_t (&v)[32]) {
+                auto minima = [&](int c, const uint32_t (&v)[16]) {
 #pragma unroll
-                    for (int qd = 0; qd < 4; ++qd)
-                        rmin[4 * c + qd] = __vimin3_s16x2(__vimin3_s16x2(v[8 * qd], v[8 * qd + 1], v[8 * qd + 2]),
+                    for (int qd = 0; qd < 2; ++qd)
+                        rmin[2 * c + qd] = __vimin3_s16x2(__vimin3_s16x2(v[8 * qd], v[8 * qd + 1], v[8 * qd + 2]),
                                                           __vimin3_s16x2(v[8 * qd + 3], v[8 * qd + 4], v[8 * qd + 5]),
                                                           __vmins2(v[8 * qd + 6], v[8 * qd + 7]));
                 };
-                auto accumulators = [&](int half, uint32_t (&v)[32]) {
-                    tmem_ld64_h2(d_s + lane_base + half * 64, v);
-                    tmem_wait_ld();
-                };
-                float q2 = publish(0);                                         // |r|^2 of this group, in its scale
-                release_and_issue(0, 0);
+                auto accumulators = [&](int c, uint32_t (&v)[16]) { tmem_ld32_h2(d_s + lane_base + c * 32, v); };
+                publish(0);
+                if (hf == 1) {
+                    nbar_arrive(7 + wg, PF_TILE);
+                } else if ((warp & 3) != 0) {
+                    nbar_arrive(1 + wg, PF_HALF);
+                } else {
+                    ring_wait(wg, 0);
+                    nbar_sync(1 + wg, PF_HALF);
+                    issue(wg, 0);
+                }
                 uint32_t codes = 0, pend = 0;
 #pragma unroll 1
                 for (int g = 0; g < ngh; ++g) {
@@ -880,32 +900,29 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                         ++n_s;
                         tc_fence_after();
                         __syncwarp();
-                        uint32_t v[32];
-                        accumulators(0, v);
-                        minima(0, v);
-                        accumulators(1, v);
-                        release_and_issue(1, g);
-                        minima(1, v);
-                    }
-                    {
-                        float q2n = 0.f;
-                        mbar_wait_mma(bar(B_S + wg), n_s & 1, abort_flag);
-                        ++n_s;
-                        tc_fence_after();
-                        __syncwarp();
-                        uint32_t v[32];
-                        accumulators(0, v);
-                        minima(2, v);
-                        accumulators(1, v);
-                        if (g + 1 < ngh) {
-                            q2n = publish(g + 1);
-                            release_and_issue(0, g + 1);
-                        } else {
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0 && hf == 0) mbar_arrive(bar(B_TFREE + w));
+                        {
+                            uint32_t v0[16], v1[16];                           // one half on its way while the other is looked at
+                            accumulators(0, v0);
+#pragma unroll
+                            for (int c = 0; c < 8; c += 2) {
+                                tmem_wait_ld16(v0);
+                                accumulators(c + 1, v1);
+                                minima(c, v0);
+                                tmem_wait_ld16(v1);
+                                if (c + 2 < 8) accumulators(c + 2, v0);
+                                else if (g + hf < ngh) hand_over(g + hf);
+                                else {                                         // (the second warpgroup is the last to read)
+                                    tc_fence_before();
+                                    __syncwarp();
+                                    if (lane == 0) mbar_arrive(bar(B_TFREE + w));
+                                }
+                                minima(c + 1, v1);
+                            }
                         }
-                        minima(3, v);
+                        if (g + 1 < ngh) {
+                            publish(g + 1);
+                            nbar_arrive(7 + wg, PF_TILE);
+                        }
                         float mf;
                         {
                             uint32_t m = __vimin3_s16x2(__vimin3_s16x2(rmin[0], rmin[1], rmin[2]), __vimin3_s16x2(rmin[3], rmin[4], rmin[5]),
@@ -925,8 +942,8 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                         }
                         const float rlen2 = fmaf(r.x, r.x, fmaf(r.y, r.y, fmaf(r.z, r.z, r.w * r.w)));
                         const float delta = fmaf(bound, cst[D + lb + g], (ksc ? 3.0e-7f : 6.0e-8f) * sqrt_approx(rlen2));
-                        const float dl = delta * cst[D + L + lb + g], sq2 = sqrt_approx(2.f * fmaxf(mf, 0.f));
-                        const float s2 = fmaf(1.1f, sq2, 2.f * sqrt_approx(q2));
+                        const float sc = cst[D + L + lb + g], dl = delta * sc, sq2 = sqrt_approx(2.f * fmaxf(mf, 0.f));
+                        const float s2 = fmaf(1.1f, sq2, 2.f * sqrt_approx(fmaf(r.x * sc, r.x * sc, fmaf(r.y * sc, r.y * sc, fmaf(r.z * sc, r.z * sc, (r.w * sc) * (r.w * sc))))));
                         float t = fmaf(2.1f * EPS_S, s2 * s2, fmaf(fmaxf(mf, 0.f), 1.0025f, 2.5f * dl * (sq2 + dl) + 4.0e-7f));
                         t *= 1.0005f;
                         const uint32_t t1 = pack_half2(t, t);
@@ -997,7 +1014,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                             const int h = warp & (PF_HELPERS - 1), n = __popc(todo);
                             int base = -1;
                             if (lane == 0) {
-                                if (atomicAdd(&s_count[h], n) + n <= PF_QUEUE) base = atomicAdd(&s_head[h], n);
+                                if (atomicAdd(&s_count[h], n) + n <= (i + 1 < n_local ? PF_QUEUE : PF_QUEUE_LAST)) base = atomicAdd(&s_head[h], n);
                                 else atomicSub(&s_count[h], n);
                             }
                             base = __shfl_sync(0xffffffffu, base, 0);
@@ -1037,7 +1054,6 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
                                 store_value_word<L>(chunk_of(page), slot, l - 3, codes, aligned, valid, lane);
                             }
                         }
-                        q2 = q2n;
                     }
                 }
                 n_use += 2 * ngh;
@@ -1111,7 +1127,7 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
             grid = g;
             a.gs = gs;
             // one unit per CTA where there are no more than SMs: a cut in cost would hand some a key and a value unit
-            a.cost_k = uk + uv <= ctx->n_sm ? 1 : (int)(ck * 64.0);
+            a.cost_k = uk + uv <= ctx->n_sm ? 1 : (int)(ck * (uk + uv >= PF_KEYS_UNITS * g ? PF_KEYS : 1.0) * 64.0);
             a.cost_v = uk + uv <= ctx->n_sm ? 1 : (int)(cv * 64.0);
         }
     }
