@@ -102,8 +102,9 @@ struct S1 {
     static constexpr int T32 = T16 + (HAS16 ? T16_BYTES : 0);
     static constexpr int VCB = T32 + T32_BYTES;                         // two copies of the value codebook
     static constexpr int P = VCB + 2 * VCB_COPY_BYTES;
-    static constexpr int Q = P + P_BYTES;                               // fp32 [HPAD][D]
-    static constexpr int BND = Q + HPAD * D * 4;                        // long [MAX_SCAN_CTAS + 1]: first unit of every CTA
+    static constexpr int Q_BYTES = HPAD * D * 4;
+    static constexpr int Q = P + P_BYTES;                               // fp32 [HPAD][D], of the present and of the next pair
+    static constexpr int BND = Q + 2 * Q_BYTES;                        // long [MAX_SCAN_CTAS + 1]: first unit of every CTA
     static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;           // int [2][PFX_CAP + 1]: page and cost prefix of small batches
     static constexpr int SMEM = PFX + 2 * (PFX_CAP + 1) * 4;
     // merge buffer (aliases the larger table once a segment's scan is done)
@@ -344,6 +345,11 @@ __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
     asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
     return d;
 }
+// to +-60000, both halves; a NaN becomes -60000
+__device__ __forceinline__ uint32_t clamp_h2(uint32_t h) {
+    asm("max.f16x2 %0, %0, %1;\n\tmin.f16x2 %0, %0, %2;" : "+r"(h) : "r"(0xfb53fb53u), "r"(0x7b537b53u));
+    return h;
+}
 __device__ __forceinline__ float ex2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -386,22 +392,24 @@ struct Segment {
 // u = kvh * P + page_prefix[b] + page, with P = page_prefix[batch] the pages of all sequences, so that
 // consecutive segments of a CTA share the KV head (and its value codebook).  page_prefix is exclusive,
 // length batch + 1.  Cooperative: every thread tests one sequence (all loads independent, one memory
-// latency), the owner publishes (b, length) through shared memory.  Contains a __syncthreads().
-__device__ __forceinline__ Segment locate(const int32_t* __restrict__ page_prefix, const int32_t* __restrict__ seq_lens,
-                                          int batch, int max_pages, long u, long u_end, int* s_found) {
-    const long P = page_prefix[batch];
-    Segment s;
-    s.kvh = (int)(u / P);
-    const long r = u - (long)s.kvh * P;
+// latency), the owner publishes sequence, length, first page and KV head through shared memory (found); a barrier, then
+// segment_at().  A CTA looks its next segment up before the scan of the present one.
+__device__ __forceinline__ void find_segment(const int32_t* __restrict__ page_prefix, const int32_t* __restrict__ seq_lens,
+                                             int batch, int max_pages, long u, int kvh, int* found) {
+    const long r = u - (long)kvh * page_prefix[batch];
     for (int t = threadIdx.x; t < batch; t += S1_THREADS) {
-        const int lo = page_prefix[t], hi = page_prefix[t + 1], len = seq_lens[t];
-        if ((long)lo <= r && r < (long)hi) { s_found[0] = t; s_found[1] = clamp_len(len, max_pages); s_found[2] = lo; }
+        const int lo = page_prefix[t], hi = page_prefix[t + 1];
+        if ((long)lo <= r && r < (long)hi) { found[0] = t; found[1] = clamp_len(seq_lens[t], max_pages); found[2] = lo; found[3] = kvh; }
     }
-    __syncthreads();
-    s.b = s_found[0];
-    s.len = s_found[1];
+}
+__device__ __forceinline__ Segment segment_at(const int32_t* __restrict__ page_prefix, int batch, long u, long u_end, const int* found) {
+    Segment s;
+    s.b = found[0];
+    s.len = found[1];
+    s.kvh = found[3];
+    const long r = u - (long)s.kvh * page_prefix[batch];
     const int pages_b = (s.len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
-    s.pg0 = (int)(r - s_found[2]);
+    s.pg0 = (int)(r - found[2]);
     const long left = u_end - u;
     s.npg = (int)(left < (long)(pages_b - s.pg0) ? left : (long)(pages_b - s.pg0));
     return s;
@@ -465,35 +473,51 @@ __device__ __noinline__ void build_score_table(unsigned char* t32, unsigned char
         // part (group = K32 + t' % (L - K32), 16 codes per pass); 16 passes either way.
         static_assert(K32 == 8 && L == 32 && S1_THREADS == 512 && HPAD == 4, "work split of the hybrid table build");
         constexpr int T32_THREADS = 16 * K32;                   // 128 = 4 warps
-        constexpr int BATCH = 8;
+        constexpr int BATCH = 4;                                // (8 or 16 in flight: spills around the call, 10 % of the scan)
         const bool is32 = threadIdx.x < T32_THREADS;
         const int tl = is32 ? threadIdx.x : threadIdx.x - T32_THREADS;
         const int g = is32 ? tl % K32 : K32 + tl % (L - K32);
         const int code0 = is32 ? tl / K32 : tl / (L - K32);
-        float4 qs[HPAD];
-#pragma unroll
-        for (int h = 0; h < HPAD; ++h) qs[h] = *reinterpret_cast<const float4*>(q_s + h * D + g * 4);
+        // q' of two heads side by side: one packed multiply-add serves both
+        uint64_t q01[4], q23[4];
+        {
+            const float4 h0 = *reinterpret_cast<const float4*>(q_s + g * 4), h1 = *reinterpret_cast<const float4*>(q_s + D + g * 4);
+            const float4 h2 = *reinterpret_cast<const float4*>(q_s + 2 * D + g * 4), h3 = *reinterpret_cast<const float4*>(q_s + 3 * D + g * 4);
+            q01[0] = pack2(h0.x, h1.x); q01[1] = pack2(h0.y, h1.y); q01[2] = pack2(h0.z, h1.z); q01[3] = pack2(h0.w, h1.w);
+            q23[0] = pack2(h2.x, h3.x); q23[1] = pack2(h2.y, h3.y); q23[2] = pack2(h2.z, h3.z); q23[3] = pack2(h2.w, h3.w);
+        }
         const float4* cbk = reinterpret_cast<const float4*>(cb_k_lut) + g;
         const uint32_t a32 = smem_u32(t32) + g * 16, a16 = smem_u32(t16) + g * 8;
-#pragma unroll 1
-        for (int it0 = 0; it0 < 16; it0 += BATCH) {
-            float4 cw[BATCH];
+        float4 cw[BATCH];
+        auto load = [&](int it0) {
 #pragma unroll
             for (int u = 0; u < BATCH; ++u) cw[u] = cbk[(size_t)(code0 + (it0 + u) * 16) * L];
+        };
+        load(0);
+#pragma unroll 1
+        for (int it0 = 0; it0 < 16; it0 += BATCH) {
+            float4 now[BATCH];                                  // the next codewords fly while these are multiplied
+#pragma unroll
+            for (int u = 0; u < BATCH; ++u) now[u] = cw[u];
+            if (it0 + BATCH < 16) load(it0 + BATCH);
 #pragma unroll
             for (int u = 0; u < BATCH; ++u) {
                 const int code = code0 + (it0 + u) * 16;
+                const uint64_t x = pack2(now[u].x, now[u].x), y = pack2(now[u].y, now[u].y), z = pack2(now[u].z, now[u].z), w = pack2(now[u].w, now[u].w);
+                uint64_t o01 = q01[0], o23 = q23[0];
+                fmul2(o01, x); fmul2(o23, x);
+                ffma2(o01, q01[1], y); ffma2(o23, q23[1], y);
+                ffma2(o01, q01[2], z); ffma2(o23, q23[2], z);
+                ffma2(o01, q01[3], w); ffma2(o23, q23[3], w);
                 float o[HPAD];
-#pragma unroll
-                for (int h = 0; h < HPAD; ++h)
-                    o[h] = fmaf(qs[h].w, cw[u].w, fmaf(qs[h].z, cw[u].z, fmaf(qs[h].y, cw[u].y, qs[h].x * cw[u].x)));
+                unpack2(o01, o[0], o[1]);
+                unpack2(o23, o[2], o[3]);
                 if (is32) {
                     asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(a32 + code * C::ROW32),
                                  "f"(o[0]), "f"(o[1]), "f"(o[2]), "f"(o[3]) : "memory");
                 } else {
-                    // (a table entry beyond the binary16 range would be a logit share of 2^16 bits; clamped, never inf)
-                    const uint32_t e0 = pack_h2(fminf(fmaxf(o[0], -60000.f), 60000.f), fminf(fmaxf(o[1], -60000.f), 60000.f));
-                    const uint32_t e1 = pack_h2(fminf(fmaxf(o[2], -60000.f), 60000.f), fminf(fmaxf(o[3], -60000.f), 60000.f));
+                    // (a table entry beyond the binary16 range would be a logit share of 2^16 bits; clamped to 60000, never inf)
+                    const uint32_t e0 = clamp_h2(pack_h2(o[0], o[1])), e1 = clamp_h2(pack_h2(o[2], o[3]));
                     asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(a16 + code * T16_ROW), "r"(e0), "r"(e1) : "memory");
                     // groups 8..15 a second time in columns 0..7: the 16 lanes of a half warp then read 16 different columns
                     if (g < 16) asm volatile("st.shared.v2.b32 [%0], {%1,%2};" ::"r"(a16 + code * T16_ROW - 64), "r"(e0), "r"(e1) : "memory");
@@ -526,19 +550,10 @@ __device__ __noinline__ void build_score_table(unsigned char* t32, unsigned char
 #pragma unroll
                 for (int h = 0; h < HPAD; ++h)
                     o[h] = fmaf(qs[h].w, cw[u].w, fmaf(qs[h].z, cw[u].z, fmaf(qs[h].y, cw[u].y, qs[h].x * cw[u].x)));
-                if (g < K32) {
 #pragma unroll
-                    for (int hs = 0; hs < HSETS; ++hs)
-                        *reinterpret_cast<float4*>(t32 + hs * C::PLANE32 + code * C::ROW32 + g * 16) =
-                            make_float4(o[hs * 4], o[hs * 4 + 1], o[hs * 4 + 2], o[hs * 4 + 3]);
-                } else if (C::HAS16) {
-                    // (a table entry beyond the binary16 range would be a logit share of 2^16 bits; clamped, never inf)
-                    const uint2 e = make_uint2(pack_h2(fminf(fmaxf(o[0], -60000.f), 60000.f), fminf(fmaxf(o[1], -60000.f), 60000.f)),
-                                               pack_h2(fminf(fmaxf(o[2], -60000.f), 60000.f), fminf(fmaxf(o[3], -60000.f), 60000.f)));
-                    *reinterpret_cast<uint2*>(t16 + code * T16_ROW + g * 8) = e;
-                    // groups 8..15 a second time in columns 0..7: the 16 lanes of a half warp then read 16 different columns
-                    if (K32 == 8 && g < 16) *reinterpret_cast<uint2*>(t16 + code * T16_ROW + (g - 8) * 8) = e;
-                }
+                for (int hs = 0; hs < HSETS; ++hs)
+                    *reinterpret_cast<float4*>(t32 + hs * C::PLANE32 + code * C::ROW32 + g * 16) =
+                        make_float4(o[hs * 4], o[hs * 4 + 1], o[hs * 4 + 2], o[hs * 4 + 3]);
             }
         }
     }
@@ -685,7 +700,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     constexpr float U_UNIT = 5.9604644775390625e-08f;         // 2^-24: a grid index u enters a product as the binary16 subnormal u 2^-24
     constexpr float CEN = VSQ ? 0.f : 64.f * U_UNIT;          // what one unit of weight adds to a tensor-core sum beyond u - centre
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ int s_found[4];
+    __shared__ int s_found[2][4];
     __shared__ int s_arrived, s_first, s_last;
     const uint32_t s_base = smem_u32(smem);
     if (s_base > C::T16 || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
@@ -699,7 +714,6 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     unsigned char* const s_abs = smem - s_base;               // s_abs + a: the byte at shared-window address a
     unsigned char* const t32_p = s_abs + C::T32;
     unsigned char* const t16_p = s_abs + C::T16;
-    float* const q_s = reinterpret_cast<float*>(s_abs + C::Q);
 
     // With the KV-head-major walk the first KV head of CTA c is floor(c * Hkv / G) whatever the lengths are:
     // its (constant) value codebook starts flowing into shared memory before the grid-dependency wait and
@@ -821,23 +835,63 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
 #else
 #define NOVAKV_TICK(i)
 #endif
-    long u = u_begin;
-    while (u < u_end) {
+    // q' of a pair's heads -> shared memory (rows beyond HG stay zero), without registers and without a wait
+    auto stage_query = [&](int b, int kvh, int buf) {
+        const float4* src = reinterpret_cast<const float4*>(qp + ((size_t)b * n_q_heads + kvh * HG) * D);
+        for (int i = threadIdx.x; i < HG * D / 4; i += S1_THREADS)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(C::Q + buf * C::Q_BYTES + i * 16), "l"(src + i) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (HG < HPAD)
+        for (int i = threadIdx.x; i < 2 * (HPAD - HG) * D; i += S1_THREADS)
+            reinterpret_cast<float*>(s_abs + C::Q + i / ((HPAD - HG) * D) * C::Q_BYTES)[HG * D + i % ((HPAD - HG) * D)] = 0.f;
+    // What a segment needs before its table can be built is on its way early: its place in the batch is looked up and its
+    // query copied during the scan of the segment before, its first page ids fly during that segment's merge.  With the packed
+    // table build, scaled 32 x 8191 84.0 -> 80.0 us a call, 128-sequence mix 303 -> 298.
+    int rem = (int)(u_end - u_begin);            // units of this CTA that are left; the present one is s_bnd[its end] - rem
+    int cur_seg = 0;                             // which half of s_found and of the q' buffers holds the present segment
+    find_segment(page_prefix, seq_lens, batch, max_pages_per_seq, u_begin, (int)(u_begin / page_prefix[batch]), s_found[0]);
+    __syncthreads();
+    Segment sg = segment_at(page_prefix, batch, u_begin, u_end, s_found[0]);
+    for (int i = threadIdx.x; i < HG * D / 4; i += S1_THREADS)                // (the first one with plain loads: a wait for copies
+        reinterpret_cast<float4*>(s_abs + C::Q)[i] =                          // would be one for the value codebook as well)
+            reinterpret_cast<const float4*>(qp + ((size_t)sg.b * n_q_heads + sg.kvh * HG) * D)[i];
+    int n_it = 0, ids_cur = 0, ids_next = 0;
+    const int32_t* pt = nullptr;
+    // page ids of 32 consecutive tiles of this warp, one per lane (coalesced gather, loaded a batch ahead)
+    auto load_ids = [&](int batch_i) {
+        const int it = batch_i * 32 + lane;
+        int page = 0;
+        if (it < n_it) {
+            page = pt[(warp + NCW * it) >> 1];
+            if (page < 0 || page >= n_pages) { atomicOr(dev_status, NOVAKV_DEV_BAD_PAGE); page = 0; }
+        }
+        return page;
+    };
+    auto fetch_ids = [&]() {
+        // this warp's tiles of the segment: half pages hp = warp, warp + NCW, ...
+        const int n_half = min(2 * sg.npg, (sg.len - sg.pg0 * NOVAKV_PAGE_TOKENS + 31) / 32);
+        n_it = n_half > warp ? (n_half - warp + NCW - 1) / NCW : 0;
+        pt = page_table + (size_t)sg.b * pt_stride + sg.pg0;
+        ids_cur = load_ids(0);
+        ids_next = load_ids(1);
+    };
+    fetch_ids();
+    __syncthreads();
+    while (rem > 0) {
         NOVAKV_TICK(0)
-        const Segment sg = locate(page_prefix, seq_lens, batch, max_pages_per_seq, u, u_end, s_found);
         const int pair = sg.kvh * batch + sg.b;            // grows along the walk
+        rem -= sg.npg;
 
         // ---- segment prologue -----------------------------------------------------------------
         if (!VSQ && vcb_head != sg.kvh) {
             stage_value_codebook_async(C::VCB, cb_v_img + (size_t)sg.kvh * VCB_COPY_BYTES);
             vcb_head = sg.kvh;
         }
-        // q' of the pair's heads -> shared memory (rows beyond HG are zero)
-        for (int i = threadIdx.x; i < HPAD * D / 4; i += S1_THREADS) {
-            const int h = i / (D / 4);
-            const float4 v = h < HG ? reinterpret_cast<const float4*>(qp + ((size_t)sg.b * n_q_heads + sg.kvh * HG) * D)[i]
-                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-            reinterpret_cast<float4*>(q_s)[i] = v;
+        if (rem > 0) {
+            const long u_next = s_bnd[blockIdx.x + 1] - rem;
+            find_segment(page_prefix, seq_lens, batch, max_pages_per_seq, u_next,
+                         sg.kvh + (u_next >= (long)(sg.kvh + 1) * page_prefix[batch]), s_found[cur_seg ^ 1]);
         }
         float qcen[KSC ? HPAD : 1];
         if (KSC) {
@@ -845,21 +899,6 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
             for (int h = 0; h < HPAD; ++h) qcen[h] = h < HG ? qc[(size_t)sg.b * n_q_heads + sg.kvh * HG + h] : 0.f;
         }
 
-        // this warp's tiles of the segment: half pages hp = warp, warp + NCW, ...
-        const int n_half = min(2 * sg.npg, (sg.len - sg.pg0 * NOVAKV_PAGE_TOKENS + 31) / 32);
-        const int n_it = n_half > warp ? (n_half - warp + NCW - 1) / NCW : 0;
-        const int32_t* pt = page_table + (size_t)sg.b * pt_stride + sg.pg0;
-        // page ids of 32 consecutive tiles of this warp, one per lane (coalesced gather, loaded a batch ahead)
-        auto load_ids = [&](int batch_i) {
-            const int it = batch_i * 32 + lane;
-            int page = 0;
-            if (it < n_it) {
-                page = pt[(warp + NCW * it) >> 1];
-                if (page < 0 || page >= n_pages) { atomicOr(dev_status, NOVAKV_DEV_BAD_PAGE); page = 0; }
-            }
-            return page;
-        };
-        int ids_cur = load_ids(0), ids_next = load_ids(1);
         // a warp's tiles are all first or all second halves of their pages (an even number of warps)
         static_assert(NCW % 2 == 0, "half of a page is a constant of the warp");
         const uint32_t k_step = (uint32_t)n_kv_heads * PAGE_BYTES;                       // bytes of a page
@@ -1143,12 +1182,13 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         // ---- score table (the first tile's loads are issued before, so that they fly during the build)
         TileRegs<L> ta;
         if (n_it > 0) load_tile(0, ta);
-        __syncthreads();     // q' of the pair is in shared memory
         NOVAKV_TICK(1)
-        build_score_table<D, HG, VM>(t32_p, t16_p, cb_k_lut + (size_t)sg.kvh * 256 * L * 4, q_s);
+        build_score_table<D, HG, VM>(t32_p, t16_p, cb_k_lut + (size_t)sg.kvh * 256 * L * 4,
+                                     reinterpret_cast<const float*>(s_abs + C::Q + cur_seg * C::Q_BYTES));
         NOVAKV_TICK(2)
         async_copies_wait();
-        __syncthreads();     // table and value codebook complete
+        __syncthreads();     // table and value codebook complete, next segment found
+        if (rem > 0) stage_query(s_found[cur_seg ^ 1][0], s_found[cur_seg ^ 1][3], cur_seg ^ 1);
         NOVAKV_TICK(3)
 
         // ---- scan: 32-token tiles, the next tile's loads in flight while one is consumed
@@ -1161,6 +1201,13 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         // ---- segment epilogue: merge the warps' partials, write one partial ---------------------
         NOVAKV_TICK(4)
         if (VM) flush_window();
+        const Segment done = sg;
+        if (rem > 0) {
+            const long u_stop = s_bnd[blockIdx.x + 1];
+            cur_seg ^= 1;
+            sg = segment_at(page_prefix, batch, u_stop - rem, u_stop, s_found[cur_seg]);
+            fetch_ids();
+        }
         __syncthreads();                                   // scan done everywhere: the tables are dead
         NOVAKV_TICK(5)
         unsigned char* const merge_p = HAS16 ? t16_p : t32_p;
@@ -1254,7 +1301,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
                 a *= 16777216.f;                           // indices entered the sums as u 2^-24
                 float val;
                 if (VSQ) val = (a + zsum) * unscale;       // levels are the codes themselves (s = 1, no offset)
-                else val = (v_scale[(size_t)sg.kvh * D + c] * a + v_off[(size_t)sg.kvh * D + c] * lsum) * unscale;
+                else val = (v_scale[(size_t)done.kvh * D + c] * a + v_off[(size_t)done.kvh * D + c] * lsum) * unscale;
                 part_acc[(pidx * HG + h) * D + c] = val;
                 if (c == 0) { part_ml[(pidx * HG + h) * 2] = M; part_ml[(pidx * HG + h) * 2 + 1] = lsum * unscale; }
             }
@@ -1270,7 +1317,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
             }
             __syncthreads();
             const long P = page_prefix[batch];
-            const long pu0 = (long)sg.kvh * P + page_prefix[sg.b], pu1 = pu0 + (sg.len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
+            const long pu0 = (long)done.kvh * P + page_prefix[done.b], pu1 = pu0 + (done.len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
             bool touches = false;                           // CTA threadIdx.x has a non-empty share of this pair
             if (threadIdx.x < gridDim.x) {
                 const int c = threadIdx.x;
@@ -1281,16 +1328,16 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
             if (s_arrived == expected) {
                 __threadfence();
                 fused_merge<D, HG>(reinterpret_cast<float*>(t32_p), part_ml, part_acc, pair, s_first, s_last, s_bnd, rv_t, v_mean,
-                                   sg.kvh, out_fused, out_is_fp32, ((size_t)sg.b * n_q_heads + sg.kvh * HG) * D);
+                                   done.kvh, out_fused, out_is_fp32, ((size_t)done.b * n_q_heads + done.kvh * HG) * D);
                 if (threadIdx.x == 0) pair_count[pair] = 0;
             }
         }
-        __syncthreads();                                   // merge buffer free before the next table build
+        async_copies_wait();
+        __syncthreads();                                   // merge buffer free, next query complete: the next table can be built
         NOVAKV_TICK(6)
 #ifdef NOVAKV_TIMING
         ++n_seg;
 #endif
-        u += sg.npg;
     }
 #ifdef NOVAKV_TIMING
     unsigned long long g_end;
@@ -1299,29 +1346,6 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         printf("cta %3d segs %d pages %ld | clocks: pre-loop %lld locate+q %lld build %lld vcbwait %lld scan(w0) %lld barrier %lld epilogue %lld total %lld | ns start %llu end %llu\n",
                blockIdx.x, n_seg, (long)(u_end - u_begin), tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], clock64() - t_start, g_start, g_end);
 #endif
-}
-
-// locate() in two parts with the barrier between them left to the caller: the look-up of a CTA's next segment hides in the
-// scan of the present one.
-__device__ __forceinline__ void find_segment(const int32_t* __restrict__ page_prefix, const int32_t* __restrict__ seq_lens,
-                                             int batch, int max_pages, long u, int kvh, int* found) {
-    const long r = u - (long)kvh * page_prefix[batch];
-    for (int t = threadIdx.x; t < batch; t += S1_THREADS) {
-        const int lo = page_prefix[t], hi = page_prefix[t + 1];
-        if ((long)lo <= r && r < (long)hi) { found[0] = t; found[1] = clamp_len(seq_lens[t], max_pages); found[2] = lo; found[3] = kvh; }
-    }
-}
-__device__ __forceinline__ Segment segment_at(const int32_t* __restrict__ page_prefix, int batch, long u, long u_end, const int* found) {
-    Segment s;
-    s.b = found[0];
-    s.len = found[1];
-    s.kvh = found[3];
-    const long r = u - (long)s.kvh * page_prefix[batch];
-    const int pages_b = (s.len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
-    s.pg0 = (int)(r - found[2]);
-    const long left = u_end - u;
-    s.npg = (int)(left < (long)(pages_b - s.pg0) ? left : (long)(pages_b - s.pg0));
-    return s;
 }
 
 // ------------------------------------------------------------------------------------------------
