@@ -21,9 +21,14 @@ namespace {
 
 constexpr int ENC_THREADS = 512;
 constexpr int ENC_TILE = 64;   // tokens per tile (search granularity)
-#ifndef NOVAKV_SMALL_APPEND_TOKENS
-#define NOVAKV_SMALL_APPEND_TOKENS 256   // batches up to this size take the per-group append kernel
-#endif
+// Batches up to this size take the per-group append kernel, larger ones the prompt encoder.  The append kernel's time grows with
+// every pass of 8 tokens a chunk, the encoder's is one unit per SM up to 256 tokens.  us, tables in the L2 / cold:
+//   d = 128 plain      64: 17.9 / 16.8 here, 18.1 / 21.5 there   96: 25.2 / 23.1, 19.2 / 23.4   256: 55 / 55, 23 / 30
+//           scaled     64: 21.5 / 21.2, 25.6 / 29.0              96: 30.3 / 29.4, 25.3 / 29.9   256: 66 / 67, 32 / 39
+//           deployed   64: 25.4 / 24.1, 25.4 / 28.5              96: 35.9 / 33.9, 25.2 / 28.5   256: 78 / 76, 32 / 37
+//   d = 64  plain     128: 14.6 / 14.0, 17.0 / 18.6             192: 20.2 / 19.3, 18.0 / 20.3   256: 21.2 / 22.8, 19.2 / 22.3
+//           scaled    128: 17.5 / 16.9, 22.0 / 24.7             192: 24.4 / 23.5, 21.7 / 24.4   256: 26.5 / 27.8, 22.6 / 26.0
+constexpr int small_append_tokens(int d) { return d == 128 ? 64 : 192; }
 
 // Shared-memory plan of the search-only kernel: codebook, one tile of coefficients, its indices.
 template <int D>
@@ -593,7 +598,7 @@ novakv_status launch_encode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     // (the append kernel reads the new rows in 16-byte pieces; rows on a 4-byte boundary take the prompt encoder, which can
     // copy them in words, whatever their number)
     const bool rows16 = (((uintptr_t)k_new | (uintptr_t)v_new) & 15) == 0;
-    if (n_tokens <= NOVAKV_SMALL_APPEND_TOKENS && rows16) {
+    if (n_tokens <= small_append_tokens(D) && rows16) {
         int tp_log2 = 0;
         while ((1 << tp_log2) < n_tokens && tp_log2 < SMALL_TP_LOG2) ++tp_log2;
         // chunks of the token list: as many as there are passes, while all CTAs are resident together, and no more than the
