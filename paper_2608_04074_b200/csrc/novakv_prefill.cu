@@ -350,6 +350,7 @@ __global__ void __launch_bounds__(PF_THREADS, 1) novakv_prefill_kernel(const __g
         if (threadIdx.x == 0) atomicOr(a.dev_status, NOVAKV_DEV_SMEM_LAYOUT);
         return;
     }
+    novakv_grid_dependency_wait();      // (the launch overlaps the preceding kernel's tail, and the next kernel's launch this one's)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int* const misc = reinterpret_cast<volatile int*>(smem + P::OFF_MISC);
     volatile int* const abort_flag = misc + 1;
@@ -1136,7 +1137,7 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
             row_map(&a.map_k, a.k_new, a.n_tokens, hkv * D) && row_map(&a.map_v, a.v_new, a.n_tokens, hkv * D);
     a.words = (((uintptr_t)a.k_pages | (uintptr_t)a.v_pages) & 3) == 0;
     novakv_prof_scope ps(ctx, 1, stream);
-    kern<<<grid, PF_THREADS, P::BYTES, stream>>>(a);
+    novakv_launch_pdl(kern, dim3(grid), dim3(PF_THREADS), P::BYTES, stream, a);
     ps.end();
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
