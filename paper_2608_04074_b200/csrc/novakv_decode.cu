@@ -105,8 +105,8 @@ struct S1 {
     static constexpr int Q_BYTES = HPAD * D * 4;
     static constexpr int Q = P + P_BYTES;                               // fp32 [HPAD][D], of the present and of the next pair
     static constexpr int BND = Q + 2 * Q_BYTES;                        // long [MAX_SCAN_CTAS + 1]: first unit of every CTA
-    static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;           // int [2][PFX_CAP + 1]: page and cost prefix of small batches
-    static constexpr int SMEM = PFX + 2 * (PFX_CAP + 1) * 4;
+    static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;           // int [3][PFX_CAP + 1]: page and cost prefix and lengths of small batches
+    static constexpr int SMEM = PFX + 3 * (PFX_CAP + 1) * 4;
     // merge buffer (aliases the larger table once a segment's scan is done)
     static constexpr int MROW = D + 4;                                  // floats per (warp, head) row of the merge buffer: 16 bytes of padding
                                                                         // keep the four head rows a warp writes at once on different banks
@@ -146,7 +146,7 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
                       const float* __restrict__ k_center /* [Hkv][D], transform domain */, float* __restrict__ qc /* [batch][Hq] or null */,
                       int32_t* __restrict__ pair_count /* [Hkv * batch] arrival counters of the fused merge, or null */,
                       void* __restrict__ out_fused /* outputs, when the scan kernel itself merges */, int out_is_fp32,
-                      int seqs_per_block) {
+                      int seqs_per_block, int form_prefix /* 0: the scan kernel forms the prefixes */) {
     const int blk = blockIdx.x;
 #ifdef NOVAKV_TIMING
     unsigned long long g_p0, g_p1;
@@ -167,6 +167,12 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
         for (int r = 0; r < ROWS; ++r) rv[r] = R[(size_t)r * D];
     }
     if (blk == (int)gridDim.x - 1) {
+        if (!form_prefix) {
+            // this grid must not complete before the preceding kernel has (the scan waits for this grid alone)
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            return;
+        }
         novakv_grid_dependency_wait();
         // exclusive prefix over sequences of their page counts; small, done by one warp.  Beside it the same
         // prefix in "cost" units, in which every non-empty sequence weighs seg_weight pages more: the scan
@@ -387,6 +393,51 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1,
 struct Segment {
     int b, kvh, pg0, npg, len;
 };
+
+// Page and cost prefixes of a batch of at most PFX_CAP sequences, and its lengths, in shared memory (pfx: [3][PFX_CAP + 1]), by
+// all threads of a scan CTA; CTA 0 also writes the prefixes for the merge kernel and reports lengths out of range.  Every
+// CTA does it by itself: a block of the kernel in front would have to wait for the append first, and the scan for that block
+// (1 x 777 step 17.6 -> 17.4 us a call, 5 x 100 of the d = 64 shape 16.7 -> 16.4, deployed band 64 x 32768 411 -> 405).
+static_assert(PFX_CAP < S1_THREADS, "a thread for every sequence");
+__device__ __forceinline__ void form_prefixes(int32_t* pfx, int (*s_part)[NCW], const int32_t* __restrict__ seq_lens, int batch, int max_pages,
+                                              int seg_weight, int32_t* __restrict__ page_prefix, int32_t* __restrict__ cost_prefix,
+                                              uint32_t* dev_status) {
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    int len = 0, pages = 0;
+    if (t < batch) {
+        const int raw = seq_lens[t];
+        len = clamp_len(raw, max_pages);
+        if (raw != len && blockIdx.x == 0) atomicOr(dev_status, NOVAKV_DEV_BAD_LENGTH);
+        pages = (len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
+    }
+    int incl = pages, incl_ne = pages > 0;
+    if (warp * 32 < batch) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(0xffffffffu, incl, o), b = __shfl_up_sync(0xffffffffu, incl_ne, o);
+            if (lane >= o) { incl += a; incl_ne += b; }
+        }
+    }
+    if (batch > 32) {
+        if (lane == 31) { s_part[0][warp] = incl; s_part[1][warp] = incl_ne; }
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) { incl += s_part[0][w]; incl_ne += s_part[1][w]; }
+    }
+    if (t < batch) {
+        const int p0 = incl - pages, c0 = p0 + seg_weight * (incl_ne - (pages > 0));
+        pfx[t] = p0;
+        pfx[PFX_CAP + 1 + t] = c0;
+        pfx[2 * (PFX_CAP + 1) + t] = len;
+        if (blockIdx.x == 0) { page_prefix[t] = p0; cost_prefix[t] = c0; }
+        if (t == batch - 1) {
+            const int c1 = incl + seg_weight * incl_ne;
+            pfx[batch] = incl;
+            pfx[PFX_CAP + 1 + batch] = c1;
+            if (blockIdx.x == 0) { page_prefix[batch] = incl; cost_prefix[batch] = c1; }
+        }
+    }
+    __syncthreads();
+}
 
 // Locate the (KV head, sequence, page) of global page unit u.  Units are ordered KV-head-major:
 // u = kvh * P + page_prefix[b] + page, with P = page_prefix[batch] the pages of all sequences, so that
@@ -680,13 +731,13 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
                             const uint8_t* __restrict__ v_pages, const __nv_bfloat16* __restrict__ k_scales,
                             const __nv_bfloat16* __restrict__ v_meta, int n_pages,
                             const int32_t* __restrict__ page_table, int max_pages_per_seq,
-                            const int32_t* __restrict__ seq_lens, const int32_t* __restrict__ page_prefix,
+                            const int32_t* __restrict__ seq_lens, int32_t* __restrict__ page_prefix_g,
                             int batch, int n_q_heads, int n_kv_heads, float* __restrict__ part_ml,
                             float* __restrict__ part_acc, uint32_t* __restrict__ dev_status, int pt_stride,
-                            const int32_t* __restrict__ cost_prefix, int seg_weight, long* __restrict__ cta_range,
+                            int32_t* __restrict__ cost_prefix_g, int seg_weight, long* __restrict__ cta_range,
                             const float* __restrict__ qc,
                             int32_t* __restrict__ pair_count, const float* __restrict__ rv_t,
-                            const float* __restrict__ v_mean, void* __restrict__ out_fused, int out_is_fp32) {
+                            const float* __restrict__ v_mean, void* __restrict__ out_fused, int out_is_fp32, int form_prefix) {
     // out_fused != null: the CTA that writes the last partial of a (sequence, KV head) pair also merges the pair's
     // partials and applies the inverse value transform (no merge kernel follows); pair_count holds one arrival
     // counter per pair, zero on entry and reset to zero by the merging CTA.  Nothing waits on another CTA.
@@ -700,7 +751,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     constexpr float U_UNIT = 5.9604644775390625e-08f;         // 2^-24: a grid index u enters a product as the binary16 subnormal u 2^-24
     constexpr float CEN = VSQ ? 0.f : 64.f * U_UNIT;          // what one unit of weight adds to a tensor-core sum beyond u - centre
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ int s_found[2][4];
+    __shared__ int s_found[2][4], s_part[2][NCW];
     __shared__ int s_arrived, s_first, s_last;
     const uint32_t s_base = smem_u32(smem);
     if (s_base > C::T16 || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
@@ -726,13 +777,14 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     else novakv_grid_dependency_wait();
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // The two prefixes are read many times (boundaries, segment look-ups): small batches keep them in shared memory.
-    if (batch <= PFX_CAP) {
+    // The two prefixes are read many times (boundaries, segment look-ups): small batches form them in shared memory.
+    const int32_t *page_prefix = page_prefix_g, *cost_prefix = cost_prefix_g;
+    if (form_prefix) {                                        // (batches of at most PFX_CAP sequences)
         int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
-        for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix[i]; pfx[PFX_CAP + 1 + i] = cost_prefix[i]; }
-        __syncthreads();
+        form_prefixes(pfx, s_part, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         page_prefix = pfx;
         cost_prefix = pfx + PFX_CAP + 1;
+
     }
     // First unit of every CTA (see scan_boundary): one thread per boundary.  This CTA owns [s_bnd[c], s_bnd[c + 1]).
     long* const s_bnd = reinterpret_cast<long*>(s_abs + C::BND);
@@ -1390,7 +1442,7 @@ struct S1M {
     static constexpr int ML = MACC + NCW * MHEADS * MROW * 4;
     static constexpr int BND = ML + NCW * HG * 8;
     static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;
-    static constexpr int SMEM = PFX + 2 * (PFX_CAP + 1) * 4;
+    static constexpr int SMEM = PFX + 3 * (PFX_CAP + 1) * 4;
     static_assert(SMEM <= S1_SMEM_BYTES, "shared memory budget");
 };
 __global__ void __launch_bounds__(S1_THREADS, 1)
@@ -1398,16 +1450,16 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
                          const float* __restrict__ k_mma_scale /* [Hkv][64] */, const uint8_t* __restrict__ cb_v_img,
                          const float* __restrict__ v_scale, const float* __restrict__ v_off, const uint8_t* __restrict__ k_pages,
                          const uint8_t* __restrict__ v_pages, int n_pages, const int32_t* __restrict__ page_table,
-                         int max_pages_per_seq, const int32_t* __restrict__ seq_lens, const int32_t* __restrict__ page_prefix,
+                         int max_pages_per_seq, const int32_t* __restrict__ seq_lens, int32_t* __restrict__ page_prefix_g,
                          int batch, int n_q_heads, int n_kv_heads, float* __restrict__ part_ml, float* __restrict__ part_acc,
-                         uint32_t* __restrict__ dev_status, int pt_stride, const int32_t* __restrict__ cost_prefix,
-                         int seg_weight, long* __restrict__ cta_range) {
+                         uint32_t* __restrict__ dev_status, int pt_stride, int32_t* __restrict__ cost_prefix_g,
+                         int seg_weight, long* __restrict__ cta_range, int form_prefix) {
     using C = S1M;
     constexpr int D = C::D, HG = C::HG, L = C::L;
     constexpr float SH = 15.f;                                // weights are scaled by 2^SH before the binary16 rounding
     constexpr float LOST = 1.0e-7f;                           // share of a logit that four truncated accumulations lose on average
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ int s_found[2][4];
+    __shared__ int s_found[2][4], s_part[2][NCW];
     const uint32_t s_base = smem_u32(smem);
     if (s_base > C::KEY || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
         // cannot happen with the shared address window of this architecture; reported, never trapped
@@ -1442,12 +1494,13 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
     novakv_grid_dependency_wait();
 
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-    if (batch <= PFX_CAP) {
+    const int32_t *page_prefix = page_prefix_g, *cost_prefix = cost_prefix_g;
+    if (form_prefix) {                                        // (batches of at most PFX_CAP sequences)
         int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
-        for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix[i]; pfx[PFX_CAP + 1 + i] = cost_prefix[i]; }
-        __syncthreads();
+        form_prefixes(pfx, s_part, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         page_prefix = pfx;
         cost_prefix = pfx + PFX_CAP + 1;
+
     }
     long* const s_bnd = reinterpret_cast<long*>(s_abs + C::BND);
     for (int c = threadIdx.x; c <= (int)gridDim.x; c += S1_THREADS)
@@ -2241,13 +2294,15 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     // kernel follows.
     const bool fuse = sink_logits == nullptr && band == nullptr && ctx->fused_merge;
 
+    // (with the merge fused in, the outputs of empty sequences are written where the prefixes are formed)
+    const int scan_prefix = batch <= PFX_CAP && !fuse;
     // sequences per prepare block: one while all pairs fit on the machine twice over, then enough to make that so
     const int seqs_per_block = max(1, min(8, (batch * hkv + 2 * ctx->n_sm - 1) / (2 * ctx->n_sm)));
     auto prepare = seqs_per_block > 1 ? novakv_prepare_kernel<D, HG, true> : novakv_prepare_kernel<D, HG, false>;
     novakv_launch_pdl(prepare, dim3((batch + seqs_per_block - 1) / seqs_per_block * hkv + 1), dim3(512), 0, stream, q, ly.rk_inv_t, seq_lens,
                       batch, hq, hkv, max_pages_per_seq, sm_scale * 1.4426950408889634f, qp, prefix, ctx->dev_status,
                       k_off_vec, qk_off, cost_prefix, ctx->seg_weight, (const float*)ly.k_center, qc,
-                      fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32, seqs_per_block);
+                      fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32, seqs_per_block, scan_prefix ? 0 : 1);
     ctx->launches++;
 
     // (before the scan: its blocks run beside the encoder of a step's append, on the SMs that leaves free)
@@ -2275,7 +2330,7 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
         novakv_launch_pdl(novakv_decode_mma_kernel, dim3(grid), dim3(S1_THREADS), S1_SMEM_BYTES, stream, qp, (const uint4*)ly.cb_k_mma,
                           (const float*)ly.k_mma_scale, (const uint8_t*)ly.cb_v_u8, (const float*)ly.v_scale, (const float*)ly.v_off,
                           k_pages, v_pages, n_pages, page_table, max_pages_per_seq, seq_lens, prefix, batch, hq, hkv, part_ml, part_acc,
-                          ctx->dev_status, pt_stride, (const int32_t*)cost_prefix, ctx->seg_weight, cta_range);
+                          ctx->dev_status, pt_stride, cost_prefix, ctx->seg_weight, cta_range, scan_prefix);
         ps.end();
         ctx->launches++;
     } else {
@@ -2292,9 +2347,9 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
                               (const uint8_t*)ly.cb_v_u8, (const float*)ly.v_scale,
                               (const float*)ly.v_off, k_pages, v_pages, k_scales, v_meta, n_pages, page_table, max_pages_per_seq,
                               seq_lens, prefix, batch, hq, hkv, part_ml, part_acc, ctx->dev_status, pt_stride,
-                              (const int32_t*)cost_prefix, ctx->seg_weight, cta_range, (const float*)qc,
+                              cost_prefix, ctx->seg_weight, cta_range, (const float*)qc,
                               pair_count, (const float*)ly.rv_t, (const float*)ly.v_mean,
-                              fuse ? out : (void*)nullptr, out_is_fp32);
+                              fuse ? out : (void*)nullptr, out_is_fp32, scan_prefix);
             ps.end();
             ctx->launches++;
         }
