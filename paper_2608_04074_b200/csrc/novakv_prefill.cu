@@ -1137,7 +1137,10 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
             row_map(&a.map_k, a.k_new, a.n_tokens, hkv * D) && row_map(&a.map_v, a.v_new, a.n_tokens, hkv * D);
     a.words = (((uintptr_t)a.k_pages | (uintptr_t)a.v_pages) & 3) == 0;
     novakv_prof_scope ps(ctx, 1, stream);
-    novakv_launch_pdl(kern, dim3(grid), dim3(PF_THREADS), P::BYTES, stream, a);
+    // A short call's launch overlaps the kernel in front.  Not a long one's: its CTAs would land on SMs in the order in which
+    // the kernel in front leaves them (32768 tokens, calls in a row: 490 us so, 501 overlapped).
+    if (a.cost_k == 1) novakv_launch_pdl(kern, dim3(grid), dim3(PF_THREADS), P::BYTES, stream, a);
+    else kern<<<grid, PF_THREADS, P::BYTES, stream>>>(a);
     ps.end();
     ctx->launches++;
     return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
