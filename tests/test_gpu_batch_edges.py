@@ -82,3 +82,31 @@ def test_append_or_prompt(cases, name, fmt, n):
             check_indices(vidx, mine, "v")
         if fmt != "plain":
             assert np.array_equal(cache.load_scales(s, 0, len(kidx)), mine["kscale"].astype(np.float32))
+
+
+@pytest.mark.parametrize("sink", [False, True])
+@pytest.mark.parametrize("beyond", [0, 1])
+def test_merge_in_halves(cases, beyond, sink):
+    """More sequences than four for every SM's block of the merge kernel: two blocks an SM, each with half of the run."""
+    from paper_2608_04074_b200.runtime import PagedCache
+    case = cases("qwen")
+    batch = 4 * (torch.cuda.get_device_properties(0).multi_processor_count // case.ctx.n_kv_heads) + beyond
+    lens = (31 * np.arange(batch) % 170).astype(np.int32)              # the first is empty
+    lens[-1] = 0
+    lens[2] = 2000                                                     # one with many pieces
+    cache = PagedCache(case.ctx, lens, seed=8)
+    k, v, _ = case.draw(710, 2000, 1)
+    e = case.oracle.encode(k.astype(np.float64), v.astype(np.float64), with_gaps=False)
+    part = [(e["kidx"][f:f + n], e["vidx"][f:f + n]) for f, n in ((13 * b % 1800 if n <= 170 else 0, n) for b, n in enumerate(lens))]
+    cache.store_logical_batch([(b, 0, *p) for b, p in enumerate(part) if lens[b]])
+    _, _, q = case.draw(711, 1, batch)
+    logits = np.linspace(-3.0, 3.0, case.ctx.n_q_heads).astype(np.float32)
+    out = cache.decode(0, torch.from_numpy(q).to(torch.bfloat16).cuda(),
+                       sink_logits=torch.from_numpy(logits).cuda() if sink else None).cpu().numpy()
+    assert case.ctx.novakv_last_device_status() == 0
+    for b, n in enumerate(lens):
+        if n == 0:
+            assert not out[b].any()
+            continue
+        args = (q[b].astype(np.float64), *part[b])
+        check_output(out[b], case.oracle.decode_sink(*args, logits.astype(np.float64)) if sink else case.oracle.decode(*args))
