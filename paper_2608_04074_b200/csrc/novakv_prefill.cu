@@ -60,13 +60,14 @@ constexpr int PF_CW_STAGES = 6;              // (the binary32 codewords are need
 static_assert(PF_OP_BYTES + PF_CW_BYTES == NOVAKV_PF_GROUP_BYTES, "codebook image");
 constexpr int PF_QUEUE = 16;                 // entries of a helper's queue
 constexpr int PF_QUEUE_LAST = 4;             // of which a segment's last tile fills so many (the CTA waits for what is queued at its end)
-// Durations the work split reckons with, microseconds per unit (measured: 19.3 for 16 groups of plain keys or values, about
-// 28 for scaled keys, which transform and norm the whole row, 11 for INT2 values).
-// Keys leave more to the helpers than values and take 7 % longer; the cut reckons with that where a CTA has enough units for
-// it to matter (32768 tokens, 28 units a CTA: 505 -> 490 us; 8191 of the d = 64 shape, 3.5 units: 73.4 -> 76).
+// Durations the work split reckons with, microseconds per unit: 18 to 19 for 16 groups of plain keys or values, about 26 for
+// scaled keys, which transform and norm the whole row, 12 to 25 for INT2 values, whose unsure tokens take the binary64 row
+// (32768 tokens, deployed / scaled: 464 / 634 us with 9 and 11 for the last two, 479 / 629 with 7 and 15, 462 / 617 so).
+// Plain keys at d = 128 leave more to the helpers than values and take 7 % longer; the cut reckons with that where a CTA has
+// enough units for it to matter (32768 tokens, 28 units a CTA: 505 -> 490 us).
 constexpr double PF_KEYS = 1.07;
 constexpr int PF_KEYS_UNITS = 8;
-constexpr double PF_US_UNIT = 3.0, PF_US_GROUP = 1.0, PF_US_SCALED = 9.0, PF_US_INT2 = 11.0;
+constexpr double PF_US_UNIT = 3.0, PF_US_GROUP = 1.0, PF_US_SCALED = 8.0, PF_US_INT2 = 13.0;
 // |coefficient - binary64 coefficient| <= KAPPA (|x| + |mean|) |R column|.  The accumulation order of the tensor core is
 // not specified; all-positive inputs (every truncation in the same direction) showed 2^-21.6, random signs 2^-23.3.
 constexpr float KAPPA = 1.4e-6f;             // > 2^-19.5
@@ -1128,7 +1129,7 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
             grid = g;
             a.gs = gs;
             // one unit per CTA where there are no more than SMs: a cut in cost would hand some a key and a value unit
-            a.cost_k = uk + uv <= ctx->n_sm ? 1 : (int)(ck * (uk + uv >= PF_KEYS_UNITS * g ? PF_KEYS : 1.0) * 64.0);
+            a.cost_k = uk + uv <= ctx->n_sm ? 1 : (int)(ck * (D == 128 && FMT == 0 && uk + uv >= PF_KEYS_UNITS * g ? PF_KEYS : 1.0) * 64.0);
             a.cost_v = uk + uv <= ctx->n_sm ? 1 : (int)(cv * 64.0);
         }
     }
