@@ -12,7 +12,7 @@
 #include "novakv.h"
 
 /* How a C argument is formed from Python argument `arg` (the context handle comes first and is not listed):
- *   I int(x)   F float(x)   P data_ptr() of a tensor, 0 for None   0, 1 shape[0], shape[1]   n, m the same, 0 for None
+ *   L an integer   I int(x)   F float(x)   P data_ptr() of a tensor, 0 for None   0, 1 shape[0], shape[1]   n, m the same, 0 for None
  *   T 1 if its dtype is float32   B its size in bytes   S the current CUDA stream (no argument) */
 typedef struct { char kind; signed char arg; } param;
 #define MAX_ARGS 28
@@ -23,39 +23,39 @@ enum { ENCODE, ENCODE_SCALED, ENCODE_DEPLOYED, DECODE, DECODE_SCALED, DECODE_SIN
 static const struct { const char* name; int n_args; param p[MAX_ARGS]; } entries[N_ENTRIES] = {
     /* layer, k_new, v_new, tok_seq, tok_pos, k_pages, v_pages, page_table, seq_lens */
     [ENCODE] = {"novakv_encode_append", 9,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'0', 5}, {'P', 7}, {'1', 7}, {'0', 7}, {'P', 8}, {'S', 0}}},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'0', 5}, {'P', 7}, {'1', 7}, {'0', 7}, {'P', 8}, {'S', 0}}},
     /* ... k_pages, v_pages, k_scales, page_table, seq_lens */
     [ENCODE_SCALED] = {"novakv_encode_append_scaled", 10,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'P', 7}, {'0', 5}, {'P', 8}, {'1', 8}, {'0', 8}, {'P', 9}, {'S', 0}}},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'P', 7}, {'0', 5}, {'P', 8}, {'1', 8}, {'0', 8}, {'P', 9}, {'S', 0}}},
     /* ... k_pages, v_pages, k_scales, v_meta, page_table, seq_lens */
     [ENCODE_DEPLOYED] = {"novakv_encode_append_deployed", 11,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'P', 7}, {'P', 8}, {'0', 5}, {'P', 9}, {'1', 9}, {'0', 9}, {'P', 10}, {'S', 0}}},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'P', 7}, {'P', 8}, {'0', 5}, {'P', 9}, {'1', 9}, {'0', 9}, {'P', 10}, {'S', 0}}},
     /* layer, q, k_pages, v_pages, page_table, seq_lens, out, workspace, sm_scale */
     [DECODE] = {"novakv_decode_attention", 9,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'0', 2}, {'P', 4}, {'1', 4}, {'P', 5}, {'0', 1}, {'F', 8}, {'P', 6}, {'T', 6}, {'P', 7}, {'B', 7}, {'S', 0}}},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'0', 2}, {'P', 4}, {'1', 4}, {'P', 5}, {'0', 1}, {'F', 8}, {'P', 6}, {'T', 6}, {'P', 7}, {'B', 7}, {'S', 0}}},
     /* layer, q, k_pages, v_pages, k_scales, page_table, seq_lens, out, workspace, sm_scale */
     [DECODE_SCALED] = {"novakv_decode_attention_scaled", 10,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'0', 2}, {'P', 5}, {'1', 5}, {'P', 6}, {'0', 1}, {'F', 9}, {'P', 7}, {'T', 7}, {'P', 8}, {'B', 8}, {'S', 0}}},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'0', 2}, {'P', 5}, {'1', 5}, {'P', 6}, {'0', 1}, {'F', 9}, {'P', 7}, {'T', 7}, {'P', 8}, {'B', 8}, {'S', 0}}},
     /* layer, q, k_pages, v_pages, k_scales, sink_logits, page_table, seq_lens, out, workspace, sm_scale */
     [DECODE_SINK] = {"novakv_decode_attention_sink", 11,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'P', 5}, {'0', 2}, {'P', 6}, {'1', 6}, {'P', 7}, {'0', 1}, {'F', 10}, {'P', 8}, {'T', 8}, {'P', 9}, {'B', 9}, {'S', 0}}},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'P', 5}, {'0', 2}, {'P', 6}, {'1', 6}, {'P', 7}, {'0', 1}, {'F', 10}, {'P', 8}, {'T', 8}, {'P', 9}, {'B', 9}, {'S', 0}}},
     /* layer, q, k_pages, v_pages, k_scales, sink_logits, page_table, quant_lens, band_k, band_v, n_sink, band_meta, out, workspace, sm_scale */
     [DECODE_BANDED] = {"novakv_decode_attention_banded", 15,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'P', 5}, {'0', 2}, {'P', 6}, {'1', 6}, {'P', 7}, {'P', 8}, {'P', 9}, {'1', 8}, {'I', 10}, {'P', 11},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'P', 5}, {'0', 2}, {'P', 6}, {'1', 6}, {'P', 7}, {'P', 8}, {'P', 9}, {'1', 8}, {'I', 10}, {'P', 11},
          {'0', 1}, {'F', 14}, {'P', 12}, {'T', 12}, {'P', 13}, {'B', 13}, {'S', 0}}},
     /* layer, q, k_pages, v_pages, k_scales, v_meta, sink_logits, page_table, quant_lens, band_k, band_v, n_sink, band_meta, out, workspace, sm_scale */
     [DECODE_DEPLOYED] = {"novakv_decode_attention_deployed", 16,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'P', 5}, {'P', 6}, {'0', 2}, {'P', 7}, {'1', 7}, {'P', 8}, {'P', 9}, {'P', 10}, {'m', 9}, {'I', 11}, {'P', 12},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'P', 5}, {'P', 6}, {'0', 2}, {'P', 7}, {'1', 7}, {'P', 8}, {'P', 9}, {'P', 10}, {'m', 9}, {'I', 11}, {'P', 12},
          {'0', 1}, {'F', 15}, {'P', 13}, {'T', 13}, {'P', 14}, {'B', 14}, {'S', 0}}},
     /* layer, k_new, v_new, band_k, band_v, n_sink, n_rec, block, band_meta, quant_lens, k_pages, v_pages, k_scales, v_meta, page_table, seq_lens, staging */
     [BAND_APPEND] = {"novakv_band_append", 17,
-        {{'I', 0}, {'P', 1}, {'P', 2}, {'0', 1}, {'P', 3}, {'P', 4}, {'1', 3}, {'I', 5}, {'I', 6}, {'I', 7}, {'P', 8}, {'P', 9}, {'P', 10}, {'P', 11}, {'P', 12}, {'P', 13},
+        {{'L', 0}, {'P', 1}, {'P', 2}, {'0', 1}, {'P', 3}, {'P', 4}, {'1', 3}, {'I', 5}, {'I', 6}, {'I', 7}, {'P', 8}, {'P', 9}, {'P', 10}, {'P', 11}, {'P', 12}, {'P', 13},
          {'0', 10}, {'P', 14}, {'1', 14}, {'P', 15}, {'P', 16}, {'B', 16}, {'S', 0}}},
     /* q, k_pages, v_pages, page_table, seq_lens, out, workspace, sm_scale, window */
     [WINDOW] = {"novakv_bf16_decode_attention", 9,
         {{'P', 0}, {'P', 1}, {'P', 2}, {'0', 1}, {'P', 3}, {'1', 3}, {'P', 4}, {'0', 0}, {'F', 7}, {'I', 8}, {'P', 5}, {'T', 5}, {'P', 6}, {'B', 6}, {'S', 0}}},
     /* layer, k_new, v_new, tok_seq, tok_pos, q, k_pages, v_pages, page_table, seq_lens, out, staging, workspace, sm_scale */
-#define HOST_PARAMS {{'I', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'P', 7}, {'0', 6}, {'P', 8}, {'1', 8}, {'P', 9}, {'0', 5}, {'F', 13}, \
+#define HOST_PARAMS {{'L', 0}, {'P', 1}, {'P', 2}, {'P', 3}, {'P', 4}, {'n', 1}, {'P', 5}, {'P', 6}, {'P', 7}, {'0', 6}, {'P', 8}, {'1', 8}, {'P', 9}, {'0', 5}, {'F', 13}, \
          {'P', 10}, {'P', 11}, {'B', 11}, {'P', 12}, {'B', 12}, {'S', 0}}
     [STEP_HOST] = {"novakv_step_host", 14, HOST_PARAMS},
     [STEP_HOST_ASYNC] = {"novakv_step_host_async", 14, HOST_PARAMS},
@@ -82,8 +82,8 @@ static long long shape_of(PyObject* x, int dim) {
     Py_DECREF(item);
     return v;
 }
-static int as_int(PyObject* x, long long* v) {
-    PyObject* n = PyNumber_Long(x);
+static int as_int(PyObject* x, int exact, long long* v) {
+    PyObject* n = exact ? PyNumber_Index(x) : PyNumber_Long(x);
     if (!n) return -1;
     *v = PyLong_AsLongLong(n);
     Py_DECREF(n);
@@ -163,7 +163,8 @@ static PyObject* entry_call(PyObject* self, PyObject* const* args, size_t nargsf
         unsigned long long u = 0;
         a[i] = 0;
         switch (p[i].kind) {
-            case 'I': if (as_int(x, &a[i])) return NULL; break;
+            case 'L': if (as_int(x, 1, &a[i])) return NULL; break;
+            case 'I': if (as_int(x, 0, &a[i])) return NULL; break;
             case 'F': f = (float)PyFloat_AsDouble(x); break;
             case 'P': if (pointer_of(x, &u)) return NULL; a[i] = (long long)u; break;
             case '0': a[i] = shape_of(x, 0); break;
