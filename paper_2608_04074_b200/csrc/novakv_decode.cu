@@ -1,7 +1,8 @@
 // Read path: decode-step attention straight from the packed index cache.
 //
-//   prepare  : q' = sm_scale*log2(e) * q rk_inv_t  per head, and a prefix sum of page counts (the
-//              work list of the scan kernel: one unit = one 64-token page of one (sequence, KV head)).
+//   prepare  : q' = sm_scale*log2(e) * q rk_inv_t  per head.  (For large batches also a prefix sum of page counts, the
+//              work list of the scan kernel: one unit = one 64-token page of one (sequence, KV head); the scan forms it
+//              itself otherwise.)
 //   stage 1  : persistent scan kernel, one CTA per SM.  Each CTA takes a contiguous range of the
 //              global page sequence, so that consecutive pages mostly belong to the same
 //              (sequence, KV head) and reuse its score table.  Per (sequence, KV head) segment:
@@ -105,8 +106,8 @@ struct S1 {
     static constexpr int Q_BYTES = HPAD * D * 4;
     static constexpr int Q = P + P_BYTES;                               // fp32 [HPAD][D], of the present and of the next pair
     static constexpr int BND = Q + 2 * Q_BYTES;                        // long [MAX_SCAN_CTAS + 1]: first unit of every CTA
-    static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;           // int [3][PFX_CAP + 1]: page and cost prefix and lengths of small batches
-    static constexpr int SMEM = PFX + 3 * (PFX_CAP + 1) * 4;
+    static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;           // int [2][PFX_CAP + 1]: page and cost prefix of small batches
+    static constexpr int SMEM = PFX + 2 * (PFX_CAP + 1) * 4;
     // merge buffer (aliases the larger table once a segment's scan is done)
     static constexpr int MROW = D + 4;                                  // floats per (warp, head) row of the merge buffer: 16 bytes of padding
                                                                         // keep the four head rows a warp writes at once on different banks
@@ -394,19 +395,18 @@ struct Segment {
     int b, kvh, pg0, npg, len;
 };
 
-// Page and cost prefixes of a batch of at most PFX_CAP sequences, and its lengths, in shared memory (pfx: [3][PFX_CAP + 1]), by
-// all threads of a scan CTA; CTA 0 also writes the prefixes for the merge kernel and reports lengths out of range.  Every
-// CTA does it by itself: a block of the kernel in front would have to wait for the append first, and the scan for that block
-// (1 x 777 step 17.6 -> 17.4 us a call, 5 x 100 of the d = 64 shape 16.7 -> 16.4, deployed band 64 x 32768 411 -> 405).
+// Page and cost prefixes of a batch of at most PFX_CAP sequences in shared memory (pfx: [2][PFX_CAP + 1]), by all threads of a
+// scan CTA; CTA 0 also writes the prefixes for the merge kernel and reports lengths out of range.  Every CTA does it by
+// itself: a block of the kernel in front would have to wait for the append first, and the scan for that block (1 x 777 step
+// 17.6 -> 17.4 us a call, 5 x 100 of the d = 64 shape 16.7 -> 16.4, deployed band 64 x 32768 411 -> 405).
 static_assert(PFX_CAP < S1_THREADS, "a thread for every sequence");
 __device__ __forceinline__ void form_prefixes(int32_t* pfx, int (*s_part)[NCW], const int32_t* __restrict__ seq_lens, int batch, int max_pages,
                                               int seg_weight, int32_t* __restrict__ page_prefix, int32_t* __restrict__ cost_prefix,
                                               uint32_t* dev_status) {
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    int len = 0, pages = 0;
+    int pages = 0;
     if (t < batch) {
-        const int raw = seq_lens[t];
-        len = clamp_len(raw, max_pages);
+        const int raw = seq_lens[t], len = clamp_len(raw, max_pages);
         if (raw != len && blockIdx.x == 0) atomicOr(dev_status, NOVAKV_DEV_BAD_LENGTH);
         pages = (len + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS;
     }
@@ -421,13 +421,13 @@ __device__ __forceinline__ void form_prefixes(int32_t* pfx, int (*s_part)[NCW], 
     if (batch > 32) {
         if (lane == 31) { s_part[0][warp] = incl; s_part[1][warp] = incl_ne; }
         __syncthreads();
-        for (int w = 0; w < warp; ++w) { incl += s_part[0][w]; incl_ne += s_part[1][w]; }
+        if (warp * 32 < batch)                                 // (the others would only keep everybody waiting)
+            for (int w = 0; w < warp; ++w) { incl += s_part[0][w]; incl_ne += s_part[1][w]; }
     }
     if (t < batch) {
         const int p0 = incl - pages, c0 = p0 + seg_weight * (incl_ne - (pages > 0));
         pfx[t] = p0;
         pfx[PFX_CAP + 1 + t] = c0;
-        pfx[2 * (PFX_CAP + 1) + t] = len;
         if (blockIdx.x == 0) { page_prefix[t] = p0; cost_prefix[t] = c0; }
         if (t == batch - 1) {
             const int c1 = incl + seg_weight * incl_ne;
@@ -784,7 +784,12 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         form_prefixes(pfx, s_part, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         page_prefix = pfx;
         cost_prefix = pfx + PFX_CAP + 1;
-
+    } else if (HG == 8 && batch <= PFX_CAP) {
+        int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
+        for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix_g[i]; pfx[PFX_CAP + 1 + i] = cost_prefix_g[i]; }
+        __syncthreads();
+        page_prefix = pfx;
+        cost_prefix = pfx + PFX_CAP + 1;
     }
     // First unit of every CTA (see scan_boundary): one thread per boundary.  This CTA owns [s_bnd[c], s_bnd[c + 1]).
     long* const s_bnd = reinterpret_cast<long*>(s_abs + C::BND);
@@ -1442,7 +1447,7 @@ struct S1M {
     static constexpr int ML = MACC + NCW * MHEADS * MROW * 4;
     static constexpr int BND = ML + NCW * HG * 8;
     static constexpr int PFX = BND + (MAX_SCAN_CTAS + 1) * 8;
-    static constexpr int SMEM = PFX + 3 * (PFX_CAP + 1) * 4;
+    static constexpr int SMEM = PFX + 2 * (PFX_CAP + 1) * 4;
     static_assert(SMEM <= S1_SMEM_BYTES, "shared memory budget");
 };
 __global__ void __launch_bounds__(S1_THREADS, 1)
@@ -1500,7 +1505,12 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
         form_prefixes(pfx, s_part, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         page_prefix = pfx;
         cost_prefix = pfx + PFX_CAP + 1;
-
+    } else if (HG == 8 && batch <= PFX_CAP) {
+        int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
+        for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix_g[i]; pfx[PFX_CAP + 1 + i] = cost_prefix_g[i]; }
+        __syncthreads();
+        page_prefix = pfx;
+        cost_prefix = pfx + PFX_CAP + 1;
     }
     long* const s_bnd = reinterpret_cast<long*>(s_abs + C::BND);
     for (int c = threadIdx.x; c <= (int)gridDim.x; c += S1_THREADS)
@@ -2295,7 +2305,10 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     const bool fuse = sink_logits == nullptr && band == nullptr && ctx->fused_merge;
 
     // (with the merge fused in, the outputs of empty sequences are written where the prefixes are formed)
-    const int scan_prefix = batch <= PFX_CAP && !fuse;
+    // Eight heads per KV head: only batches of one warp.  The append (d = 64, about 6 us) then ends before the queries are
+    // transformed, and a block of the prepare kernel has formed the prefixes by the time the scan could (70 sequences
+    // of 400 tokens: 44.1 us so, 44.6 in the scan; 5 of 100: 16.7 and 16.4).
+    const int scan_prefix = batch <= (HG == 8 ? 32 : PFX_CAP) && !fuse;
     // sequences per prepare block: one while all pairs fit on the machine twice over, then enough to make that so
     const int seqs_per_block = max(1, min(8, (batch * hkv + 2 * ctx->n_sm - 1) / (2 * ctx->n_sm)));
     auto prepare = seqs_per_block > 1 ? novakv_prepare_kernel<D, HG, true> : novakv_prepare_kernel<D, HG, false>;
