@@ -136,6 +136,7 @@ __device__ __forceinline__ int clamp_len(int len, int max_pages) {
 // false: the loop's registers cost 0.7 us of 4.1, cold, at 8 sequences x 8 heads); once there are more pairs than the
 // machine holds blocks, runs save the 64 KB per pair that re-reading the transform costs: 128 sequences x 8 heads,
 // d = 128: 13.5 -> 8.2 us.
+constexpr int PREPARE_RUN = 8;                 // sequences per block at most
 template <int D, int HG, bool RUNS>
 __global__ void __launch_bounds__(512)
 novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict__ rk_inv_t,
@@ -158,22 +159,17 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
     const int c = threadIdx.x % D, part = threadIdx.x / D;
     // The query transform depends on nothing the preceding kernel of the stream (normally the append of this
     // step's tokens) writes: queries are produced before that kernel started, the transform is a constant.  So
-    // the blocks that transform queries never wait on the grid dependency: they run beside the preceding
-    // kernel.  Only the block that forms the page prefix (it reads seq_lens, which an append updates) waits;
-    // since a grid completes only when all its blocks have, the scan kernel's own wait still covers both.
+    // the blocks that transform queries run beside the preceding kernel.  They write nothing before it has completed: it
+    // may still read what shares memory with this call's workspace (the partials of another call on that scratch, new
+    // rows whose tensor has been freed).
+    const int n_query_blocks = (int)gridDim.x - form_prefix;
     float rv[ROWS];
-    if (blk < (int)gridDim.x - 1) {
+    if (blk < n_query_blocks) {
         const float* R = rk_inv_t + (size_t)kvh * D * D + (size_t)part * ROWS * D + c;
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) rv[r] = R[(size_t)r * D];
     }
-    if (blk == (int)gridDim.x - 1) {
-        if (!form_prefix) {
-            // this grid must not complete before the preceding kernel has (the scan waits for this grid alone)
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            return;
-        }
+    if (blk == n_query_blocks) {
         novakv_grid_dependency_wait();
         // exclusive prefix over sequences of their page counts; small, done by one warp.  Beside it the same
         // prefix in "cost" units, in which every non-empty sequence weighs seg_weight pages more: the scan
@@ -225,12 +221,14 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
         return;
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    static_assert(HG * D <= 512, "a thread for every coordinate of a KV head's queries");
+    constexpr int RUN = RUNS ? PREPARE_RUN : 1;
     __shared__ float q_s[HG][D];
     __shared__ float red_s[PARTS][HG][D];
+    __shared__ float qp_s[RUN][HG * D], qk_s[RUN][HG], qc_s[RUN][HG];            // results, until they may be written
     const int b0 = RUNS ? run * seqs_per_block : run, b_end = RUNS ? min(batch, b0 + seqs_per_block) : run + 1;
     for (int b = b0; b < b_end; ++b) {
         if (RUNS && b != b0) __syncthreads();                  // the shared arrays are free
-        if (pair_count != nullptr && threadIdx.x == 0) pair_count[kvh * batch + b] = 0;
         for (int i = threadIdx.x; i < HG * D; i += 512)
             q_s[i / D][i % D] = __bfloat162float(q[((size_t)b * n_q_heads + kvh * HG) * D + i]);
         __syncthreads();
@@ -244,13 +242,13 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
 #pragma unroll
         for (int h = 0; h < HG; ++h) red_s[part][h][c] = acc[h];
         __syncthreads();
-        for (int i = threadIdx.x; i < HG * D; i += 512) {
-            const int h = i / D, cc = i % D;
+        if (threadIdx.x < HG * D) {
+            const int h = threadIdx.x / D, cc = threadIdx.x % D;
             float v = 0.f;
 #pragma unroll
             for (int p = 0; p < PARTS; ++p) v += red_s[p][h][cc];
             v *= scale_log2;
-            qp[((size_t)b * n_q_heads + kvh * HG + h) * D + cc] = v;
+            qp_s[b - b0][threadIdx.x] = v;
             if (qc != nullptr) red_s[0][h][cc] = v * k_center[(size_t)kvh * D + cc];       // (each thread rewrites only what it read)
         }
         // the constant the read path drops from every logit of a query, q . k_mean * sm_scale (base-2 units):
@@ -260,9 +258,7 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
             float acc = 0.f;
             for (int i = lane; i < D; i += 32) acc = fmaf(q_s[h][i], k_mean[(size_t)kvh * D + i], acc);
             acc = warp_sum_f(acc);
-            // (the merge kernel of a preceding decode call on this workspace reads qk_off: its grid must have completed)
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            if (lane == 0) qk_off[(size_t)b * n_q_heads + kvh * HG + h] = acc * scale_log2;
+            if (lane == 0) qk_s[b - b0][h] = acc * scale_log2;
         }
         // scaled key format: the table is built from centred codewords, and the centre's share <q', centre> of
         // every logit is added back before the per-token scale multiplies it
@@ -273,13 +269,24 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
                 float acc = 0.f;
                 for (int i = lane; i < D; i += 32) acc += red_s[0][h][i];
                 acc = warp_sum_f(acc);
-                if (lane == 0) qc[(size_t)b * n_q_heads + kvh * HG + h] = acc;
+                if (lane == 0) qc_s[b - b0][h] = acc;
             }
         }
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (qk_off != nullptr || qc != nullptr) __syncthreads();    // (qp_s: every thread writes out what it put there)
+    for (int b = b0; b < b_end; ++b) {
+        const size_t row = (size_t)b * n_q_heads + kvh * HG;
+        if (threadIdx.x < HG * D) qp[row * D + threadIdx.x] = qp_s[b - b0][threadIdx.x];
+        if (threadIdx.x < HG) {
+            if (qk_off != nullptr) qk_off[row + threadIdx.x] = qk_s[b - b0][threadIdx.x];
+            if (qc != nullptr) qc[row + threadIdx.x] = qc_s[b - b0][threadIdx.x];
+        }
+        if (pair_count != nullptr && threadIdx.x == 0) pair_count[kvh * batch + b] = 0;
+    }
 #ifdef NOVAKV_TIMING
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(g_p1));
-    if (threadIdx.x == 0 && (blk == 0 || blk == (int)gridDim.x - 2))
+    if (threadIdx.x == 0 && (blk == 0 || blk == n_query_blocks - 1))
         printf("prepare block %d | ns start %llu end %llu\n", blk, g_p0, g_p1);
 #endif
 }
@@ -2310,9 +2317,9 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     // of 400 tokens: 44.1 us so, 44.6 in the scan; 5 of 100: 16.7 and 16.4).
     const int scan_prefix = batch <= (HG == 8 ? 32 : PFX_CAP) && !fuse;
     // sequences per prepare block: one while all pairs fit on the machine twice over, then enough to make that so
-    const int seqs_per_block = max(1, min(8, (batch * hkv + 2 * ctx->n_sm - 1) / (2 * ctx->n_sm)));
+    const int seqs_per_block = max(1, min(PREPARE_RUN, (batch * hkv + 2 * ctx->n_sm - 1) / (2 * ctx->n_sm)));
     auto prepare = seqs_per_block > 1 ? novakv_prepare_kernel<D, HG, true> : novakv_prepare_kernel<D, HG, false>;
-    novakv_launch_pdl(prepare, dim3((batch + seqs_per_block - 1) / seqs_per_block * hkv + 1), dim3(512), 0, stream, q, ly.rk_inv_t, seq_lens,
+    novakv_launch_pdl(prepare, dim3((batch + seqs_per_block - 1) / seqs_per_block * hkv + (scan_prefix ? 0 : 1)), dim3(512), 0, stream, q, ly.rk_inv_t, seq_lens,
                       batch, hq, hkv, max_pages_per_seq, sm_scale * 1.4426950408889634f, qp, prefix, ctx->dev_status,
                       k_off_vec, qk_off, cost_prefix, ctx->seg_weight, (const float*)ly.k_center, qc,
                       fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32, seqs_per_block, scan_prefix ? 0 : 1);

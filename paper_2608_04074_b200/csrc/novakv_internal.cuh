@@ -142,8 +142,9 @@ novakv_status novakv_launch_bf16_decode(novakv_ctx* ctx, const __nv_bfloat16* q,
 // touches anything a preceding kernel may write, which blocks until the predecessor grid has completed
 // and its writes are visible.  Before the wait a kernel only reads calibration constants (uploaded
 // synchronously by novakv_load_calibration, never written by a kernel) into registers or its own shared
-// memory, so the launch latency and that staging overlap the predecessor's tail.  There is no unbounded
-// wait in user code.
+// memory, so the launch latency and that staging overlap the predecessor's tail; the query transform also reads q, which
+// the public header asks to be complete by then.  Nothing is written to global memory before the wait: workspaces, staging
+// buffers and freed tensors share memory with what the predecessor may still read.  There is no unbounded wait in user code.
 __device__ __forceinline__ void novakv_grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
