@@ -2325,14 +2325,6 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
                       fuse ? pair_count : (int32_t*)nullptr, fuse ? out : (void*)nullptr, out_is_fp32, seqs_per_block, scan_prefix ? 0 : 1);
     ctx->launches++;
 
-    // (before the scan: its blocks run beside the encoder of a step's append, on the SMs that leaves free)
-    if (band != nullptr) {
-        novakv_launch_pdl(novakv_band_kernel<D, HG>, dim3(batch * hkv), dim3(BAND_WARPS * 32), 0, stream, q, band->k, band->v,
-                          band->cap, band->n_sink, band->meta, hq, hkv, sm_scale * 1.4426950408889634f, k_off_vec, band_ml,
-                          band_acc);
-        ctx->launches++;
-    }
-
     // d = 64 with eight query heads per KV head, plain format: the kernel that takes the logits from tensor cores.  (At
     // d = 128 its two copies of the key codewords do not fit; with four heads a look-up in the table reads no more bytes than
     // a gather of a codeword; the scaled format has not been built with it.)  Not for short calls: its CTAs stage 192 KB of
@@ -2373,6 +2365,13 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
             ps.end();
             ctx->launches++;
         }
+    }
+    // (behind the scan, whose CTAs let it start when they have seen everything in front of this call complete)
+    if (band != nullptr) {
+        novakv_launch_pdl(novakv_band_kernel<D, HG>, dim3(batch * hkv), dim3(BAND_WARPS * 32), 0, stream, q, band->k, band->v,
+                          band->cap, band->n_sink, band->meta, hq, hkv, sm_scale * 1.4426950408889634f, k_off_vec, band_ml,
+                          band_acc);
+        ctx->launches++;
     }
     if (fuse) return cudaGetLastError() == cudaSuccess ? NOVAKV_OK : NOVAKV_ECUDA;
     const bool ext = sink_logits != nullptr || band != nullptr;

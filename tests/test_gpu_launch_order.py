@@ -115,6 +115,38 @@ def test_new_rows_in_the_scratch_of_the_decode(cases, name, fmt, n):
     assert ctx.novakv_last_device_status() == 0
 
 
+@pytest.mark.parametrize("fmt", ["scaled", "deployed"])
+def test_band_rows_from_the_call_in_front(cases, fmt):
+    """Band rows that the kernel directly before the decode call writes, having let its dependents start (here: the output of
+    another decode): the band kernel has to see them."""
+    from paper_2608_04074_b200.runtime import BandedCache
+    case = cases("qwen", True)
+    ctx = case.ctx
+    other, q_other = _cache(case, np.full(32, 3000, np.int32), 31, key_scale=True)
+    banded = BandedCache(ctx, 4, 2000, seed=5, key_scale=fmt == "scaled", int2_values=fmt == "deployed")
+    for b, n in enumerate((1500, 700, 330, 60)):
+        k, v, _ = case.draw(3200 + b, n, 1)
+        banded.prefill(0, b, _dev(k, torch.bfloat16), _dev(v, torch.bfloat16))
+    _, _, q = case.draw(3300, 1, 4)
+    q = _dev(q, torch.bfloat16)
+    rows = banded.band_v.view(-1)[:q_other.numel()].view(q_other.shape)      # the first rows of the band
+    before = rows.clone()
+
+    def calls(wait):
+        rows.copy_(before)
+        other.decode(0, q_other, out=rows)
+        if wait:
+            torch.cuda.synchronize()
+        return banded.decode(0, q)
+
+    expected = calls(True)
+    rows.copy_(before)
+    assert not torch.equal(banded.decode(0, q), expected)
+    for _ in range(TIMES):
+        assert torch.equal(calls(False), expected)
+    assert ctx.novakv_last_device_status() == 0
+
+
 @pytest.mark.parametrize("batch", [2, 9, 64])
 def test_band_staging_in_the_scratch_of_the_decode(cases, batch):
     """The rows that leave the band are encoded out of a staging buffer; the decode that follows may use the same scratch."""
