@@ -8,6 +8,7 @@ import os
 import shutil
 import subprocess
 import sysconfig
+import warnings
 from pathlib import Path
 
 PKG_DIR = Path(__file__).resolve().parent
@@ -15,7 +16,8 @@ CSRC = PKG_DIR / "csrc"
 INCLUDE = PKG_DIR.parent / "include"
 LIB_CUDA = PKG_DIR / "libnovakv.so"
 LIB_CALIB = PKG_DIR / "libnovakv_calib.so"
-LIB_CALLS = PKG_DIR / "_novakv_calls.so"
+# (a C extension: named after the interpreter it is built for, so that another one does not load it)
+LIB_CALLS = PKG_DIR / ("_novakv_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 CUDA_SOURCES = ["novakv_api.cu", "novakv_encode.cu", "novakv_prefill.cu", "novakv_decode.cu", "novakv_bf16_decode.cu",
                 "novakv_noalloc.cu"]
@@ -36,8 +38,17 @@ def _nvcc() -> str:
 
 
 def build_cuda(force: bool = False, verbose: bool = False) -> Path:
+    """The C library, and its Python entry where Python's headers are (a C caller needs only the library)."""
+    lib = _build_library(force, verbose)
+    try:
+        build_calls(force)
+    except (OSError, RuntimeError) as e:
+        warnings.warn(f"{lib.name} is built, its Python entry is not: {e}")
+    return lib
+
+
+def _build_library(force: bool, verbose: bool) -> Path:
     srcs = [CSRC / s for s in CUDA_SOURCES if (CSRC / s).exists()]
-    build_calls(force)
     deps = srcs + sorted(CSRC.glob("*.cuh")) + sorted(INCLUDE.glob("*.h"))
     if not force and _newer(LIB_CUDA, deps):
         return LIB_CUDA
