@@ -446,6 +446,25 @@ __device__ __forceinline__ void form_prefixes(int32_t* pfx, int (*s_part)[NCW], 
     __syncthreads();
 }
 
+// A scan CTA that cannot run leaves an empty range; the merge kernel reads the prefixes all the same and needs them whole.
+__device__ __noinline__ void leave_unscanned(long* cta_range, int form_prefix, const int32_t* seq_lens, int batch, int max_pages, int seg_weight,
+                                             int32_t* page_prefix, int32_t* cost_prefix, uint32_t* dev_status) {
+    novakv_grid_dependency_wait();
+    if (threadIdx.x != 0) return;
+    atomicOr(dev_status, NOVAKV_DEV_SMEM_LAYOUT);
+    cta_range[blockIdx.x * 2] = 0;
+    cta_range[blockIdx.x * 2 + 1] = 0;
+    if (!form_prefix || blockIdx.x != 0) return;
+    int pages = 0, cost = 0;
+    for (int b = 0; b <= batch; ++b) {
+        page_prefix[b] = pages;
+        cost_prefix[b] = cost;
+        const int n = b < batch ? (clamp_len(seq_lens[b], max_pages) + NOVAKV_PAGE_TOKENS - 1) / NOVAKV_PAGE_TOKENS : 0;
+        pages += n;
+        cost += n > 0 ? n + seg_weight : 0;
+    }
+}
+
 // Locate the (KV head, sequence, page) of global page unit u.  Units are ordered KV-head-major:
 // u = kvh * P + page_prefix[b] + page, with P = page_prefix[batch] the pages of all sequences, so that
 // consecutive segments of a CTA share the KV head (and its value codebook).  page_prefix is exclusive,
@@ -763,10 +782,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     const uint32_t s_base = smem_u32(smem);
     if (s_base > C::T16 || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
         // cannot happen with the shared address window of this architecture; reported, never trapped
-        if (threadIdx.x == 0) {
-            atomicOr(dev_status, NOVAKV_DEV_SMEM_LAYOUT);
-            cta_range[blockIdx.x * 2] = 0; cta_range[blockIdx.x * 2 + 1] = 0;
-        }
+        leave_unscanned(cta_range, form_prefix, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         return;
     }
     unsigned char* const s_abs = smem - s_base;               // s_abs + a: the byte at shared-window address a
@@ -1475,10 +1491,7 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
     const uint32_t s_base = smem_u32(smem);
     if (s_base > C::KEY || C::SMEM - s_base > (uint32_t)S1_SMEM_BYTES) {
         // cannot happen with the shared address window of this architecture; reported, never trapped
-        if (threadIdx.x == 0) {
-            atomicOr(dev_status, NOVAKV_DEV_SMEM_LAYOUT);
-            cta_range[blockIdx.x * 2] = 0; cta_range[blockIdx.x * 2 + 1] = 0;
-        }
+        leave_unscanned(cta_range, form_prefix, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         return;
     }
     unsigned char* const s_abs = smem - s_base;               // s_abs + a: the byte at shared-window address a
