@@ -414,7 +414,7 @@ novakv_status novakv_debug_set_value_path(novakv_ctx* ctx, int path);
  * cuts the walk into one contiguous piece per CTA.  Each pair a CTA touches costs it a fixed set-up (the
  * per-query score table), so the cut is even not in pages but in pages + `pages` per pair touched: a CTA
  * that has to set up several pairs gets fewer pages.  `pages` = 0 gives the even split in pages; the
- * default is 24.  Results do not depend on it beyond binary32 rounding (it only moves split points).
+ * default is 34 at d = 128 and 24 at d = 64.  Results do not depend on it beyond binary32 rounding (it only moves split points).
  */
 novakv_status novakv_debug_set_segment_weight(novakv_ctx* ctx, int pages);
 
@@ -435,6 +435,13 @@ novakv_status novakv_debug_set_fused_merge(novakv_ctx* ctx, int on);
  * nothing else is touched.
  */
 novakv_status novakv_debug_set_wait_limit(novakv_ctx* ctx, long clocks);
+
+/*
+ * Largest number of new tokens that a call of this context's shape hands to the append kernel (binary64 coefficients, derived
+ * bounds); larger calls, and rows off a 16-byte boundary, take the prompt encoder (tensor cores, measured bounds, binary64 where
+ * these leave a decision open).  For tests that compare the two.
+ */
+int novakv_debug_append_kernel_tokens(const novakv_ctx* ctx);
 
 /* Kernels this library launched since the context was created (all kinds). */
 long novakv_launch_count(const novakv_ctx* ctx);

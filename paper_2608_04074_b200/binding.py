@@ -27,6 +27,7 @@ EXPORTED = [
     "novakv_value_meta_page_bytes", "novakv_encode_append_deployed", "novakv_decode_attention_deployed",
     "novakv_debug_set_segment_weight", "novakv_debug_set_fused_merge",
     "novakv_band_append_staging_bytes", "novakv_band_append", "novakv_debug_set_wait_limit",
+    "novakv_debug_append_kernel_tokens",
 ]
 
 
@@ -119,6 +120,7 @@ def load_library(path=None):
                                                  c_size_t, c_void_p]
     lib.novakv_profile_enable.argtypes = [c_void_p, c_int]
     lib.novakv_profile_read.argtypes = [c_void_p, c_int, POINTER(c_double), POINTER(c_long)]
+    lib.novakv_debug_append_kernel_tokens.argtypes = [c_void_p]
     lib.novakv_launch_count.argtypes = [c_void_p]
     lib.novakv_debug_set_scan_ctas.argtypes = [c_void_p, c_int]
     lib.novakv_debug_set_value_path.argtypes = [c_void_p, c_int]
@@ -342,6 +344,9 @@ class Context:
 
     def novakv_debug_set_wait_limit(self, clocks):
         _check(self.lib, self.lib.novakv_debug_set_wait_limit(self.handle, int(clocks)), "novakv_debug_set_wait_limit")
+
+    def novakv_debug_append_kernel_tokens(self):
+        return int(self.lib.novakv_debug_append_kernel_tokens(self.handle))
 
     def novakv_launch_count(self):
         return int(self.lib.novakv_launch_count(self.handle))

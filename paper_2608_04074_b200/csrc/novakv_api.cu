@@ -668,6 +668,8 @@ extern "C" novakv_status novakv_debug_set_scan_ctas(novakv_ctx* ctx, int n_ctas)
     return NOVAKV_OK;
 }
 
+extern "C" int novakv_debug_append_kernel_tokens(const novakv_ctx* ctx) { return ctx ? novakv_append_kernel_tokens(ctx) : 0; }
+
 extern "C" novakv_status novakv_debug_set_segment_weight(novakv_ctx* ctx, int pages) {
     if (!ctx || pages < 0 || pages > 4096) return NOVAKV_EINVAL;
     ctx->seg_weight = pages;

@@ -21,15 +21,6 @@ namespace {
 
 constexpr int ENC_THREADS = 512;
 constexpr int ENC_TILE = 64;   // tokens per tile (search granularity)
-// Batches up to this size take the per-group append kernel, larger ones the prompt encoder.  The append kernel's time grows with
-// every pass of 8 tokens a chunk, the encoder's is one unit per SM up to 256 tokens.  us, tables in the L2 / cold:
-//   d = 128 plain      64: 17.9 / 16.8 here, 18.1 / 21.5 there   96: 25.2 / 23.1, 19.2 / 23.4   256: 55 / 55, 23 / 30
-//           scaled     64: 21.5 / 21.2, 25.6 / 29.0              96: 30.3 / 29.4, 25.3 / 29.9   256: 66 / 67, 32 / 39
-//           deployed   64: 25.4 / 24.1, 25.4 / 28.5              96: 35.9 / 33.9, 25.2 / 28.5   256: 78 / 76, 32 / 37
-//   d = 64  plain     128: 14.6 / 14.0, 17.0 / 18.6             192: 20.2 / 19.3, 18.0 / 20.3   256: 21.2 / 22.8, 19.2 / 22.3
-//           scaled    128: 17.5 / 16.9, 22.0 / 24.7             192: 24.4 / 23.5, 21.7 / 24.4   256: 26.5 / 27.8, 22.6 / 26.0
-constexpr int small_append_tokens(int d) { return d == 128 ? 64 : 192; }
-
 // Shared-memory plan of the search-only kernel: codebook, one tile of coefficients, its indices.
 template <int D>
 struct EncSmem {
@@ -272,6 +263,29 @@ __device__ __forceinline__ int exact_search_warp(const double (&rd)[4], const fl
 
 constexpr int SMALL_CTAS_PER_SM = 5;             // (shared memory allows six at d = 128; five leave a thread 96 registers)
 constexpr int SMALL_TP_LOG2 = 3;
+// Chunks of the token list that run side by side: all of their CTAs are resident together.
+int small_append_chunks(const novakv_ctx* ctx) {
+    return max(1, SMALL_CTAS_PER_SM * ctx->n_sm / (ctx->n_groups / 4 * ctx->cfg.n_kv_heads * 2));
+}
+// Batches up to this size take the append kernel, larger ones the prompt encoder.  The append kernel's time grows with every
+// pass of 8 tokens of its longest chunk, and fewer KV heads leave room for more chunks; the encoder's is one unit per SM.  So the
+// line lies behind two passes (never above 256 tokens).  us in a stream of calls, append kernel / encoder:
+//                 heads   two passes at most                      three or more
+//   d = 128 plain     1   256: 10.2 / 20.0
+//                     2   128: 10.3 / 17.8   256: 17.7 / 21.7
+//                     4    64: 10.2 / 17.7   160: 18.4 / 22.2     192: 25.2 / 22.3   256: 26.0 / 24.4
+//                     8    32: 10.2 / 19.0    64: 17.7 / 19.5      96: 25.2 / 20.1   256: 55.8 / 25.6
+//           scaled    1, 2, 4, 8 heads: 256: 11.9 / 30.7   256: 21.2 / 28.5   160: 21.8 / 26.5   64: 21.2 / 21.8, 96: 30.4 / 22.1
+//           deployed                    256: 14.0 / 30.8   256: 25.5 / 27.2   160: 26.2 / 26.5   64: 25.4 / 21.8, 96: 36.4 / 21.9
+//   d = 64  plain                       256:  5.0 / 16.6   256:  8.2 / 17.2   256: 14.4 / 18.3  160: 14.7 / 17.9, 192: 20.3 / 18.3
+//           scaled                      256:  6.5 / 17.7   256:  9.5 / 19.6   256: 17.0 / 21.2  160: 17.0 / 19.3, 192: 24.2 / 19.4
+// With eight heads and more it lies a little or a lot too high (16 / 32 heads, d = 128, 64 tokens: 32.5 / 20.0, 62 / 30): up to 64
+// (d = 128) or 192 tokens (d = 64) the append kernel keeps its calls, whose bounds are derived where the encoder's are measured.
+constexpr int SMALL_PASSES = 2;
+constexpr int small_always(int d) { return d == 128 ? 64 : 192; }
+int small_append_tokens(const novakv_ctx* ctx) {
+    return max(small_always(ctx->cfg.head_dim), min(256, (small_append_chunks(ctx) * SMALL_PASSES) << SMALL_TP_LOG2));
+}
 template <int D, int FMT>
 __global__ void __launch_bounds__(128, SMALL_CTAS_PER_SM)
 novakv_encode_small_kernel(const __nv_bfloat16* __restrict__ k_new, const __nv_bfloat16* __restrict__ v_new,
@@ -598,14 +612,13 @@ novakv_status launch_encode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
     // (the append kernel reads the new rows in 16-byte pieces; rows on a 4-byte boundary take the prompt encoder, which can
     // copy them in words, whatever their number)
     const bool rows16 = (((uintptr_t)k_new | (uintptr_t)v_new) & 15) == 0;
-    if (n_tokens <= small_append_tokens(D) && rows16) {
+    if (n_tokens <= small_append_tokens(ctx) && rows16) {
         int tp_log2 = 0;
         while ((1 << tp_log2) < n_tokens && tp_log2 < SMALL_TP_LOG2) ++tp_log2;
         // chunks of the token list: as many as there are passes, while all CTAs are resident together, and no more than the
         // longest chunk needs (every chunk stages the constants): 64 tokens, d = 128, plain: 5 chunks 23.4 us cold and 18.0
         // warm, 4 chunks 20.5 and 17.4
-        const int passes = (n_tokens + (1 << tp_log2) - 1) >> tp_log2, per_chunk = D / NOVAKV_G / 4 * ctx->cfg.n_kv_heads * 2;
-        const int resident = max(1, min(passes, SMALL_CTAS_PER_SM * ctx->n_sm / per_chunk));
+        const int passes = (n_tokens + (1 << tp_log2) - 1) >> tp_log2, resident = min(passes, small_append_chunks(ctx));
         const int longest = (passes + resident - 1) / resident, chunks = (passes + longest - 1) / longest;
         dim3 grid(D / NOVAKV_G / 4, ctx->cfg.n_kv_heads, 2 * chunks);
         novakv_prof_scope ps(ctx, 1, stream);
@@ -662,6 +675,8 @@ novakv_status launch_search_t(novakv_ctx* ctx, const novakv_layer& ly, int which
 }
 
 }  // namespace
+
+int novakv_append_kernel_tokens(const novakv_ctx* ctx) { return small_append_tokens(ctx); }
 
 novakv_status novakv_launch_encode(novakv_ctx* ctx, const novakv_layer& ly, const __nv_bfloat16* k_new,
     const __nv_bfloat16* v_new, const int32_t* tok_seq, const int32_t* tok_pos, int n_tokens,

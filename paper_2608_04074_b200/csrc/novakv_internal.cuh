@@ -80,6 +80,7 @@ struct novakv_prof_scope {
 };
 
 // encode
+int novakv_append_kernel_tokens(const novakv_ctx* ctx);
 novakv_status novakv_launch_encode(novakv_ctx* ctx, const novakv_layer& ly, const __nv_bfloat16* k_new,
     const __nv_bfloat16* v_new, const int32_t* tok_seq, const int32_t* tok_pos, int n_tokens,
     uint8_t* k_pages, uint8_t* v_pages, int n_pages, const int32_t* page_table,

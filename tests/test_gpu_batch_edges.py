@@ -1,11 +1,12 @@
 """Batches on both sides of the sizes at which a call takes another way: the scan's own prefixes (up to 511 sequences; warps of
-32), and the append kernel or the prompt encoder (64 tokens at d = 128, 192 at d = 64).  Outputs: 2e-3 of the largest
+32), and the append kernel or the prompt encoder (two passes of eight tokens for every chunk that fits on the machine, which
+depends on the KV heads).  Outputs: 2e-3 of the largest
 (check_output); indices and scales equal the oracle's (check_indices)."""
 import numpy as np
 import pytest
 
 from gpu_common import Case, check_indices, check_output
-from paper_2608_04074_b200 import cache_format, workloads
+from paper_2608_04074_b200 import cache_format, synth, workloads
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -55,11 +56,8 @@ def test_prefixes(cases, name, batch):
     assert case.ctx.novakv_last_device_status() == NOVAKV_DEV_BAD_LENGTH
 
 
-@pytest.mark.parametrize("n", [64, 65, 192, 193])
-@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("qwen", "scaled"), ("qwen", "deployed"), ("gptoss", "plain"), ("gptoss", "scaled")])
-def test_append_or_prompt(cases, name, fmt, n):
+def _append_or_prompt(case, fmt, n):
     from paper_2608_04074_b200.runtime import PagedCache
-    case = cases(name, fmt != "plain")
     cache = PagedCache(case.ctx, np.zeros(2, np.int32), capacity_tokens=np.array([n, n]), seed=6, key_scale=fmt == "scaled",
                        int2_values=fmt == "deployed")
     k, v, _ = case.draw(900 + n, n, 1)
@@ -82,6 +80,28 @@ def test_append_or_prompt(cases, name, fmt, n):
             check_indices(vidx, mine, "v")
         if fmt != "plain":
             assert np.array_equal(cache.load_scales(s, 0, len(kidx)), mine["kscale"].astype(np.float32))
+
+
+@pytest.mark.parametrize("n", [64, 65, 192, 193, "line", "line + 1"])
+@pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("qwen", "scaled"), ("qwen", "deployed"), ("gptoss", "plain"), ("gptoss", "scaled")])
+def test_append_or_prompt(cases, name, fmt, n):
+    case = cases(name, fmt != "plain")
+    line = case.ctx.novakv_debug_append_kernel_tokens()
+    _append_or_prompt(case, fmt, {"line": line, "line + 1": line + 1}.get(n, n))
+
+
+@pytest.mark.parametrize("fmt", ["plain", "deployed"])
+@pytest.mark.parametrize("hkv,d", [(1, 64), (1, 128), (2, 128), (3, 128), (4, 128), (16, 64), (16, 128)])
+def test_append_or_prompt_by_heads(hkv, d, fmt):
+    wl = workloads.Workload("heads", synth.LayerShape(hkv, hkv, d), np.array([1024], np.int32), 7, n_outlier=2, calib_tokens=1024,
+                            calib_queries_for_values=128, lloyd_iters=2)
+    case = Case(wl, key_scale=fmt != "plain")
+    line = case.ctx.novakv_debug_append_kernel_tokens()
+    chunks = max(1, 5 * torch.cuda.get_device_properties(0).multi_processor_count // (d // 16 * hkv * 2))
+    assert line == max(64 if d == 128 else 192, min(256, 16 * chunks))
+    for n in (line // 2 + 3, line, line + 1):
+        _append_or_prompt(case, fmt, n)
+    case.ctx.close()
 
 
 @pytest.mark.parametrize("sink", [False, True])
