@@ -72,11 +72,11 @@ def test_search_from_oracle_coefficients_is_exact(name, request):
 
 
 # --------------------------------------------------------------------------- T2: transform + search + paged store
-@pytest.mark.parametrize("add", [[200, 64, 1, 130], [20, 7, 1, 3], [1, 0, 0, 0], [70, 60, 50, 40], [0, 2, 0, 0]])
+@pytest.mark.parametrize("add", [[200, 64, 1, 130], [20, 7, 1, 3], [1, 0, 0, 0], [70, 60, 50, 40], [20, 9, 14, 13], [0, 2, 0, 0]])
 @pytest.mark.parametrize("name", ["tiny", "qwen", "gptoss"])
 def test_encode_append_matches_oracle_indices(name, add, request):
-    """395 tokens take the tiled (prefill) kernel; 31, 1, 220 and 2 tokens the per-group append kernel with
-    1, 1, 7 and 1 passes and 1, 32, 1 and 16 lane groups per token."""
+    """395 tokens take the prompt encoder, 220 either kernel (by shape: novakv_debug_append_kernel_tokens); 31, 1, 56 and 2
+    tokens the per-group append kernel with 4, 1, 7 and 1 passes and 4, 32, 4 and 16 lane groups per token."""
     case = request.getfixturevalue(name)
     lens0 = np.array([0, 5, 63, 130], np.int32)          # existing lengths; tokens are appended after them
     add = np.array(add, np.int32)
@@ -584,11 +584,11 @@ def gptoss_scaled():
     return Case(workloads.gpt_oss_20b(batch=2, seq_len=2048, calib_tokens=4096, lloyd_iters=6), key_scale=True)
 
 
-@pytest.mark.parametrize("add", [[200, 64, 1, 130], [20, 7, 1, 3], [1, 0, 0, 0], [70, 60, 50, 40]])
+@pytest.mark.parametrize("add", [[200, 64, 1, 130], [20, 7, 1, 3], [1, 0, 0, 0], [70, 60, 50, 40], [20, 9, 14, 13]])
 @pytest.mark.parametrize("name", ["qwen_scaled", "gptoss_scaled"])
 def test_scaled_encode_matches_oracle_indices_and_scales(name, add, request):
-    """Append on the scaled key format, through the tiled kernel (395 tokens: a long run, a ragged tail, a
-    single token) and through the clustered append kernel (31, 1 and 220 tokens: one, one and seven passes):
+    """Append on the scaled key format, through the prompt encoder (395 and 220 tokens: a long run, a ragged tail, a
+    single token) and through the clustered append kernel (31, 1 and 56 tokens: four, one and seven passes):
     indices as in the unscaled test, scales bit for bit (bfloat16)."""
     from paper_2608_04074_b200.runtime import PagedCache
     case = request.getfixturevalue(name)
@@ -879,7 +879,7 @@ def test_banded_with_scale_and_sink(qwen_scaled):
 
 
 # --------------------------------------------------------------------------- deployed format: scaled VQ keys + INT2 values
-@pytest.mark.parametrize("add", [[200, 64, 1, 130], [20, 7, 1, 3], [1, 0, 0, 0], [70, 60, 50, 40]])
+@pytest.mark.parametrize("add", [[200, 64, 1, 130], [20, 7, 1, 3], [1, 0, 0, 0], [70, 60, 50, 40], [20, 9, 14, 13]])
 @pytest.mark.parametrize("name", ["qwen_scaled", "gptoss_scaled"])
 def test_deployed_encode_matches_oracle(name, add, request):
     """Keys as in the scaled format; value bytes (four 2-bit levels each) and (scale, zero) bit for bit."""

@@ -1,6 +1,8 @@
-"""Prompt encoder (more than 256 tokens per call) at the edges of its tiling: 256-token units of two 128-token halves,
-runs of units cut across (KV head, side, part of the groups) boundaries, and the exact re-search of close decisions.
-Indices, scales and (scale, zero) pairs must equal the oracle's; only float64 near-ties may differ (gpu_common)."""
+"""Prompt encoder (more tokens per call than the append kernel takes, which the context tells) at the edges of its tiling:
+256-token units of two 128-token halves, runs of units cut across (KV head, side, part of the groups) boundaries, and the
+exact re-search of close decisions.  Indices, scales and (scale, zero) pairs must equal the oracle's; only float64 near-ties may
+differ (gpu_common).  Where the append kernel is the witness - its bounds are derived, the encoder's measured -, the same tokens
+are stored in one call and in steps of the largest size that the append kernel takes."""
 import dataclasses
 
 import numpy as np
@@ -27,6 +29,13 @@ def _make(name, key_scale):
 @pytest.fixture(scope="module")
 def cases():
     return {(n, s): _make(n, s) for n in ("qwen", "gptoss") for s in (False, True)}
+
+
+def _append_step(case):
+    """Tokens per call of the append kernel, at most: one more and the encoder would be compared with itself."""
+    step = case.ctx.novakv_debug_append_kernel_tokens()
+    assert 8 <= step < 257                              # (every test of the encoder has more tokens in a call)
+    return step
 
 
 def _run(case, fmt, n, start, permute, holes, scale=1.0, offset=0):
@@ -128,7 +137,7 @@ def test_prefill_bounds_hold_on_hard_inputs(cases, name, fmt, kind):
     k, v = x.to(torch.bfloat16)
     seq, pos = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.arange(n, dtype=torch.int32, device="cuda")
     stored = []
-    for step in (n, 256):
+    for step in (n, _append_step(case)):
         cache = PagedCache(case.ctx, np.array([0], np.int32), capacity_tokens=np.array([n], np.int32), seed=7, key_scale=fmt == "scaled")
         for i in range(0, n, step):
             cache.append(0, k[i:i + step], v[i:i + step], seq[i:i + step], pos[i:i + step])
@@ -173,7 +182,7 @@ def test_prefill_squares_that_underflow(cases, name, fmt, factor):
     k[:, :, ::16] *= 40.0                                  # a few large elements: small coefficients with large errors beside them
     seq, pos = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.arange(n, dtype=torch.int32, device="cuda")
     stored = []
-    for step in (n, 256):
+    for step in (n, _append_step(case)):
         cache = PagedCache(case.ctx, np.array([0], np.int32), capacity_tokens=np.array([n], np.int32), seed=7,
                            key_scale=fmt == "scaled", int2_values=fmt == "deployed")
         for i in range(0, n, step):
@@ -205,11 +214,13 @@ def test_prefill_pools_off_a_word_boundary(cases, name, fmt, shift):
     assert all(torch.equal(a, b) for a, b in zip(*stored))
 
 
-@pytest.mark.parametrize("n", [24, 41, 100, 256])
+@pytest.mark.parametrize("n", [24, 41, 57, "most"])
 @pytest.mark.parametrize("name,fmt", [("qwen", "plain"), ("gptoss", "plain"), ("qwen", "scaled"), ("gptoss", "deployed")])
 def test_append_batches_of_several_chunks(cases, name, fmt, n):
     """Batches that still take the append kernel but span several of its passes and chunks of the token list."""
-    _run(cases[name, fmt != "plain"], fmt, n, 40, True, n == 100)
+    most = _append_step(cases[name, fmt != "plain"])
+    assert most >= 57
+    _run(cases[name, fmt != "plain"], fmt, most if n == "most" else n, 40, True, n == 57)
 
 
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
@@ -235,7 +246,7 @@ def test_prefill_token_that_is_not_finite(cases, name, fmt, bad):
         assert case.ctx.novakv_last_device_status() == 0
         return [*cache.load_logical(0, 0, n), *([cache.load_scales(0, 0, n)] if fmt != "plain" else [])]
 
-    clean, prompt, small = stored(None, n), stored(bad, n), stored(bad, 150)
+    clean, prompt, small = stored(None, n), stored(bad, n), stored(bad, min(150, _append_step(case)))
     for c, p, s in zip(clean, prompt, small):
         assert np.array_equal(p[t], s[t])
         assert np.array_equal(np.delete(p, t, 0), np.delete(c, t, 0))
