@@ -35,7 +35,9 @@ def calls():
     assert build.LIB_CALLS.exists()
     from paper_2608_04074_b200 import _novakv_calls
     _novakv_calls.setup(lambda device: 0, lambda: 0, torch.float32)
-    return _novakv_calls.bind(binding.load_library()._handle)
+    yield _novakv_calls.bind(binding.load_library()._handle)
+    if torch.cuda.is_available():                        # (contexts of other tests ask the same functions)
+        _novakv_calls.setup(torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice, torch.float32)
 
 
 def _args(kinds):
