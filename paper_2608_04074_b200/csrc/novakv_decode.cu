@@ -807,7 +807,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
         form_prefixes(pfx, s_part, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         page_prefix = pfx;
         cost_prefix = pfx + PFX_CAP + 1;
-    } else if (HG == 8 && batch <= PFX_CAP) {
+    } else if (batch <= PFX_CAP) {
         int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
         for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix_g[i]; pfx[PFX_CAP + 1 + i] = cost_prefix_g[i]; }
         __syncthreads();
@@ -1525,7 +1525,7 @@ novakv_decode_mma_kernel(const float* __restrict__ qp, const uint4* __restrict__
         form_prefixes(pfx, s_part, seq_lens, batch, max_pages_per_seq, seg_weight, page_prefix_g, cost_prefix_g, dev_status);
         page_prefix = pfx;
         cost_prefix = pfx + PFX_CAP + 1;
-    } else if (HG == 8 && batch <= PFX_CAP) {
+    } else if (batch <= PFX_CAP) {
         int32_t* pfx = reinterpret_cast<int32_t*>(s_abs + C::PFX);
         for (int i = threadIdx.x; i <= batch; i += S1_THREADS) { pfx[i] = page_prefix_g[i]; pfx[PFX_CAP + 1 + i] = cost_prefix_g[i]; }
         __syncthreads();
