@@ -161,7 +161,9 @@ novakv_prepare_kernel(const __nv_bfloat16* __restrict__ q, const float* __restri
     // step's tokens) writes: queries are produced before that kernel started, the transform is a constant.  So
     // the blocks that transform queries run beside the preceding kernel.  They write nothing before it has completed: it
     // may still read what shares memory with this call's workspace (the partials of another call on that scratch, new
-    // rows whose tensor has been freed).
+    // rows whose tensor has been freed).  The blocks keep their place until then, so the scan's come later: append + decode of
+    // 1 x 777 18.1 -> 18.3 us, 32 x 8191 scaled 80.8 -> 82.2, the 128-sequence mix 281 -> 286 against writing at once.  (Fewer blocks, as
+    // many as SMs: the mix 285, but 64 x 200 36.2 -> 38.9.)
     const int n_query_blocks = (int)gridDim.x - form_prefix;
     float rv[ROWS];
     if (blk < n_query_blocks) {
@@ -404,8 +406,9 @@ struct Segment {
 
 // Page and cost prefixes of a batch of at most PFX_CAP sequences in shared memory (pfx: [2][PFX_CAP + 1]), by all threads of a
 // scan CTA; CTA 0 also writes the prefixes for the merge kernel and reports lengths out of range.  Every CTA does it by
-// itself: a block of the kernel in front would have to wait for the append first, and the scan for that block (1 x 777 step
-// 17.6 -> 17.4 us a call, 5 x 100 of the d = 64 shape 16.7 -> 16.4, deployed band 64 x 32768 411 -> 405).
+// itself: a block of the kernel in front would have to wait for the append, load the lengths and write, and the scan for that
+// block (append + decode, that block / here: 1 x 777 19.0 / 18.4 us, 8 x 16384 42.4 / 42.0, 128 x 1000 102.9 / 102.3; 5 x 100 of the
+// d = 64 shape 17.0 / 16.5).
 static_assert(PFX_CAP < S1_THREADS, "a thread for every sequence");
 __device__ __forceinline__ void form_prefixes(int32_t* pfx, int (*s_part)[NCW], const int32_t* __restrict__ seq_lens, int batch, int max_pages,
                                               int seg_weight, int32_t* __restrict__ page_prefix, int32_t* __restrict__ cost_prefix,
@@ -794,8 +797,7 @@ novakv_decode_stage1_kernel(const float* __restrict__ qp, const float* __restric
     // lands behind the segment lookup and the first table build.
     int vcb_head = (int)(((long)blockIdx.x * n_kv_heads) / gridDim.x);   // KV head whose value codebook is resident
     if (!VSQ) stage_value_codebook_async(C::VCB, cb_v_img + (size_t)vcb_head * VCB_COPY_BYTES);
-    // With the merge fused in, the kernels that follow (the query transform of the next call writes the same
-    // workspace) must not start before this grid is done: no early release of the dependents.
+    // With the merge fused in this grid writes the outputs: its dependents are not let in before it is done.
     if (out_fused != nullptr) asm volatile("griddepcontrol.wait;" ::: "memory");
     else novakv_grid_dependency_wait();
 
@@ -2326,8 +2328,8 @@ novakv_status launch_decode_t(novakv_ctx* ctx, const novakv_layer& ly, const __n
 
     // (with the merge fused in, the outputs of empty sequences are written where the prefixes are formed)
     // Eight heads per KV head: only batches of one warp.  The append (d = 64, about 6 us) then ends before the queries are
-    // transformed, and a block of the prepare kernel has formed the prefixes by the time the scan could (70 sequences
-    // of 400 tokens: 44.1 us so, 44.6 in the scan; 5 of 100: 16.7 and 16.4).
+    // transformed, and a block of the prepare kernel has formed the prefixes by the time the scan could (append + decode, a block
+    // of the prepare kernel / the scan: 33 x 1000 32.7 / 33.2 us, 70 x 400 43.1 / 43.6, 128 x 1000 81.0 / 81.8; 5 x 100 17.0 / 16.5).
     const int scan_prefix = batch <= (HG == 8 ? 32 : PFX_CAP) && !fuse;
     // sequences per prepare block: one while all pairs fit on the machine twice over, then enough to make that so
     const int seqs_per_block = max(1, min(PREPARE_RUN, (batch * hkv + 2 * ctx->n_sm - 1) / (2 * ctx->n_sm)));

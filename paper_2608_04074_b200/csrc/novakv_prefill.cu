@@ -112,7 +112,8 @@ enum { B_R = 0, B_X = 1 /* +slot */, B_XFREE = 4 /* +slot */, B_T = 7 /* +half *
        B_RING = 15 /* +stage */, B_RINGFREE = 19, B_CW = 23 /* +stage */, B_CWFREE = B_CW + PF_CW_STAGES,
        B_DRAIN = B_CW + 2 * PF_CW_STAGES, B_COUNT };
 static_assert(B_COUNT * 8 <= 288, "barrier block");
-// named barriers: 1 + wg among the four warps of a warpgroup, 5 + half among the eight of a half tile
+// named barriers: 1 + wg among the four warps of a warpgroup, 5 + half among the eight of a half tile, 7 + wg: the other
+// warpgroup of the half tile has read its distances, wg has written its operand
 __device__ __forceinline__ void nbar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void nbar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
@@ -1119,6 +1120,7 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
     // cheaper: when there are too few units to give every SM one, or a few whole ones.
     double best = 1e30;
     int grid = 1;
+    bool one_each = false;              // no more units than SMs
     for (int gs = L / P::GU; gs <= L / 8; gs *= 2) {
         const double cp = PF_US_UNIT + PF_US_GROUP * (L / gs), ck = cp + (FMT ? PF_US_SCALED : 0.0), cv = FMT == 2 ? PF_US_INT2 : cp;
         const int uk = hkv * gs * n_tiles, uv = FMT == 2 ? hkv * n_tiles : uk;
@@ -1128,9 +1130,10 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
             best = longest;
             grid = g;
             a.gs = gs;
-            // one unit per CTA where there are no more than SMs: a cut in cost would hand some a key and a value unit
-            a.cost_k = uk + uv <= ctx->n_sm ? 1 : (int)(ck * (D == 128 && FMT == 0 && uk + uv >= PF_KEYS_UNITS * g ? PF_KEYS : 1.0) * 64.0);
-            a.cost_v = uk + uv <= ctx->n_sm ? 1 : (int)(cv * 64.0);
+            // (then one unit per CTA: a cut in cost would hand some a key and a value unit)
+            one_each = uk + uv <= ctx->n_sm;
+            a.cost_k = one_each ? 1 : (int)(ck * (D == 128 && FMT == 0 && uk + uv >= PF_KEYS_UNITS * g ? PF_KEYS : 1.0) * 64.0);
+            a.cost_v = one_each ? 1 : (int)(cv * 64.0);
         }
     }
     // tensor maps of the new rows (rebuilt on every call: the buffers are the caller's)
@@ -1140,7 +1143,7 @@ novakv_status launch_prefill_t(novakv_ctx* ctx, const PrefillArgs& args, cudaStr
     novakv_prof_scope ps(ctx, 1, stream);
     // A short call's launch overlaps the kernel in front.  Not a long one's: its CTAs would land on SMs in the order in which
     // the kernel in front leaves them (32768 tokens, calls in a row: 490 us so, 501 overlapped).
-    if (a.cost_k == 1) novakv_launch_pdl(kern, dim3(grid), dim3(PF_THREADS), P::BYTES, stream, a);
+    if (one_each) novakv_launch_pdl(kern, dim3(grid), dim3(PF_THREADS), P::BYTES, stream, a);
     else kern<<<grid, PF_THREADS, P::BYTES, stream>>>(a);
     ps.end();
     ctx->launches++;
