@@ -51,7 +51,8 @@ NOALLOC_SCRATCH_BYTES = 4 << 20      # NOVAKV_NOALLOC_SCRATCH_BYTES of the publi
 
 
 def load_library(path=None):
-    """Load libnovakv.so (built in-tree by ``build.build_cuda``); raises if it is absent."""
+    """Load libnovakv.so (built in-tree by ``build.build_cuda``); raises if it is absent.  The argument types cover the
+    per-step calls too, which ``Context`` makes through the extension: for callers of the library through ctypes."""
     global _lib
     if _lib is not None and path is None:
         return _lib
